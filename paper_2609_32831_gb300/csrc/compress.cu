@@ -1,7 +1,7 @@
 // Segment compression kernels (§3.4; App. E "Physical, type-aware KV
 // storage" and "Batched GQA token selection") and the decode-time append.
 //
-//  topk_select     exact per-(sequence, KV head) top-k by radix select on
+//  topk            exact per-(sequence, KV head) top-k by radix select on
 //                  order-preserving score keys, ties to the lower index,
 //                  kept indices written in ascending order
 //  gather_rows     compaction of the kept bf16 rows (eviction)
@@ -30,25 +30,13 @@ __device__ __forceinline__ uint32_t score_key(float f) {
 }
 
 constexpr int kTopkThreads = 1024;
-
-// Block-wide exclusive scan of one flag per thread; returns the prefix and
-// writes the block total to *total. Uses `scratch` [32] ints.
-__device__ __forceinline__ int block_excl_scan(int flag, int* scratch, int* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned bal = __ballot_sync(0xffffffffu, flag);
-  const int in_warp = __popc(bal & ((1u << lane) - 1u));
-  if (lane == 0) scratch[warp] = __popc(bal);
-  __syncthreads();
-  int before = 0, sum = 0;
-  for (int w = 0; w < kTopkThreads / 32; ++w) {
-    const int c = scratch[w];
-    before += (w < warp) ? c : 0;
-    sum += c;
-  }
-  __syncthreads();
-  *total = sum;
-  return before + in_warp;
-}
+constexpr int kTopkWarps = kTopkThreads / 32;
+constexpr int kTopkRows = 16;      // 32-candidate rows of a warp kept in registers between the passes
+constexpr int kTopkBins = 2048;    // radix digits of 11, 11 and 10 bits
+constexpr int kTopkMaxCluster = 8;
+// Candidates a CTA takes before the list is spread over a cluster: below, a
+// cluster barrier per pass costs more than the shorter lists save.
+constexpr int kTopkPerCta = 8192;
 
 // Score of candidate i: scores[i], or scores[idx[i]] through the source's
 // logical indices; an index outside the score array flags UC_ERR_RANGE and
@@ -64,124 +52,26 @@ __device__ __forceinline__ float candidate_score(const float* s, const int32_t* 
   return s[t];
 }
 
-__global__ void __launch_bounds__(kTopkThreads) topk_select_kernel(TopkArgs a) {
-  const int bh = blockIdx.x;
-  const int b = bh / a.n_kv_heads;
-  const int keep = a.keep[b];
-  const float* s = a.scores + (int64_t)bh * a.scores_stride + a.scores_offset;
-  int32_t* out = a.kept_idx + (int64_t)bh * a.cap;
-  const int32_t* sidx = a.score_idx ? a.score_idx + (int64_t)bh * a.score_idx_stride : nullptr;
-  const int r = min(a.n_recent, keep);
-  const int n_old = a.src_n[b] - r;
-  const int k_old = keep - r;
-
-  __shared__ uint32_t hist[256];
-  __shared__ uint32_t sh_prefix, sh_mask, sh_remaining;
-  __shared__ int scratch[32];
-  __shared__ int sh_nan;
-
-  if (threadIdx.x == 0) {
-    sh_prefix = 0;
-    sh_mask = 0;
-    sh_remaining = (uint32_t)k_old;
-    sh_nan = 0;
-  }
-  __syncthreads();
-
-  if (k_old > 0) {
-    for (int shift = 24; shift >= 0; shift -= 8) {
-      for (int i = threadIdx.x; i < 256; i += kTopkThreads) hist[i] = 0;
-      __syncthreads();
-      const uint32_t prefix = sh_prefix, mask = sh_mask;
-      for (int i = threadIdx.x; i < n_old; i += kTopkThreads) {
-        int bad = 0;
-        const float f = candidate_score(s, sidx, a.score_limit, i, &bad);
-        if (shift == 24 && (isnan(f) || bad)) sh_nan = bad ? 2 : 1;
-        const uint32_t key = score_key(f);
-        if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
-      }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        uint32_t rem = sh_remaining, cum = 0;
-        int digit = 0;
-        for (int d = 255; d >= 0; --d) {
-          const uint32_t h = hist[d];
-          if (cum + h >= rem) {
-            digit = d;
-            break;
-          }
-          cum += h;
-        }
-        sh_remaining = rem - cum;
-        sh_prefix = prefix | ((uint32_t)digit << shift);
-        sh_mask = mask | (255u << shift);
-      }
-      __syncthreads();
-    }
-  }
-  if (sh_nan) {
-    // the result is undefined, but later kernels of the call must still find
-    // in-range row indices: keep rows 0 .. keep-1
-    for (int t = threadIdx.x; t < keep; t += kTopkThreads) out[t] = t;
-    if (bh % a.n_kv_heads == 0 && threadIdx.x == 0) a.n_kept[b] = keep;
-    if (threadIdx.x == 0) set_status(a.status, UC_ERR_RANGE, sh_nan);
-    return;
-  }
-  const uint32_t thr = sh_prefix;
-  const int need_eq = (int)sh_remaining;
-  int out_base = 0, eq_base = 0;
-  if (k_old > 0) {
-    for (int base = 0; base < n_old; base += kTopkThreads) {
-      const int i = base + threadIdx.x;
-      uint32_t key = 0;
-      int bad = 0;
-      if (i < n_old) key = score_key(candidate_score(s, sidx, a.score_limit, i, &bad));
-      const int gt = (i < n_old) && key > thr;
-      const int eq = (i < n_old) && key == thr;
-      int eq_total, take_total;
-      const int eq_rank = eq_base + block_excl_scan(eq, scratch, &eq_total);
-      const int take = gt || (eq && eq_rank < need_eq);
-      const int pos = out_base + block_excl_scan(take, scratch, &take_total);
-      if (take) out[pos] = i;
-      eq_base += eq_total;
-      out_base += take_total;
-    }
-  }
-  for (int t = threadIdx.x; t < r; t += kTopkThreads) out[k_old + t] = n_old + t;
-  if (bh % a.n_kv_heads == 0 && threadIdx.x == 0) a.n_kept[b] = keep;
-}
-
-// The same selection for long candidate lists (the long-context workloads:
-// ~118K image tokens per (sequence, KV head) at 128K context): one cluster of
-// kTopkCluster CTAs per (sequence, KV head), each CTA histogramming its share
-// of the candidates into rank 0's shared-memory histogram (distributed shared
-// memory) between cluster barriers, then counting its (greater, equal) keys
-// so that each CTA writes its kept indices at their global rank. Every CTA
-// runs every cluster barrier, and none leaves while another may still read
-// its shared memory.
-constexpr int kTopkCluster = 8;
-// The cluster kernel serves calls with long candidate lists and few (sequence,
-// KV head) pairs (128K context, batch 2: 8 pairs x 118K candidates, 405 ->
-// 109 us); with many pairs one CTA each already fills the GPU (32K context,
-// batch 16: 64 pairs x 29K candidates, 150 us single vs 236 us clustered).
-constexpr int kTopkClusterMinN = 16384;
-constexpr int kTopkClusterMaxPairs = 32;
-
-__device__ __forceinline__ int block_sum(int v, int* scratch) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
-  __syncthreads();
-  int s = 0;
-  for (int w = 0; w < kTopkThreads / 32; ++w) s += scratch[w];
-  __syncthreads();
-  return s;
-}
-
-__global__ void __cluster_dims__(kTopkCluster, 1, 1) __launch_bounds__(kTopkThreads)
-    topk_cluster_kernel(TopkArgs a) {
+// Exact top-k of one (sequence, KV head) by a cluster of 1 .. 8 CTAs (chosen
+// by launch_topk from the list's length). Every warp owns a contiguous run of
+// 32-candidate rows whose keys it loads once (coalesced) and keeps in
+// registers, so that the three radix passes, the count and the emission read
+// no memory (rows past kTopkRows, beyond 131072 candidates per cluster of 8,
+// are read again each time). Per pass: a shared-memory histogram, one cluster
+// barrier, then every CTA sums the cluster's histograms through distributed
+// shared memory and finds the digit with one block scan (each pass has a
+// histogram of its own, so no second barrier is needed). Emission order:
+// counts of (greater, equal) keys per warp, prefix over the warps and CTAs,
+// then per row two ballots give every kept index its ascending place.
+// What bounds it is the chain of barriers and the histogram's atomics. An
+// eviction of 29492 to 5898 tokens and a re-eviction of those to 2949 (16
+// pairs, gather and quantization included) took 161 us with the selection
+// that read the scores again in each of five passes and searched its 256 bins
+// with one thread (64.5 and 40 us of it), 99.5 us with this one.
+__global__ void __launch_bounds__(kTopkThreads) topk_kernel(TopkArgs a) {
   cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int bh = blockIdx.x / kTopkCluster;
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int bh = blockIdx.x / C;
   const int b = bh / a.n_kv_heads;
   const int keep = a.keep[b];
   const float* s = a.scores + (int64_t)bh * a.scores_stride + a.scores_offset;
@@ -190,125 +80,165 @@ __global__ void __cluster_dims__(kTopkCluster, 1, 1) __launch_bounds__(kTopkThre
   const int r = min(a.n_recent, keep);
   const int n_old = a.src_n[b] - r;
   const int k_old = keep - r;
-  const int lo = (int)((int64_t)n_old * rank / kTopkCluster);
-  const int hi = (int)((int64_t)n_old * (rank + 1) / kTopkCluster);
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-  __shared__ uint32_t hist[256];   // this CTA's histogram of the pass
-  __shared__ uint32_t ghist[256];  // the cluster's histogram (rank 0's copy)
-  __shared__ uint32_t sh_prefix, sh_mask, sh_remaining;
+  __shared__ __align__(16) uint32_t hist[3][kTopkBins];
+  __shared__ int warp_cnt[kTopkWarps][2];  // (greater, equal) keys of each warp; scan scratch before
+  __shared__ int cta_cnt[2];
+  __shared__ uint32_t sh_digit, sh_rem;
   __shared__ int sh_nan;
-  __shared__ int counts[kTopkCluster][2];  // rank 0: (greater, equal) keys per CTA
-  __shared__ int scratch[32];
-  uint32_t* g_hist = cluster.map_shared_rank(ghist, 0);
-  int* g_nan = cluster.map_shared_rank(&sh_nan, 0);
 
-  for (int i = tid; i < 256; i += kTopkThreads) ghist[i] = 0;
-  if (tid == 0) {
-    sh_prefix = 0;
-    sh_mask = 0;
-    sh_remaining = (uint32_t)max(k_old, 0);
-    sh_nan = 0;
-  }
-  cluster.sync();  // every CTA's shared memory is set before any other adds into it
-
-  uint32_t prefix = 0, mask = 0;
   if (k_old > 0) {  // the same for every CTA of the cluster (one sequence)
-    for (int shift = 24; shift >= 0; shift -= 8) {
-      for (int i = tid; i < 256; i += kTopkThreads) hist[i] = 0;
-      __syncthreads();
-      for (int i = lo + tid; i < hi; i += kTopkThreads) {
+    for (int i = tid; i < 3 * kTopkBins; i += kTopkThreads) hist[0][i] = 0;
+    if (tid == 0) sh_nan = 0;
+    const int rows = (n_old + 31) / 32;
+    const int per_warp = (rows + C * kTopkWarps - 1) / (C * kTopkWarps);
+    const int row0 = (rank * kTopkWarps + warp) * per_warp;
+    uint32_t keys[kTopkRows];
+    int flag = 0;
+#pragma unroll
+    for (int e = 0; e < kTopkRows; ++e) {
+      const int i = (row0 + e) * 32 + lane;
+      keys[e] = 0u;
+      if (e < per_warp && i < n_old) {
         int bad = 0;
         const float f = candidate_score(s, sidx, a.score_limit, i, &bad);
-        if (shift == 24 && (isnan(f) || bad)) atomicOr(g_nan, bad ? 2 : 1);
-        const uint32_t key = score_key(f);
-        if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
+        if (bad)
+          flag = 2;
+        else if (isnan(f))
+          flag = max(flag, 1);
+        keys[e] = score_key(f);
+      }
+    }
+    // body(key, valid, i) over the warp's rows, in index order; every lane
+    // of the warp takes every row
+    auto each_row = [&](auto&& body) {
+#pragma unroll
+      for (int e = 0; e < kTopkRows; ++e) {
+        if (e < per_warp) {
+          const int i = (row0 + e) * 32 + lane;
+          body(keys[e], i < n_old, i);
+        }
+      }
+      for (int e = kTopkRows; e < per_warp; ++e) {
+        const int i = (row0 + e) * 32 + lane;
+        uint32_t key = 0u;
+        if (i < n_old) {
+          int bad = 0;
+          const float f = candidate_score(s, sidx, a.score_limit, i, &bad);
+          if (bad)
+            flag = 2;
+          else if (isnan(f))
+            flag = max(flag, 1);
+          key = score_key(f);
+        }
+        body(key, i < n_old, i);
+      }
+    };
+    __syncthreads();
+    uint32_t prefix = 0, mask = 0, rem = (uint32_t)k_old;
+    int nan = 0;
+#pragma unroll 1
+    for (int pass = 0; pass < 3; ++pass) {
+      const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
+      const uint32_t dmask = pass == 2 ? 1023u : 2047u;
+      each_row([&](uint32_t key, bool valid, int) {
+        if (valid && (key & mask) == prefix) atomicAdd(&hist[pass][(key >> shift) & dmask], 1u);
+      });
+      if (pass == 0 && flag) atomicMax(&sh_nan, flag);
+      if (C > 1)
+        cluster.sync();
+      else
+        __syncthreads();
+      // thread t: bins 2047 - 2t and 2046 - 2t (descending keys), summed over the cluster
+      uint32_t h1 = 0, h0 = 0;
+      for (int q = 0; q < C; ++q) {
+        const uint2 v = *reinterpret_cast<const uint2*>(
+            (C > 1 ? cluster.map_shared_rank(&hist[pass][0], q) : &hist[pass][0]) + (kTopkBins - 2 - 2 * tid));
+        h0 += v.x;
+        h1 += v.y;
+        if (pass == 0) nan = max(nan, C > 1 ? *cluster.map_shared_rank(&sh_nan, q) : sh_nan);
+      }
+      const uint32_t c = h1 + h0;
+      uint32_t incl = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      if (lane == 31) warp_cnt[warp][0] = (int)incl;
+      __syncthreads();
+      uint32_t before = lane < warp ? (uint32_t)warp_cnt[lane][0] : 0u;
+      before = __reduce_add_sync(0xffffffffu, before);
+      const uint32_t excl = before + incl - c;
+      if (excl < rem && rem <= excl + c) {
+        const bool hi = rem <= excl + h1;
+        sh_digit = (uint32_t)(kTopkBins - 1 - 2 * tid - (hi ? 0 : 1));
+        sh_rem = rem - excl - (hi ? 0u : h1);
       }
       __syncthreads();
-      for (int i = tid; i < 256; i += kTopkThreads)
-        if (hist[i]) atomicAdd(&g_hist[i], hist[i]);
-      cluster.sync();
+      prefix |= sh_digit << shift;
+      mask |= dmask << shift;
+      rem = sh_rem;
+    }
+    if (nan) {
+      // the result is undefined, but later kernels of the call must still find
+      // in-range row indices: keep rows 0 .. keep-1
       if (rank == 0) {
-        if (tid == 0) {
-          uint32_t rem = sh_remaining, cum = 0;
-          int digit = 0;
-          for (int d = 255; d >= 0; --d) {
-            const uint32_t h = ghist[d];
-            if (cum + h >= rem) {
-              digit = d;
-              break;
-            }
-            cum += h;
-          }
-          sh_remaining = rem - cum;
-          sh_prefix |= (uint32_t)digit << shift;
-          sh_mask |= 255u << shift;
-        }
-        __syncthreads();
-        for (int i = tid; i < 256; i += kTopkThreads) ghist[i] = 0;
+        for (int t = tid; t < keep; t += kTopkThreads) out[t] = t;
+        if (bh % a.n_kv_heads == 0 && tid == 0) a.n_kept[b] = keep;
+        if (tid == 0) set_status(a.status, UC_ERR_RANGE, nan);
+      }
+      if (C > 1) cluster.sync();  // no CTA leaves while another may still read its shared memory
+      return;
+    }
+    const uint32_t thr = prefix;
+    const int need_eq = (int)rem;
+    int gt = 0, eq = 0;
+    each_row([&](uint32_t key, bool valid, int) {
+      gt += __popc(__ballot_sync(0xffffffffu, valid && key > thr));
+      eq += __popc(__ballot_sync(0xffffffffu, valid && key == thr));
+    });
+    // (the last pass's barrier follows its reads of warp_cnt)
+    if (lane == 0) {
+      warp_cnt[warp][0] = gt;
+      warp_cnt[warp][1] = eq;
+    }
+    __syncthreads();
+    const int wg = warp_cnt[lane][0], we = warp_cnt[lane][1];
+    int g_before = __reduce_add_sync(0xffffffffu, lane < warp ? wg : 0);
+    int e_before = __reduce_add_sync(0xffffffffu, lane < warp ? we : 0);
+    if (C > 1) {
+      const int g_all = __reduce_add_sync(0xffffffffu, wg), e_all = __reduce_add_sync(0xffffffffu, we);
+      if (tid == 0) {
+        cta_cnt[0] = g_all;
+        cta_cnt[1] = e_all;
       }
       cluster.sync();
-      prefix = *cluster.map_shared_rank(&sh_prefix, 0);
-      mask = *cluster.map_shared_rank(&sh_mask, 0);
+      for (int q = 0; q < rank; ++q) {
+        const int* cc = cluster.map_shared_rank(&cta_cnt[0], q);
+        g_before += cc[0];
+        e_before += cc[1];
+      }
     }
+    int pos = g_before + min(e_before, need_eq);
+    int eq_rank0 = e_before;
+    const unsigned below = (1u << lane) - 1u;
+    each_row([&](uint32_t key, bool valid, int i) {
+      const bool is_eq = valid && key == thr;
+      const unsigned me = __ballot_sync(0xffffffffu, is_eq);
+      const bool take = (valid && key > thr) || (is_eq && eq_rank0 + __popc(me & below) < need_eq);
+      const unsigned mt = __ballot_sync(0xffffffffu, take);
+      if (take) out[pos + __popc(mt & below)] = i;
+      pos += __popc(mt);
+      eq_rank0 += __popc(me);
+    });
+    if (C > 1) cluster.sync();  // no CTA leaves while another may still read its shared memory
   }
-  const int nan = *g_nan;
-  const uint32_t thr = prefix;
-  const int need_eq = (int)*cluster.map_shared_rank(&sh_remaining, 0);
-  if (nan) {
-    // the result is undefined, but later kernels of the call must still find
-    // in-range row indices: keep rows 0 .. keep-1
-    if (rank == 0) {
-      for (int t = tid; t < keep; t += kTopkThreads) out[t] = t;
-      if (bh % a.n_kv_heads == 0 && tid == 0) a.n_kept[b] = keep;
-      if (tid == 0) set_status(a.status, UC_ERR_RANGE, nan);
-    }
-  } else if (k_old > 0) {
-    // this CTA's (greater, equal) counts, then the global rank of its first take
-    int gt = 0, eq = 0;
-    for (int i = lo + tid; i < hi; i += kTopkThreads) {
-      int bad = 0;
-      const uint32_t key = score_key(candidate_score(s, sidx, a.score_limit, i, &bad));
-      gt += key > thr;
-      eq += key == thr;
-    }
-    gt = block_sum(gt, scratch);
-    eq = block_sum(eq, scratch);
-    if (tid == 0) {
-      int* c = cluster.map_shared_rank(&counts[0][0], 0);
-      c[2 * rank] = gt;
-      c[2 * rank + 1] = eq;
-    }
-    cluster.sync();
-    int eq_base = 0, out_base = 0;
-    for (int q = 0; q < rank; ++q) {
-      const int* c = cluster.map_shared_rank(&counts[q][0], 0);
-      const int g_q = c[0], e_q = c[1];
-      out_base += g_q + min(e_q, max(0, need_eq - eq_base));
-      eq_base += e_q;
-    }
-    for (int base = lo; base < hi; base += kTopkThreads) {
-      const int i = base + tid;
-      uint32_t key = 0;
-      int bad = 0;
-      if (i < hi) key = score_key(candidate_score(s, sidx, a.score_limit, i, &bad));
-      const int g1 = (i < hi) && key > thr;
-      const int e1 = (i < hi) && key == thr;
-      int eq_total, take_total;
-      const int eq_rank = eq_base + block_excl_scan(e1, scratch, &eq_total);
-      const int take = g1 || (e1 && eq_rank < need_eq);
-      const int pos = out_base + block_excl_scan(take, scratch, &take_total);
-      if (take) out[pos] = i;
-      eq_base += eq_total;
-      out_base += take_total;
-    }
-  }
-  if (!nan && rank == 0) {
+  if (rank == 0) {
     for (int t = tid; t < r; t += kTopkThreads) out[k_old + t] = n_old + t;
     if (bh % a.n_kv_heads == 0 && tid == 0) a.n_kept[b] = keep;
   }
-  if (nan || k_old <= 0) cluster.sync();  // the count exchange's barrier of the other path
-  cluster.sync();  // no CTA leaves while another may still read its shared memory
 }
 
 // Kept indices of a segment that keeps every token (QUANT).
@@ -625,15 +555,42 @@ __global__ void append_token_kernel(AppendArgs a) {
 
 // ---------------------------------------------------------------- launchers
 
+static int compress_sms() {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(sms, 1);
+  }
+  return sms;
+}
+
+// CTAs per (sequence, KV head): one up to kTopkPerCta candidates, then as many
+// (a power of two up to 8) as share the list at no fewer than that each and
+// fit the GPU at one CTA per SM.
 void launch_topk(const TopkArgs& a, int n_blocks, bool evict, cudaStream_t st) {
+  if (!evict) {
+    iota_kernel<<<n_blocks, 256, 0, st>>>(a);
+    count_launch();
+    return;
+  }
   int max_src = 0;
   for (int b = 0; b < UC_MAX_BATCH; ++b) max_src = std::max(max_src, a.src_n[b]);
-  if (evict && max_src >= kTopkClusterMinN && n_blocks <= kTopkClusterMaxPairs)
-    topk_cluster_kernel<<<n_blocks * kTopkCluster, kTopkThreads, 0, st>>>(a);
-  else if (evict)
-    topk_select_kernel<<<n_blocks, kTopkThreads, 0, st>>>(a);
-  else
-    iota_kernel<<<n_blocks, 256, 0, st>>>(a);
+  int c = 1;
+  while (c < kTopkMaxCluster && max_src > c * kTopkPerCta && n_blocks * c * 2 <= compress_sms()) c *= 2;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)c;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n_blocks * c));
+  cfg.blockDim = dim3(kTopkThreads);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, topk_kernel, a);
   count_launch();
 }
 
@@ -658,16 +615,9 @@ void launch_gather(const GatherArgs& a, cudaStream_t st) {
 }
 
 void launch_quantize(const GatherArgs& a, int bits, cudaStream_t st) {
-  static int sms = 0;
   static bool attr4 = false, attr2 = false;
-  if (sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    sms = std::max(sms, 1);
-  }
   const int warps = a.batch * a.n_kv_heads * a.max_chunks;
-  const int blocks = std::min((warps + kQuantWarps - 1) / kQuantWarps, kQuantCtasPerSm * sms);
+  const int blocks = std::min((warps + kQuantWarps - 1) / kQuantWarps, kQuantCtasPerSm * compress_sms());
   if (blocks > 0) {
     if (bits == 4) {
       if (!attr4)

@@ -195,6 +195,32 @@ def test_evict_topk_parity_long(n, keeps, recent, ties):
             np.testing.assert_array_equal(idx[b * hkv + j, :keeps[b]], ref)
 
 
+@pytest.mark.parametrize("n,keep,recent,bh", [
+    (8192, 8191, 0, 1), (8193, 31, 0, 1), (16385, 5000, 7, 2), (32769, 32769, 0, 1),   # cluster sizes 1, 2, 4, 8
+    (131073, 40000, 33, 1), (140001, 1, 0, 1),         # rows past the register-resident ones
+    (32, 32, 0, 3), (33, 1, 0, 3), (1024, 1, 1, 2),    # one row, a ragged row, recent tokens only
+    (9000, 2222, 0, 96)])                              # too many pairs for a cluster each
+def test_topk_split_edges(n, keep, recent, bh):
+    """Kept indices at the edges of the top-k's split (rows per warp, CTAs per
+    pair), with values over 60 octaves, ties across every boundary, negative
+    scores and both infinities: bit-exact with the oracle's full sort."""
+    rng = np.random.default_rng(n + keep)
+    B, hkv = (bh // 8, 8) if bh > 8 else (1, bh)
+    s = (rng.standard_normal((B, hkv, n)) * np.exp2(rng.integers(-30, 30, (B, hkv, n)))).astype(np.float32)
+    s[..., ::3] = np.float32(0.5)
+    s[..., 5], s[..., n // 2] = np.inf, -np.inf
+    k = torch.zeros((B, hkv, n, 128), dtype=torch.bfloat16, device=DEV)
+    seg = uc.Segment("evict", 16, B, hkv, n, keep, DEV)
+    seg.set_keep([keep] * B)
+    ws = uc.Workspace(DEV)
+    uc.compress_segment(k, k, seg, scores=torch.from_numpy(s).to(DEV), n_recent=recent, ws=ws)
+    assert ws.status() == 0
+    idx = seg.tensor("kept_idx").view(B, hkv, keep).cpu().numpy()
+    for b in range(B):
+        for j in range(hkv):
+            np.testing.assert_array_equal(idx[b, j], osel.topk_keep(s[b, j], keep, recent))
+
+
 def test_evict_nan_score_reports_range():
     B, hkv, n = 1, 4, 100
     k, v = synth.make_kv(5, B, hkv, n)

@@ -556,7 +556,7 @@ uc_status uc_compress_segment(const void* k_src, const void* v_src, int64_t src_
     t.keep[b] = seg->n_kept_host[b];
     t.src_n[b] = seg->n_src;
   }
-  launch_topk(t, nbh, evict, cs);
+  if (evict) launch_topk(t, nbh, cs);  // else the quantizer writes the indices itself
 
   GatherArgs g;
   memset(&g, 0, sizeof(g));
@@ -565,6 +565,8 @@ uc_status uc_compress_segment(const void* k_src, const void* v_src, int64_t src_
   g.src_row_stride = src_row_stride;
   g.src_row_offset = src_row_offset;
   g.kept_idx = seg->kept_idx;
+  g.identity = evict ? 0 : 1;
+  g.n_kept = seg->n_kept;
   g.k_dst = static_cast<__nv_bfloat16*>(seg->k);
   g.v_dst = static_cast<__nv_bfloat16*>(seg->v);
   g.dst_row_stride = seg->row_stride;
@@ -710,9 +712,10 @@ uc_status uc_recompress_segment(const uc_segment* src, const float* scores, int6
     t.keep[b] = dst->n_kept_host[b];
     t.src_n[b] = src->n_kept_host[b];
   }
-  launch_topk(t, nbh, evict, cs);
+  if (evict) launch_topk(t, nbh, cs);  // else the quantizer writes the indices itself
 
-  // 3. gather or quantize the kept rows into the destination.
+  // 3. gather or quantize the kept rows into the destination; kept_idx moves
+  // from stored rows to the source's logical token indices on the way.
   GatherArgs g;
   memset(&g, 0, sizeof(g));
   g.k_src = k_rows;
@@ -720,6 +723,10 @@ uc_status uc_recompress_segment(const uc_segment* src, const float* scores, int6
   g.src_row_stride = rows_stride;
   g.src_row_offset = rows_offset;
   g.kept_idx = dst->kept_idx;
+  g.identity = evict ? 0 : 1;
+  g.n_kept = dst->n_kept;
+  g.src_idx = src->kept_idx;  // NULL for FULL sources: stored row i is token i
+  g.src_cap = src->cap;
   g.k_dst = static_cast<__nv_bfloat16*>(dst->k);
   g.v_dst = static_cast<__nv_bfloat16*>(dst->v);
   g.dst_row_stride = dst->row_stride;
@@ -742,18 +749,6 @@ uc_status uc_recompress_segment(const uc_segment* src, const float* scores, int6
   } else {
     g.max_chunks = std::max(1, (max_keep + 31) / 32);
     launch_gather(g, cs);
-  }
-
-  // 4. stored-row indices -> the source's logical token indices.
-  if (src->kept_idx != nullptr) {
-    ComposeArgs c;
-    c.kept_idx = dst->kept_idx;
-    c.src_idx = src->kept_idx;
-    c.n_kept = dst->n_kept;
-    c.n_kv_heads = dst->n_kv_heads;
-    c.cap = dst->cap;
-    c.src_cap = src->cap;
-    launch_compose_idx(c, nbh, cs);
   }
   return cuda_check("uc_recompress_segment");
 }

@@ -5,8 +5,8 @@
 //                  order-preserving score keys, ties to the lower index,
 //                  kept indices written in ascending order
 //  gather_rows     compaction of the kept bf16 rows (eviction)
-//  quantize_groups int4 / int2 group quantization of the kept sequence
-//  copy_tail       the bf16 residual tail (n_kept mod 32 last kept tokens)
+//  quantize_groups int4 / int2 group quantization of the kept sequence and
+//                  its bf16 residual tail (n_kept mod 32 last kept tokens)
 //  append_token    one decode token per sequence into a segment
 #include <algorithm>
 
@@ -241,15 +241,6 @@ __global__ void __launch_bounds__(kTopkThreads) topk_kernel(TopkArgs a) {
   }
 }
 
-// Kept indices of a segment that keeps every token (QUANT).
-__global__ void iota_kernel(TopkArgs a) {
-  const int bh = blockIdx.x;
-  const int b = bh / a.n_kv_heads;
-  int32_t* out = a.kept_idx + (int64_t)bh * a.cap;
-  for (int t = threadIdx.x; t < a.keep[b]; t += blockDim.x) out[t] = t;
-  if (bh % a.n_kv_heads == 0 && threadIdx.x == 0) a.n_kept[b] = a.keep[b];
-}
-
 // -------------------------------------------------- re-compression helpers
 
 // One warp per (b, kvh, 32 kept tokens) of a packed segment: rebuild the K and
@@ -317,45 +308,63 @@ __global__ void dequant_rows_kernel(DequantArgs a) {
   }
 }
 
-__global__ void compose_idx_kernel(ComposeArgs a) {
-  const int bh = blockIdx.x;
-  const int b = bh / a.n_kv_heads;
-  int32_t* idx = a.kept_idx + (int64_t)bh * a.cap;
-  const int32_t* src = a.src_idx + (int64_t)bh * a.src_cap;
-  for (int t = threadIdx.x; t < a.n_kept[b]; t += blockDim.x) idx[t] = src[idx[t]];
+// ----------------------------------------------------------------- gather
+
+// Source row of kept token t of block bh; a re-compression's kept index moves
+// on to the logical token of that row (every entry has one reader, the lane
+// that also rewrites it), a segment that keeps every token gets its indices
+// here (`identity`: row t is kept token t).
+__device__ __forceinline__ int32_t take_row(const GatherArgs& a, int bh, int t) {
+  int32_t* e = a.kept_idx + (int64_t)bh * a.cap + t;
+  const int32_t row = a.identity ? t : *e;
+  if (a.src_idx != nullptr)
+    *e = a.src_idx[(int64_t)bh * a.src_cap + row];
+  else if (a.identity)
+    *e = row;
+  return row;
 }
 
-// ----------------------------------------------------------------- gather
+// Copy kept tokens t0 .. t0 + cnt - 1 (cnt <= 32) of block bh to the rows
+// dst_row .. of k_dst / v_dst. Lane t holds token t0 + t's source row; two
+// rows per step (16 lanes x 16 bytes each), eight rows' K and V in flight.
+__device__ __forceinline__ void copy_rows(const GatherArgs& a, int bh, int t0, int cnt, int64_t dst_row) {
+  const int lane = threadIdx.x & 31;
+  const int32_t row = lane < cnt ? take_row(a, bh, t0 + lane) : 0;
+  const int64_t src_base = (int64_t)bh * a.src_row_stride + a.src_row_offset;
+  const int c = (lane & 15) * 8;
+  for (int q0 = 0; q0 < cnt; q0 += 8) {
+    uint4 kx[4], vx[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int t = q0 + 2 * u + (lane >> 4);
+      const int64_t sr = (src_base + __shfl_sync(0xffffffffu, row, t & 31)) * kHeadDim + c;
+      if (t < cnt) {
+        kx[u] = *reinterpret_cast<const uint4*>(a.k_src + sr);
+        vx[u] = *reinterpret_cast<const uint4*>(a.v_src + sr);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int t = q0 + 2 * u + (lane >> 4);
+      if (t < cnt) {
+        *reinterpret_cast<uint4*>(a.k_dst + (dst_row + t) * kHeadDim + c) = kx[u];
+        *reinterpret_cast<uint4*>(a.v_dst + (dst_row + t) * kHeadDim + c) = vx[u];
+      }
+    }
+  }
+}
 
 // One warp per (b, kvh, 32 kept tokens): copy the kept K and V rows into the
 // compacted bf16 storage (rows_per_block = cap, offset 0).
 __global__ void gather_rows_kernel(GatherArgs a) {
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
   const int per_bh = a.max_chunks;
   const int bh = warp / per_bh;
   if (bh >= a.batch * a.n_kv_heads) return;
-  const int b = bh / a.n_kv_heads;
   const int t0 = (warp % per_bh) * 32;
-  const int n = a.keep[b];
+  const int n = a.keep[bh / a.n_kv_heads];
   if (t0 >= n) return;
-  const int32_t* idx = a.kept_idx + (int64_t)bh * a.cap;
-  const int64_t src_base = (int64_t)bh * a.src_row_stride + a.src_row_offset;
-  const int64_t dst_base = (int64_t)bh * a.dst_row_stride + a.dst_row_offset;
-  const int cnt = min(32, n - t0);
-  // two rows per pass: lanes 0..15 row 2q, lanes 16..31 row 2q+1
-  for (int q = 0; q < (cnt + 1) / 2; ++q) {
-    const int t = t0 + 2 * q + (lane >> 4);
-    if (t < t0 + cnt) {
-      const int64_t sr = src_base + idx[t];
-      const int64_t dr = dst_base + t;
-      const int c = (lane & 15) * 8;
-      *reinterpret_cast<uint4*>(a.k_dst + dr * kHeadDim + c) =
-          *reinterpret_cast<const uint4*>(a.k_src + sr * kHeadDim + c);
-      *reinterpret_cast<uint4*>(a.v_dst + dr * kHeadDim + c) =
-          *reinterpret_cast<const uint4*>(a.v_src + sr * kHeadDim + c);
-    }
-  }
+  copy_rows(a, bh, t0, min(32, n - t0), (int64_t)bh * a.dst_row_stride + a.dst_row_offset + t0);
 }
 
 // ---------------------------------------------------------- quantization
@@ -391,15 +400,17 @@ __global__ void __launch_bounds__(kQuantWarps * 32, kQuantCtasPerSm) quantize_gr
   const int n_warps = gridDim.x * kQuantWarps;
   const int per_bh = a.max_chunks;
   const int total = a.batch * a.n_kv_heads * per_bh;
-  // the first valid group at or after w (groups past a sequence's full
-  // groups are skipped)
+  const int all = total + a.batch * a.n_kv_heads;  // then one residual tail per (b, kvh)
+  // the first valid group or tail at or after w (groups past a sequence's
+  // full groups and empty tails are skipped)
   auto valid_from = [&](int w) {
-    for (; w < total; w += n_warps) {
-      const int b = (w / per_bh) / a.n_kv_heads;
-      if (w % per_bh < a.keep[b] / kGroup) break;
+    for (; w < all; w += n_warps) {
+      const int b = (w < total ? w / per_bh : w - total) / a.n_kv_heads;
+      if (w < total ? w % per_bh < a.keep[b] / kGroup : a.keep[b] % kGroup != 0) break;
     }
     return w;
   };
+  if (a.identity && blockIdx.x == 0 && threadIdx.x < a.batch) a.n_kept[threadIdx.x] = a.keep[threadIdx.x];
   if (lane == 0) {
     for (int k = 0; k < kQuantBufs; ++k) mbar_init(&sm.bar[k], 1);
     fence_barrier_init();
@@ -408,7 +419,7 @@ __global__ void __launch_bounds__(kQuantWarps * 32, kQuantCtasPerSm) quantize_gr
   // kept index of this lane's row of group w (loaded a group ahead, so that
   // the request does not wait for it)
   auto row_index = [&](int w) {
-    return w < total ? a.kept_idx[(int64_t)(w / per_bh) * a.cap + (w % per_bh) * kGroup + lane] : 0;
+    return w < total ? take_row(a, w / per_bh, (w % per_bh) * kGroup + lane) : 0;
   };
   // rows of group w (K if kv == 0, else V) into buffer `buf`
   auto request = [&](int w, int buf, int kv, int32_t idx) {
@@ -423,10 +434,11 @@ __global__ void __launch_bounds__(kQuantWarps * 32, kQuantCtasPerSm) quantize_gr
   auto krow = [&](int t) { return reinterpret_cast<const __nv_bfloat16*>(sm.rows[0] + t * kQuantRowBytes); };
   auto vrow = [&](int t) { return reinterpret_cast<const __nv_bfloat16*>(sm.rows[kVBuf] + t * kQuantRowBytes); };
   int w = valid_from(blockIdx.x * kQuantWarps + (threadIdx.x >> 5));
-  if (w >= total) return;
   int32_t idx = row_index(w);
-  request(w, 0, 0, idx);
-  if constexpr (kQuantBufs == 2) request(w, 1, 1, idx);
+  if (w < total) {
+    request(w, 0, 0, idx);
+    if constexpr (kQuantBufs == 2) request(w, 1, 1, idx);
+  }
   // phase of the next completion of each buffer's barrier
   uint32_t ph_k = 0, ph_v = 0;
   bool failed = false;
@@ -474,28 +486,14 @@ __global__ void __launch_bounds__(kQuantWarps * 32, kQuantCtasPerSm) quantize_gr
     // released: wait for each barrier's pending phase (bounded again)
     mbar_wait(&sm.bar[0], ph_k, nullptr, 0, a.wait_ns);
     if constexpr (kQuantBufs == 2) mbar_wait(&sm.bar[1], ph_v, nullptr, 0, a.wait_ns);
+    return;
   }
-}
-
-// The residual tail: the last (n mod 32) kept tokens, copied to the bf16
-// tail block (32 rows per (b, kvh)). One warp per (b, kvh).
-__global__ void copy_tail_kernel(GatherArgs a) {
-  const int bh = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (bh >= a.batch * a.n_kv_heads) return;
-  const int b = bh / a.n_kv_heads;
-  const int n = a.keep[b];
-  const int t0 = (n / kGroup) * kGroup;
-  const int32_t* idx = a.kept_idx + (int64_t)bh * a.cap;
-  const int64_t src_base = (int64_t)bh * a.src_row_stride + a.src_row_offset;
-  for (int t = t0 + (lane >> 4); t < n; t += 2) {
-    const int64_t sr = src_base + idx[t];
-    const int64_t dr = (int64_t)bh * kGroup + (t - t0);
-    const int c = (lane & 15) * 8;
-    *reinterpret_cast<uint4*>(a.k_dst + dr * kHeadDim + c) =
-        *reinterpret_cast<const uint4*>(a.k_src + sr * kHeadDim + c);
-    *reinterpret_cast<uint4*>(a.v_dst + dr * kHeadDim + c) =
-        *reinterpret_cast<const uint4*>(a.v_src + sr * kHeadDim + c);
+  // the residual tails: the last (n mod 32) kept tokens of a (b, kvh), copied
+  // to its bf16 tail block of 32 rows
+  for (; w < all; w = valid_from(w + n_warps)) {
+    const int bh = w - total;
+    const int n = a.keep[bh / a.n_kv_heads];
+    copy_rows(a, bh, n / kGroup * kGroup, n % kGroup, (int64_t)bh * kGroup);
   }
 }
 
@@ -569,12 +567,7 @@ static int compress_sms() {
 // CTAs per (sequence, KV head): one up to kTopkPerCta candidates, then as many
 // (a power of two up to 8) as share the list at no fewer than that each and
 // fit the GPU at one CTA per SM.
-void launch_topk(const TopkArgs& a, int n_blocks, bool evict, cudaStream_t st) {
-  if (!evict) {
-    iota_kernel<<<n_blocks, 256, 0, st>>>(a);
-    count_launch();
-    return;
-  }
+void launch_topk(const TopkArgs& a, int n_blocks, cudaStream_t st) {
   int max_src = 0;
   for (int b = 0; b < UC_MAX_BATCH; ++b) max_src = std::max(max_src, a.src_n[b]);
   int c = 1;
@@ -603,11 +596,6 @@ void launch_dequant_rows(const DequantArgs& a, cudaStream_t st) {
   count_launch();
 }
 
-void launch_compose_idx(const ComposeArgs& a, int nbh, cudaStream_t st) {
-  compose_idx_kernel<<<nbh, 256, 0, st>>>(a);
-  count_launch();
-}
-
 void launch_gather(const GatherArgs& a, cudaStream_t st) {
   const int warps = a.batch * a.n_kv_heads * a.max_chunks;
   gather_rows_kernel<<<(warps + 3) / 4, 128, 0, st>>>(a);
@@ -616,24 +604,19 @@ void launch_gather(const GatherArgs& a, cudaStream_t st) {
 
 void launch_quantize(const GatherArgs& a, int bits, cudaStream_t st) {
   static bool attr4 = false, attr2 = false;
-  const int warps = a.batch * a.n_kv_heads * a.max_chunks;
+  const int warps = a.batch * a.n_kv_heads * (a.max_chunks + 1);  // groups and tails
   const int blocks = std::min((warps + kQuantWarps - 1) / kQuantWarps, kQuantCtasPerSm * compress_sms());
-  if (blocks > 0) {
-    if (bits == 4) {
-      if (!attr4)
-        attr4 = cudaFuncSetAttribute(quantize_groups_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kQuantSmemBytes) == cudaSuccess;
-      quantize_groups_kernel<4><<<blocks, kQuantWarps * 32, kQuantSmemBytes, st>>>(a);
-    } else {
-      if (!attr2)
-        attr2 = cudaFuncSetAttribute(quantize_groups_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kQuantSmemBytes) == cudaSuccess;
-      quantize_groups_kernel<2><<<blocks, kQuantWarps * 32, kQuantSmemBytes, st>>>(a);
-    }
-    count_launch();
+  if (bits == 4) {
+    if (!attr4)
+      attr4 = cudaFuncSetAttribute(quantize_groups_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)kQuantSmemBytes) == cudaSuccess;
+    quantize_groups_kernel<4><<<blocks, kQuantWarps * 32, kQuantSmemBytes, st>>>(a);
+  } else {
+    if (!attr2)
+      attr2 = cudaFuncSetAttribute(quantize_groups_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)kQuantSmemBytes) == cudaSuccess;
+    quantize_groups_kernel<2><<<blocks, kQuantWarps * 32, kQuantSmemBytes, st>>>(a);
   }
-  const int tw = a.batch * a.n_kv_heads;
-  copy_tail_kernel<<<(tw + 3) / 4, 128, 0, st>>>(a);
   count_launch();
 }
 

@@ -88,7 +88,11 @@ struct GatherArgs {
   const __nv_bfloat16* k_src;
   const __nv_bfloat16* v_src;
   int64_t src_row_stride, src_row_offset;
-  const int32_t* kept_idx;
+  int32_t* kept_idx;       // source rows of the kept tokens (see identity, src_idx)
+  int identity;            // 1: every token is kept: kept_idx and n_kept are written here
+  const int32_t* src_idx;  // re-compression: kept_idx is rewritten to src_idx[row] (logical tokens); or NULL
+  int src_cap;
+  int32_t* n_kept;         // written when identity
   __nv_bfloat16* k_dst;  // EVICT: compacted rows; quantized: the tail block
   __nv_bfloat16* v_dst;
   int64_t dst_row_stride, dst_row_offset;
@@ -135,19 +139,10 @@ struct DequantArgs {
   int batch, n_kv_heads, cap, bits, max_groups;
 };
 
-// kept_idx[i] = src_idx[kept_idx[i]] for the first n_kept[b] entries.
-struct ComposeArgs {
-  int32_t* kept_idx;
-  const int32_t* src_idx;
-  const int32_t* n_kept;
-  int n_kv_heads, cap, src_cap;
-};
-
-void launch_topk(const TopkArgs& a, int n_blocks, bool evict, cudaStream_t st);
+void launch_topk(const TopkArgs& a, int n_blocks, cudaStream_t st);
 void launch_dequant_rows(const DequantArgs& a, cudaStream_t st);
 void launch_attention_mass(const float* mass, int batch, int rows, int n_seg, float scale,
                            bool accumulate, float* out, cudaStream_t st);
-void launch_compose_idx(const ComposeArgs& a, int nbh, cudaStream_t st);
 void launch_gather(const GatherArgs& a, cudaStream_t st);
 void launch_quantize(const GatherArgs& a, int bits, cudaStream_t st);
 void launch_append(const AppendArgs& a, int bits, cudaStream_t st);

@@ -19,9 +19,19 @@ from ._lib import (GROUP, HEAD_DIM, KIND_EVICT, KIND_EVICT_QUANT, KIND_FULL, KIN
 KIND_NAMES = {"full": KIND_FULL, "evict": KIND_EVICT, "quant": KIND_QUANT, "evict_quant": KIND_EVICT_QUANT}
 
 
-def _stream(stream=None) -> C.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+_raw_stream = None   # torch's handle lookup without a Stream object, once CUDA is initialised
+
+
+def _stream(stream=None) -> int:
+    """The cudaStream_t of ``stream``, else of the current device's current stream."""
+    global _raw_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        handle = torch.cuda.current_stream().cuda_stream
+        _raw_stream = torch._C._cuda_getCurrentRawStream
+        return handle
+    return _raw_stream(torch._C._cuda_getDevice())
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -456,6 +466,11 @@ def attention_mass(mass: torch.Tensor, out: Optional[torch.Tensor] = None, weigh
     return out
 
 
+def _seg_array(segs: Sequence[Segment]):
+    """A C array of the segments' addresses (valid while ``segs`` are)."""
+    return (C.c_void_p * len(segs))(*[C.addressof(s.c) for s in segs])
+
+
 def attend(q: torch.Tensor, segs: Sequence[Segment], out: Optional[torch.Tensor] = None,
            lse: Optional[torch.Tensor] = None, mass: Optional[torch.Tensor] = None,
            want_lse: bool = True, want_mass: bool = True, ws: Optional[Workspace] = None,
@@ -464,18 +479,27 @@ def attend(q: torch.Tensor, segs: Sequence[Segment], out: Optional[torch.Tensor]
     mass fp32 [B, Hq, T, n_seg])."""
     B, hq, T, d = q.shape
     ns = len(segs)
-    arr = (C.POINTER(UcSegment) * ns)(*[C.pointer(s.c) for s in segs])
+    arr = _seg_array(segs)
     if out is None:
         out = torch.empty_like(q)
     if want_lse and lse is None:
-        lse = torch.empty((B, hq, T), dtype=torch.float32, device=q.device)
+        lse = q.new_empty((B, hq, T), dtype=torch.float32)
     if want_mass and mass is None:
-        mass = torch.empty((B, hq, T, ns), dtype=torch.float32, device=q.device)
+        mass = q.new_empty((B, hq, T, ns), dtype=torch.float32)
     ws = ws or default_workspace(q.device)
-    wp, wn = ws.get(lib().uc_attend_workspace_size(C.cast(arr, C.c_void_p), ns, hq, T), "attend")
-    check("uc_attend", lib().uc_attend(
-        _ptr(q), hq, T, C.cast(arr, C.c_void_p), ns, _ptr(out), _ptr(lse), _ptr(mass), wp, wn,
-        _stream(stream)))
+    L = lib()
+    # the call plans once and says if the workspace at hand is too small for
+    # it (nothing is launched then): only then is the size asked for
+    buf = ws.bufs.get("attend")
+    wp, wn = (buf.data_ptr(), buf.numel()) if buf is not None else \
+        ws.get(L.uc_attend_workspace_size(arr, ns, hq, T), "attend")
+    args = (q.data_ptr(), hq, T, arr, ns, out.data_ptr(), _ptr(lse), _ptr(mass))
+    st = _stream(stream)
+    code = L.uc_attend(*args, wp, wn, st)
+    if code == _lib.UC_ERR_OOM:
+        wp, wn = ws.get(L.uc_attend_workspace_size(arr, ns, hq, T), "attend")
+        code = L.uc_attend(*args, wp, wn, st)
+    check("uc_attend", code)
     return out, lse, mass
 
 
@@ -500,38 +524,48 @@ def attend_batch(calls, ws: Optional[Workspace] = None, stream=None):
     of (q, segs) or (q, segs, out, lse, mass) with q [B, Hq, T, 128] bf16
     (T <= 8; every call the same number of 8-row query tiles). Returns the
     list of (O, lse, mass) per call."""
-    from ._lib import UcAttendCall
     n = len(calls)
-    arr = (UcAttendCall * n)()
-    keep = []
-    results = []
-    for i, call in enumerate(calls):
+    given = [(list(call[2:5]) + [None, None, None])[:3] for call in calls]
+    shapes = [(B, hq, T, len(call[1])) for call in calls for B, hq, T, _ in [call[0].shape]]
+    dev = calls[0][0].device
+    if n > 1 and all(g[1] is None and g[2] is None for g in given) and all(x == shapes[0] for x in shapes) \
+            and all(call[0].device == dev for call in calls):
+        # one allocation each for the calls' lse and masses
+        B, hq, T, ns = shapes[0]
+        lses = torch.empty((n, B, hq, T), dtype=torch.float32, device=dev).unbind(0)
+        masses = torch.empty((n, B, hq, T, ns), dtype=torch.float32, device=dev).unbind(0)
+        given = [(g[0], lses[i], masses[i]) for i, g in enumerate(given)]
+    keep, results, structs = [], [], []
+    for call, (out, lse, mass), (B, hq, T, ns) in zip(calls, given, shapes):
         q, segs = call[0], call[1]
-        out, lse, mass = (list(call[2:5]) + [None, None, None])[:3]
-        B, hq, T, d = q.shape
-        ns = len(segs)
         if out is None:
             out = torch.empty_like(q)
         if lse is None:
-            lse = torch.empty((B, hq, T), dtype=torch.float32, device=q.device)
+            lse = q.new_empty((B, hq, T), dtype=torch.float32)
         if mass is None:
-            mass = torch.empty((B, hq, T, ns), dtype=torch.float32, device=q.device)
-        sp = (C.POINTER(UcSegment) * ns)(*[C.pointer(s.c) for s in segs])
+            mass = q.new_empty((B, hq, T, ns), dtype=torch.float32)
+        sp = _seg_array(segs)
         keep.append(sp)
-        arr[i].q, arr[i].n_q_heads, arr[i].n_qtok = _ptr(q), hq, T
-        arr[i].segs, arr[i].n_seg = C.cast(sp, C.c_void_p), ns
-        arr[i].out, arr[i].lse, arr[i].mass = _ptr(out), _ptr(lse), _ptr(mass)
+        structs.append(_lib.UcAttendCall(q.data_ptr(), hq, T, C.addressof(sp), ns, out.data_ptr(), lse.data_ptr(),
+                                         mass.data_ptr()))
         results.append((out, lse, mass))
-    ws = ws or default_workspace(calls[0][0].device)
-    wp, wn = ws.get(lib().uc_attend_batch_workspace_size(C.cast(arr, C.c_void_p), n), "attend_batch")
-    check("uc_attend_batch", lib().uc_attend_batch(C.cast(arr, C.c_void_p), n, wp, wn, _stream(stream)))
+    arr = (_lib.UcAttendCall * n)(*structs)
+    ws = ws or default_workspace(dev)
+    L = lib()
+    buf = ws.bufs.get("attend_batch")   # as in attend(): the size is asked for only when the call needs more
+    wp, wn = (buf.data_ptr(), buf.numel()) if buf is not None else \
+        ws.get(L.uc_attend_batch_workspace_size(arr, n), "attend_batch")
+    st = _stream(stream)
+    code = L.uc_attend_batch(arr, n, wp, wn, st)
+    if code == _lib.UC_ERR_OOM:
+        wp, wn = ws.get(L.uc_attend_batch_workspace_size(arr, n), "attend_batch")
+        code = L.uc_attend_batch(arr, n, wp, wn, st)
+    check("uc_attend_batch", code)
     return results
 
 
 def attend_workspace_size(segs: Sequence[Segment], n_q_heads: int, n_qtok: int) -> int:
-    ns = len(segs)
-    arr = (C.POINTER(UcSegment) * ns)(*[C.pointer(s.c) for s in segs])
-    return int(lib().uc_attend_workspace_size(C.cast(arr, C.c_void_p), ns, n_q_heads, n_qtok))
+    return int(lib().uc_attend_workspace_size(_seg_array(segs), len(segs), n_q_heads, n_qtok))
 
 
 def append(seg: Segment, k_new: torch.Tensor, v_new: torch.Tensor, position: int,

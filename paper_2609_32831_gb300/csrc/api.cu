@@ -1051,24 +1051,22 @@ constexpr size_t kCounterBlock = (size_t)UC_MAX_BATCH * 8 * 4;
 static_assert(kCounterBlock % 256 == 0, "counter block alignment");
 
 // Partial outputs of one decode call.
-size_t decode_part_bytes(const uc_segment* const* segs, int n_seg, int mtiles, int nbh_launch,
-                         int forced_ipb = 0) {
-  const AttnPlan p = plan_attend(segs, n_seg, mtiles, nbh_launch, forced_ipb);
-  return ((size_t)p.n_items * attend_part_floats(mtiles) * 4 + 255) / 256 * 256;
+size_t decode_part_bytes(const AttnPlan& p) {
+  return ((size_t)p.n_items * attend_part_floats(p.mtiles) * 4 + 255) / 256 * 256;
 }
 
-// Kernel parameters of one checked decode call whose counters start at
-// `counters` (a kCounterBlock) and partial outputs at `parts`.
+size_t decode_workspace(const AttnPlan& p) { return 256 + kCounterBlock + decode_part_bytes(p); }
+
+// Kernel parameters of one checked and planned decode call whose counters
+// start at `counters` (a kCounterBlock) and partial outputs at `parts`.
 uc_status build_decode_call(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_segment* const* segs,
-                            int32_t n_seg, void* out, float* lse, float* mass, int nbh_launch, int forced_ipb,
-                            uint8_t* counters, uint8_t* parts, DevStatus* status, AttnParams* p,
-                            AttnPlan* plan) {
+                            int32_t n_seg, void* out, float* lse, float* mass, const AttnPlan* plan,
+                            uint8_t* counters, uint8_t* parts, DevStatus* status, AttnParams* p) {
   memset(p, 0, sizeof(*p));
   const int B = segs[0]->batch, hkv = segs[0]->n_kv_heads;
   const int group = n_q_heads / hkv;
   const int rows = group * n_qtok;
-  const int mtiles = (rows + 7) / 8;
-  *plan = plan_attend(segs, n_seg, mtiles, nbh_launch, forced_ipb);
+  const int mtiles = plan->mtiles;
   for (int s = 0; s < n_seg; ++s) {
     const uc_segment* sg = segs[s];
     SegDev& d = p->seg[s];
@@ -1131,6 +1129,33 @@ void batch_items(const uc_attend_call* calls, int n_calls, int mtiles, int* ipb)
   }
 }
 
+// uc_attend's checks before it looks at its workspace and the call's plan: a
+// decode call's work items in *plan (T <= UC_MAX_QTOKENS), a dense call's key
+// tiles in *dp; *need: the workspace bytes the call takes.
+uc_status check_and_plan(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_segment* const* segs,
+                         int32_t n_seg, const void* out, const char* name, AttnPlan* plan, DensePlan* dp,
+                         size_t* need) {
+  uc_status st = check_call(q, n_q_heads, n_qtok, segs, n_seg, out, name);
+  if (st != UC_OK) return st;
+  const int hkv = segs[0]->n_kv_heads;
+  if (n_qtok > UC_MAX_QTOKENS) {
+    if (!plan_dense(segs, n_seg, dp)) {
+      set_error("%s: more than %d key tiles of %d", name, kMaxDenseTiles, kDenseKeys);
+      return UC_ERR_SHAPE;
+    }
+    *need = dense_workspace(*dp, segs[0]->batch * hkv);
+    return UC_OK;
+  }
+  const int mtiles = decode_mtiles(n_q_heads, hkv, n_qtok);
+  if (mtiles > 8) {
+    set_error("%s: (Hq / Hkv) * T = %d rows exceed 64", name, n_q_heads / hkv * n_qtok);
+    return UC_ERR_SHAPE;
+  }
+  *plan = plan_attend(segs, n_seg, mtiles, segs[0]->batch * hkv);
+  *need = decode_workspace(*plan);
+  return UC_OK;
+}
+
 }  // namespace
 }  // extern "C"
 
@@ -1143,24 +1168,9 @@ size_t attend_counter_bytes() { return kCounterBlock; }
 
 uc_status attend_precheck(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_segment* const* segs,
                           int32_t n_seg, const void* out, const char* name, size_t* need) {
-  uc_status st = check_call(q, n_q_heads, n_qtok, segs, n_seg, out, name);
-  if (st != UC_OK) return st;
-  const int hkv = segs[0]->n_kv_heads;
-  if (n_qtok > UC_MAX_QTOKENS) {
-    static thread_local DensePlan dp;
-    if (!plan_dense(segs, n_seg, &dp)) {
-      set_error("%s: more than %d key tiles of %d", name, kMaxDenseTiles, kDenseKeys);
-      return UC_ERR_SHAPE;
-    }
-    *need = dense_workspace(dp, segs[0]->batch * hkv);
-    return UC_OK;
-  }
-  if (decode_mtiles(n_q_heads, hkv, n_qtok) > 8) {
-    set_error("%s: (Hq / Hkv) * T = %d rows exceed 64", name, n_q_heads / hkv * n_qtok);
-    return UC_ERR_SHAPE;
-  }
-  *need = 256 + kCounterBlock + decode_part_bytes(segs, n_seg, decode_mtiles(n_q_heads, hkv, n_qtok), segs[0]->batch * hkv);
-  return UC_OK;
+  AttnPlan plan;
+  static thread_local DensePlan dp;
+  return check_and_plan(q, n_q_heads, n_qtok, segs, n_seg, out, name, &plan, &dp, need);
 }
 
 uint64_t wait_limit_ns() { return g_wait_limit_ns.load(); }
@@ -1186,7 +1196,7 @@ size_t uc_attend_workspace_size(const uc_segment* const* segs, int32_t n_seg, in
   const int hkv = segs[0]->n_kv_heads;
   if (hkv < 1 || n_q_heads % hkv) return 0;
   const int mtiles = decode_mtiles(n_q_heads, hkv, n_qtok);
-  return 256 + kCounterBlock + decode_part_bytes(segs, n_seg, mtiles, segs[0]->batch * hkv);
+  return decode_workspace(plan_attend(segs, n_seg, mtiles, segs[0]->batch * hkv));
 }
 
 uc_status uc_attend_plan(const uc_segment* const* segs, int32_t n_seg, int32_t n_q_heads, int32_t n_qtok,
@@ -1254,24 +1264,20 @@ uc_status uc_attend(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_s
     set_error("uc_attend: null or misaligned workspace");
     return UC_ERR_ARG;
   }
-  size_t need_checked = 0;
-  uc_status st = uc::attend_precheck(q, n_q_heads, n_qtok, segs, n_seg, out, "uc_attend", &need_checked);
+  size_t need = 0;
+  AttnPlan plan;
+  static thread_local DensePlan dp;
+  uc_status st = check_and_plan(q, n_q_heads, n_qtok, segs, n_seg, out, "uc_attend", &plan, &dp, &need);
   if (st != UC_OK) return st;
+  if (workspace_bytes < need) {
+    set_error("uc_attend: workspace %zu < %zu bytes", workspace_bytes, need);
+    return UC_ERR_OOM;
+  }
   const int B = segs[0]->batch, hkv = segs[0]->n_kv_heads;
   const int group = n_q_heads / hkv;
   if (n_qtok > UC_MAX_QTOKENS) {
     // many query tokens (denoising / editing): tensor-core dense path
-    static thread_local DensePlan dp;
-    if (!plan_dense(segs, n_seg, &dp)) {
-      set_error("uc_attend: more than %d key tiles of %d", kMaxDenseTiles, kDenseKeys);
-      return UC_ERR_SHAPE;
-    }
     const int nbh = B * hkv;
-    const size_t need = dense_workspace(dp, nbh);
-    if (workspace_bytes < need) {
-      set_error("uc_attend: workspace %zu < %zu bytes", workspace_bytes, need);
-      return UC_ERR_OOM;
-    }
     static thread_local DenseParams d;
     memset(&d, 0, sizeof(d));
     uint8_t* ws = static_cast<uint8_t*>(workspace);
@@ -1320,21 +1326,10 @@ uc_status uc_attend(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_s
     launch_dense(d, reinterpret_cast<cudaStream_t>(stream));
     return cuda_check("uc_attend (dense)");
   }
-  const int mtiles = decode_mtiles(n_q_heads, hkv, n_qtok);
-  if (mtiles > 8) {
-    set_error("uc_attend: (Hq / Hkv) * T = %d rows exceed 64", group * n_qtok);
-    return UC_ERR_SHAPE;
-  }
-  const size_t need = uc_attend_workspace_size(segs, n_seg, n_q_heads, n_qtok);
-  if (workspace_bytes < need) {
-    set_error("uc_attend: workspace %zu < %zu bytes", workspace_bytes, need);
-    return UC_ERR_OOM;
-  }
   static thread_local AttnParams p;
-  AttnPlan plan;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  st = build_decode_call(q, n_q_heads, n_qtok, segs, n_seg, out, lse, mass, B * hkv, 0, ws + 256,
-                         ws + 256 + kCounterBlock, reinterpret_cast<DevStatus*>(ws), &p, &plan);
+  st = build_decode_call(q, n_q_heads, n_qtok, segs, n_seg, out, lse, mass, &plan, ws + 256,
+                         ws + 256 + kCounterBlock, reinterpret_cast<DevStatus*>(ws), &p);
   if (st != UC_OK) return st;
   p.defer_merge = merge_kernel_for(plan.items_per_bh);
   launch_attend(p, plan.grid, reinterpret_cast<cudaStream_t>(stream));
@@ -1360,7 +1355,7 @@ size_t uc_attend_batch_workspace_size(const uc_attend_call* calls, int32_t n_cal
   for (int c = 0; c < n_calls; ++c) {
     const uc_attend_call& k = calls[c];
     const int mt = decode_mtiles(k.n_q_heads, k.segs[0]->n_kv_heads, k.n_qtok);
-    n += decode_part_bytes(k.segs, k.n_seg, mt, nbh_launch, ipb[c]);
+    n += decode_part_bytes(plan_attend(k.segs, k.n_seg, mt, nbh_launch, ipb[c]));
   }
   return n;
 }
@@ -1395,27 +1390,30 @@ uc_status uc_attend_batch(const uc_attend_call* calls, int32_t n_calls, void* wo
     mtiles = mt;
     nbh_launch += k.segs[0]->batch * k.segs[0]->n_kv_heads;
   }
-  const size_t need = uc_attend_batch_workspace_size(calls, n_calls);
-  if (need == 0 || workspace_bytes < need) {
+  int ipb[UC_MAX_CALLS];
+  batch_items(calls, n_calls, mtiles, ipb);
+  AttnPlan plans[UC_MAX_CALLS];
+  size_t need = 256 + UC_MAX_CALLS * kCounterBlock;
+  for (int c = 0; c < n_calls; ++c) {
+    plans[c] = plan_attend(calls[c].segs, calls[c].n_seg, mtiles, nbh_launch, ipb[c]);
+    need += decode_part_bytes(plans[c]);
+  }
+  if (workspace_bytes < need) {
     set_error("uc_attend_batch: workspace %zu < %zu bytes", workspace_bytes, need);
     return UC_ERR_OOM;
   }
-  int ipb[UC_MAX_CALLS];
-  batch_items(calls, n_calls, mtiles, ipb);
-  static thread_local MultiAttnParams m;
-  memset(&m, 0, sizeof(m));
+  static thread_local MultiAttnParams m;  // each call's parameters are cleared by build_decode_call
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   DevStatus* status = reinterpret_cast<DevStatus*>(ws);
   size_t off = 256 + UC_MAX_CALLS * kCounterBlock;
   int heavy = 0, light = 0, grid = 0;
   for (int c = 0; c < n_calls; ++c) {
     const uc_attend_call& k = calls[c];
-    AttnPlan plan;
+    const AttnPlan& plan = plans[c];
     const uc_status st = build_decode_call(k.q, k.n_q_heads, k.n_qtok, k.segs, k.n_seg, k.out, k.lse, k.mass,
-                                           nbh_launch, ipb[c], ws + 256 + c * kCounterBlock, ws + off, status,
-                                           &m.call[c], &plan);
+                                           &plan, ws + 256 + c * kCounterBlock, ws + off, status, &m.call[c]);
     if (st != UC_OK) return st;
-    off += decode_part_bytes(k.segs, k.n_seg, mtiles, nbh_launch, ipb[c]);
+    off += decode_part_bytes(plan);
     const int nbh = k.segs[0]->batch * k.segs[0]->n_kv_heads;
     m.heavy_begin[c] = heavy;
     m.light_begin[c] = light;

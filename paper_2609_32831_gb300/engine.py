@@ -208,6 +208,7 @@ class RequestCache:
             if scores_out is not None:
                 scores_out[:] = scores
         tables = self._budgets(lambda l: scores[l]) if auto else None
+        configs: Dict[tuple, tuple] = {}    # the layers of a chunk share its tables: one configuration per type
         for l in range(self.L):
             segs = []
             for a, ty in enumerate(self.types):
@@ -216,7 +217,9 @@ class RequestCache:
                     continue
                 if ty.policy == "auto":
                     c = l // self.layer_chunk
-                    kind, bits, full_view, keep = api.plan_batch(tables[c * self.B:(c + 1) * self.B], a)
+                    if (c, a) not in configs:
+                        configs[c, a] = api.plan_batch(tables[c * self.B:(c + 1) * self.B], a)
+                    kind, bits, full_view, keep = configs[c, a]
                     if full_view:
                         segs.append(self._view((l, a), k[l], v[l], self.begin[a], ty.n))
                         continue

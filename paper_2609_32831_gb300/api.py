@@ -483,9 +483,9 @@ def attend(q: torch.Tensor, segs: Sequence[Segment], out: Optional[torch.Tensor]
     if out is None:
         out = torch.empty_like(q)
     if want_lse and lse is None:
-        lse = q.new_empty((B, hq, T), dtype=torch.float32)
+        lse = torch.empty((B, hq, T), dtype=torch.float32, device=q.device)
     if want_mass and mass is None:
-        mass = q.new_empty((B, hq, T, ns), dtype=torch.float32)
+        mass = torch.empty((B, hq, T, ns), dtype=torch.float32, device=q.device)
     ws = ws or default_workspace(q.device)
     L = lib()
     # the call plans once and says if the workspace at hand is too small for
@@ -541,9 +541,9 @@ def attend_batch(calls, ws: Optional[Workspace] = None, stream=None):
         if out is None:
             out = torch.empty_like(q)
         if lse is None:
-            lse = q.new_empty((B, hq, T), dtype=torch.float32)
+            lse = torch.empty((B, hq, T), dtype=torch.float32, device=q.device)
         if mass is None:
-            mass = q.new_empty((B, hq, T, ns), dtype=torch.float32)
+            mass = torch.empty((B, hq, T, ns), dtype=torch.float32, device=q.device)
         sp = _seg_array(segs)
         keep.append(sp)
         structs.append(_lib.UcAttendCall(q.data_ptr(), hq, T, C.addressof(sp), ns, out.data_ptr(), lse.data_ptr(),

@@ -782,13 +782,26 @@ double tile_bytes_host(const uc_segment* s) {
   return groups_per_tile(s->bits) * (2.0 * 32 * 128 * s->bits / 8 + 1024);
 }
 
-// Stored bytes one (sequence, KV head) of a call streams (longest sequence).
-double call_cost(const uc_segment* const* segs, int nseg) {
+// What a tile costs, for sharing a call's tiles among its items. One n-tile
+// of query rows runs at bf16 and int4 rates near the memory's, so a tile
+// costs its bytes. With more n-tiles a launch is bound by its instructions:
+// a 32-key packed group takes about 3.3 times those of a 16-key bf16 block
+// (scores, softmax, values), so the four groups of an int4 tile cost as much
+// as 13 blocks and a 64-row bf16 tile four (4 x 16K tokens, 4 query tokens,
+// half of the bytes bf16: the busiest SM worked twice the mean when items
+// were equal in bytes).
+double tile_cost_host(const uc_segment* s, int mtiles) {
+  if (mtiles <= 1) return tile_bytes_host(s);
+  return is_quant(s->kind) ? 3.3 * groups_per_tile(s->bits) : 4.0;
+}
+
+// Cost of one (sequence, KV head) of a call (longest sequence).
+double call_cost(const uc_segment* const* segs, int nseg, int mtiles) {
   double total = 0.0;
   for (int s = 0; s < nseg; ++s) {
     int mx = 0;
     for (int b = 0; b < segs[s]->batch; ++b) mx = std::max(mx, segs[s]->n_kept_host[b]);
-    total += seg_tiles_host(segs[s], mx) * tile_bytes_host(segs[s]);
+    total += seg_tiles_host(segs[s], mx) * tile_cost_host(segs[s], mtiles);
   }
   return total;
 }
@@ -806,17 +819,17 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
   const int nbh = B * hkv;
   const int slots = slots_in > 0 ? slots_in : std::max(1, attend_ctas_per_sm(mtiles)) * num_sms();
   // heavy tiles of each segment (a packed segment's bf16 tail is a light
-  // item of its own) and their bytes
+  // item of its own) and their cost
   int htiles[UC_MAX_SEGMENTS];
-  double tbytes[UC_MAX_SEGMENTS], hbytes[UC_MAX_SEGMENTS];
+  double tcost[UC_MAX_SEGMENTS], hcost[UC_MAX_SEGMENTS];
   bool heavy[UC_MAX_SEGMENTS];
   for (int s = 0; s < nseg; ++s) {
     int mx = 0;
     for (int b = 0; b < B; ++b) mx = std::max(mx, segs[s]->n_kept_host[b]);
     const int nt = seg_tiles_host(segs[s], mx);
     htiles[s] = is_quant(segs[s]->kind) ? nt - ((mx % UC_GROUP) ? 1 : 0) : nt;
-    tbytes[s] = tile_bytes_host(segs[s]);
-    hbytes[s] = htiles[s] * tbytes[s];
+    tcost[s] = tile_cost_host(segs[s], mtiles);
+    hcost[s] = htiles[s] * tcost[s];
     heavy[s] = htiles[s] > 0;
   }
   // Heavy items per (b, kvh): the fewest (at least one per heavy segment, at
@@ -836,7 +849,7 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
       const bool q = is_quant(segs[s]->kind);
       if (heavy[s]) {
         ++nh;
-        tot += hbytes[s];
+        tot += hcost[s];
         nl += q ? 1 : 0;
       } else {
         nl += (q && htiles[s] > 0) ? 2 : 1;
@@ -879,7 +892,7 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
     }
     bool changed = false;
     for (int s = 0; s < nseg; ++s)
-      if (heavy[s] && H > 0 && hbytes[s] < 0.5 * tot / H) {
+      if (heavy[s] && H > 0 && hcost[s] < 0.5 * tot / H) {
         heavy[s] = false;
         changed = true;
       }
@@ -903,7 +916,7 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
     double worst = 0.0;
     for (int s = 0; s < nseg; ++s) {
       if (!heavy[s] || hc[s] >= htiles[s]) continue;
-      const double item = std::ceil((double)htiles[s] / hc[s]) * tbytes[s];
+      const double item = std::ceil((double)htiles[s] / hc[s]) * tcost[s];
       if (item > worst) {
         worst = item;
         pick = s;
@@ -1120,7 +1133,7 @@ void batch_items(const uc_attend_call* calls, int n_calls, int mtiles, int* ipb)
   const int slots = std::max(1, attend_ctas_per_sm(mtiles)) * num_sms();
   double cost[UC_MAX_CALLS], total = 0.0;
   for (int c = 0; c < n_calls; ++c) {
-    cost[c] = call_cost(calls[c].segs, calls[c].n_seg);
+    cost[c] = call_cost(calls[c].segs, calls[c].n_seg, mtiles);
     total += cost[c] * calls[c].segs[0]->batch * calls[c].segs[0]->n_kv_heads;
   }
   for (int c = 0; c < n_calls; ++c) {

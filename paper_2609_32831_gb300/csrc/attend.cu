@@ -6,7 +6,7 @@
 // Design (GB300, HBM-bound): persistent CTAs walk a static list of work
 // items; an item is one chunk of 64-token tiles of one segment of one
 // (sequence, KV head). Per CTA one producer warp streams tiles into a
-// 2- or 3-stage shared-memory ring (TMA 2D loads with 128-byte swizzle for bf16
+// 2-stage shared-memory ring (TMA 2D loads with 128-byte swizzle for bf16
 // rows, 1D bulk copies for packed codes and parameters) and four consumer
 // warps compute with mma.sync m16n8k16:
 //   bf16 rows:  S = Q K^T in bf16 (exact products), P split into bf16 hi + lo
@@ -19,6 +19,7 @@
 // Each item leaves an unnormalised partial (O, m, l); the last CTA to finish
 // a (sequence, KV head) merges its items by log-sum-exp, writes O, lse and
 // the per-segment probability mass, and re-arms the counter.
+#include <atomic>
 #include <mutex>
 
 #include "common.cuh"
@@ -27,13 +28,12 @@
 namespace uc {
 
 constexpr int kTileTok = 64;
-constexpr int kMaxStages = 3;
-// Ring stages: one query n-tile runs 3 CTAs per SM with 2 stages each (the
-// register budget is 128), larger calls 1 CTA per SM with 3.
+constexpr int kStages = 2;  // ring slots of a CTA
+// CTAs per SM the register budget is set for: 3 for one query n-tile (128
+// registers), 2 for more (200; the query buffers of up to seven n-tiles leave
+// room for two CTAs' shared memory, eight run one).
 template <int NTW>
-__host__ __device__ constexpr int stages_for() { return NTW == 1 ? 2 : 3; }
-template <int NTW>
-__host__ __device__ constexpr int ctas_for() { return NTW == 1 ? 3 : 1; }
+__host__ __device__ constexpr int ctas_for() { return NTW == 1 ? 3 : 2; }
 constexpr int kConsumers = 4;
 constexpr int kAttnThreads = 32 * (kConsumers + 1);
 constexpr int kSlotBytes = 32768;
@@ -55,42 +55,38 @@ constexpr int kItemQ = 2;  // items handed from the producer to the consumers ah
 struct AttnSmem {
   float merge_w[kMaxItemsPerBh * 8];  // per (item, row of an 8-row block): m, then weight
   float merge_l[kMaxItemsPerBh * 8];
-  uint64_t full[kMaxStages];
-  uint64_t empty[kMaxStages];
+  uint64_t full[kStages];
+  uint64_t empty[kStages];
   uint64_t item_full[kItemQ];   // producer -> consumers: item position and its query rows
   uint64_t item_empty[kItemQ];  // consumers -> producer: the entry is free again
   int item_pos[kItemQ];         // processing position, -1: no more work
   int n_pending;                    // (sequence, KV head) merges this CTA owes
   int pending[kMaxPendingMerges];
-  alignas(1024) uint8_t slot[kMaxStages][kSlotBytes];  // only stages_for<NTW>() are allocated
+  alignas(1024) uint8_t slot[kStages][kSlotBytes];
 };
 
 // Query fragments of the current item live in shared memory (2 KB per
 // n-tile of 8 query rows): for one n-tile in the merge staging arrays, which
 // are idle while an item runs (merges happen between items), keeping three
-// CTAs per SM; for up to eight n-tiles after the ring.
-template <int NTW>
-__host__ __device__ constexpr int qfrag_tiles() { return NTW == 1 ? 0 : 8; }
+// CTAs per SM; for more n-tiles after the ring. The bf16 query rows of an
+// item as the producer copies them (g * T rows) take as much again per entry
+// of the item queue.
+constexpr int kQTileBytes = 2048;
+static_assert(kQTileBytes == 8 * kHeadDim * 2, "bf16 rows of an n-tile");
+__host__ __device__ constexpr int qfrag_tiles(int ntiles) { return ntiles <= 1 ? 0 : ntiles; }
 
-// bf16 query rows of one item as copied by the producer (g * T rows)
-template <int NTW>
-__host__ __device__ constexpr int qrow_bytes() { return NTW == 1 ? 8 * 256 : 64 * 256; }
-
-template <int NTW>
-__host__ __device__ constexpr size_t attend_smem_bytes() {
-  return offsetof(AttnSmem, slot) + (size_t)stages_for<NTW>() * kSlotBytes + (size_t)qfrag_tiles<NTW>() * 2048 +
-         (size_t)kItemQ * qrow_bytes<NTW>() + 1024;
+constexpr size_t attend_smem_bytes(int ntiles) {
+  return offsetof(AttnSmem, slot) + (size_t)kStages * kSlotBytes +
+         (size_t)(qfrag_tiles(ntiles) + kItemQ * ntiles) * kQTileBytes + 1024;
 }
 
-// Shared-memory regions after the ring: query fragments (NTW > 1), then the
-// producer's query-row buffers.
-template <int NTW>
+// Shared-memory regions after the ring: query fragments (more than one
+// n-tile), then the producer's query-row buffers.
 __device__ __forceinline__ uint8_t* after_ring(AttnSmem& sm) {
-  return reinterpret_cast<uint8_t*>(sm.slot) + stages_for<NTW>() * kSlotBytes;
+  return reinterpret_cast<uint8_t*>(sm.slot) + kStages * kSlotBytes;
 }
-template <int NTW>
-__device__ __forceinline__ uint8_t* qrows_buf(AttnSmem& sm, int k) {
-  return after_ring<NTW>(sm) + qfrag_tiles<NTW>() * 2048 + k * qrow_bytes<NTW>();
+__device__ __forceinline__ uint8_t* qrows_buf(AttnSmem& sm, int k, int ntiles) {
+  return after_ring(sm) + (qfrag_tiles(ntiles) + k * ntiles) * kQTileBytes;
 }
 
 __host__ __device__ size_t attend_part_floats(int ntiles) { return (size_t)ntiles * 8 * (kHeadDim + 2); }
@@ -248,7 +244,7 @@ __device__ __forceinline__ uint2 lds64(uint32_t a) {
 // contiguous) along with it.
 template <int NTW, class W>
 __device__ void produce(const W& w, AttnSmem& sm) {
-  constexpr int ST = stages_for<NTW>();
+  constexpr int ST = kStages;
   const AttnParams& p0 = w.call(0);
   int* sched = p0.sched;
   uint32_t seq = 0;
@@ -275,7 +271,7 @@ __device__ void produce(const W& w, AttnSmem& sm) {
     const __nv_bfloat16* qsrc =
         p.q + (size_t)(ii.b * p.n_q_heads + (ii.bh % p.n_kv_heads) * p.group) * p.n_qtok * kHeadDim;
     mbar_arrive_expect_tx(&sm.item_full[k], qbytes);
-    bulk_load(qrows_buf<NTW>(sm, k), qsrc, qbytes, &sm.item_full[k]);
+    bulk_load(qrows_buf(sm, k, p.mtiles), qsrc, qbytes, &sm.item_full[k]);
     for (int t = ii.tb; t < ii.te; ++t, ++seq) {
       const int slot = seq % ST;
       if (seq >= ST && !mbar_wait(&sm.empty[slot], ((seq / ST) - 1) & 1, p.status, 10, p.wait_ns)) {
@@ -771,10 +767,9 @@ __device__ __forceinline__ void group_quant(WarpState<NTW>& st, uint32_t qsm,
     }
 #pragma unroll
     for (int blk = 0; blk < 2; ++blk) {
-      x[blk][nt][0] = ((sa[blk][nt][0] + sl[blk][nt][0]) + bt0) * scale;
-      x[blk][nt][1] = ((sa[blk][nt][1] + sl[blk][nt][1]) + bt1) * scale;
-      x[blk][nt][2] = ((sa[blk][nt][2] + sl[blk][nt][2]) + bt0) * scale;
-      x[blk][nt][3] = ((sa[blk][nt][3] + sl[blk][nt][3]) + bt1) * scale;
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        x[blk][nt][e] = ((sa[blk][nt][e] + sl[blk][nt][e]) + (e & 1 ? bt1 : bt0)) * scale;
     }
   }
 
@@ -896,22 +891,25 @@ __device__ __forceinline__ void zero_v_rows(uint8_t* slot, int u, int valid) {
 // Weights of the 8-row block r0: m_of(i, rr), l_of(i, rr) read item i's
 // values; the normalised weights go to merge_l[i * 8 + rr]; lse and the
 // per-segment mass are written for the block's nr valid rows.
-template <class MOf, class LOf>
+//
+// PARTS threads per query row (128 / PARTS rows at once); wts[i * stride + rr].
+template <int PARTS = 16, class MOf, class LOf>
 __device__ __forceinline__ void merge_weights(const AttnParams& p, float* wts, int b, int kvh, int r0,
-                                              int nr, MOf m_of, LOf l_of, bool outputs = true) {
+                                              int nr, MOf m_of, LOf l_of, bool outputs = true, int stride = 8) {
   const int tid = threadIdx.x;
   const int I = p.items_per_bh;
-  const int rr = tid >> 4, part = tid & 15;
+  const int rr = tid / PARTS, part = tid % PARTS;
+  const int i0 = PARTS == 16 || rr < stride ? part : I;  // threads past the padded rows have no items
   float M = kNegInf;
-  for (int i = part; i < I; i += 16) M = fmaxf(M, m_of(i, rr));
+  for (int i = i0; i < I; i += PARTS) M = fmaxf(M, m_of(i, rr));
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  for (int o = PARTS / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
   const float Mu = (M == kNegInf) ? 0.f : M;
   float L = 0.f;
   float Ls[UC_MAX_SEGMENTS];
 #pragma unroll
   for (int q = 0; q < UC_MAX_SEGMENTS; ++q) Ls[q] = 0.f;
-  for (int i = part; i < I; i += 16) {
+  for (int i = i0; i < I; i += PARTS) {
     int sg = 0;
 #pragma unroll
     for (int q = 1; q < UC_MAX_SEGMENTS; ++q) sg += (q < p.nseg && i >= p.seg[q].chunk_begin) ? 1 : 0;
@@ -922,17 +920,17 @@ __device__ __forceinline__ void merge_weights(const AttnParams& p, float* wts, i
 #pragma unroll
     for (int q = 0; q < UC_MAX_SEGMENTS; ++q)
       if (q == sg) Ls[q] += lw;
-    wts[i * 8 + rr] = w;  // unnormalised weight
+    wts[i * stride + rr] = w;  // unnormalised weight
   }
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) {
+  for (int o = PARTS / 2; o > 0; o >>= 1) {
     L += __shfl_xor_sync(0xffffffffu, L, o);
 #pragma unroll
     for (int q = 0; q < UC_MAX_SEGMENTS; ++q)
       if (q < p.nseg) Ls[q] += __shfl_xor_sync(0xffffffffu, Ls[q], o);
   }
   const float inv = (L > 0.f) ? 1.f / L : 0.f;
-  for (int i = part; i < I; i += 16) wts[i * 8 + rr] *= inv;
+  for (int i = i0; i < I; i += PARTS) wts[i * stride + rr] *= inv;
   if (outputs && part == 0 && rr < nr) {
     const int r = r0 + rr;
     const int hl = r / p.n_qtok, t = r % p.n_qtok;
@@ -963,7 +961,7 @@ __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t*
   const int rows_pad = 8 * p.mtiles;
   const int I = p.items_per_bh;
   const float* base = p.part + (size_t)bh * I * pf;
-  constexpr int ST = stages_for<NTW>();
+  constexpr int ST = kStages;
 
   // ---- one n-tile, few items: whole partials through the ring at once
   constexpr int kWholeFloats = 8 * (kHeadDim + 2);              // O, m, l of one n-tile
@@ -1010,6 +1008,71 @@ __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t*
 
   constexpr int kPerSlot = kSlotBytes / (8 * kHeadDim * 4);  // 8-row blocks of O per ring slot
   const int nb = (I + kPerSlot - 1) / kPerSlot;
+
+  // ---- several n-tiles after the CTA's last item: the weights of all rows
+  // at once (in the query buffers, idle by then), while the row blocks of O
+  // stream through the ring back to back. Block by block, each with its own
+  // loads, weights and first copies, the merge of 28 rows x 19 items held the
+  // launch for as long as its items: 4 x 16K tokens, 4 query tokens 65 us.
+  if constexpr (NTW > 1) {
+    if (seq != nullptr) {
+      float* wts = reinterpret_cast<float*>(after_ring(sm));  // [I][rows_pad] weights, then l
+      float* ls = wts + I * rows_pad;
+      const int total = nb * p.mtiles;
+      auto issue_all = [&](int n) {  // batch n: items of row block n / nb (thread 0)
+        const uint32_t sq = *seq + n;
+        uint64_t* bar = &sm.full[sq % ST];
+        const int i0 = (n % nb) * kPerSlot, cnt = min(kPerSlot, I - i0);
+        mbar_arrive_expect_tx(bar, (uint32_t)cnt * 8 * kHeadDim * 4);
+        for (int k = 0; k < cnt; ++k)
+          bulk_load(sm.slot[sq % ST] + k * 8 * kHeadDim * 4, base + (i0 + k) * pf + (size_t)(n / nb) * 8 * kHeadDim,
+                    8 * kHeadDim * 4, bar);
+      };
+      if (tid == 0) {
+        fence_proxy_async_global();
+        for (int n = 0; n < min(ST, total); ++n) issue_all(n);
+      }
+      for (int x = tid; x < I * rows_pad; x += 128) {
+        const int i = x / rows_pad, r = x % rows_pad;
+        const float* ml = base + i * pf + rows_pad * kHeadDim + r;
+        wts[x] = r < p.rows ? __ldcg(ml) : kNegInf;
+        ls[x] = r < p.rows ? __ldcg(ml + rows_pad) : 0.f;
+      }
+      consumer_sync();
+      auto m_of = [&](int i, int r) { return wts[i * rows_pad + r]; };
+      auto l_of = [&](int i, int r) { return ls[i * rows_pad + r]; };
+      if (p.mtiles <= 2)
+        merge_weights<8>(p, wts, b, kvh, 0, p.rows, m_of, l_of, true, rows_pad);
+      else if (p.mtiles <= 4)
+        merge_weights<4>(p, wts, b, kvh, 0, p.rows, m_of, l_of, true, rows_pad);
+      else
+        merge_weights<2>(p, wts, b, kvh, 0, p.rows, m_of, l_of, true, rows_pad);
+      consumer_sync();
+      float acc[8];
+      for (int n = 0; n < total; ++n) {
+        const int r0 = n / nb * 8, i0 = (n % nb) * kPerSlot, cnt = min(kPerSlot, I - i0);
+        if (i0 == 0) {
+#pragma unroll
+          for (int rr = 0; rr < 8; ++rr) acc[rr] = 0.f;
+        }
+        const uint32_t sq = *seq + n;
+        const bool ok = mbar_wait(&sm.full[sq % ST], (sq / ST) & 1, p.status, 14, p.wait_ns);
+        const float* buf = reinterpret_cast<const float*>(sm.slot[sq % ST]);
+        if (ok) {
+          for (int k = 0; k < cnt; ++k)
+#pragma unroll
+            for (int rr = 0; rr < 8; ++rr)
+              acc[rr] += wts[(i0 + k) * rows_pad + r0 + rr] * buf[(k * 8 + rr) * kHeadDim + tid];
+        }
+        consumer_sync();  // the slot is read: refill it
+        if (tid == 0 && n + ST < total) issue_all(n + ST);
+        if (i0 + kPerSlot >= I) merge_store(p, b, kvh, r0, min(8, p.rows - r0), acc);
+      }
+      *seq += total;
+      consumer_sync();
+      return;
+    }
+  }
   auto issue = [&](int r0, int j) {  // batch j of the 8-row block r0 (thread 0)
     const uint32_t sq = *seq + j;
     uint64_t* bar = &sm.full[sq % ST];
@@ -1303,8 +1366,8 @@ __device__ __forceinline__ void run_item(const AttnParams& p, AttnSmem& sm, cons
                                          uint32_t& seq, bool& aborted, int NG, int KS, int grp, int ks) {
   const int lane = threadIdx.x & 31;
   uint32_t* qf = NTW == 1 ? reinterpret_cast<uint32_t*>(sm.merge_w)
-                          : reinterpret_cast<uint32_t*>(after_ring<NTW>(sm));
-  store_q<BITS == 16>(p, qf, qrows_buf<NTW>(sm, k));
+                          : reinterpret_cast<uint32_t*>(after_ring(sm));
+  store_q<BITS == 16>(p, qf, qrows_buf(sm, k, p.mtiles));
   consumer_sync();
   if (lane == 0) mbar_arrive(&sm.item_empty[k]);  // the query rows are no longer needed
   const uint32_t qs = smem_u32(qf) + grp * NTW * 2048;
@@ -1312,7 +1375,7 @@ __device__ __forceinline__ void run_item(const AttnParams& p, AttnSmem& sm, cons
   state_init<NTW>(st);
   int last_slot = -1;
   for (int t = ii.tb; t < ii.te; ++t, ++seq) {
-    constexpr int ST = stages_for<NTW>();
+    constexpr int ST = kStages;
     const int slot = seq % ST;
     if (!aborted && !mbar_wait(&sm.full[slot], (seq / ST) & 1, p.status, 11, p.wait_ns)) aborted = true;
     const uint32_t sbase = smem_u32(sm.slot[slot]);
@@ -1446,7 +1509,7 @@ __global__ void __launch_bounds__(kAttnThreads, ctas_for<NTW>()) attend_kernel(c
   griddep_launch_dependents();
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < stages_for<NTW>(); ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(&sm.full[s], 1);
       mbar_init(&sm.empty[s], kConsumers);
     }
@@ -1477,42 +1540,40 @@ __global__ void __launch_bounds__(kAttnThreads, ctas_for<NTW>()) attend_kernel(c
 static void attend_setup_once() {
   static std::once_flag once;
   std::call_once(once, [] {
-    cudaFuncSetAttribute(attend_kernel<1, AttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)attend_smem_bytes<1>());
-    cudaFuncSetAttribute(attend_kernel<2, AttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)attend_smem_bytes<2>());
-    cudaFuncSetAttribute(attend_kernel<1, MultiAttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)attend_smem_bytes<1>());
-    cudaFuncSetAttribute(attend_kernel<2, MultiAttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)attend_smem_bytes<2>());
+    const int one = (int)attend_smem_bytes(1), most = (int)attend_smem_bytes(8);
+    cudaFuncSetAttribute(attend_kernel<1, AttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize, one);
+    cudaFuncSetAttribute(attend_kernel<2, AttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(attend_kernel<1, MultiAttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize, one);
+    cudaFuncSetAttribute(attend_kernel<2, MultiAttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   });
 }
 
-// Resident CTAs per SM of the instantiation used for `ntiles` n-tiles.
+// Resident CTAs per SM of a call with `ntiles` n-tiles (1 .. 8).
 int attend_ctas_per_sm(int ntiles) {
-  static int cached[2] = {0, 0};
-  const int w = ntiles <= 1 ? 0 : 1;
-  if (cached[w] == 0) {
+  static std::atomic<int> cached[9];
+  int n = cached[ntiles].load(std::memory_order_relaxed);
+  if (n == 0) {
     attend_setup_once();
-    int n = 0;
-    if (w == 0)
+    if (ntiles <= 1)
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, attend_kernel<1, AttnParams>, kAttnThreads,
-                                                    attend_smem_bytes<1>());
+                                                    attend_smem_bytes(1));
     else
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, attend_kernel<2, AttnParams>, kAttnThreads,
-                                                    attend_smem_bytes<2>());
-    cached[w] = n > 0 ? n : 1;
+                                                    attend_smem_bytes(ntiles));
+    n = n > 0 ? n : 1;
+    cached[ntiles].store(n, std::memory_order_relaxed);
   }
-  return cached[w];
+  return n;
 }
 
 void launch_attend(const AttnParams& p, int grid, cudaStream_t st) {
   attend_setup_once();
   const bool pdl = pdl_enabled();
+  const size_t smem = attend_smem_bytes(p.mtiles);
   if (p.mtiles <= 1)
-    launch_maybe_pdl(pdl, attend_kernel<1, AttnParams>, grid, kAttnThreads, attend_smem_bytes<1>(), st, p);
+    launch_maybe_pdl(pdl, attend_kernel<1, AttnParams>, grid, kAttnThreads, smem, st, p);
   else
-    launch_maybe_pdl(pdl, attend_kernel<2, AttnParams>, grid, kAttnThreads, attend_smem_bytes<2>(), st, p);
+    launch_maybe_pdl(pdl, attend_kernel<2, AttnParams>, grid, kAttnThreads, smem, st, p);
   count_launch();
   if (p.defer_merge) {
     // always launched programmatically: its CTAs take the SM slots the
@@ -1525,10 +1586,11 @@ void launch_attend(const AttnParams& p, int grid, cudaStream_t st) {
 
 void launch_attend_multi(const MultiAttnParams& m, int grid, cudaStream_t st) {
   attend_setup_once();
+  const size_t smem = attend_smem_bytes(m.call[0].mtiles);
   if (m.call[0].mtiles <= 1)
-    attend_kernel<1, MultiAttnParams><<<grid, kAttnThreads, attend_smem_bytes<1>(), st>>>(m);
+    attend_kernel<1, MultiAttnParams><<<grid, kAttnThreads, smem, st>>>(m);
   else
-    attend_kernel<2, MultiAttnParams><<<grid, kAttnThreads, attend_smem_bytes<2>(), st>>>(m);
+    attend_kernel<2, MultiAttnParams><<<grid, kAttnThreads, smem, st>>>(m);
   count_launch();
 }
 

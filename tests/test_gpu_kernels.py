@@ -321,6 +321,27 @@ def test_attend_parity(mix, T):
     assert (np.abs(host(mass) - rm) <= 2 * bound[..., None]).all()
 
 
+@pytest.mark.parametrize("hq,T", [(28, 3), (28, 4), (28, 6), (32, 8), (24, 8), (8, 8)])
+def test_attend_query_tiles_many_items(hq, T):
+    """2 to 8 query n-tiles with enough items per (b, kvh) that their merge
+    takes several batches per row block (two sequences: up to 32 items)."""
+    B, hkv = 2, 4
+    sizes, kinds = [1500, 9000, 4000], ["full", "quant", "evict_quant"]
+    gsegs, osegs = _build_mix(hq + T, B, hkv, sizes, kinds, [1500, 9000, [2000, 1333]], [16, 4, 2])
+    items = uc.attend_plan(gsegs, hq, T)["items_per_bh"]
+    assert items > 8, items
+    q = synth.make_q(T + hq, B, hq, T)
+    rO, rl, rm = oattn.attend(q, osegs, hkv)
+    bound = _packed.logit_error_bound(q, osegs, hkv, [False, True, True])
+    ws = uc.Workspace(DEV)
+    for _ in range(2):
+        O, lse, mass = uc.attend(dev(q), gsegs, ws=ws)
+        assert _packed.attention_error(host(O), rO) <= _packed.ATTN_RTOL
+        assert (np.abs(host(lse) - rl) <= bound).all()
+        assert (np.abs(host(mass) - rm) <= 2 * bound[..., None]).all()
+    assert ws.status() == 0
+
+
 LONG_MIXES = {
     # few (sequence, KV head) pairs and long segments: more than 32 items per
     # pair, merged by the separate merge kernel

@@ -53,7 +53,7 @@ constexpr int kMaxPendingMerges = 64;
 constexpr int kItemQ = 2;  // items handed from the producer to the consumers ahead
 
 struct AttnSmem {
-  float merge_w[kMaxItemsPerBh * 8];  // per (item, row of an 8-row block): m, then weight
+  alignas(16) float merge_w[kMaxItemsPerBh * 8];  // per (item, row of an 8-row block): m, then weight
   float merge_l[kMaxItemsPerBh * 8];
   uint64_t full[kStages];
   uint64_t empty[kStages];
@@ -876,32 +876,26 @@ __device__ __forceinline__ void zero_v_rows(uint8_t* slot, int u, int valid) {
 
 // Partial layout per item: [rows_pad][128] O (unnormalised), [rows_pad] m,
 // [rows_pad] l, rows_pad = 8 * (number of n-tiles).
-//
-// The merge runs on the 128 consumer threads of the CTA that finished the
-// last item of a (sequence, KV head), per block of 8 query rows: the
-// log-sum-exp weights of every item (16 threads per row), then each thread
-// (one output channel) sums the weighted partial outputs. After the CTA's
-// last item the ring is idle (`seq` given) and the partials come through it
-// by bulk copies continuing the consumers' tile sequence: for one n-tile and
-// at most seven items per stage, the whole partials (O, m, l) in one round
-// trip; otherwise (m, l) by loads and the 4 KB row blocks of O eight items
-// per slot, copies issued ahead. Without `seq` (a merge between items) each
-// thread loads the partial outputs, eight items at a time.
-//
-// Weights of the 8-row block r0: m_of(i, rr), l_of(i, rr) read item i's
-// values; the normalised weights go to merge_l[i * 8 + rr]; lse and the
-// per-segment mass are written for the block's nr valid rows.
-//
-// PARTS threads per query row (128 / PARTS rows at once); wts[i * stride + rr].
-template <int PARTS = 16, class MOf, class LOf>
-__device__ __forceinline__ void merge_weights(const AttnParams& p, float* wts, int b, int kvh, int r0,
-                                              int nr, MOf m_of, LOf l_of, bool outputs = true, int stride = 8) {
-  const int tid = threadIdx.x;
+
+// Output row of query row r of a KV head (r = head * T + token).
+__device__ __forceinline__ size_t out_row(const AttnParams& p, int b, int kvh, int r) {
+  const int hl = p.n_qtok == 1 ? r : r / p.n_qtok, t = p.n_qtok == 1 ? 0 : r % p.n_qtok;
+  return (size_t)(b * p.n_q_heads + kvh * p.group + hl) * p.n_qtok + t;
+}
+
+// Log-sum-exp weights of query rows r0 .. r0 + nr - 1 over every item:
+// ml[i * stride + rr] holds item i's m, ll[...] its l; the normalised weights
+// replace m. PARTS threads per row (128 / PARTS rows at once, stride of them
+// real); lse and the per-segment mass are written for the valid rows.
+template <int PARTS>
+__device__ __forceinline__ void merge_weights(const AttnParams& p, float* ml, const float* ll, int stride, int b,
+                                              int kvh, int r0, int nr, bool outputs = true) {
   const int I = p.items_per_bh;
-  const int rr = tid / PARTS, part = tid % PARTS;
+  const int rr = threadIdx.x / PARTS, part = threadIdx.x % PARTS;
   const int i0 = PARTS == 16 || rr < stride ? part : I;  // threads past the padded rows have no items
+  const bool mass = outputs && p.mass != nullptr;
   float M = kNegInf;
-  for (int i = i0; i < I; i += PARTS) M = fmaxf(M, m_of(i, rr));
+  for (int i = i0; i < I; i += PARTS) M = fmaxf(M, ml[i * stride + rr]);
 #pragma unroll
   for (int o = PARTS / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
   const float Mu = (M == kNegInf) ? 0.f : M;
@@ -910,245 +904,139 @@ __device__ __forceinline__ void merge_weights(const AttnParams& p, float* wts, i
 #pragma unroll
   for (int q = 0; q < UC_MAX_SEGMENTS; ++q) Ls[q] = 0.f;
   for (int i = i0; i < I; i += PARTS) {
-    int sg = 0;
-#pragma unroll
-    for (int q = 1; q < UC_MAX_SEGMENTS; ++q) sg += (q < p.nseg && i >= p.seg[q].chunk_begin) ? 1 : 0;
-    const float mi = m_of(i, rr);
+    const float mi = ml[i * stride + rr];
     const float w = (mi == kNegInf) ? 0.f : exp2f(mi - Mu);
-    const float lw = l_of(i, rr) * w;
+    const float lw = ll[i * stride + rr] * w;
     L += lw;
+    if (mass) {
+      int sg = 0;
 #pragma unroll
-    for (int q = 0; q < UC_MAX_SEGMENTS; ++q)
-      if (q == sg) Ls[q] += lw;
-    wts[i * stride + rr] = w;  // unnormalised weight
+      for (int q = 1; q < UC_MAX_SEGMENTS; ++q) sg += (q < p.nseg && i >= p.seg[q].chunk_begin) ? 1 : 0;
+#pragma unroll
+      for (int q = 0; q < UC_MAX_SEGMENTS; ++q)
+        if (q == sg) Ls[q] += lw;
+    }
+    ml[i * stride + rr] = w;  // unnormalised weight (this thread's own entry)
   }
 #pragma unroll
-  for (int o = PARTS / 2; o > 0; o >>= 1) {
-    L += __shfl_xor_sync(0xffffffffu, L, o);
-#pragma unroll
-    for (int q = 0; q < UC_MAX_SEGMENTS; ++q)
-      if (q < p.nseg) Ls[q] += __shfl_xor_sync(0xffffffffu, Ls[q], o);
-  }
+  for (int o = PARTS / 2; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
   const float inv = (L > 0.f) ? 1.f / L : 0.f;
-  for (int i = i0; i < I; i += PARTS) wts[i * stride + rr] *= inv;
+  for (int i = i0; i < I; i += PARTS) ml[i * stride + rr] *= inv;
+  if (mass) {
+#pragma unroll
+    for (int q = 0; q < UC_MAX_SEGMENTS; ++q)
+      if (q < p.nseg)
+#pragma unroll
+        for (int o = PARTS / 2; o > 0; o >>= 1) Ls[q] += __shfl_xor_sync(0xffffffffu, Ls[q], o);
+  }
   if (outputs && part == 0 && rr < nr) {
-    const int r = r0 + rr;
-    const int hl = r / p.n_qtok, t = r % p.n_qtok;
-    const size_t orow = ((size_t)(b * p.n_q_heads + kvh * p.group + hl) * p.n_qtok + t);
+    const size_t orow = out_row(p, b, kvh, r0 + rr);
     if (p.lse) p.lse[orow] = (L > 0.f) ? (M + log2f(L)) * kLn2 : kNegInf;
-    if (p.mass)
+    if (mass)
       for (int q = 0; q < p.nseg; ++q) p.mass[orow * p.nseg + q] = Ls[q] * inv;
   }
 }
 
-__device__ __forceinline__ void merge_store(const AttnParams& p, int b, int kvh, int r0, int nr,
-                                            const float (&acc)[8]) {
-#pragma unroll
-  for (int rr = 0; rr < 8; ++rr) {
-    if (rr >= nr) continue;
-    const int r = r0 + rr;
-    const int hl = r / p.n_qtok, t = r % p.n_qtok;
-    const size_t orow = ((size_t)(b * p.n_q_heads + kvh * p.group + hl) * p.n_qtok + t);
-    p.out[orow * kHeadDim + threadIdx.x] = __float2bfloat16_rn(acc[rr]);
-  }
-}
-
+// The merge runs on the 128 consumer threads of the CTA that finished the
+// last item of a (sequence, KV head): the weights of every item and row, then
+// per 8-row block the weighted sums of the items' O, four channels of two
+// rows per thread (16-byte shared-memory reads; one 4-byte read per value
+// with its weight held the merge of 13 items for 5 us). After the CTA's last
+// item the ring is idle (`seq` given): the row blocks of O stream through it
+// back to back, eight items per slot, by bulk copies continuing the consumers'
+// tile sequence, the first ones in flight while the weights are formed.
+// Without `seq` (a merge between items) the threads load them.
 template <int NTW>
 __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t* seq) {
-  const int tid = threadIdx.x;  // 0..127 = channel
+  const int tid = threadIdx.x;
   const int b = bh / p.n_kv_heads, kvh = bh % p.n_kv_heads;
   const size_t pf = attend_part_floats(p.mtiles);
   const int rows_pad = 8 * p.mtiles;
   const int I = p.items_per_bh;
   const float* base = p.part + (size_t)bh * I * pf;
-  constexpr int ST = kStages;
-
-  // ---- one n-tile, few items: whole partials through the ring at once
-  constexpr int kWholeFloats = 8 * (kHeadDim + 2);              // O, m, l of one n-tile
-  constexpr int kWhole = kSlotBytes / (kWholeFloats * 4);       // items per slot (7)
-  static_assert(NTW != 1 || kWhole * ST == kWholeMergeItems, "planner's whole-merge item limit");
-  if (seq != nullptr && p.mtiles == 1 && I <= kWhole * ST) {
-    const int nbw = (I + kWhole - 1) / kWhole;
-    if (tid == 0) {
-      // the partials were written by other CTAs (generic proxy) and acquired
-      // at GPU scope; order that acquire before the copy engine's reads
-      fence_proxy_async_global();
-      for (int j = 0; j < nbw; ++j) {
-        const uint32_t sq = *seq + j;
-        uint64_t* bar = &sm.full[sq % ST];
-        const int i0 = j * kWhole, cnt = min(kWhole, I - i0);
-        mbar_arrive_expect_tx(bar, (uint32_t)(cnt * kWholeFloats * 4));
-        for (int k = 0; k < cnt; ++k)
-          bulk_load(sm.slot[sq % ST] + k * kWholeFloats * 4, base + (i0 + k) * pf, kWholeFloats * 4, bar);
-      }
-    }
-    for (int j = 0; j < nbw; ++j) {
-      const uint32_t sq = *seq + j;
-      mbar_wait(&sm.full[sq % ST], (sq / ST) & 1, p.status, 14, p.wait_ns);
-    }
-    auto item = [&](int i) {
-      return reinterpret_cast<const float*>(sm.slot[(*seq + i / kWhole) % ST]) + (i % kWhole) * kWholeFloats;
-    };
-    merge_weights(p, sm.merge_l, b, kvh, 0, p.rows, [&](int i, int rr) { return item(i)[8 * kHeadDim + rr]; },
-                  [&](int i, int rr) { return item(i)[8 * kHeadDim + 8 + rr]; });
-    consumer_sync();
-    float acc[8];
-#pragma unroll
-    for (int rr = 0; rr < 8; ++rr) acc[rr] = 0.f;
-    for (int i = 0; i < I; ++i) {
-      const float* o = item(i);
-#pragma unroll
-      for (int rr = 0; rr < 8; ++rr) acc[rr] += sm.merge_l[i * 8 + rr] * o[rr * kHeadDim + tid];
-    }
-    merge_store(p, b, kvh, 0, p.rows, acc);
-    consumer_sync();  // the slots are read before any later copy into them
-    *seq += nbw;
-    return;
-  }
-
   constexpr int kPerSlot = kSlotBytes / (8 * kHeadDim * 4);  // 8-row blocks of O per ring slot
   const int nb = (I + kPerSlot - 1) / kPerSlot;
-
-  // ---- several n-tiles after the CTA's last item: the weights of all rows
-  // at once (in the query buffers, idle by then), while the row blocks of O
-  // stream through the ring back to back. Block by block, each with its own
-  // loads, weights and first copies, the merge of 28 rows x 19 items held the
-  // launch for as long as its items: 4 x 16K tokens, 4 query tokens 65 us.
-  if constexpr (NTW > 1) {
-    if (seq != nullptr) {
-      float* wts = reinterpret_cast<float*>(after_ring(sm));  // [I][rows_pad] weights, then l
-      float* ls = wts + I * rows_pad;
-      const int total = nb * p.mtiles;
-      auto issue_all = [&](int n) {  // batch n: items of row block n / nb (thread 0)
-        const uint32_t sq = *seq + n;
-        uint64_t* bar = &sm.full[sq % ST];
-        const int i0 = (n % nb) * kPerSlot, cnt = min(kPerSlot, I - i0);
-        mbar_arrive_expect_tx(bar, (uint32_t)cnt * 8 * kHeadDim * 4);
-        for (int k = 0; k < cnt; ++k)
-          bulk_load(sm.slot[sq % ST] + k * 8 * kHeadDim * 4, base + (i0 + k) * pf + (size_t)(n / nb) * 8 * kHeadDim,
-                    8 * kHeadDim * 4, bar);
-      };
-      if (tid == 0) {
-        fence_proxy_async_global();
-        for (int n = 0; n < min(ST, total); ++n) issue_all(n);
-      }
-      for (int x = tid; x < I * rows_pad; x += 128) {
-        const int i = x / rows_pad, r = x % rows_pad;
-        const float* ml = base + i * pf + rows_pad * kHeadDim + r;
-        wts[x] = r < p.rows ? __ldcg(ml) : kNegInf;
-        ls[x] = r < p.rows ? __ldcg(ml + rows_pad) : 0.f;
-      }
-      consumer_sync();
-      auto m_of = [&](int i, int r) { return wts[i * rows_pad + r]; };
-      auto l_of = [&](int i, int r) { return ls[i * rows_pad + r]; };
-      if (p.mtiles <= 2)
-        merge_weights<8>(p, wts, b, kvh, 0, p.rows, m_of, l_of, true, rows_pad);
-      else if (p.mtiles <= 4)
-        merge_weights<4>(p, wts, b, kvh, 0, p.rows, m_of, l_of, true, rows_pad);
-      else
-        merge_weights<2>(p, wts, b, kvh, 0, p.rows, m_of, l_of, true, rows_pad);
-      consumer_sync();
-      float acc[8];
-      for (int n = 0; n < total; ++n) {
-        const int r0 = n / nb * 8, i0 = (n % nb) * kPerSlot, cnt = min(kPerSlot, I - i0);
-        if (i0 == 0) {
-#pragma unroll
-          for (int rr = 0; rr < 8; ++rr) acc[rr] = 0.f;
-        }
-        const uint32_t sq = *seq + n;
-        const bool ok = mbar_wait(&sm.full[sq % ST], (sq / ST) & 1, p.status, 14, p.wait_ns);
-        const float* buf = reinterpret_cast<const float*>(sm.slot[sq % ST]);
-        if (ok) {
-          for (int k = 0; k < cnt; ++k)
-#pragma unroll
-            for (int rr = 0; rr < 8; ++rr)
-              acc[rr] += wts[(i0 + k) * rows_pad + r0 + rr] * buf[(k * 8 + rr) * kHeadDim + tid];
-        }
-        consumer_sync();  // the slot is read: refill it
-        if (tid == 0 && n + ST < total) issue_all(n + ST);
-        if (i0 + kPerSlot >= I) merge_store(p, b, kvh, r0, min(8, p.rows - r0), acc);
-      }
-      *seq += total;
-      consumer_sync();
-      return;
-    }
-  }
-  auto issue = [&](int r0, int j) {  // batch j of the 8-row block r0 (thread 0)
-    const uint32_t sq = *seq + j;
-    uint64_t* bar = &sm.full[sq % ST];
-    const int i0 = j * kPerSlot, cnt = min(kPerSlot, I - i0);
+  const int total = nb * p.mtiles;
+  auto issue = [&](int n) {  // batch n: eight items of row block n / nb (thread 0)
+    const uint32_t sq = *seq + n;
+    uint64_t* bar = &sm.full[sq % kStages];
+    const int i0 = (n % nb) * kPerSlot, cnt = min(kPerSlot, I - i0);
     mbar_arrive_expect_tx(bar, (uint32_t)cnt * 8 * kHeadDim * 4);
     for (int k = 0; k < cnt; ++k)
-      bulk_load(sm.slot[sq % ST] + k * 8 * kHeadDim * 4, base + (i0 + k) * pf + (size_t)r0 * kHeadDim,
+      bulk_load(sm.slot[sq % kStages] + k * 8 * kHeadDim * 4, base + (i0 + k) * pf + (size_t)(n / nb) * 8 * kHeadDim,
                 8 * kHeadDim * 4, bar);
   };
-  for (int r0 = 0; r0 < p.rows; r0 += 8) {
-    const int nr = min(8, p.rows - r0);
-    if (seq != nullptr && tid == 0) {
-      fence_proxy_async_global();
-      for (int j = 0; j < min(ST, nb); ++j) issue(r0, j);
-    }
-    for (int x = tid; x < I * 8; x += 128) {
-      const int i = x >> 3, rr = x & 7;
-      float m = kNegInf, l = 0.f;
-      if (rr < nr) {
-        m = __ldcg(base + i * pf + rows_pad * kHeadDim + r0 + rr);
-        l = __ldcg(base + i * pf + rows_pad * kHeadDim + rows_pad + r0 + rr);
-      }
-      sm.merge_w[x] = m;
-      sm.merge_l[x] = l;
-    }
-    consumer_sync();
-    merge_weights(p, sm.merge_l, b, kvh, r0, nr, [&](int i, int rr) { return sm.merge_w[i * 8 + rr]; },
-                  [&](int i, int rr) { return sm.merge_l[i * 8 + rr]; });
-    consumer_sync();
-    float acc[8];
-#pragma unroll
-    for (int rr = 0; rr < 8; ++rr) acc[rr] = 0.f;
-    int i = 0;
-    if (seq != nullptr) {
-      for (int j = 0; j < nb; ++j) {
-        const uint32_t sq = *seq + j;
-        const bool ok = mbar_wait(&sm.full[sq % ST], (sq / ST) & 1, p.status, 14, p.wait_ns);
-        const float* buf = reinterpret_cast<const float*>(sm.slot[sq % ST]);
-        const int i0 = j * kPerSlot, cnt = min(kPerSlot, I - i0);
-        if (ok) {
-          for (int k = 0; k < cnt; ++k)
-#pragma unroll
-            for (int rr = 0; rr < 8; ++rr)
-              acc[rr] += sm.merge_l[(i0 + k) * 8 + rr] * buf[(k * 8 + rr) * kHeadDim + tid];
-        }
-        consumer_sync();  // the slot is read: refill it
-        if (tid == 0 && j + ST < nb) issue(r0, j + ST);
-      }
-      *seq += nb;
-      i = I;
-    }
-    for (; i + 8 <= I; i += 8) {
-      // eight items' loads in flight at once
-      float v[8][8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const float* pi = base + (i + k) * pf + (size_t)r0 * kHeadDim + tid;
-#pragma unroll
-        for (int rr = 0; rr < 8; ++rr) v[k][rr] = (rr < nr) ? __ldcg(pi + rr * kHeadDim) : 0.f;
-      }
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-#pragma unroll
-        for (int rr = 0; rr < 8; ++rr) acc[rr] += sm.merge_l[(i + k) * 8 + rr] * v[k][rr];
-    }
-    for (; i < I; ++i) {
-      const float* pi = base + i * pf + (size_t)r0 * kHeadDim + tid;
-      float v[8];
-#pragma unroll
-      for (int rr = 0; rr < 8; ++rr) v[rr] = (rr < nr) ? __ldcg(pi + rr * kHeadDim) : 0.f;
-#pragma unroll
-      for (int rr = 0; rr < 8; ++rr) acc[rr] += sm.merge_l[i * 8 + rr] * v[rr];
-    }
-    merge_store(p, b, kvh, r0, nr, acc);
-    consumer_sync();
+  if (seq != nullptr && tid == 0) {
+    // the partials were written by other CTAs (generic proxy) and acquired
+    // at GPU scope; order that acquire before the copy engine's reads
+    fence_proxy_async_global();
+    for (int n = 0; n < min(kStages, total); ++n) issue(n);
   }
+  // rows whose weights are formed at once: every row when the query buffers
+  // behind the ring are idle too, else the 8 rows the merge arrays hold
+  const int set = NTW == 1 || seq == nullptr ? 8 : rows_pad;
+  float* wts = NTW == 1 || seq == nullptr ? sm.merge_w : reinterpret_cast<float*>(after_ring(sm));  // [I][set]
+  float* ls = NTW == 1 || seq == nullptr ? sm.merge_l : wts + I * set;
+  const int cq = tid & 31, rg = tid >> 5;  // channels 4 cq .. + 3, rows 2 rg, 2 rg + 1 of a block
+  for (int s0 = 0; s0 < p.rows; s0 += set) {
+    for (int x = tid; x < I * set; x += 128) {
+      const int i = x / set, r = s0 + x % set;
+      const float* mp = base + i * pf + rows_pad * kHeadDim + r;
+      wts[x] = r < p.rows ? __ldcg(mp) : kNegInf;
+      ls[x] = r < p.rows ? __ldcg(mp + rows_pad) : 0.f;
+    }
+    consumer_sync();
+    const int nr = min(set, p.rows - s0);
+    if (NTW == 1 || set == 8)
+      merge_weights<16>(p, wts, ls, 8, b, kvh, s0, nr);
+    else if (p.mtiles <= 2)
+      merge_weights<8>(p, wts, ls, set, b, kvh, s0, nr);
+    else if (p.mtiles <= 4)
+      merge_weights<4>(p, wts, ls, set, b, kvh, s0, nr);
+    else
+      merge_weights<2>(p, wts, ls, set, b, kvh, s0, nr);
+    consumer_sync();
+    for (int r0 = s0; r0 < min(s0 + set, p.rows); r0 += 8) {
+      float acc[2][4] = {};
+      auto add = [&](int i, float4 x0, float4 x1) {
+        const float2 w = *reinterpret_cast<const float2*>(&wts[i * set + (r0 - s0) + 2 * rg]);
+        acc[0][0] += w.x * x0.x; acc[0][1] += w.x * x0.y; acc[0][2] += w.x * x0.z; acc[0][3] += w.x * x0.w;
+        acc[1][0] += w.y * x1.x; acc[1][1] += w.y * x1.y; acc[1][2] += w.y * x1.z; acc[1][3] += w.y * x1.w;
+      };
+      if (seq != nullptr) {
+        for (int j = 0; j < nb; ++j) {
+          const int n = r0 / 8 * nb + j, i0 = j * kPerSlot, cnt = min(kPerSlot, I - i0);
+          const uint32_t sq = *seq + n;
+          const bool ok = mbar_wait(&sm.full[sq % kStages], (sq / kStages) & 1, p.status, 14, p.wait_ns);
+          const float4* buf = reinterpret_cast<const float4*>(sm.slot[sq % kStages]) + 2 * rg * 32 + cq;
+          if (ok) {
+#pragma unroll
+            for (int k = 0; k < kPerSlot; ++k)
+              if (k < cnt) add(i0 + k, buf[k * 256], buf[k * 256 + 32]);
+          }
+          if (n + kStages < total) {
+            consumer_sync();  // the slot is read: refill it
+            if (tid == 0) issue(n + kStages);
+          }
+        }
+      } else {
+#pragma unroll 4
+        for (int i = 0; i < I; ++i) {
+          const float4* pi = reinterpret_cast<const float4*>(base + i * pf + (size_t)(r0 + 2 * rg) * kHeadDim) + cq;
+          add(i, __ldcg(pi), __ldcg(pi + 32));
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = r0 + 2 * rg + h;
+        if (r < p.rows)
+          *reinterpret_cast<uint2*>(p.out + out_row(p, b, kvh, r) * kHeadDim + 4 * cq) =
+              make_uint2(pack_bf16(acc[h][0], acc[h][1]), pack_bf16(acc[h][2], acc[h][3]));
+      }
+    }
+    consumer_sync();  // the weights and the slots are read
+  }
+  if (seq != nullptr) *seq += total;
 }
 
 // Split-K merge as a kernel of its own, for calls with many items per
@@ -1160,7 +1048,7 @@ __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t*
 // partials and skips its own merges (`defer_merge`).
 constexpr int kMergeChunks = kHeadDim / 32;
 __global__ void __launch_bounds__(256) merge_partials_kernel(const __grid_constant__ AttnParams p) {
-  __shared__ float s_m[kMaxItemsPerBh * 8], s_w[kMaxItemsPerBh * 8];
+  __shared__ float s_m[kMaxItemsPerBh * 8], s_w[kMaxItemsPerBh * 8];  // m, then the weights; l
   __shared__ float s_red[8][8][33];
   griddep_wait();  // the attention launch whose partials this merges has completed
   griddep_launch_dependents();
@@ -1187,9 +1075,7 @@ __global__ void __launch_bounds__(256) merge_partials_kernel(const __grid_consta
     s_w[x] = l;
   }
   __syncthreads();
-  if (tid < 128)
-    merge_weights(p, s_w, b, kvh, r0, nr, [&](int i, int rr) { return s_m[i * 8 + rr]; },
-                  [&](int i, int rr) { return s_w[i * 8 + rr]; }, ch == 0);
+  if (tid < 128) merge_weights<16>(p, s_m, s_w, 8, b, kvh, r0, nr, ch == 0);
   __syncthreads();
   const int c = ch * 32 + lane;
   float v[kMaxItemsPerBh / 8][8];
@@ -1208,7 +1094,7 @@ __global__ void __launch_bounds__(256) merge_partials_kernel(const __grid_consta
     const int i = warp + 8 * k;
     if (i < I)
 #pragma unroll
-      for (int rr = 0; rr < 8; ++rr) acc[rr] += s_w[i * 8 + rr] * v[k][rr];
+      for (int rr = 0; rr < 8; ++rr) acc[rr] += s_m[i * 8 + rr] * v[k][rr];
   }
 #pragma unroll
   for (int rr = 0; rr < 8; ++rr) s_red[warp][rr][lane] = acc[rr];
@@ -1219,10 +1105,7 @@ __global__ void __launch_bounds__(256) merge_partials_kernel(const __grid_consta
 #pragma unroll
     for (int w = 0; w < 8; ++w) sum += s_red[w][rr][lane];
     if (rr < nr) {
-      const int r = r0 + rr;
-      const int hl = r / p.n_qtok, t = r % p.n_qtok;
-      const size_t orow = ((size_t)(b * p.n_q_heads + kvh * p.group + hl) * p.n_qtok + t);
-      p.out[orow * kHeadDim + c] = __float2bfloat16_rn(sum);
+      p.out[out_row(p, b, kvh, r0 + rr) * kHeadDim + c] = __float2bfloat16_rn(sum);
     }
   }
 }

@@ -506,6 +506,9 @@ size_t uc_attend_workspace_size(const uc_segment* const* segs, int32_t n_seg, in
  * head); heavy items split the long segments so that one round of them fills
  * the CTA slots, light items (the bf16 tails of packed segments, segments
  * under half an average heavy item) run last on CTAs that finished early.
+ * Short calls of one 8-row query tile run the same items as one cluster of
+ * CTAs per (sequence, KV head) (one for each heavy item, one for the light
+ * ones), merged inside the cluster.
  * slots: resident CTAs the launch may use; <= 0 asks this device's
  * occupancy (then a CUDA device must be current; otherwise the call touches
  * no device). Reads kind, bits, batch, n_kv_heads and n_kept_host of each
@@ -515,7 +518,7 @@ size_t uc_attend_workspace_size(const uc_segment* const* segs, int32_t n_seg, in
 typedef struct {
   int32_t items_per_bh;                 /* partials per (sequence, KV head), <= 64 */
   int32_t n_heavy, n_light;             /* heavy / light items per (sequence, KV head) */
-  int32_t grid;                         /* CTAs the launch starts */
+  int32_t grid;                         /* CTAs that walk the items as a work queue */
   int32_t merge_kernel;                 /* 1: the split-K merge runs as a kernel of its own */
   int32_t n_chunks[UC_MAX_SEGMENTS];    /* items of each segment */
   int32_t light[UC_MAX_SEGMENTS];       /* 1: every item of the segment is light */

@@ -759,6 +759,7 @@ namespace {
 
 struct AttnPlan {
   int items_per_bh, n_items, grid, mtiles, n_heavy, n_light;
+  int cluster;  // > 0: short call, a cluster of this many CTAs per (sequence, KV head)
   int chunk_begin[UC_MAX_SEGMENTS], n_chunks[UC_MAX_SEGMENTS];
   int16_t heavy_local[128], light_local[2 * UC_MAX_SEGMENTS];
 };
@@ -806,6 +807,58 @@ double call_cost(const uc_segment* const* segs, int nseg, int mtiles) {
   return total;
 }
 
+// Splits h items among the heavy segments so that the largest item is
+// smallest (one more item at a time to the segment whose items are largest);
+// hc: items per segment.
+void split_items(int h, int nseg, const bool* heavy, const int* htiles, const double* tcost, int* hc) {
+  int nh = 0;
+  for (int s = 0; s < nseg; ++s) {
+    hc[s] = heavy[s] ? 1 : 0;
+    nh += hc[s];
+  }
+  for (int left = h - nh; left > 0; --left) {
+    int pick = -1;
+    double worst = 0.0;
+    for (int s = 0; s < nseg; ++s) {
+      if (!heavy[s] || hc[s] >= htiles[s]) continue;
+      const double item = ((htiles[s] + hc[s] - 1) / hc[s]) * tcost[s];
+      if (item > worst) {
+        worst = item;
+        pick = s;
+      }
+    }
+    if (pick < 0) break;
+    ++hc[pick];
+  }
+}
+
+// Clusters of c CTAs that a GB300 runs at once with three CTAs per SM (the
+// occupancy query's answer: clusters stay inside a GPC, so not slots / c).
+constexpr int kClusterFit[kMaxClusterItems + 1] = {0,  456, 228, 148, 110, 87, 74, 59, 51,
+                                                   46, 43,  36,  36,  28,  26, 26, 21};
+constexpr int kClusterSlots = 456;
+
+// Time (us) of a tile on an SM that runs three CTAs (one 32K layer by the
+// planner at 3, 2 and 1 CTAs per SM: int2 75, 83, 124 us, int4 84, 93, 146).
+double tile_us(const uc_segment* s) { return !is_quant(s->kind) ? 0.75 : (s->bits == 4 ? 0.68 : 1.16); }
+
+// Time until a single-n-tile call's longest items (`item` us of SM time each,
+// h per pair) end: the CTAs of the busiest SM share it, and one or two of
+// them leave part of its rate unused.
+double items_us(double item, int h, int nbh) {
+  const int n = (h * nbh + 151) / 152;
+  return n * item * (n >= 3 ? 1.0 : (n == 2 ? 1.32 : 2.0));
+}
+// The queue's merge (arrival counter, partials through global memory) ends
+// later than the cluster's by about kQueueMergeUs; a cluster has no idle CTAs
+// to take light items and its CTAs lie less evenly over the SMs
+// (kClusterSpread). Cluster / queue, us on the device: 1K batch 1 7.8 / 9.4,
+// 8K batch 8 (int4, bf16) 14.3 / 16.5, and where the rule takes the queue 8K
+// batch 8 int2 20.6 / 19.8, 8K batch 1 int2 12.3 / 11.7, 32K batch 4 int2
+// 39.3 / 31.7.
+constexpr double kQueueMergeUs = 1.5, kClusterSpread = 1.15;
+constexpr double kLightItemUs = 0.4;  // SM time of a light item's start and end
+
 // nbh_launch: (sequence, KV head) pairs of every call sharing the launch.
 // forced_ipb > 0 fixes the items per (sequence, KV head) instead of
 // searching for the count that fills whole rounds of CTA slots.
@@ -823,6 +876,7 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
   int htiles[UC_MAX_SEGMENTS];
   double tcost[UC_MAX_SEGMENTS], hcost[UC_MAX_SEGMENTS];
   bool heavy[UC_MAX_SEGMENTS];
+  int longest = 0;
   for (int s = 0; s < nseg; ++s) {
     int mx = 0;
     for (int b = 0; b < B; ++b) mx = std::max(mx, segs[s]->n_kept_host[b]);
@@ -831,7 +885,14 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
     tcost[s] = tile_cost_host(segs[s], mtiles);
     hcost[s] = htiles[s] * tcost[s];
     heavy[s] = htiles[s] > 0;
+    longest = std::max(longest, htiles[s]);
   }
+  // Generated tokens of up to one tile are a light item like none at all, so
+  // that a plan frozen before the first of them (a captured decode step) and
+  // the plans of the steps after it form the same items in the same places.
+  if (mtiles == 1 && forced_ipb <= 0 && longest > 1)
+    for (int s = 0; s < nseg; ++s)
+      if (segs[s]->kind == UC_KIND_EVICT && htiles[s] == 1) heavy[s] = false;
   // Heavy items per (b, kvh): the fewest (at least one per heavy segment, at
   // most 56 and at most 64 with the light items, the partials one merge
   // stages) that keep >= 90 % of the CTA slots busy in every round, else the
@@ -890,6 +951,37 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
       const int hr = std::min(hmax, slots / std::max(1, nbh_launch));
       if (hr > H) H = hr;
     }
+    // short calls: the items of a pair on one cluster where that, with the
+    // number of items a cluster can have, is expected to end sooner
+    p.cluster = 0;
+    if (mtiles == 1 && forced_ipb <= 0 && slots == kClusterSlots && nh > 0) {
+      auto longest_us = [&](int h) {
+        int hc[UC_MAX_SEGMENTS];
+        split_items(h, nseg, heavy, htiles, tcost, hc);
+        double us = 0.0;
+        for (int s = 0; s < nseg; ++s)
+          if (heavy[s]) us = std::max(us, ((htiles[s] + hc[s] - 1) / hc[s]) * tile_us(segs[s]));
+        return us;
+      };
+      double best = items_us(longest_us(H), H, nbh_launch) + kQueueMergeUs;
+      double light = nl * kLightItemUs;
+      for (int s = 0; s < nseg; ++s)
+        if (!heavy[s] && htiles[s] > 1) light += htiles[s] * tile_us(segs[s]);
+      // ranks for the light items: one each, or one for all of them
+      for (int lr = nl;; lr = 1) {
+        int h = std::min(kMaxClusterItems - lr, hmax);
+        while (h >= nh && kClusterFit[h + lr] < nbh_launch) --h;
+        if (h >= nh) {
+          const double us = kClusterSpread * items_us(std::max(light / std::max(1, lr), longest_us(h)), h + lr, nbh_launch);
+          if (us < best) {
+            best = us;
+            p.cluster = lr + 1;
+            H = h;
+          }
+        }
+        if (lr <= 1) break;
+      }
+    }
     bool changed = false;
     for (int s = 0; s < nseg; ++s)
       if (heavy[s] && H > 0 && hcost[s] < 0.5 * tot / H) {
@@ -898,33 +990,15 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
       }
     if (!changed) break;
   }
-  // split them among the heavy segments so that the largest item is
-  // smallest (one more item at a time to the segment whose items are
-  // largest). Where the launch merges its own partials, drop then the items
-  // that do not shrink a segment's largest item: each would only bring its
-  // start, cross-warp reduction and merge share (8K understanding layer: text
-  // 8 tiles as 4 items of 2 instead of 5 items of 1-2, 13 items per (b, kvh)
-  // instead of 14, 12694 -> 13221 tokens/s). With the separate merge kernel
-  // an item is cheap and more of them even out the SMs' loads.
-  int hc[UC_MAX_SEGMENTS], nh = 0;
-  for (int s = 0; s < nseg; ++s) {
-    hc[s] = heavy[s] ? 1 : 0;
-    nh += hc[s];
-  }
-  for (int left = H - nh; left > 0; --left) {
-    int pick = -1;
-    double worst = 0.0;
-    for (int s = 0; s < nseg; ++s) {
-      if (!heavy[s] || hc[s] >= htiles[s]) continue;
-      const double item = std::ceil((double)htiles[s] / hc[s]) * tcost[s];
-      if (item > worst) {
-        worst = item;
-        pick = s;
-      }
-    }
-    if (pick < 0) break;
-    ++hc[pick];
-  }
+  // Split them among the heavy segments. Where the launch merges its own
+  // partials, drop then the items that do not shrink a segment's largest
+  // item: each would only bring its start, cross-warp reduction and merge
+  // share (8K understanding layer: text 8 tiles as 4 items of 2 instead of 5
+  // items of 1-2, 13 items per (b, kvh) instead of 14, 12694 -> 13221
+  // tokens/s). With the separate merge kernel an item is cheap and more of
+  // them even out the SMs' loads.
+  int hc[UC_MAX_SEGMENTS];
+  split_items(H, nseg, heavy, htiles, tcost, hc);
   {
     int trimmed[UC_MAX_SEGMENTS], items = 0;
     for (int s = 0; s < nseg; ++s) {
@@ -963,6 +1037,7 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
     }
     cb += p.n_chunks[s];
   }
+  if (p.cluster) p.cluster = p.n_heavy > 0 ? p.n_heavy + p.cluster - 1 : 0;  // light ranks + 1 so far
   p.items_per_bh = assigned;  // at most 64 (the merge staging)
   p.n_items = assigned * nbh;
   p.grid = std::min(p.n_items, slots);
@@ -1344,7 +1419,9 @@ uc_status uc_attend(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_s
   st = build_decode_call(q, n_q_heads, n_qtok, segs, n_seg, out, lse, mass, &plan, ws + 256,
                          ws + 256 + kCounterBlock, reinterpret_cast<DevStatus*>(ws), &p);
   if (st != UC_OK) return st;
-  p.defer_merge = merge_kernel_for(plan.items_per_bh);
+  // (a device whose clusters fit less well than planned for takes the queue)
+  p.cluster = plan.cluster > 0 && attend_clusters(plan.cluster) >= B * hkv ? plan.cluster : 0;
+  p.defer_merge = p.cluster ? 0 : merge_kernel_for(plan.items_per_bh);
   launch_attend(p, plan.grid, reinterpret_cast<cudaStream_t>(stream));
   return cuda_check("uc_attend");
 }

@@ -18,7 +18,9 @@
 //               accumulation.
 // Each item leaves an unnormalised partial (O, m, l); the last CTA to finish
 // a (sequence, KV head) merges its items by log-sum-exp, writes O, lse and
-// the per-segment probability mass, and re-arms the counter.
+// the per-segment probability mass, and re-arms the counter. In short calls
+// the items of a (sequence, KV head) run on one thread-block cluster instead,
+// which merges them through distributed shared memory.
 #include <atomic>
 #include <mutex>
 
@@ -203,6 +205,22 @@ struct WorkOf<MultiAttnParams> {
 
 __device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
+// consumer_sync with a vote: true if `ok` holds in every consumer warp.
+__device__ __forceinline__ bool consumer_all(bool ok) {
+  uint32_t all;
+  asm volatile(
+      "{\n"
+      ".reg .pred p, q;\n"
+      "setp.ne.u32 p, %1, 0;\n"
+      "barrier.cta.red.and.pred q, 1, 128, p;\n"
+      "selp.u32 %0, 1, 0, q;\n"
+      "}\n"
+      : "=r"(all)
+      : "r"((uint32_t)ok)
+      : "memory");
+  return all != 0;
+}
+
 // Arrival on a (sequence, KV head) counter, acquire-release at GPU scope:
 // after a CTA barrier, the partial outputs every consumer thread wrote are
 // ordered before the increment (release is cumulative over the barrier), and
@@ -242,7 +260,10 @@ __device__ __forceinline__ uint2 lds64(uint32_t a) {
 // start it), hands each position to the consumers through a two-entry queue
 // and copies the item's query rows (the g * T rows of one KV head are
 // contiguous) along with it.
-template <int NTW, class W>
+//
+// In a cluster launch rank r < n_heavy takes its pair's heavy item r, the
+// ranks after them (one, or one each) share the pair's light items.
+template <int NTW, bool CLUSTER, class W>
 __device__ void produce(const W& w, AttnSmem& sm) {
   constexpr int ST = kStages;
   const AttnParams& p0 = w.call(0);
@@ -253,6 +274,13 @@ __device__ void produce(const W& w, AttnSmem& sm) {
   // the item count); later items come from the launch-wide counter, so the
   // first copies are issued without waiting for an atomic's round trip
   int pos = blockIdx.x;
+  int end = 0;
+  if constexpr (CLUSTER) {
+    const int pair = blockIdx.x / p0.cluster, rank = blockIdx.x % p0.cluster;
+    const int light0 = p0.n_heavy * p0.batch * p0.n_kv_heads + pair * p0.n_light;
+    pos = rank < p0.n_heavy ? pair * p0.n_heavy + rank : light0 + rank - p0.n_heavy;
+    end = rank < p0.n_heavy ? 0 : light0 + p0.n_light;
+  }
   for (uint32_t iseq = 0;; ++iseq) {
     const int k = iseq % kItemQ;
     if (iseq >= kItemQ && !mbar_wait(&sm.item_empty[k], ((iseq / kItemQ) - 1) & 1, p0.status, 12, p0.wait_ns))
@@ -315,16 +343,23 @@ __device__ void produce(const W& w, AttnSmem& sm) {
       }
     }
     if (stop) break;
-    pos = (int)gridDim.x + atomicAdd(sched, 1);
+    if constexpr (CLUSTER) {
+      pos += p0.cluster - p0.n_heavy;
+      if (pos >= end) pos = w.n_items();
+    } else {
+      pos = (int)gridDim.x + atomicAdd(sched, 1);
+    }
   }
   // This producer claims nothing more: the last producer of the launch to
   // get here re-arms the work queue for the next launch. Done here rather
   // than at the CTA's exit, so that the fence and the atomic stay off the
   // path of the consumers' final merges.
-  __threadfence();
-  if (atomicAdd(sched + 1, 1) == (int)gridDim.x - 1) {
-    sched[0] = 0;
-    sched[1] = 0;
+  if constexpr (!CLUSTER) {
+    __threadfence();
+    if (atomicAdd(sched + 1, 1) == (int)gridDim.x - 1) {
+      sched[0] = 0;
+      sched[1] = 0;
+    }
   }
   // A consumer that gave up on a bounded wait (the status word is set) no
   // longer waits for the copies this producer issued: they land before the
@@ -1129,15 +1164,11 @@ __device__ __forceinline__ void store_q(const AttnParams& p, uint32_t* qf, const
   }
 }
 
-// Merge the warps that share n-tiles (through the item's last slot), then
-// write this item's partial.
+// Adds the zero-point term of packed values to O: channel group gi of query
+// rows 2j, 2j + 1 sits in lane (gi, j).
 template <int NTW>
-__device__ __forceinline__ void finish_item(const AttnParams& p, AttnSmem& sm, WarpState<NTW>& st,
-                                            int it, int last_slot, int NG, int KS, int grp, int ks) {
-  const int lane = threadIdx.x & 31;
-  const int g = lane >> 2, j = lane & 3;
-  // zero-point term of packed values: channel group gi of query rows 2j,
-  // 2j + 1 sits in lane (gi, j)
+__device__ __forceinline__ void fold_zero_points(WarpState<NTW>& st) {
+  const int j = threadIdx.x & 3;
 #pragma unroll
   for (int nt = 0; nt < NTW; ++nt)
 #pragma unroll
@@ -1152,7 +1183,11 @@ __device__ __forceinline__ void finish_item(const AttnParams& p, AttnSmem& sm, W
         st.o[nt][2 * gi + mh][3] += z1;
       }
     }
-  // full row sums: add the shares of the 8 key lanes (g)
+}
+
+// Full row sums: adds the shares of the 8 key lanes (g).
+template <int NTW>
+__device__ __forceinline__ void reduce_row_sums(WarpState<NTW>& st) {
 #pragma unroll
   for (int nt = 0; nt < NTW; ++nt)
 #pragma unroll
@@ -1163,6 +1198,17 @@ __device__ __forceinline__ void finish_item(const AttnParams& p, AttnSmem& sm, W
       v += __shfl_xor_sync(0xffffffffu, v, 16);
       st.l[nt][h] = v;
     }
+}
+
+// Merge the warps that share n-tiles (through the item's last slot), then
+// write this item's partial.
+template <int NTW>
+__device__ __forceinline__ void finish_item(const AttnParams& p, AttnSmem& sm, WarpState<NTW>& st,
+                                            int it, int last_slot, int NG, int KS, int grp, int ks) {
+  const int lane = threadIdx.x & 31;
+  const int g = lane >> 2, j = lane & 3;
+  fold_zero_points<NTW>(st);
+  reduce_row_sums<NTW>(st);
   constexpr int kVals = NTW * 36;
   if (KS > 1 && last_slot >= 0) {
     float* buf = reinterpret_cast<float*>(sm.slot[last_slot]);
@@ -1242,11 +1288,13 @@ __device__ __forceinline__ void finish_item(const AttnParams& p, AttnSmem& sm, W
   }
 }
 
-// All tiles of one item: bf16 rows (BITS = 16: bf16 segments and the tails
-// of packed segments) or packed groups (BITS = 4 / 2).
+// All tiles of one item added to a warp's state: bf16 rows (BITS = 16: bf16
+// segments and the tails of packed segments) or packed groups (BITS = 4 / 2).
+// With `keep_last` the item's last slot is not handed back; returns it (-1: none).
 template <int NTW, int BITS>
-__device__ __forceinline__ void run_item(const AttnParams& p, AttnSmem& sm, const ItemInfo& ii, int it, int k,
-                                         uint32_t& seq, bool& aborted, int NG, int KS, int grp, int ks) {
+__device__ __forceinline__ int run_tiles(const AttnParams& p, AttnSmem& sm, const ItemInfo& ii, int k, uint32_t& seq,
+                                         bool& aborted, int KS, int grp, int ks, bool keep_last,
+                                         WarpState<NTW>& st) {
   const int lane = threadIdx.x & 31;
   uint32_t* qf = NTW == 1 ? reinterpret_cast<uint32_t*>(sm.merge_w)
                           : reinterpret_cast<uint32_t*>(after_ring(sm));
@@ -1254,8 +1302,6 @@ __device__ __forceinline__ void run_item(const AttnParams& p, AttnSmem& sm, cons
   consumer_sync();
   if (lane == 0) mbar_arrive(&sm.item_empty[k]);  // the query rows are no longer needed
   const uint32_t qs = smem_u32(qf) + grp * NTW * 2048;
-  WarpState<NTW> st;
-  state_init<NTW>(st);
   int last_slot = -1;
   for (int t = ii.tb; t < ii.te; ++t, ++seq) {
     constexpr int ST = kStages;
@@ -1299,7 +1345,7 @@ __device__ __forceinline__ void run_item(const AttnParams& p, AttnSmem& sm, cons
         for (; gl < ngt; gl += KS) group_quant<NTW, BITS>(st, qs, sbase, gl, p.scale_log2, none);
       }
     }
-    if (t + 1 < ii.te || KS == 1) {
+    if (t + 1 < ii.te || !keep_last) {
       // reads alone need no proxy fence before the slot is handed back to
       // the copy engine; the zeroed rows of a partial bf16 tile do
       if (wrote) fence_proxy_async();
@@ -1309,7 +1355,205 @@ __device__ __forceinline__ void run_item(const AttnParams& p, AttnSmem& sm, cons
       last_slot = slot;
     }
   }
+  return last_slot;
+}
+
+template <int NTW, int BITS>
+__device__ __forceinline__ void run_item(const AttnParams& p, AttnSmem& sm, const ItemInfo& ii, int it, int k,
+                                         uint32_t& seq, bool& aborted, int NG, int KS, int grp, int ks) {
+  WarpState<NTW> st;
+  state_init<NTW>(st);
+  const int last_slot = run_tiles<NTW, BITS>(p, sm, ii, k, seq, aborted, KS, grp, ks, KS > 1, st);
   finish_item<NTW>(p, sm, st, it, last_slot, NG, KS, grp, ks);
+}
+
+// ---- cluster launches (one n-tile): a (sequence, KV head)'s items on the
+// CTAs of one cluster. A warp carries its state from item to item (the row
+// sums go to its bank per segment, for the masses); the CTA's four warps meet
+// in its idle ring, and after one cluster barrier rank r's warps each finish
+// query rows of the pair from every CTA's shared memory. No partial output
+// goes through global memory, and no CTA waits for an arrival counter's
+// answer, copies partials in and weighs them after everyone else has left:
+// those took 2 + 5 us at the end of a 20 us call (8K context, batch 8).
+struct ClusterPart {
+  float o[8][kHeadDim];                // unnormalised O of this CTA's items
+  float m[8];                          // per query row, log2 units
+  float l[UC_MAX_SEGMENTS][8];         // row sums per segment
+};
+struct ClusterSmem {
+  float o[kConsumers][8][kHeadDim];    // the warps' O
+  ClusterPart part;
+};
+static_assert(sizeof(ClusterSmem) <= (size_t)kStages * kSlotBytes, "in the idle ring");
+// per warp, segment and row: the row sum so far and the maximum it refers to
+using RowBank = float2[kConsumers][UC_MAX_SEGMENTS][8];
+static_assert(sizeof(RowBank) <= sizeof(float) * kMaxItemsPerBh * 8, "in the merge array the queries leave free");
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// Shared address of the same variable in another CTA of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const void* local, int rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(local)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t a) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(a)
+               : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void consume_cluster(const AttnParams& p, AttnSmem& sm) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = lane >> 2, j = lane & 3;
+  uint32_t seq = 0;
+  bool aborted = false;
+  RowBank& bank = *reinterpret_cast<RowBank*>(sm.merge_l);
+  for (int x = lane; x < UC_MAX_SEGMENTS * 8; x += 32) bank[warp][x >> 3][x & 7] = make_float2(kNegInf, 0.f);
+  __syncwarp();
+  WarpState<1> st;
+  state_init<1>(st);
+  for (uint32_t iseq = 0;; ++iseq) {
+    const int k = iseq % kItemQ;
+    // one decision for the CTA's warps (a wait that ran out in one of them ends
+    // the loop in all, so their barriers stay in step); it also separates the
+    // last item's reads of the query fragments from this item's writes
+    if (!consumer_all(mbar_wait(&sm.item_full[k], (iseq / kItemQ) & 1, p.status, 13, p.wait_ns))) break;
+    const int pos = sm.item_pos[k];
+    if (pos < 0) break;
+    int it;
+    const ItemInfo ii = decode_item(p, pos, &it);
+    const SegDev& sd = p.seg[ii.s];
+    if (seg_is_bf16(sd.kind) || ii.tail)
+      run_tiles<1, 16>(p, sm, ii, k, seq, aborted, kConsumers, 0, warp, false, st);
+    else if (sd.bits == 4)
+      run_tiles<1, 4>(p, sm, ii, k, seq, aborted, kConsumers, 0, warp, false, st);
+    else
+      run_tiles<1, 2>(p, sm, ii, k, seq, aborted, kConsumers, 0, warp, false, st);
+    reduce_row_sums<1>(st);
+    if (g == 0) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float2& e = bank[warp][ii.s][2 * j + h];
+        const float old = e.y == 0.f ? 0.f : e.y * exp2f(e.x - st.m[0][h]);
+        e = make_float2(st.m[0][h], old + st.l[0][h]);
+      }
+    }
+    st.l[0][0] = st.l[0][1] = 0.f;
+    __syncwarp();
+  }
+  // the CTA's part: O of the four warps, row maxima, row sums per segment
+  fold_zero_points<1>(st);
+  ClusterSmem& cs = *reinterpret_cast<ClusterSmem*>(sm.slot[0]);
+  consumer_sync();  // every warp is past its last tile: the ring is idle
+#pragma unroll
+  for (int mt = 0; mt < 8; ++mt)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) cs.o[warp][2 * j + (e & 1)][16 * mt + g + 8 * (e >> 1)] = st.o[0][mt][e];
+  float* wm = sm.merge_w;  // the warps' row maxima (the query fragments are no longer needed)
+  if (g == 0) {
+    wm[warp * 8 + 2 * j] = st.m[0][0];
+    wm[warp * 8 + 2 * j + 1] = st.m[0][1];
+  }
+  consumer_sync();
+  {
+    const int row = threadIdx.x >> 4;  // 16 threads per row, two float4 each
+    float M = kNegInf, wt[kConsumers];
+#pragma unroll
+    for (int w = 0; w < kConsumers; ++w) M = fmaxf(M, wm[w * 8 + row]);
+#pragma unroll
+    for (int w = 0; w < kConsumers; ++w) {
+      const float m = wm[w * 8 + row];
+      wt[w] = m == kNegInf ? 0.f : exp2f(m - M);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = 4 * (threadIdx.x & 15) + 64 * h;
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int w = 0; w < kConsumers; ++w) {
+        const float4 x = *reinterpret_cast<const float4*>(&cs.o[w][row][c]);
+        a.x += wt[w] * x.x; a.y += wt[w] * x.y; a.z += wt[w] * x.z; a.w += wt[w] * x.w;
+      }
+      *reinterpret_cast<float4*>(&cs.part.o[row][c]) = a;
+    }
+    const int s = threadIdx.x & 15;
+    if (s < p.nseg) {
+      float l = 0.f;
+#pragma unroll
+      for (int w = 0; w < kConsumers; ++w) {
+        const float2 e = bank[w][s][row];
+        if (e.y != 0.f) l += e.y * exp2f(e.x - M);
+      }
+      cs.part.l[s][row] = l;
+    }
+    if (s == 0) cs.part.m[row] = M;
+  }
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();
+  // one warp per query row: the rows of the pair over the warps of the cluster
+  const int C = p.cluster, rank = blockIdx.x % C;
+  const int pair = blockIdx.x / C, b = pair / p.n_kv_heads, kvh = pair % p.n_kv_heads;
+  for (int r = rank + C * warp; r < p.rows; r += C * kConsumers) {
+    const uint32_t pb = cluster_addr(&cs.part, lane < C ? lane : 0);  // lane c: CTA c's part
+    float m = kNegInf, l = 0.f, ls[UC_MAX_SEGMENTS];
+#pragma unroll
+    for (int s = 0; s < UC_MAX_SEGMENTS; ++s) ls[s] = 0.f;
+    if (lane < C) {
+      m = ld_cluster(pb + (uint32_t)offsetof(ClusterPart, m) + 4 * r);
+#pragma unroll
+      for (int s = 0; s < UC_MAX_SEGMENTS; ++s)
+        if (s < p.nseg) ls[s] = ld_cluster(pb + (uint32_t)offsetof(ClusterPart, l) + (s * 8 + r) * 4);
+    }
+    float4 x[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c)
+      if (c < C) x[c] = ld_cluster4(cluster_addr(&cs.part.o[r][4 * lane], c));
+    float M = m;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    const float w = m == kNegInf ? 0.f : exp2f(m - M);
+#pragma unroll
+    for (int s = 0; s < UC_MAX_SEGMENTS; ++s) l += ls[s];
+    l *= w;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    const float inv = l > 0.f ? 1.f / l : 0.f;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int c = 0; c < 16; ++c)
+      if (c < C) {
+        const float wc = __shfl_sync(0xffffffffu, w, c) * inv;
+        a.x += wc * x[c].x; a.y += wc * x[c].y; a.z += wc * x[c].z; a.w += wc * x[c].w;
+      }
+    const size_t orow = out_row(p, b, kvh, r);
+    *reinterpret_cast<uint2*>(p.out + orow * kHeadDim + 4 * lane) = make_uint2(pack_bf16(a.x, a.y), pack_bf16(a.z, a.w));
+    if (lane == 0 && p.lse) p.lse[orow] = l > 0.f ? (M + log2f(l)) * kLn2 : kNegInf;
+    if (p.mass) {
+#pragma unroll
+      for (int s = 0; s < UC_MAX_SEGMENTS; ++s) {
+        if (s < p.nseg) {
+          ls[s] *= w;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) ls[s] += __shfl_xor_sync(0xffffffffu, ls[s], o);
+          if (lane == 0) p.mass[orow * p.nseg + s] = ls[s] * inv;
+        }
+      }
+    }
+  }
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();  // no CTA leaves while another may still read its shared memory
 }
 
 template <int NTW, class W>
@@ -1377,7 +1621,7 @@ __device__ void consume(const W& w, AttnSmem& sm) {
   }
 }
 
-template <int NTW, class P>
+template <int NTW, class P, bool CLUSTER = false>
 __global__ void __launch_bounds__(kAttnThreads, ctas_for<NTW>()) attend_kernel(const __grid_constant__ P params) {
   const typename WorkOf<P>::type w{params};
   extern __shared__ uint8_t dyn_smem[];
@@ -1413,10 +1657,13 @@ __global__ void __launch_bounds__(kAttnThreads, ctas_for<NTW>()) attend_kernel(c
           prefetch_tmap(&p.tmap[2 * s + 1]);
         }
       }
-      produce<NTW>(w, sm);
+      produce<NTW, CLUSTER>(w, sm);
     }
   } else {
-    consume<NTW>(w, sm);
+    if constexpr (CLUSTER)
+      consume_cluster(params, sm);
+    else
+      consume<NTW>(w, sm);
   }
 }
 
@@ -1426,6 +1673,8 @@ static void attend_setup_once() {
     const int one = (int)attend_smem_bytes(1), most = (int)attend_smem_bytes(8);
     cudaFuncSetAttribute(attend_kernel<1, AttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize, one);
     cudaFuncSetAttribute(attend_kernel<2, AttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(attend_kernel<1, AttnParams, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, one);
+    cudaFuncSetAttribute(attend_kernel<1, AttnParams, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaFuncSetAttribute(attend_kernel<1, MultiAttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize, one);
     cudaFuncSetAttribute(attend_kernel<2, MultiAttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   });
@@ -1449,9 +1698,51 @@ int attend_ctas_per_sm(int ntiles) {
   return n;
 }
 
+static cudaLaunchConfig_t cluster_config(int c, int grid, cudaStream_t st, cudaLaunchAttribute* attr) {
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)c;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kAttnThreads);
+  cfg.dynamicSmemBytes = attend_smem_bytes(1);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cfg;
+}
+
+// Clusters of c CTAs this device runs at once (0: none).
+int attend_clusters(int c) {
+  static std::atomic<int> cached[kMaxClusterItems + 1];  // count + 1
+  if (c < 1 || c > kMaxClusterItems) return 0;
+  int n = cached[c].load(std::memory_order_relaxed) - 1;
+  if (n < 0) {
+    attend_setup_once();
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = cluster_config(c, c, nullptr, attr);
+    if (cudaOccupancyMaxActiveClusters(&n, attend_kernel<1, AttnParams, true>, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    cached[c].store(n + 1, std::memory_order_relaxed);
+  }
+  return n;
+}
+
 void launch_attend(const AttnParams& p, int grid, cudaStream_t st) {
   attend_setup_once();
   const bool pdl = pdl_enabled();
+  if (p.cluster) {
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = cluster_config(p.cluster, p.cluster * p.batch * p.n_kv_heads, st, attr);
+    cudaLaunchKernelEx(&cfg, attend_kernel<1, AttnParams, true>, p);
+    count_launch();
+    return;
+  }
   const size_t smem = attend_smem_bytes(p.mtiles);
   if (p.mtiles <= 1)
     launch_maybe_pdl(pdl, attend_kernel<1, AttnParams>, grid, kAttnThreads, smem, st, p);

@@ -213,6 +213,9 @@ struct AttnParams {
   int n_heavy, n_light;
   int16_t heavy_local[128];
   int16_t light_local[2 * UC_MAX_SEGMENTS];
+  // > 0: a cluster of this many CTAs per (sequence, KV head) instead of the
+  // work queue: one per heavy item, then one for the light items or one each
+  int cluster;
   int defer_merge;  // 1: the attend launch only leaves partials; a merge kernel follows
   float scale_log2;
   uint64_t wait_ns;  // limit of every bounded wait of the launch (UC_ERR_TIMEOUT past it)
@@ -267,6 +270,8 @@ size_t dense_smem_bytes();
 void launch_dense(const DenseParams& p, cudaStream_t st);
 
 int attend_ctas_per_sm(int ntiles);
+constexpr int kMaxClusterItems = 16;  // CTAs of the largest cluster
+int attend_clusters(int c);
 __host__ __device__ size_t attend_part_floats(int mtiles);
 void launch_attend(const AttnParams& p, int grid, cudaStream_t st);
 void launch_attend_multi(const MultiAttnParams& m, int grid, cudaStream_t st);

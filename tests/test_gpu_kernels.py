@@ -342,6 +342,43 @@ def test_attend_query_tiles_many_items(hq, T):
     assert ws.status() == 0
 
 
+CLUSTER_MIXES = {
+    # (B, Hkv, sizes, kinds, keeps, bits): clusters of 1, few and 16 CTAs, more
+    # light items than ranks, eight segments, sequences that hold nothing of a
+    # segment, 64 pairs (six CTAs each), and one pair too many for any cluster
+    "one_token": (1, 1, [1], ["full"], [1], [16]),
+    "tails_only": (2, 2, [20, 33, 31], ["quant", "quant", "quant"], [20, 33, 31], [4, 2, 4]),
+    "eight_segments": (1, 4, [40, 64, 100, 33, 257, 7, 90, 300],
+                       ["full", "quant", "evict", "quant", "evict_quant", "full", "quant", "evict_quant"],
+                       [40, 64, 20, 33, 130, 7, 90, 250], [16, 4, 16, 2, 2, 16, 4, 4]),
+    "sixteen_ranks": (1, 1, [3000, 4100], ["full", "quant"], [3000, 4100], [16, 4]),
+    "ragged": (5, 4, [700, 900], ["evict", "evict_quant"], [[1, 700, 64, 65, 128], [900, 1, 32, 64, 31]], [16, 2]),
+    "pairs_64": (8, 8, [300, 1000], ["full", "quant"], [300, 1000], [16, 2]),
+    "pairs_512": (64, 8, [70], ["full"], [70], [16]),
+}
+
+
+@pytest.mark.parametrize("mix", list(CLUSTER_MIXES))
+def test_attend_short_calls(mix):
+    B, hkv, sizes, kinds, keeps, bits = CLUSTER_MIXES[mix]
+    hq = 7 * hkv
+    gsegs, osegs = _build_mix(len(mix), B, hkv, sizes, kinds, keeps, bits)
+    q = synth.make_q(B, B, hq, 1)
+    rO, rl, rm = oattn.attend(q, osegs, hkv)
+    bound = _packed.logit_error_bound(q, osegs, hkv, [kd in ("quant", "evict_quant") for kd in kinds])
+    ws = uc.Workspace(DEV)
+    first = None
+    for _ in range(2):
+        O, lse, mass = uc.attend(dev(q), gsegs, ws=ws)
+        assert _packed.attention_error(host(O), rO) <= _packed.ATTN_RTOL
+        assert (np.abs(host(lse) - rl) <= bound).all()
+        assert (np.abs(host(mass) - rm) <= 2 * bound[..., None]).all()
+        if first is not None:
+            assert all(torch.equal(x, y) for x, y in zip(first, (O, lse, mass)))   # a fixed summation order
+        first = (O, lse, mass)
+    assert ws.status() == 0
+
+
 LONG_MIXES = {
     # few (sequence, KV head) pairs and long segments: more than 32 items per
     # pair, merged by the separate merge kernel

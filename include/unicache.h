@@ -172,14 +172,12 @@ int32_t uc_version(void);
 /* Number of kernels this library has launched in this process. */
 uint64_t uc_launch_count(void);
 
-/* Issue order of the dense (many-query) attention kernel, process-wide.
- * 1 (default): the issuing thread waits for a Q tile's P V to complete
- * before the next Q K^T of that tile, which overwrites P's tensor-memory
- * columns. 0: that Q K^T is issued right behind the P V; this relies on the
- * tensor pipe reading P before the later MMA writes those columns, an
- * ordering the two MMAs (different accumulators) are not documented to
- * have. On GB300 both orders give bit-identical results (tested) and 0 is
- * 2.8 % faster on the denoising workload. Returns the previous setting. */
+/* Issue order of the dense (many-query) attention kernel, process-wide: a
+ * setting kept for its callers. 1 (default) asked for a wait between the P V
+ * of a Q tile and the next Q K^T, which overwrote P's tensor-memory columns; 0
+ * left that wait out and relied on the tensor pipe's order. P has columns of
+ * its own now and nothing is overwritten early: both settings run the same
+ * code without the wait. Returns the previous setting. */
 int32_t uc_set_dense_serial_pv(int32_t serial);
 
 /* Limit, in nanoseconds, of every bounded wait inside the decode attention

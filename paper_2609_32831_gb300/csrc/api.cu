@@ -1410,7 +1410,6 @@ uc_status uc_attend(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_s
     d.n_qtok = n_qtok;
     d.group = group;
     d.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)UC_HEAD_DIM));
-    d.serial_pv = g_dense_serial_pv.load();
     launch_dense(d, reinterpret_cast<cudaStream_t>(stream));
     return cuda_check("uc_attend (dense)");
   }

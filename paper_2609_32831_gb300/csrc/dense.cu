@@ -12,17 +12,18 @@
 // 2. dense_kernel: one CTA per 256 query rows (two Q tiles of 128) of one
 //    query head; keys in tiles of 128. Warpgroup roles:
 //      WG0, WG1   softmax of Q tile 0 / 1: one query row per thread (= one
-//                 TMEM lane); S read from TMEM, P = 2^(S - m) written back
-//                 over S as fp16 pairs; online softmax with a lazily moved
+//                 TMEM lane); S read from TMEM (which frees it for the other
+//                 tile's S), P = 2^(S - m) written to the tile's own columns
+//                 as fp16 pairs; online softmax with a lazily moved
 //                 reference max (O is rescaled only when a row's max grows
 //                 by more than 2^8, so P <= 256 stays exact enough in fp16);
 //      WG2        warp 8: TMA producer of K hi / K lo tiles (3-slot ring) and
 //                 V tiles (2-slot ring); warp 9: allocates TMEM and issues
-//                 every tcgen05.mma from one thread, alternating the Q tiles:
+//                 every tcgen05.mma from one lane, alternating the Q tiles:
 //                 S_x = Q_x K^T (M=128, N=128, K=128, both from shared
 //                 memory) and O_x += P_x V (A = P from TMEM, B = V from shared
 //                 memory), so that one tile's softmax overlaps the other
-//                 tile's MMAs. TMEM: S/P and O of both tiles, 512 columns.
+//                 tile's MMAs. TMEM: one S, P and O of both tiles, 512 columns.
 //    The warpgroups rebalance registers with setmaxnreg (softmax 216, the
 //    producer / MMA group 56).
 #include <mutex>
@@ -37,17 +38,17 @@ namespace uc {
 // (Q) and B (K) offsets step 32 B inside a 128-B swizzled row, then 16 KB
 // to the second 64-channel block.
 template <int ACC0>
-__device__ __forceinline__ void issue_qk(uint32_t d, uint32_t q_lo, uint32_t k_lo, uint32_t hi, uint32_t idesc) {
-  umma_ss_off<0, 0, ACC0>(d, q_lo, k_lo, hi, idesc);
-  umma_ss_off<2, 2, 1>(d, q_lo, k_lo, hi, idesc);
-  umma_ss_off<4, 4, 1>(d, q_lo, k_lo, hi, idesc);
-  umma_ss_off<6, 6, 1>(d, q_lo, k_lo, hi, idesc);
-  umma_ss_off<1024, 1024, 1>(d, q_lo, k_lo, hi, idesc);
-  umma_ss_off<1026, 1026, 1>(d, q_lo, k_lo, hi, idesc);
-  umma_ss_off<1028, 1028, 1>(d, q_lo, k_lo, hi, idesc);
-  umma_ss_off<1030, 1030, 1>(d, q_lo, k_lo, hi, idesc);
+__device__ __forceinline__ void issue_qk(uint32_t lead, uint32_t d, uint32_t q_lo, uint32_t k_lo, uint32_t hi,
+                                         uint32_t idesc) {
+  umma_ss_lead<0, 0, ACC0>(lead, d, q_lo, k_lo, hi, idesc);
+  umma_ss_lead<2, 2, 1>(lead, d, q_lo, k_lo, hi, idesc);
+  umma_ss_lead<4, 4, 1>(lead, d, q_lo, k_lo, hi, idesc);
+  umma_ss_lead<6, 6, 1>(lead, d, q_lo, k_lo, hi, idesc);
+  umma_ss_lead<1024, 1024, 1>(lead, d, q_lo, k_lo, hi, idesc);
+  umma_ss_lead<1026, 1026, 1>(lead, d, q_lo, k_lo, hi, idesc);
+  umma_ss_lead<1028, 1028, 1>(lead, d, q_lo, k_lo, hi, idesc);
+  umma_ss_lead<1030, 1030, 1>(lead, d, q_lo, k_lo, hi, idesc);
 }
-
 
 // Two fp32 lanes in one 64-bit register: packed FMA / add (sm_100 family).
 __device__ __forceinline__ uint64_t f2_pack(float a, float b) {
@@ -74,22 +75,6 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return d;
 }
 
-// Non-blocking test of an mbarrier phase (issued early; its result is used
-// later, so the check overlaps the MMAs queued meanwhile).
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n"
-      ".reg .pred p;\n"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n"
-      "}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
 template <int N>
 __device__ __forceinline__ void setmaxnreg_inc() {
   asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
@@ -114,11 +99,17 @@ constexpr int kDThreads = 384;     // WG0, WG1: softmax of Q tile 0, 1; WG2: TMA
 constexpr int kRegSoftmax = 216;
 constexpr int kRegOther = 56;
 static_assert(2 * 128 * kRegSoftmax + 128 * kRegOther <= kDThreads * 168, "register split");
-constexpr int kTmemCols = 512;     // per Q tile X: S/P [256X, 256X+128), O [256X+128, 256X+256)
+// Tensor memory columns. Both Q tiles' S go through one buffer: a softmax
+// thread holds its whole row of S in registers right after the loads, long
+// before the other tile's S is due, and P has columns of its own, so no MMA
+// overwrites what an earlier one reads and S(j+1) follows P(j) V(j) into the
+// pipe at once. (With P in S's columns the issuing thread had to wait for P V
+// to complete first: 235 idle cycles per tile and key tile, 180 us of the 4096
+// x 8448 keys batch 4 call, 1793 us.)
+constexpr int kTmemCols = 512;
+constexpr uint32_t kTmemP = 128;   // + 64 x
+constexpr uint32_t kTmemO = 256;   // + 128 x
 constexpr float kDNegInf = -INFINITY;
-// Issue S(j+1) of a Q tile only after P(j) V(j) of that tile has completed
-// (P(j) lives in S's TMEM columns). false: rely on the in-order execution of
-// the tensor pipe for that write-after-read.
 
 struct DenseSmem {
   uint8_t q[kDQT][2][16384];       // Q fp16 [128 rows][2 x 64 cols], K-major, 128B swizzle
@@ -128,8 +119,7 @@ struct DenseSmem {
   uint8_t tseg[kMaxDenseTiles];    // segment of tile j
   uint8_t tlo[kMaxDenseTiles];     // 1 if tile j has K lo rows (packed segment)
   uint64_t k_full[kDKSlots], k_empty[kDKSlots], v_full[kDVSlots], v_empty[kDVSlots];
-  uint64_t s_full[kDQT], p_full[kDQT], q_full[kDQT], o_full[kDQT];
-  uint64_t pv_done[kDQT];  // serial order only: P V of the Q tile completed
+  uint64_t s_full[kDQT], s_free[kDQT], p_full[kDQT], q_full[kDQT], o_full[kDQT];
   uint32_t tmem_base;
 };
 static_assert(sizeof(DenseSmem) + 1024 <= 232448, "dense kernel shared memory");
@@ -358,7 +348,7 @@ __global__ void __launch_bounds__(kDThreads, 1) dense_kernel(const __grid_consta
   extern __shared__ uint8_t dyn_smem[];
   DenseSmem& sm = *reinterpret_cast<DenseSmem*>(
       (reinterpret_cast<uintptr_t>(dyn_smem) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int n_qp = (p.n_qtok + kDQ * kDQT - 1) / (kDQ * kDQT);
   const int qp = blockIdx.x % n_qp;
   const int bhq = blockIdx.x / n_qp;  // b * Hq + h
@@ -380,7 +370,7 @@ __global__ void __launch_bounds__(kDThreads, 1) dense_kernel(const __grid_consta
       mbar_init(&sm.s_full[x], 1);
       mbar_init(&sm.p_full[x], kDQ);
       mbar_init(&sm.q_full[x], kDQ);
-      mbar_init(&sm.pv_done[x], 1);
+      mbar_init(&sm.s_free[x], kDQ);
       mbar_init(&sm.o_full[x], 1);
     }
     fence_barrier_init();
@@ -422,16 +412,17 @@ __global__ void __launch_bounds__(kDThreads, 1) dense_kernel(const __grid_consta
         tma_load_2d(sm.v[s][1], &p.tmap_v, 64, row, &sm.v_full[s]);
       }
     }
-    if (warp == 9 && lane == 0) {
+    if (warp == 9) {
       // ----------------------------------------------------- MMA issuer
-      // One thread issues every MMA, alternating the Q tiles so that one
-      // tile's softmax overlaps the other tile's MMAs:
+      // One lane issues every MMA, the whole warp waits (see elect_one),
+      // alternating the Q tiles so that one tile's softmax overlaps the other
+      // tile's MMAs:
       //   S_0(0), S_1(0); for each key tile j:
       //     O_0 += P_0(j) V(j), S_0(j+1);  O_1 += P_1(j) V(j), S_1(j+1).
-      // This thread shares its SM sub-partition with busy softmax warps, so
-      // it keeps its instructions per MMA to a minimum: descriptor low
-      // words plus constants, slot counters without divisions, and barrier
-      // checks issued as non-blocking tests between MMAs.
+      // A commit covers every MMA before it, so s_full of S_x(j+1) also says
+      // that P_x(j) V(j) is complete: O_x is final and P_x's columns are free.
+      const uint32_t lead = elect_one();
+      const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
       constexpr uint32_t id_s = idesc_f16(kDQ, kDK, 0, 0);
       constexpr uint32_t id_o = idesc_f16(kDQ, kHeadDim, 0, 1);
       const uint32_t dhi = (uint32_t)(smem_desc_sw128(0, 16) >> 32);  // SBO, version, swizzle
@@ -444,114 +435,86 @@ __global__ void __launch_bounds__(kDThreads, 1) dense_kernel(const __grid_consta
       // K ring position: slot and phase of the next K part to consume
       int ks = 0;
       uint32_t kph = 0;
-      auto k_next = [&]() {
+      int hs = 0, ls = -1;  // slots of the tile whose S is issued next
+      auto k_take_part = [&](int where) -> bool {
+        if (!dwait_warp(&sm.k_full[ks], kph, p.status, where, aborted)) return false;
         if (++ks == kDKSlots) {
           ks = 0;
           kph ^= 1u;
         }
-      };
-      int hs = 0, ls = -1;  // slots of the tile whose S is issued next
-      // issues S_x = Q_x K^T (+ Q_x K_lo^T) of the current (hs, ls)
-      auto issue_s = [&](uint32_t q_lo, uint32_t d) {
-        issue_qk<0>(d, q_lo, k_lo0 + (uint32_t)hs * kSlotStep, dhi, id_s);
-        if (ls >= 0) issue_qk<1>(d, q_lo, k_lo0 + (uint32_t)ls * kSlotStep, dhi, id_s);
-      };
-      // O_x += P_x V(j), K steps 0-3 or 4-7: A = P in TMEM (columns of S_x)
-      auto issue_pv_lo = [&](uint32_t d_s, uint32_t vb, uint32_t acc0) {
-        umma_ts_off<0>(d_s + 128, d_s, vb, dhi, id_o, acc0);
-        umma_ts_off<1>(d_s + 128, d_s, vb, dhi, id_o, 1u);
-        umma_ts_off<2>(d_s + 128, d_s, vb, dhi, id_o, 1u);
-        umma_ts_off<3>(d_s + 128, d_s, vb, dhi, id_o, 1u);
-      };
-      auto issue_pv_hi = [&](uint32_t d_s, uint32_t vb) {
-        umma_ts_off<4>(d_s + 128, d_s, vb, dhi, id_o, 1u);
-        umma_ts_off<5>(d_s + 128, d_s, vb, dhi, id_o, 1u);
-        umma_ts_off<6>(d_s + 128, d_s, vb, dhi, id_o, 1u);
-        umma_ts_off<7>(d_s + 128, d_s, vb, dhi, id_o, 1u);
-      };
-      // takes the K parts of tile j (waits unless a test already saw them)
-      auto k_take = [&](bool lo, bool known_ready) -> bool {
-        hs = ks;
-        if (!known_ready && !dwait(&sm.k_full[ks], kph, p.status, 32, aborted)) return false;
-        k_next();
-        ls = -1;
-        if (lo) {
-          ls = ks;
-          if (!known_ready && !dwait(&sm.k_full[ks], kph, p.status, 33, aborted)) return false;
-          k_next();
-        }
         return true;
       };
-      auto k_test = [&](bool lo) -> bool {
-        bool ok = mbar_test(&sm.k_full[ks], kph);
-        if (lo) {
-          const int s2 = ks + 1 == kDKSlots ? 0 : ks + 1;
-          ok = mbar_test(&sm.k_full[s2], s2 == 0 ? kph ^ 1u : kph) && ok;
-        }
-        return ok;
+      auto k_take = [&](bool lo) -> bool {
+        hs = ks;
+        if (!k_take_part(32)) return false;
+        ls = lo ? ks : -1;
+        return !lo || k_take_part(33);
       };
-      const uint32_t d_s0 = tmem, d_s1 = tmem + 256;
-      bool ok = dwait(&sm.q_full[0], 0, p.status, 34, aborted) && dwait(&sm.q_full[1], 0, p.status, 34, aborted);
-      if (ok && T > 0 && k_take(sm.tlo[0] != 0, false)) {
+      // S_x = Q_x K^T (+ Q_x K_lo^T) of the current (hs, ls)
+      auto issue_s = [&](uint32_t q_lo) {
+        issue_qk<0>(lead, tm, q_lo, k_lo0 + (uint32_t)hs * kSlotStep, dhi, id_s);
+        if (ls >= 0) issue_qk<1>(lead, tm, q_lo, k_lo0 + (uint32_t)ls * kSlotStep, dhi, id_s);
+      };
+      // O_x += P_x V(j): A = P in TMEM
+      auto issue_pv = [&](uint32_t x, uint32_t vb, uint32_t acc0) {
+        const uint32_t d = tm + kTmemO + 128 * x, a = tm + kTmemP + 64 * x;
+        umma_ts_lead<0>(lead, d, a, vb, dhi, id_o, acc0);
+        umma_ts_lead<1>(lead, d, a, vb, dhi, id_o, 1u);
+        umma_ts_lead<2>(lead, d, a, vb, dhi, id_o, 1u);
+        umma_ts_lead<3>(lead, d, a, vb, dhi, id_o, 1u);
+        umma_ts_lead<4>(lead, d, a, vb, dhi, id_o, 1u);
+        umma_ts_lead<5>(lead, d, a, vb, dhi, id_o, 1u);
+        umma_ts_lead<6>(lead, d, a, vb, dhi, id_o, 1u);
+        umma_ts_lead<7>(lead, d, a, vb, dhi, id_o, 1u);
+      };
+      // S_1(j) once S_0(j) is in registers; its K slots are free after it
+      auto second_s = [&](int j) -> bool {
+        if (!dwait_warp(&sm.s_free[0], j & 1, p.status, 37, aborted)) return false;
         tc_fence_after();
-        issue_s(q_lo0, d_s0);
-        umma_commit(&sm.s_full[0]);
-        issue_s(q_lo1, d_s1);
-        umma_commit(&sm.s_full[1]);
-        umma_commit(&sm.k_empty[hs]);
-        if (ls >= 0) umma_commit(&sm.k_empty[ls]);
-        bool v_ok = false;
-        bool lo_next = T > 1 && sm.tlo[1] != 0;
-        int vs = 0;
-        uint32_t vph = 0;
-        for (int j = 0; j < T; ++j) {
-          const bool more = j + 1 < T;
-          const uint32_t vb = v_lo0 + (uint32_t)vs * kVSlotStep;
-          // ---- Q tile 0: O_0 += P_0(j) V(j), then S_0(j+1)
-          if (!dwait(&sm.p_full[0], j & 1, p.status, 35, aborted)) break;
-          if (!v_ok && !dwait(&sm.v_full[vs], vph, p.status, 36, aborted)) break;
-          tc_fence_after();
-          issue_pv_lo(d_s0, vb, j > 0);
-          const bool k_ok = more && k_test(lo_next);
-          issue_pv_hi(d_s0, vb);
-          bool pb_ok = false;
-          if (more) {
-            if (p.serial_pv) {
-              umma_commit(&sm.pv_done[0]);
-              if (!dwait(&sm.pv_done[0], j & 1, p.status, 37, aborted)) break;
-            }
-            if (!k_take(lo_next, k_ok)) break;
+        issue_s(q_lo1);
+        umma_commit_lead(lead, &sm.s_full[1]);
+        umma_commit_lead(lead, &sm.k_empty[hs]);
+        if (ls >= 0) umma_commit_lead(lead, &sm.k_empty[ls]);
+        return true;
+      };
+      bool ok = dwait_warp(&sm.q_full[0], 0, p.status, 34, aborted) &&
+                dwait_warp(&sm.q_full[1], 0, p.status, 34, aborted);
+      if (ok && T > 0 && k_take(sm.tlo[0] != 0)) {
+        tc_fence_after();
+        issue_s(q_lo0);
+        umma_commit_lead(lead, &sm.s_full[0]);
+        if (second_s(0)) {
+          int vs = 0;
+          uint32_t vph = 0;
+          for (int j = 0; j < T; ++j) {
+            const bool more = j + 1 < T;
+            const uint32_t vb = v_lo0 + (uint32_t)vs * kVSlotStep;
+            // ---- Q tile 0: O_0 += P_0(j) V(j), then S_0(j+1) once S_1(j) is in registers
+            if (!dwait_warp(&sm.p_full[0], j & 1, p.status, 35, aborted)) break;
+            if (!dwait_warp(&sm.v_full[vs], vph, p.status, 36, aborted)) break;
             tc_fence_after();
-            pb_ok = mbar_test(&sm.p_full[1], j & 1);
-            issue_s(q_lo0, d_s0);
-            umma_commit(&sm.s_full[0]);
-          }
-          // ---- Q tile 1: O_1 += P_1(j) V(j), then S_1(j+1)
-          if (!pb_ok && !dwait(&sm.p_full[1], j & 1, p.status, 38, aborted)) break;
-          tc_fence_after();
-          issue_pv_lo(d_s1, vb, j > 0);
-          const int vs_n = vs + 1 == kDVSlots ? 0 : vs + 1;
-          const uint32_t vph_n = vs_n == 0 ? vph ^ 1u : vph;
-          v_ok = more && mbar_test(&sm.v_full[vs_n], vph_n);
-          issue_pv_hi(d_s1, vb);
-          umma_commit(&sm.v_empty[vs]);
-          vs = vs_n;
-          vph = vph_n;
-          if (more) {
-            if (p.serial_pv) {
-              umma_commit(&sm.pv_done[1]);
-              if (!dwait(&sm.pv_done[1], j & 1, p.status, 39, aborted)) break;
+            issue_pv(0, vb, j > 0);
+            if (more) {
+              if (!k_take(sm.tlo[j + 1] != 0)) break;
+              if (!dwait_warp(&sm.s_free[1], j & 1, p.status, 39, aborted)) break;
               tc_fence_after();
+              issue_s(q_lo0);
+              umma_commit_lead(lead, &sm.s_full[0]);
             }
-            issue_s(q_lo1, d_s1);
-            umma_commit(&sm.s_full[1]);
-            umma_commit(&sm.k_empty[hs]);
-            if (ls >= 0) umma_commit(&sm.k_empty[ls]);
-            lo_next = j + 2 < T && sm.tlo[j + 2] != 0;
+            // ---- Q tile 1: O_1 += P_1(j) V(j), then S_1(j+1)
+            if (!dwait_warp(&sm.p_full[1], j & 1, p.status, 38, aborted)) break;
+            tc_fence_after();
+            issue_pv(1, vb, j > 0);
+            umma_commit_lead(lead, &sm.v_empty[vs]);
+            if (++vs == kDVSlots) {
+              vs = 0;
+              vph ^= 1u;
+            }
+            if (more && !second_s(j + 1)) break;
           }
         }
-        umma_commit(&sm.o_full[0]);
-        umma_commit(&sm.o_full[1]);
+        umma_commit_lead(lead, &sm.o_full[0]);
+        umma_commit_lead(lead, &sm.o_full[1]);
       }
     }
   } else {
@@ -585,7 +548,7 @@ __global__ void __launch_bounds__(kDThreads, 1) dense_kernel(const __grid_consta
       softmax_bar();
     }
     const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
-    const uint32_t s_col = x * 256, o_col = x * 256 + 128;
+    const uint32_t p_col = kTmemP + 64 * x, o_col = kTmemO + 128 * x;
     const float sl2 = p.scale_log2;
     float m_ref = kDNegInf, l = 0.f;
     float ls[MAXSEG];
@@ -596,90 +559,40 @@ __global__ void __launch_bounds__(kDThreads, 1) dense_kernel(const __grid_consta
       if (!dwait_warp(&sm.s_full[x], j & 1, p.status, 40, aborted)) break;
       tc_fence_after();
       const int vld = sm.valid[j];
-      uint32_t pk[2][32];
-      float sum[4];
-      // One pass: P = 2^(S sl2 - m_ref) with the current reference max while
-      // the tile max is taken alongside (no max -> exp dependency). Redone,
-      // from S reloaded out of TMEM (P is not stored yet), for the first
-      // tile and whenever a row's max grows by more than 8 (P <= 2^8).
-      bool redo = !__all_sync(0xffffffffu, m_ref != kDNegInf);
-      if (!redo) {
-        uint32_t sr[4][32];
+      uint32_t sr[4][32];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) tmem_ld32(tmem + lane_off + s_col + 32 * c, sr[c]);
-        tmem_wait_ld();
-        if (vld < kDK) {
+      for (int c = 0; c < 4; ++c) tmem_ld32(tmem + lane_off + 32 * c, sr[c]);
+      tmem_wait_ld();
+      tc_fence_before();
+      mbar_arrive(&sm.s_free[x]);  // the other tile's S may take the columns
+      if (vld < kDK) {
 #pragma unroll
-          for (int c = 0; c < kDK; ++c)
-            if (c >= vld) sr[c >> 5][c & 31] = __float_as_uint(kDNegInf);
-        }
-        const uint64_t nm2 = f2_pack(-m_ref, -m_ref);
-        float mx[4] = {kDNegInf, kDNegInf, kDNegInf, kDNegInf};
-        uint64_t acc[2] = {0ull, 0ull};
-#pragma unroll
-        for (int c2 = 0; c2 < kDK / 2; ++c2) {
-          const float s0 = __uint_as_float(sr[(2 * c2) >> 5][(2 * c2) & 31]);
-          const float s1 = __uint_as_float(sr[(2 * c2 + 1) >> 5][(2 * c2 + 1) & 31]);
-          mx[c2 & 3] = fmax3(mx[c2 & 3], s0, s1);
-          float e0, e1;
-          f2_unpack(f2_fma(f2_pack(s0, s1), sl2_2, nm2), e0, e1);
-          const float a = ex2_approx(e0), bb = ex2_approx(e1);
-          acc[c2 & 1] = f2_add(acc[c2 & 1], f2_pack(a, bb));
-          pk[c2 >> 5][c2 & 31] = pack_f16(a, bb);
-        }
-        const float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
-        f2_unpack(acc[0], sum[0], sum[1]);
-        f2_unpack(acc[1], sum[2], sum[3]);
-        redo = __any_sync(0xffffffffu, tmax > m_ref + 8.f);
+        for (int c = 0; c < kDK; ++c)
+          if (c >= vld) sr[c >> 5][c & 31] = __float_as_uint(kDNegInf);
       }
-      if (redo) {
-        uint32_t sr[4][32];
+      float mx[4] = {kDNegInf, kDNegInf, kDNegInf, kDNegInf};
 #pragma unroll
-        for (int c = 0; c < 4; ++c) tmem_ld32(tmem + lane_off + s_col + 32 * c, sr[c]);
-        tmem_wait_ld();
-        if (vld < kDK) {
-#pragma unroll
-          for (int c = 0; c < kDK; ++c)
-            if (c >= vld) sr[c >> 5][c & 31] = __float_as_uint(kDNegInf);
-        }
-        float mx[4] = {kDNegInf, kDNegInf, kDNegInf, kDNegInf};
-#pragma unroll
-        for (int c2 = 0; c2 < kDK / 2; ++c2)
-          mx[c2 & 3] = fmax3(mx[c2 & 3], __uint_as_float(sr[(2 * c2) >> 5][(2 * c2) & 31]),
-                             __uint_as_float(sr[(2 * c2 + 1) >> 5][(2 * c2 + 1) & 31]));
-        const float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
-        // lazy rescale: the reference max moves only when the tile's max
-        // exceeds it by more than 8; O in TMEM, final since the previous
-        // P V completed before S of this tile, is rescaled warp-wide
-        const bool grow = tmax > m_ref + 8.f;
+      for (int c2 = 0; c2 < kDK / 2; ++c2)
+        mx[c2 & 3] = fmax3(mx[c2 & 3], __uint_as_float(sr[(2 * c2) >> 5][(2 * c2) & 31]),
+                           __uint_as_float(sr[(2 * c2 + 1) >> 5][(2 * c2 + 1) & 31]));
+      const float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
+      // lazy rescale: the reference max moves only when the tile's max exceeds
+      // it by more than 8 (P <= 2^8); O in TMEM, final since P V of the last
+      // key tile completed before this S, is then rescaled warp-wide
+      const bool grow = tmax > m_ref + 8.f;
+      if (__any_sync(0xffffffffu, grow)) {
         const float m_new = grow ? tmax : m_ref;
         const bool need_o = grow && m_ref != kDNegInf;
-        const float mb = (m_new == kDNegInf) ? 0.f : m_new;
-        const uint64_t nm2 = f2_pack(-mb, -mb);
-        uint64_t acc[2] = {0ull, 0ull};
-#pragma unroll
-        for (int c2 = 0; c2 < kDK / 2; ++c2) {
-          float e0, e1;
-          f2_unpack(f2_fma(f2_pack(__uint_as_float(sr[(2 * c2) >> 5][(2 * c2) & 31]),
-                                   __uint_as_float(sr[(2 * c2 + 1) >> 5][(2 * c2 + 1) & 31])),
-                           sl2_2, nm2),
-                    e0, e1);
-          const float a = ex2_approx(e0), bb = ex2_approx(e1);
-          acc[c2 & 1] = f2_add(acc[c2 & 1], f2_pack(a, bb));
-          pk[c2 >> 5][c2 & 31] = pack_f16(a, bb);
-        }
-        f2_unpack(acc[0], sum[0], sum[1]);
-        f2_unpack(acc[1], sum[2], sum[3]);
         if (__any_sync(0xffffffffu, need_o)) {
           const float alpha = need_o ? ex2_approx(m_ref - m_new) : 1.f;
 #pragma unroll 1
-          for (int cb = 0; cb < 4; ++cb) {
-            uint32_t o[32];
-            tmem_ld32(tmem + lane_off + o_col + cb * 32, o);
+          for (int cb = 0; cb < 8; ++cb) {
+            uint32_t o[16];
+            tmem_ld16(tmem + lane_off + o_col + cb * 16, o);
             tmem_wait_ld();
 #pragma unroll
-            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-            tmem_st32(tmem + lane_off + o_col + cb * 32, o);
+            for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+            tmem_st16(tmem + lane_off + o_col + cb * 16, o);
           }
           l *= alpha;
 #pragma unroll
@@ -687,8 +600,26 @@ __global__ void __launch_bounds__(kDThreads, 1) dense_kernel(const __grid_consta
         }
         m_ref = m_new;
       }
-      tmem_st32(tmem + lane_off + s_col, pk[0]);
-      tmem_st32(tmem + lane_off + s_col + 32, pk[1]);
+      const float mb = (m_ref == kDNegInf) ? 0.f : m_ref;
+      const uint64_t nm2 = f2_pack(-mb, -mb);
+      uint32_t pk[2][32];
+      float sum[4];
+      uint64_t acc[2] = {0ull, 0ull};
+#pragma unroll
+      for (int c2 = 0; c2 < kDK / 2; ++c2) {
+        float e0, e1;
+        f2_unpack(f2_fma(f2_pack(__uint_as_float(sr[(2 * c2) >> 5][(2 * c2) & 31]),
+                                 __uint_as_float(sr[(2 * c2 + 1) >> 5][(2 * c2 + 1) & 31])),
+                         sl2_2, nm2),
+                  e0, e1);
+        const float a = ex2_approx(e0), bb = ex2_approx(e1);
+        acc[c2 & 1] = f2_add(acc[c2 & 1], f2_pack(a, bb));
+        pk[c2 >> 5][c2 & 31] = pack_f16(a, bb);
+      }
+      f2_unpack(acc[0], sum[0], sum[1]);
+      f2_unpack(acc[1], sum[2], sum[3]);
+      tmem_st32(tmem + lane_off + p_col, pk[0]);
+      tmem_st32(tmem + lane_off + p_col + 32, pk[1]);
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive(&sm.p_full[x]);

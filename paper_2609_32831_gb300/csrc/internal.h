@@ -262,7 +262,6 @@ struct DenseParams {
   DevStatus* status;
   int64_t rows_per_bh, lo_rows_per_bh;
   int n_tiles, nseg, batch, n_kv_heads, n_q_heads, n_qtok, group;
-  int serial_pv;  // 1: wait for P V of a Q tile before its next Q K^T
   float scale_log2;
 };
 

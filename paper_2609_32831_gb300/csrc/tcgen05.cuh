@@ -26,8 +26,36 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
+// One lane of a converged warp. The MMA warps run their loops with all 32
+// lanes and predicate the issuing instructions on this lane: in warp-uniform
+// control flow the descriptors stay in uniform registers. Issued from a
+// branch of one lane instead, every MMA first moved its operands over, and an
+// M = N = 128 MMA took 130 cycles of the issuing thread against 86 on the
+// tensor pipe.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n"
+      ".reg .pred q;\n"
+      "elect.sync _|q, 0xffffffff;\n"
+      "selp.u32 %0, 1, 0, q;\n"
+      "}\n"
+      : "=r"(p));
+  return p;
+}
+
 // Arrive once on an mbarrier when every tcgen05.mma issued so far by this
-// thread has completed.
+// thread has completed (`lead`: the lane that issues).
+__device__ __forceinline__ void umma_commit_lead(uint32_t lead, uint64_t* bar) {
+  asm volatile(
+      "{\n"
+      ".reg .pred q;\n"
+      "setp.ne.b32 q, %1, 0;\n"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+      "}\n" ::"r"(smem_u32(bar)),
+      "r"(lead)
+      : "memory");
+}
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                    smem_u32(bar))
@@ -57,6 +85,23 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
       "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]),
       "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]),
       "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+}
+
+// 16 consecutive 32-bit TMEM columns of this thread's lane.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
 
@@ -108,24 +153,45 @@ __device__ __forceinline__ void umma_ss_off(uint32_t d_tmem, uint32_t a_lo, uint
       "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "n"(OA), "n"(OB), "n"(ACC)
       : "memory");
 }
-template <int KK>
-__device__ __forceinline__ void umma_ts_off(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc,
-                                            uint32_t acc) {
+// The same from a converged warp, one lane issuing; A from shared memory (ss)
+// or tensor memory (ts).
+template <int OA, int OB, int ACC>
+__device__ __forceinline__ void umma_ss_lead(uint32_t lead, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
+                                             uint32_t idesc) {
   asm volatile(
       "{\n"
-      ".reg .pred p;\n"
+      ".reg .pred p, q;\n"
+      ".reg .b32 al, bl;\n"
+      ".reg .b64 da, db;\n"
+      "setp.ne.b32 q, %8, 0;\n"
+      "add.u32 al, %1, %5;\n"
+      "add.u32 bl, %2, %6;\n"
+      "setp.ne.b32 p, %7, 0;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n"
+      "}\n" ::"r"(d_tmem),
+      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "n"(OA), "n"(OB), "n"(ACC), "r"(lead)
+      : "memory");
+}
+template <int KK>
+__device__ __forceinline__ void umma_ts_lead(uint32_t lead, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo,
+                                             uint32_t hi, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n"
+      ".reg .pred p, q;\n"
       ".reg .b32 at, bl;\n"
       ".reg .b64 db;\n"
+      "setp.ne.b32 q, %8, 0;\n"
       "add.u32 at, %1, %5;\n"
       "add.u32 bl, %2, %6;\n"
       "setp.ne.b32 p, %7, 0;\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p;\n"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p;\n"
       "}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "n"(8 * KK), "n"(128 * KK), "r"(acc)
+      "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "n"(8 * KK), "n"(128 * KK), "r"(acc), "r"(lead)
       : "memory");
 }
-
 
 // Instruction descriptor, kind::f16 with bf16 A and B, fp32 D.
 __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n, int a_mn_major, int b_mn_major) {

@@ -63,15 +63,16 @@ __device__ __forceinline__ bool sc_wait_warp(uint64_t* bar, uint32_t parity, Dev
 // 32 B inside their 128-B swizzled rows, then jump to their second channel
 // half (offsets in units of 16 B).
 template <int AH, int BH>
-__device__ __forceinline__ void sc_issue(uint32_t d, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc) {
-  umma_ss_off<0, 0, 0>(d, a_lo, b_lo, hi, idesc);
-  umma_ss_off<2, 2, 1>(d, a_lo, b_lo, hi, idesc);
-  umma_ss_off<4, 4, 1>(d, a_lo, b_lo, hi, idesc);
-  umma_ss_off<6, 6, 1>(d, a_lo, b_lo, hi, idesc);
-  umma_ss_off<AH, BH, 1>(d, a_lo, b_lo, hi, idesc);
-  umma_ss_off<AH + 2, BH + 2, 1>(d, a_lo, b_lo, hi, idesc);
-  umma_ss_off<AH + 4, BH + 4, 1>(d, a_lo, b_lo, hi, idesc);
-  umma_ss_off<AH + 6, BH + 6, 1>(d, a_lo, b_lo, hi, idesc);
+__device__ __forceinline__ void sc_issue(uint32_t lead, uint32_t d, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
+                                         uint32_t idesc) {
+  umma_ss_lead<0, 0, 0>(lead, d, a_lo, b_lo, hi, idesc);
+  umma_ss_lead<2, 2, 1>(lead, d, a_lo, b_lo, hi, idesc);
+  umma_ss_lead<4, 4, 1>(lead, d, a_lo, b_lo, hi, idesc);
+  umma_ss_lead<6, 6, 1>(lead, d, a_lo, b_lo, hi, idesc);
+  umma_ss_lead<AH, BH, 1>(lead, d, a_lo, b_lo, hi, idesc);
+  umma_ss_lead<AH + 2, BH + 2, 1>(lead, d, a_lo, b_lo, hi, idesc);
+  umma_ss_lead<AH + 4, BH + 4, 1>(lead, d, a_lo, b_lo, hi, idesc);
+  umma_ss_lead<AH + 6, BH + 6, 1>(lead, d, a_lo, b_lo, hi, idesc);
 }
 
 // Both passes on the 5th-generation tensor cores, bf16 operands, fp32 in
@@ -91,7 +92,7 @@ __global__ void __launch_bounds__(kScThreads, 1) score_kernel(const __grid_const
   extern __shared__ uint8_t dyn_smem[];
   ScoreSmem& sm = *reinterpret_cast<ScoreSmem*>(
       (reinterpret_cast<uintptr_t>(dyn_smem) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int bh = blockIdx.x / a.chunks, chunk = blockIdx.x % a.chunks;
   const int b = bh / a.n_kv_heads, kvh = bh % a.n_kv_heads;
   const int group = a.n_q_heads / a.n_kv_heads;
@@ -153,30 +154,39 @@ __global__ void __launch_bounds__(kScThreads, 1) score_kernel(const __grid_const
       }
     }
   } else if (warp == kScMmaWarp) {
-    if (lane == 0) {
-      // ------------------------------------------------------ MMA issue
-      const uint32_t hi = (uint32_t)(smem_desc_sw128(0, 16) >> 32);
-      const uint32_t q_lo = (uint32_t)smem_desc_sw128(smem_u32(sm.q[0]), 16);
-      const int xt = (a.rows + 127) / 128;  // query-row tiles of pass 1
-      uint32_t seq = 0;
-      for (int t = t_begin; t < t_end; ++t, ++seq) {
-        const int slot = seq % kScStages, buf = seq & 1;
-        if (!mbar_wait(&sm.k_full[slot], (seq / kScStages) & 1, a.status, 22)) break;
-        if (seq >= 2 && !mbar_wait(&sm.s_free[buf], ((seq >> 1) - 1) & 1, a.status, 23)) break;
-        tc_fence_after();
-        const uint32_t k_lo = (uint32_t)smem_desc_sw128(smem_u32(sm.k[slot][0]), 16);
-        const uint32_t d = tmem + buf * 256;
-        if (!PASS2) {
-          constexpr uint32_t id = idesc_bf16(128, kScTile, 0, 0);
-          // Q rows 128x .. : 16 KB further in each channel half (32 KB apart)
-          sc_issue<2048, 1024>(d, q_lo, k_lo, hi, id);
-          if (xt > 1) sc_issue<2048, 1024>(d + 128, q_lo + (16384 >> 4), k_lo, hi, id);
-        } else {
-          constexpr uint32_t id = idesc_bf16(kScTile, kScMaxRows, 0, 0);
-          sc_issue<1024, 2048>(d, k_lo, q_lo, hi, id);
-        }
-        umma_commit(&sm.k_empty[slot]);
-        umma_commit(&sm.s_full[buf]);
+    // -------------------------------------------------------- MMA issue
+    // (one lane issues, the whole warp waits: see elect_one)
+    const uint32_t lead = elect_one();
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t hi = (uint32_t)(smem_desc_sw128(0, 16) >> 32);
+    const uint32_t q_lo = (uint32_t)smem_desc_sw128(smem_u32(sm.q[0]), 16);
+    const uint32_t k_lo0 = (uint32_t)smem_desc_sw128(smem_u32(sm.k[0][0]), 16);
+    constexpr uint32_t kSlotStep = sizeof(sm.k[0]) >> 4;  // descriptor units per K slot
+    const int xt = (a.rows + 127) / 128;  // query-row tiles of pass 1
+    uint32_t seq = 0;
+    int slot = 0;
+    uint32_t kph = 0;
+    for (int t = t_begin; t < t_end; ++t, ++seq) {
+      const int buf = seq & 1;
+      if (!sc_wait_warp(&sm.k_full[slot], kph, a.status, 22, aborted)) break;
+      if (seq >= 2 && !sc_wait_warp(&sm.s_free[buf], ((seq >> 1) - 1) & 1, a.status, 23, aborted)) break;
+      tc_fence_after();
+      const uint32_t k_lo = k_lo0 + (uint32_t)slot * kSlotStep;
+      const uint32_t d = tm + buf * 256;
+      if (!PASS2) {
+        constexpr uint32_t id = idesc_bf16(128, kScTile, 0, 0);
+        // Q rows 128x .. : 16 KB further in each channel half (32 KB apart)
+        sc_issue<2048, 1024>(lead, d, q_lo, k_lo, hi, id);
+        if (xt > 1) sc_issue<2048, 1024>(lead, d + 128, q_lo + (16384 >> 4), k_lo, hi, id);
+      } else {
+        constexpr uint32_t id = idesc_bf16(kScTile, kScMaxRows, 0, 0);
+        sc_issue<1024, 2048>(lead, d, k_lo, q_lo, hi, id);
+      }
+      umma_commit_lead(lead, &sm.k_empty[slot]);
+      umma_commit_lead(lead, &sm.s_full[buf]);
+      if (++slot == kScStages) {
+        slot = 0;
+        kph ^= 1u;
       }
     }
   } else {

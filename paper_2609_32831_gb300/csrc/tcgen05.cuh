@@ -56,11 +56,6 @@ __device__ __forceinline__ void umma_commit_lead(uint32_t lead, uint64_t* bar) {
       "r"(lead)
       : "memory");
 }
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
-}
 
 // 32 consecutive 32-bit TMEM columns of this thread's lane.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -130,31 +125,11 @@ __host__ __device__ constexpr uint32_t idesc_f16(int m, int n, int a_mn_major, i
          ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-// tcgen05.mma kind::f16 issued by one thread, D in TMEM: A and B from
-// shared memory (ss) or A from TMEM (ts). Descriptors are given as the low
-// 32-bit words of their bases (start address field + leading offset) and a shared high word;
-// each K step's offset (bytes >> 4) is an immediate added inside, so the
-// issuing thread keeps only the base words in registers.
-template <int OA, int OB, int ACC>
-__device__ __forceinline__ void umma_ss_off(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
-                                            uint32_t idesc) {
-  asm volatile(
-      "{\n"
-      ".reg .pred p;\n"
-      ".reg .b32 al, bl;\n"
-      ".reg .b64 da, db;\n"
-      "add.u32 al, %1, %5;\n"
-      "add.u32 bl, %2, %6;\n"
-      "setp.ne.b32 p, %7, 0;\n"
-      "mov.b64 da, {al, %3};\n"
-      "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n"
-      "}\n" ::"r"(d_tmem),
-      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "n"(OA), "n"(OB), "n"(ACC)
-      : "memory");
-}
-// The same from a converged warp, one lane issuing; A from shared memory (ss)
-// or tensor memory (ts).
+// tcgen05.mma kind::f16 from a converged warp, issued by its lane `lead`; D
+// in TMEM, A from shared memory (ss) or TMEM (ts), B from shared memory.
+// Descriptors are given as the low 32-bit words of their bases (start address
+// field + leading offset) and a shared high word; each K step's offset (bytes
+// >> 4) is an immediate.
 template <int OA, int OB, int ACC>
 __device__ __forceinline__ void umma_ss_lead(uint32_t lead, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
                                              uint32_t idesc) {

@@ -36,16 +36,35 @@ struct ScoreSmem {
   uint8_t k[kScStages][2][kScTile * 128];
   float part[2][2][kScTile];      // pass 2: per pair, the second half's key sums (double-buffered)
   float2 ml[2][kScMaxRows];       // pass 1: (max, sum) of each row's two key halves
-  float lse2[kScMaxRows];
+  alignas(16) float nlse2[kScMaxRows];  // pass 2: minus the rows' log2-sum-exp, -inf past the window
   uint64_t k_full[kScStages], k_empty[kScStages];
   uint64_t s_full[2], s_free[2];
   uint32_t tmem_base;
 };
 
-__device__ __forceinline__ float fmax3(float a, float b, float c) {
-  float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
+// sum over 32 logits (two per packed FMA and add) of 2^(x sl2 + bias); bias:
+// one pair for all (nm) or a pair per two columns from shared memory.
+template <bool PER_COL>
+__device__ __forceinline__ float exp_sum32(const uint32_t (&x)[32], uint64_t sl2, uint64_t nm, const float* bias) {
+  uint64_t acc[2] = {0ull, 0ull};
+#pragma unroll
+  for (int e = 0; e < 32; e += 4) {
+    uint64_t b0 = nm, b1 = nm;
+    if constexpr (PER_COL) {
+      const float4 v = *reinterpret_cast<const float4*>(bias + e);
+      b0 = f2_pack(v.x, v.y);
+      b1 = f2_pack(v.z, v.w);
+    }
+    float e0, e1, e2, e3;
+    f2_unpack(f2_fma(f2_pack(__uint_as_float(x[e]), __uint_as_float(x[e + 1])), sl2, b0), e0, e1);
+    f2_unpack(f2_fma(f2_pack(__uint_as_float(x[e + 2]), __uint_as_float(x[e + 3])), sl2, b1), e2, e3);
+    acc[0] = f2_add(acc[0], f2_pack(ex2_approx(e0), ex2_approx(e1)));
+    acc[1] = f2_add(acc[1], f2_pack(ex2_approx(e2), ex2_approx(e3)));
+  }
+  float s0, s1, s2, s3;
+  f2_unpack(acc[0], s0, s1);
+  f2_unpack(acc[1], s2, s3);
+  return (s0 + s1) + (s2 + s3);
 }
 
 __device__ __forceinline__ void sc_sync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
@@ -128,7 +147,7 @@ __global__ void __launch_bounds__(kScThreads, 1) score_kernel(const __grid_const
     }
     if (PASS2)
       for (int r = threadIdx.x; r < kScMaxRows; r += 32 * kScCompute)
-        sm.lse2[r] = r < a.rows ? a.lse2[(size_t)bh * rows_pad + r] : INFINITY;
+        sm.nlse2[r] = r < a.rows ? -a.lse2[(size_t)bh * rows_pad + r] : -INFINITY;
     fence_proxy_async_smem();
   }
   tc_fence_before();
@@ -195,10 +214,15 @@ __global__ void __launch_bounds__(kScThreads, 1) score_kernel(const __grid_const
     // (every other tile), so one pair's tensor-memory loads overlap the
     // other pair's exp2 work. Pass 1: warpgroup w takes row tile w % 2 of its
     // pair's tiles; pass 2: the query rows (columns of S^T) 128 (w % 2) ..
-    // 128 (w % 2) + 127. Each tile is read in two 64-column chunks.
+    // 128 (w % 2) + 127. Each tile is read in 32-column chunks, the next one on
+    // its way while this one is summed; S goes back to the MMA warp before
+    // the last chunk's sums. (With 64-column chunks, each loaded, waited for
+    // and then summed with one FMA and add per logit, S handed back after
+    // the sums, a 32K layer of batch 16 took 294 us.)
     const int wg = warp >> 2, par = wg >> 1, hw = wg & 1;
     const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
     const float sl2 = a.scale_log2;
+    const uint64_t sl2_2 = f2_pack(sl2, sl2);
     if (!PASS2) {
       const int row = hw * 128 + 32 * (warp & 3) + lane;  // query row = TMEM lane of S tile hw
       const bool active = hw * 128 + 32 * (warp & 3) < a.rows;
@@ -209,48 +233,48 @@ __global__ void __launch_bounds__(kScThreads, 1) score_kernel(const __grid_const
         if (!sc_wait_warp(&sm.s_full[buf], (seq >> 1) & 1, a.status, 24, aborted)) break;
         tc_fence_after();
         const int valid_t = min(kScTile, a.n_ctx - t * kScTile);
-        if (active) {
-#pragma unroll 1
-          for (int kh = 0; kh < 2; ++kh) {
-            const int valid = valid_t - 64 * kh;
-            if (valid <= 0) break;
-            uint32_t sr[2][32];
+        auto release = [&]() {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sm.s_free[buf]);
+        };
+        if (!active) {
+          release();
+          continue;
+        }
+        const uint32_t col0 = tmem + lane_off + buf * 256 + hw * 128;
+        uint32_t sr[2][32];
+        tmem_ld32(col0, sr[0]);
+        tmem_wait_ld32(sr[0]);
 #pragma unroll
-            for (int c = 0; c < 2; ++c) tmem_ld32(tmem + lane_off + buf * 256 + hw * 128 + kh * 64 + 32 * c, sr[c]);
-            tmem_wait_ld();
-            // the chunk's max on the raw logits (sl2 > 0), two per 3-input max
-            if (valid < 64) {
+        for (int c = 0; c < 4; ++c) {
+          uint32_t(&x)[32] = sr[c & 1];
+          if (c < 3)
+            tmem_ld32(col0 + 32 * (c + 1), sr[(c + 1) & 1]);
+          else
+            release();
+          const int valid = valid_t - 32 * c;
+          if (valid > 0) {
+            if (valid < 32) {
 #pragma unroll
-              for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int e = 0; e < 32; ++e)
-                  if (32 * c + e >= valid) sr[c][e] = __float_as_uint(-INFINITY);
+              for (int e = 0; e < 32; ++e)
+                if (e >= valid) x[e] = __float_as_uint(-INFINITY);
             }
+            // the chunk's max on the raw logits (sl2 > 0), two per 3-input max
             float mr[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-              for (int e = 0; e < 32; e += 2)
-                mr[c] = fmax3(mr[c], __uint_as_float(sr[c][e]), __uint_as_float(sr[c][e + 1]));
+            for (int e = 0; e < 32; e += 2)
+              mr[(e >> 1) & 1] = fmax3(mr[(e >> 1) & 1], __uint_as_float(x[e]), __uint_as_float(x[e + 1]));
             const float mx = fmaxf(mr[0], mr[1]) * sl2;
             // reference max moved only when exceeded by more than 8
             if (mx > m_ref + 8.f) {
               l = (m_ref == -INFINITY) ? 0.f : l * ex2_approx(m_ref - mx);
               m_ref = mx;
             }
-            const float nm = -m_ref;
-            float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-              for (int e = 0; e < 32; ++e)
-                acc[(c << 1) | (e & 1)] += ex2_approx(fmaf(__uint_as_float(sr[c][e]), sl2, nm));
-            l += (acc[0] + acc[1]) + (acc[2] + acc[3]);
+            l += exp_sum32<false>(x, sl2_2, f2_pack(-m_ref, -m_ref), nullptr);
           }
+          if (c < 3) tmem_wait_ld32(sr[(c + 1) & 1]);
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.s_free[buf]);
       }
       // the row's two pairs meet in shared memory
       sm.ml[par][row] = make_float2(m_ref, l);
@@ -274,27 +298,28 @@ __global__ void __launch_bounds__(kScThreads, 1) score_kernel(const __grid_const
         const bool ok = sc_wait_warp(&sm.s_full[buf], (seq >> 1) & 1, a.status, 25, aborted);
         tc_fence_after();
         float sum = 0.f;
-        if (ok) {
-#pragma unroll 1
-          for (int ch = 0; ch < 2; ++ch) {
-            const int col0 = 128 * hw + 64 * ch;  // query rows of this chunk (lse = +inf past the window)
-            if (col0 >= a.rows) break;
-            uint32_t sr[2][32];
+        // query rows (columns of S^T) of this warpgroup in chunks of 32 (lse =
+        // +inf past the window); chunks wholly past it are skipped
+        const int chunks = ok ? min(4, (a.rows - 128 * hw + 31) / 32) : 0;
+        const uint32_t col0 = tmem + lane_off + buf * 256 + 128 * hw;
+        uint32_t sr[2][32];
+        if (chunks > 0) {
+          tmem_ld32(col0, sr[0]);
+          tmem_wait_ld32(sr[0]);
+        }
 #pragma unroll
-            for (int c = 0; c < 2; ++c) tmem_ld32(tmem + lane_off + buf * 256 + col0 + 32 * c, sr[c]);
-            tmem_wait_ld();
-            float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-              for (int e = 0; e < 32; ++e)
-                acc[(c << 1) | (e & 1)] += ex2_approx(fmaf(__uint_as_float(sr[c][e]), sl2, -sm.lse2[col0 + 32 * c + e]));
-            sum += (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        for (int c = 0; c < 4; ++c) {
+          if (c < chunks) {
+            if (c + 1 < chunks) tmem_ld32(col0 + 32 * (c + 1), sr[(c + 1) & 1]);
+            sum += exp_sum32<true>(sr[c & 1], sl2_2, 0ull, &sm.nlse2[128 * hw + 32 * c]);
+            if (c + 1 < chunks) tmem_wait_ld32(sr[(c + 1) & 1]);
+          }
+          if (c == 2) {  // every chunk is in registers
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.s_free[buf]);
           }
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.s_free[buf]);
         // the pair's two row halves of the key meet in shared memory (double
         // buffered: one warpgroup of the pair is at most one tile ahead)
         const int pb = (seq >> 1) & 1;

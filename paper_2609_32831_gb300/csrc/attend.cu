@@ -11,10 +11,9 @@
 // warps compute with mma.sync m16n8k16:
 //   bf16 rows:  S = Q K^T in bf16 (exact products), P split into bf16 hi + lo
 //               parts so P V keeps ~16 mantissa bits;
-//   packed:     each pair of codes -> an exact fp16 pair 2^(10-B) + code with
-//               one LOP3 (magic-number trick; the offset is removed exactly
-//               by small extra MMAs), scales folded into the queries (keys)
-//               and the probabilities (values), S and P V in fp16 with fp32
+//   packed:     each pair of codes -> an exact pair of (subnormal) fp16 values
+//               with one LOP3, scales folded into the queries (keys) and the
+//               probabilities (values), S and P V in fp16 with fp32
 //               accumulation.
 // Each item leaves an unnormalised partial (O, m, l); the last CTA to finish
 // a (sequence, KV head) merges its items by log-sum-exp, writes O, lse and
@@ -408,6 +407,16 @@ __device__ __forceinline__ void state_init(WarpState<NTW>& st) {
   }
 }
 
+template <int NTW>
+__device__ __forceinline__ void scale_o(WarpState<NTW>& st, float f) {
+#pragma unroll
+  for (int nt = 0; nt < NTW; ++nt)
+#pragma unroll
+    for (int mt = 0; mt < 8; ++mt)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) st.o[nt][mt][e] *= f;
+}
+
 // Online softmax over NB 16-key blocks: x[blk][nt][e] (e: 0/1 key g, 2/3 key
 // g+8; e & 1 selects the row), in log2 units. Writes probabilities into pr.
 // The reference max m moves only when a row's max exceeds it by more than
@@ -543,102 +552,112 @@ __device__ __forceinline__ void block_bf16(WarpState<NTW>& st, uint32_t qs,
 //
 // A code word holds 16 int2 or 8 int4 codes as pairs: pair p is the code at
 // bit p * BITS of the low half and the one at the same bit of the high half.
-// One LOP3 turns a pair into the exact fp16 pair (2^(10-B) + a, 2^(10-B) + b)
-// when both codes sit at mantissa bit B (OR-ing exponent 25 - B). Shifted
-// copies of the word bring every pair to such a bit:
-//   int2  L = w << 6, M = w, R = w >> 6:  p0 L@6, p1 L@8, p2 M@4, p3 M@6,
-//                                         p4 M@8, p5 R@4, p6 R@6, p7 R@8
-//   int4  L = w << 4, M = w, R = w >> 4, R2 = w >> 8: p0..p3 at bit 4
-// (bits that a shift moves across the half boundary fall outside the masks).
-// The offset 2^(10-B) (64, 16 or 4) is removed exactly by extra MMAs with
-// fp16 powers of two, so no rounded zero-point absorbs it.
+// Masking a (shifted) copy of the word leaves the codes in the mantissas of
+// two subnormal fp16 values: a code at bit B is exactly code * 2^(B - 24), one
+// LOP3 per pair and no offset to remove. The tensor cores take subnormal
+// operands as they are; the powers of two are put right elsewhere:
+//   keys    the query of the pair's channels carries 2^(4 - B) and the logit
+//           scale 2^20: int2 copies w << 6, w, w >> 6 with codes at bits 4, 6,
+//           8 (queries times 1, 1/4, 1/16: none overflows for it), int4 copies
+//           w << 4, w, w >> 4, w >> 8 with every code at bit 4 (a query times
+//           1/16 would leave its fp16 lo part too few bits beside codes up to
+//           15: lse of 8192 tokens 3.7e-7 off instead of 4.3e-8);
+//   values  one HFMA2 per pair centres the codes and brings every pair to
+//           2^-9 (code - C): copies w and w >> 10 (int2) or w >> 8 (int4).
+// (With the exponent 2^(10-B) OR-ed in instead, each pair carried an offset of
+// 64, 16 or 4 through the fp32 accumulators, removed by extra rows of the beta
+// MMAs; value copies took two or three shifts per word. One 32K layer, batch
+// 16: int2 70.1 us, now 67.0; lse of 8192 tokens 2.7e-7 (int2) and 1.2e-7
+// (int4) off, now 4.8e-8 and 4.3e-8.)
 template <int BITS>
-struct Words {
+struct KeyWords {
   uint32_t l, m, r, r2;
 };
-
 template <int BITS>
-__device__ __forceinline__ Words<BITS> words(uint32_t w) {
+__device__ __forceinline__ KeyWords<BITS> key_words(uint32_t w) {
   if constexpr (BITS == 2)
-    return Words<BITS>{w << 6, w, w >> 6, 0u};
+    return KeyWords<BITS>{w << 6, w, w >> 6, 0u};
   else
-    return Words<BITS>{w << 4, w, w >> 4, w >> 8};
+    return KeyWords<BITS>{w << 4, w, w >> 4, w >> 8};
 }
 
-template <int BITS, int P>
-struct PairAt {
-  // bit of the pair in its source copy and the offset 2^(10 - bit)
-  static constexpr int kBit = BITS == 4 ? 4 : (P % 3 == 2 ? 4 : (P % 3 == 0 ? 6 : 8));
-  static constexpr int kOff = 1 << (10 - kBit);
-};
+// Bit of key pair p in its copy and the class of the pair's channels: queries
+// scaled by 1 / class_scale.
+constexpr int kKeyBit0 = 4;
+template <int BITS>
+__host__ __device__ constexpr int key_bit(int p) {
+  return BITS == 4 ? 4 : (p % 3 == 2 ? 4 : (p % 3 == 0 ? 6 : 8));
+}
+template <int BITS>
+__host__ __device__ constexpr int key_classes() { return BITS == 4 ? 1 : 3; }
+template <int BITS>
+__host__ __device__ constexpr int key_class(int p) { return (key_bit<BITS>(p) - kKeyBit0) / 2; }
+__host__ __device__ constexpr float class_scale(int c) { return (float)(1 << (2 * c)); }  // 2^(B - 4)
 
 template <int BITS, int P>
-__device__ __forceinline__ uint32_t pair_h2(const Words<BITS>& c) {
-  constexpr int B = PairAt<BITS, P>::kBit;
-  constexpr uint32_t qmax = (1u << BITS) - 1u;
-  constexpr uint32_t mask = (qmax << B) | (qmax << (B + 16));
-  constexpr uint32_t expo = ((uint32_t)(25 - B) << 10) | ((uint32_t)(25 - B) << 26);
+__device__ __forceinline__ uint32_t key_pair(const KeyWords<BITS>& c) {
+  constexpr uint32_t code = ((1u << BITS) - 1u) << key_bit<BITS>(P);
   uint32_t src;
   if constexpr (BITS == 2)
     src = P < 2 ? c.l : (P < 5 ? c.m : c.r);
   else
     src = P == 0 ? c.l : (P == 1 ? c.m : (P == 2 ? c.r : c.r2));
-  uint32_t x;
-  asm("lop3.b32 %0, %1, %2, %3, 0xea;" : "=r"(x) : "r"(src), "n"(mask), "n"(expo));
-  return x;
+  return src & (code | (code << 16));
 }
 
-// The same pair centred: (a - C, b - C) with C = qmax / 2, exact (one more
-// HSUB2 of 2^(10-B) + C). Used for values, whose accumulator sums thousands
-// of tokens: uncentred values would carry off * sum(s p) next to the signal.
-template <int BITS, int P>
-__device__ __forceinline__ uint32_t pair_centred_h2(const Words<BITS>& c) {
-  constexpr int B = PairAt<BITS, P>::kBit;
-  // 2^(10-B) + C in fp16: exponent 25 - B, mantissa C * 2^B (C = qmax / 2)
-  constexpr uint32_t sub = ((uint32_t)(25 - B) << 10) | (((1u << BITS) - 1u) << (B - 1));
-  const uint32_t x = pair_h2<BITS, P>(c);
-  const __half m = __ushort_as_half((unsigned short)sub);
-  __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&x), __halves2half2(m, m));
-  return *reinterpret_cast<uint32_t*>(&h);
-}
-
-// -offset of pair P as an fp16 pair (a power of two, exact)
-template <int BITS, int P>
-__device__ __forceinline__ constexpr uint32_t neg_off_h2() {
-  constexpr int off = PairAt<BITS, P>::kOff;
-  // -2^k in fp16: sign 1, exponent k + 15, mantissa 0
-  constexpr uint32_t h = 0x8000u | ((uint32_t)((off == 64 ? 6 : (off == 16 ? 4 : 2)) + 15) << 10);
-  return h | (h << 16);
-}
-
-// Row of the beta MMA that collects s . q for the channels of pair P:
-// offset 64 -> row 1, 16 -> row 2, 4 -> row 3.
 template <int BITS>
-__host__ __device__ constexpr int off_row(int p) {
-  return BITS == 4 ? 1 : (p % 3 == 2 ? 1 : (p % 3 == 0 ? 2 : 3));
-}
+struct ValueWords {
+  uint32_t m, r;
+};
 template <int BITS>
-__host__ __device__ constexpr int off_of_row(int r) {
-  return BITS == 4 ? (r == 1 ? 64 : 0) : (r == 1 ? 64 : (r == 2 ? 16 : 4));
+__device__ __forceinline__ ValueWords<BITS> value_words(uint32_t w) {
+  return ValueWords<BITS>{w, BITS == 2 ? w >> 10 : w >> 8};
+}
+constexpr float kValueScale = 1.f / 512.f;  // of the codes value_pair returns
+
+// Value pair p: 2^-9 (code - C), C = qmax / 2, exact. Centred, because the
+// accumulator sums thousands of tokens: uncentred values would carry
+// C * sum(s p) next to the signal.
+template <int BITS, int P>
+__device__ __forceinline__ uint32_t value_pair(const ValueWords<BITS>& c) {
+  constexpr int B = BITS == 4 ? 4 * (P & 1) : 2 * (P % 5);
+  constexpr uint32_t code = ((1u << BITS) - 1u) << B;
+  const uint32_t x = ((BITS == 2 ? P < 5 : P < 2) ? c.m : c.r) & (code | (code << 16));
+  // 2^(15 - B) and -C 2^-9 = -(qmax 2^-10) in fp16 (qmax = 1.1b or 1.111b binary)
+  constexpr uint32_t mul = (uint32_t)(15 - B + 15) << 10;
+  constexpr uint32_t add = 0x8000u | ((uint32_t)(BITS - 1 - 10 + 15) << 10) |
+                           ((((1u << BITS) - 1u) << (11 - BITS)) & 0x3ffu);
+  return hfma2_u32(x, mul | (mul << 16), add | (add << 16));
 }
 
 // One quantization group (32 keys = two 16-key blocks) of a packed tile.
-// With codes entering as c + off (off per pair position, see above) and
-// x_hat = c * s + z:
-//   S^T  = (c + off)_K . (s_K (.) Q)^T + beta,
-//          beta = z_K . Q^T - sum_off off * (s_K . Q^T over that offset's channels)
-//          (one MMA per 16 channels: A rows z, s|off=64, s|off=16, s|off=4, all
-//          against the unscaled query: exact fp16 products, fp32 sums)
+// With x_hat = c * s + z (the powers of two of the codes left out):
+//   S^T  = c_K . (s_K (.) Q)^T + beta,  beta = z_K . Q^T
+//          (one MMA per 16 channels: A row r holds z over the channels of
+//          class r, whose queries carry 1 / class_scale(r): exact fp16
+//          products, fp32 sums)
 //   O^T += (c - C)_V^T . (s_V (.) P^T) + z'_V^T . P^T,  C = qmax / 2,
-//          z' = fp16(z + C s)  (centred values: their accumulator sums
-//          thousands of tokens, so no offset may ride along)
+//          z' = fp16(z + C s)
 // The per-channel key scales fold into the queries as fp16 hi + lo parts (the
 // scaled query keeps ~22 bits) and the per-token value scales into the
 // probabilities.
-// beta of two groups of one tile with one set of MMAs: A rows 0..3 hold
-// group a's (z, s over the channels of the offsets 64, 16, 4), rows 4..7
-// group b's, against the unscaled query. bt[h][nt] = beta of group h for
-// query rows 2j, 2j + 1 of n-tile nt.
+// Class rows of a beta accumulator (lanes 4 (first + r) + j) summed with their
+// scales: beta of query rows 2j, 2j + 1.
+template <int BITS>
+__device__ __forceinline__ void beta_rows(const float (&bq)[4], int first, float (&bt)[2]) {
+  const int j = threadIdx.x & 3;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    bt[h] = __shfl_sync(0xffffffffu, bq[h], 4 * first + j);
+#pragma unroll
+    for (int r = 1; r < key_classes<BITS>(); ++r)
+      bt[h] = fmaf(class_scale(r), __shfl_sync(0xffffffffu, bq[h], 4 * (first + r) + j), bt[h]);
+  }
+}
+
+// beta of two groups of one tile with one set of MMAs: A rows 0..3 hold group
+// a's zero points by class, rows 4..7 group b's. bt[h][nt] = beta of group h
+// for query rows 2j, 2j + 1 of n-tile nt.
 template <int NTW, int BITS>
 __device__ __forceinline__ void group_beta_pair(uint32_t qsm, uint32_t base, int ga, int gb,
                                                 float (&bt)[2][NTW][2]) {
@@ -647,13 +666,12 @@ __device__ __forceinline__ void group_beta_pair(uint32_t qsm, uint32_t base, int
   float bq[NTW][4];
 #pragma unroll
   for (int nt = 0; nt < NTW; ++nt) bq[nt][0] = bq[nt][1] = bq[nt][2] = bq[nt][3] = 0.f;
-  const uint32_t kp = base + kSlotKParams + (g < 4 ? ga : gb) * 512 + j * 16;
+  const uint32_t kp = base + kSlotKParams + (g < 4 ? ga : gb) * 512 + j * 16 + 8;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const uint4 P = lds128(kp + i * 64);  // s(c0 c1), s(c8 c9), z(c0 c1), z(c8 c9)
+    const uint2 z = lds64(kp + i * 64);  // z(c0 c1), z(c8 c9)
     const int p0 = BITS == 4 ? 2 * (i & 1) : 2 * (i & 3);
-    const int r0 = off_row<BITS>(p0), r1 = off_row<BITS>(p0 + 1);
-    const uint32_t az[4] = {gg == 0 ? P.z : (gg == r0 ? P.x : 0u), 0u, gg == 0 ? P.w : (gg == r1 ? P.y : 0u), 0u};
+    const uint32_t az[4] = {gg == key_class<BITS>(p0) ? z.x : 0u, 0u, gg == key_class<BITS>(p0 + 1) ? z.y : 0u, 0u};
 #pragma unroll
     for (int nt = 0; nt < NTW; ++nt) {
       const uint2 qv = lds64(qsm + ((nt * 8 + i) * 32 + lane) * 8);
@@ -663,21 +681,7 @@ __device__ __forceinline__ void group_beta_pair(uint32_t qsm, uint32_t base, int
 #pragma unroll
   for (int nt = 0; nt < NTW; ++nt)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      // row r of group h sits in lanes 4 (4h + r) + j
-      float b0 = __shfl_sync(0xffffffffu, bq[nt][0], 16 * h + j);
-      float b1 = __shfl_sync(0xffffffffu, bq[nt][1], 16 * h + j);
-#pragma unroll
-      for (int r = 1; r < 4; ++r) {
-        const float w = -(float)off_of_row<BITS>(r);
-        if (w != 0.f) {
-          b0 = fmaf(w, __shfl_sync(0xffffffffu, bq[nt][0], 16 * h + 4 * r + j), b0);
-          b1 = fmaf(w, __shfl_sync(0xffffffffu, bq[nt][1], 16 * h + 4 * r + j), b1);
-        }
-      }
-      bt[h][nt][0] = b0;
-      bt[h][nt][1] = b1;
-    }
+    for (int h = 0; h < 2; ++h) beta_rows<BITS>(bq[nt], 4 * h, bt[h][nt]);
 }
 
 // kBeta = false: the group's beta comes in bt_in (from group_beta_pair)
@@ -694,9 +698,6 @@ __device__ __forceinline__ void group_quant(WarpState<NTW>& st, uint32_t qsm,
 
   // ---- per 16 channels: scaled queries (fp16 hi + lo), beta, and S of both
   // 16-key blocks (four independent MMA chains; beta is added at the end)
-  // beta rows: 0: z . q, 1..3: s . q over the channels whose pairs carry the
-  // offset 64, 16, 4 (exact fp16 products, fp32 sums); beta = row 0 - 64 row 1
-  // - 16 row 2 - 4 row 3 is formed in fp32 afterwards.
   float bq[NTW][4];
   float sa[2][NTW][4], sl[2][NTW][4];
 #pragma unroll
@@ -728,42 +729,41 @@ __device__ __forceinline__ void group_quant(WarpState<NTW>& st, uint32_t qsm,
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const uint4 P = lds128(kp + i * 64);  // s(c0 c1), s(c8 c9), z(c0 c1), z(c8 c9)
-    // offset rows of the pairs of channels (16i + 2j, +1) and (16i + 2j + 8, +9)
+    // pairs of channels (16i + 2j, +1) and (16i + 2j + 8, +9)
     const int p0 = BITS == 4 ? 2 * (i & 1) : 2 * (i & 3);
-    const int r0 = off_row<BITS>(p0), r1 = off_row<BITS>(p0 + 1);
-    const uint32_t az[4] = {kBeta ? (g == 0 ? P.z : (g == r0 ? P.x : 0u)) : 0u, 0u,
-                            kBeta ? (g == 0 ? P.w : (g == r1 ? P.y : 0u)) : 0u, 0u};
+    const uint32_t az[4] = {kBeta && g == key_class<BITS>(p0) ? P.z : 0u, 0u,
+                            kBeta && g == key_class<BITS>(p0 + 1) ? P.w : 0u, 0u};
     // A fragments of both blocks for channels 16 i .. 16 i + 15
     uint32_t af[2][4];
     const int q = BITS == 4 ? (i >> 1) : (i >> 2);
 #pragma unroll
     for (int blk = 0; blk < 2; ++blk) {
-      const Words<BITS> w0 = words<BITS>(kw[2 * blk][q]), w1 = words<BITS>(kw[2 * blk + 1][q]);
+      const KeyWords<BITS> w0 = key_words<BITS>(kw[2 * blk][q]), w1 = key_words<BITS>(kw[2 * blk + 1][q]);
       if constexpr (BITS == 4) {
         if ((i & 1) == 0) {
-          af[blk][0] = pair_h2<4, 0>(w0); af[blk][1] = pair_h2<4, 0>(w1);
-          af[blk][2] = pair_h2<4, 1>(w0); af[blk][3] = pair_h2<4, 1>(w1);
+          af[blk][0] = key_pair<4, 0>(w0); af[blk][1] = key_pair<4, 0>(w1);
+          af[blk][2] = key_pair<4, 1>(w0); af[blk][3] = key_pair<4, 1>(w1);
         } else {
-          af[blk][0] = pair_h2<4, 2>(w0); af[blk][1] = pair_h2<4, 2>(w1);
-          af[blk][2] = pair_h2<4, 3>(w0); af[blk][3] = pair_h2<4, 3>(w1);
+          af[blk][0] = key_pair<4, 2>(w0); af[blk][1] = key_pair<4, 2>(w1);
+          af[blk][2] = key_pair<4, 3>(w0); af[blk][3] = key_pair<4, 3>(w1);
         }
       } else {
         switch (i & 3) {
           case 0:
-            af[blk][0] = pair_h2<2, 0>(w0); af[blk][1] = pair_h2<2, 0>(w1);
-            af[blk][2] = pair_h2<2, 1>(w0); af[blk][3] = pair_h2<2, 1>(w1);
+            af[blk][0] = key_pair<2, 0>(w0); af[blk][1] = key_pair<2, 0>(w1);
+            af[blk][2] = key_pair<2, 1>(w0); af[blk][3] = key_pair<2, 1>(w1);
             break;
           case 1:
-            af[blk][0] = pair_h2<2, 2>(w0); af[blk][1] = pair_h2<2, 2>(w1);
-            af[blk][2] = pair_h2<2, 3>(w0); af[blk][3] = pair_h2<2, 3>(w1);
+            af[blk][0] = key_pair<2, 2>(w0); af[blk][1] = key_pair<2, 2>(w1);
+            af[blk][2] = key_pair<2, 3>(w0); af[blk][3] = key_pair<2, 3>(w1);
             break;
           case 2:
-            af[blk][0] = pair_h2<2, 4>(w0); af[blk][1] = pair_h2<2, 4>(w1);
-            af[blk][2] = pair_h2<2, 5>(w0); af[blk][3] = pair_h2<2, 5>(w1);
+            af[blk][0] = key_pair<2, 4>(w0); af[blk][1] = key_pair<2, 4>(w1);
+            af[blk][2] = key_pair<2, 5>(w0); af[blk][3] = key_pair<2, 5>(w1);
             break;
           default:
-            af[blk][0] = pair_h2<2, 6>(w0); af[blk][1] = pair_h2<2, 6>(w1);
-            af[blk][2] = pair_h2<2, 7>(w0); af[blk][3] = pair_h2<2, 7>(w1);
+            af[blk][0] = key_pair<2, 6>(w0); af[blk][1] = key_pair<2, 6>(w1);
+            af[blk][2] = key_pair<2, 7>(w0); af[blk][3] = key_pair<2, 7>(w1);
             break;
         }
       }
@@ -784,28 +784,17 @@ __device__ __forceinline__ void group_quant(WarpState<NTW>& st, uint32_t qsm,
     }
   }
   float x[2][NTW][4];
+  const float ks = scale * (float)(1 << (24 - kKeyBit0));  // the codes' power of two
 #pragma unroll
   for (int nt = 0; nt < NTW; ++nt) {
-    float bt0 = bt_in[nt][0], bt1 = bt_in[nt][1];
-    if constexpr (kBeta) {
-      // rows 0..3 of bq sit in lanes (0..3, j)
-      bt0 = __shfl_sync(0xffffffffu, bq[nt][0], j);
-      bt1 = __shfl_sync(0xffffffffu, bq[nt][1], j);
+    float bt[2] = {bt_in[nt][0], bt_in[nt][1]};
+    if constexpr (kBeta) beta_rows<BITS>(bq[nt], 0, bt);
+    bt[0] *= scale;
+    bt[1] *= scale;
 #pragma unroll
-      for (int r = 1; r < 4; ++r) {
-        const float w = -(float)off_of_row<BITS>(r);
-        if (w != 0.f) {
-          bt0 = fmaf(w, __shfl_sync(0xffffffffu, bq[nt][0], 4 * r + j), bt0);
-          bt1 = fmaf(w, __shfl_sync(0xffffffffu, bq[nt][1], 4 * r + j), bt1);
-        }
-      }
-    }
+    for (int blk = 0; blk < 2; ++blk)
 #pragma unroll
-    for (int blk = 0; blk < 2; ++blk) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        x[blk][nt][e] = ((sa[blk][nt][e] + sl[blk][nt][e]) + (e & 1 ? bt1 : bt0)) * scale;
-    }
+      for (int e = 0; e < 4; ++e) x[blk][nt][e] = fmaf(sa[blk][nt][e] + sl[blk][nt][e], ks, bt[e & 1]);
   }
 
   // ---- softmax over the group's 32 keys
@@ -837,20 +826,20 @@ __device__ __forceinline__ void group_quant(WarpState<NTW>& st, uint32_t qsm,
 #pragma unroll
       for (int nt = 0; nt < NTW; ++nt) mma_f16(st.z[nt], az, b[nt][0], b[nt][1]);
     }
-    Words<BITS> vc[2 * KW];
+    ValueWords<BITS> vc[2 * KW];
     {
       const uint32_t va = base + kSlotVCodes + (u * 32 + lane) * (BITS * 8);
       const uint4 v0 = lds128(va);
-      vc[0] = words<BITS>(v0.x);
-      vc[1] = words<BITS>(v0.y);
-      vc[2] = words<BITS>(v0.z);
-      vc[3] = words<BITS>(v0.w);
+      vc[0] = value_words<BITS>(v0.x);
+      vc[1] = value_words<BITS>(v0.y);
+      vc[2] = value_words<BITS>(v0.z);
+      vc[3] = value_words<BITS>(v0.w);
       if constexpr (BITS == 4) {
         const uint4 v1 = lds128(va + 16);
-        vc[2 * KW > 4 ? 4 : 0] = words<BITS>(v1.x);
-        vc[2 * KW > 5 ? 5 : 1] = words<BITS>(v1.y);
-        vc[2 * KW > 6 ? 6 : 2] = words<BITS>(v1.z);
-        vc[2 * KW > 7 ? 7 : 3] = words<BITS>(v1.w);
+        vc[2 * KW > 4 ? 4 : 0] = value_words<BITS>(v1.x);
+        vc[2 * KW > 5 ? 5 : 1] = value_words<BITS>(v1.y);
+        vc[2 * KW > 6 ? 6 : 2] = value_words<BITS>(v1.z);
+        vc[2 * KW > 7 ? 7 : 3] = value_words<BITS>(v1.w);
       }
     }
 #pragma unroll
@@ -869,23 +858,23 @@ __device__ __forceinline__ void group_quant(WarpState<NTW>& st, uint32_t qsm,
         // a0 / a1 tokens 2j, 2j + 1 (pair p0), a2 / a3 tokens 2j + 8, 2j + 9 (p0 + 1)
         if constexpr (BITS == 4) {
           // m = 2mt + h: word m >> 1 = mt, p0 = 2 (m & 1) = 2h
-          a[0] = pair_centred_h2<4, 0>(vc[mt]);
-          a[2] = pair_centred_h2<4, 1>(vc[mt]);
-          a[1] = pair_centred_h2<4, 2>(vc[mt]);
-          a[3] = pair_centred_h2<4, 3>(vc[mt]);
+          a[0] = value_pair<4, 0>(vc[mt]);
+          a[2] = value_pair<4, 1>(vc[mt]);
+          a[1] = value_pair<4, 2>(vc[mt]);
+          a[3] = value_pair<4, 3>(vc[mt]);
         } else {
           // word m >> 2 = mt >> 1, p0 = 2 (m & 3) = 4 (mt & 1) + 2h
           const int q = mt >> 1;
           if ((mt & 1) == 0) {
-            a[0] = pair_centred_h2<2, 0>(vc[q]);
-            a[2] = pair_centred_h2<2, 1>(vc[q]);
-            a[1] = pair_centred_h2<2, 2>(vc[q]);
-            a[3] = pair_centred_h2<2, 3>(vc[q]);
+            a[0] = value_pair<2, 0>(vc[q]);
+            a[2] = value_pair<2, 1>(vc[q]);
+            a[1] = value_pair<2, 2>(vc[q]);
+            a[3] = value_pair<2, 3>(vc[q]);
           } else {
-            a[0] = pair_centred_h2<2, 4>(vc[q]);
-            a[2] = pair_centred_h2<2, 5>(vc[q]);
-            a[1] = pair_centred_h2<2, 6>(vc[q]);
-            a[3] = pair_centred_h2<2, 7>(vc[q]);
+            a[0] = value_pair<2, 4>(vc[q]);
+            a[2] = value_pair<2, 5>(vc[q]);
+            a[1] = value_pair<2, 6>(vc[q]);
+            a[3] = value_pair<2, 7>(vc[q]);
           }
         }
 #pragma unroll
@@ -1145,11 +1134,12 @@ __global__ void __launch_bounds__(256) merge_partials_kernel(const __grid_consta
   }
 }
 
-// Query rows of every n-tile as Q^T B fragments (bf16 for BF16, else fp16)
+// Query rows of every n-tile as Q^T B fragments (bf16 for bf16 rows, else
+// fp16 scaled for the key pairs of their channels)
 // in shared memory: word w of lane (g, j) for channels 16i + 2j (+8) of row
 // 8 nt + g at [((nt * 8 + i) * 32 + lane) * 2 + w], from the bf16 rows the
 // producer copied (row r = head * T + token). All consumer threads.
-template <bool BF16>
+template <int BITS>
 __device__ __forceinline__ void store_q(const AttnParams& p, uint32_t* qf, const uint8_t* rows) {
   for (int x = threadIdx.x; x < p.mtiles * 512; x += 128) {
     const int nt = x >> 9, i = (x >> 6) & 7, ln = (x >> 1) & 31, w = x & 1;
@@ -1157,8 +1147,12 @@ __device__ __forceinline__ void store_q(const AttnParams& p, uint32_t* qf, const
     const int c = 16 * i + 2 * (ln & 3) + 8 * w;
     uint32_t word = 0u;
     if (r < p.rows) {
-      const uint32_t w0 = *reinterpret_cast<const uint32_t*>(rows + (r * kHeadDim + c) * 2);
-      word = BF16 ? w0 : pack_f16(bf16_lo(w0), bf16_hi(w0));
+      word = *reinterpret_cast<const uint32_t*>(rows + (r * kHeadDim + c) * 2);
+      if constexpr (BITS != 16) {
+        // 1 / class_scale of the channels' key pair
+        const float f = 1.f / class_scale(key_class<BITS>(BITS == 4 ? 2 * (i & 1) + w : 2 * (i & 3) + w));
+        word = pack_f16(bf16_lo(word) * f, bf16_hi(word) * f);
+      }
     }
     qf[x] = word;
   }
@@ -1298,10 +1292,12 @@ __device__ __forceinline__ int run_tiles(const AttnParams& p, AttnSmem& sm, cons
   const int lane = threadIdx.x & 31;
   uint32_t* qf = NTW == 1 ? reinterpret_cast<uint32_t*>(sm.merge_w)
                           : reinterpret_cast<uint32_t*>(after_ring(sm));
-  store_q<BITS == 16>(p, qf, qrows_buf(sm, k, p.mtiles));
+  store_q<BITS>(p, qf, qrows_buf(sm, k, p.mtiles));
   consumer_sync();
   if (lane == 0) mbar_arrive(&sm.item_empty[k]);  // the query rows are no longer needed
   const uint32_t qs = smem_u32(qf) + grp * NTW * 2048;
+  // packed values enter O as kValueScale times theirs
+  if constexpr (BITS != 16) scale_o<NTW>(st, kValueScale);
   int last_slot = -1;
   for (int t = ii.tb; t < ii.te; ++t, ++seq) {
     constexpr int ST = kStages;
@@ -1355,6 +1351,7 @@ __device__ __forceinline__ int run_tiles(const AttnParams& p, AttnSmem& sm, cons
       last_slot = slot;
     }
   }
+  if constexpr (BITS != 16) scale_o<NTW>(st, 1.f / kValueScale);
   return last_slot;
 }
 

@@ -771,6 +771,7 @@ int groups_per_tile(int bits) { return bits == 2 ? 8 : 4; }
 // (b, kvh) runs on one SM; 128K batch 2, 54 items: 10 us of a 55 us
 // launch). Below 33 items the second launch costs more than it saves.
 constexpr int kMergeKernelItems = 32;
+constexpr int kInLaunchMerge = 40;  // items x n-tiles
 
 int seg_tiles_host(const uc_segment* s, int n) {
   if (!is_quant(s->kind)) return (n + 63) / 64;
@@ -917,6 +918,10 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
       }
     }
     const int hmax = std::max(nh, std::min(56, 64 - nl));
+    // few pairs with several n-tiles: where they cannot fill two CTAs per SM
+    // they fill one (two on half of the SMs ended later: 7 query tokens over
+    // 43K bf16 tokens, batch 1)
+    const int fill = mtiles > 1 && 10 * hmax * nbh_launch < 9 * slots ? std::max(1, slots / 2) : slots;
     H = forced_ipb;
     if (nh == 0) {
       H = 0;
@@ -924,7 +929,7 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
       double best_eff = -1.0;
       for (int h = nh; h <= hmax; ++h) {
         const double all = (double)h * nbh_launch;
-        const double eff = all / (std::ceil(all / slots) * slots);
+        const double eff = all / (std::ceil(all / fill) * fill);
         if (eff >= 0.9) {
           H = h;
           break;
@@ -944,11 +949,32 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
       const double all = (double)hw * nbh_launch;
       if (all / (std::ceil(all / slots) * slots) >= 0.8) H = hw;
     }
+    // Several n-tiles: an in-launch merge takes about 0.2 us per item and
+    // n-tile on the one SM that runs it (4 x 16K tokens, 4 query tokens: 15 of
+    // 46 us). Past kInLaunchMerge of them, where at most twice the items make
+    // it so, the call takes enough, in full rounds, for the merge kernel, which
+    // spreads them over many SMs (that call 45.3 -> 40.6 us, 8 query tokens
+    // 74.3 -> 63.5; from 12 items per pair up, batch 16: 117 -> 135).
+    if (mtiles > 1 && forced_ipb <= 0 && (H + nl) * mtiles > kInLaunchMerge && 2 * (H + nl) > kMergeKernelItems &&
+        H + nl <= kMergeKernelItems) {
+      int tiles = 0;
+      for (int s = 0; s < nseg; ++s) tiles += heavy[s] ? htiles[s] : 0;
+      double best_eff = -1.0;
+      for (int h = kMergeKernelItems + 1 - nl; h <= std::min(hmax, tiles); ++h) {
+        const double all = (double)h * nbh_launch;
+        const double eff = all / (std::ceil(all / slots) * slots);
+        if (eff > best_eff + 1e-9) {
+          best_eff = eff;
+          H = h;
+        }
+        if (eff >= 0.9) break;
+      }
+    }
     // calls whose merge is the separate kernel: there an item costs no
     // merge work, so take the most heavy items that still start in the
     // first round (128K batch 2: 52 -> 56 heavy items, 50.3 -> 47.8 us)
     if (forced_ipb <= 0 && H + nl > kMergeKernelItems) {
-      const int hr = std::min(hmax, slots / std::max(1, nbh_launch));
+      const int hr = std::min(hmax, fill / std::max(1, nbh_launch));
       if (hr > H) H = hr;
     }
     // short calls: the items of a pair on one cluster where that, with the
@@ -1199,6 +1225,7 @@ uc_status build_decode_call(const void* q, int32_t n_q_heads, int32_t n_qtok, co
   p->scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)UC_HEAD_DIM));
   p->wait_ns = uc::wait_limit_ns();
   p->withhold_pos = uc::take_withhold_pos();
+  p->stages = 2;
   return UC_OK;
 }
 
@@ -1421,6 +1448,7 @@ uc_status uc_attend(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_s
   // (a device whose clusters fit less well than planned for takes the queue)
   p.cluster = plan.cluster > 0 && attend_clusters(plan.cluster) >= B * hkv ? plan.cluster : 0;
   p.defer_merge = p.cluster ? 0 : merge_kernel_for(plan.items_per_bh);
+  if (plan.mtiles > 1 && plan.grid <= num_sms()) p.stages = 3;
   launch_attend(p, plan.grid, reinterpret_cast<cudaStream_t>(stream));
   return cuda_check("uc_attend");
 }

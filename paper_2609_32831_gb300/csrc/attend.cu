@@ -29,12 +29,15 @@
 namespace uc {
 
 constexpr int kTileTok = 64;
-constexpr int kStages = 2;  // ring slots of a CTA
-// CTAs per SM the register budget is set for: 3 for one query n-tile (128
-// registers), 2 for more (200; the query buffers of up to seven n-tiles leave
-// room for two CTAs' shared memory, eight run one).
-template <int NTW>
-__host__ __device__ constexpr int ctas_for() { return NTW == 1 ? 3 : 2; }
+// Ring slots (ST) of a CTA and CTAs per SM the register budget is set for:
+// two slots, three CTAs with one query n-tile (128 registers), two with more
+// (168; the query buffers of up to seven n-tiles leave room for two CTAs'
+// shared memory, eight run one). A launch with several n-tiles and no more
+// CTAs than SMs takes three slots and all registers (7 query tokens over 43K
+// bf16 tokens, batch 1: 47.5 us otherwise).
+constexpr int kStages = 2, kMaxStages = 3;
+template <int NTW, int ST>
+__host__ __device__ constexpr int ctas_for() { return NTW == 1 ? 3 : (ST == kMaxStages ? 1 : 2); }
 constexpr int kConsumers = 4;
 constexpr int kAttnThreads = 32 * (kConsumers + 1);
 constexpr int kSlotBytes = 32768;
@@ -56,14 +59,14 @@ constexpr int kItemQ = 2;  // items handed from the producer to the consumers ah
 struct AttnSmem {
   alignas(16) float merge_w[kMaxItemsPerBh * 8];  // per (item, row of an 8-row block): m, then weight
   float merge_l[kMaxItemsPerBh * 8];
-  uint64_t full[kStages];
-  uint64_t empty[kStages];
+  uint64_t full[kMaxStages];
+  uint64_t empty[kMaxStages];
   uint64_t item_full[kItemQ];   // producer -> consumers: item position and its query rows
   uint64_t item_empty[kItemQ];  // consumers -> producer: the entry is free again
   int item_pos[kItemQ];         // processing position, -1: no more work
   int n_pending;                    // (sequence, KV head) merges this CTA owes
   int pending[kMaxPendingMerges];
-  alignas(1024) uint8_t slot[kStages][kSlotBytes];
+  alignas(1024) uint8_t slot[kMaxStages][kSlotBytes];  // as many as the launch has
 };
 
 // Query fragments of the current item live in shared memory (2 KB per
@@ -76,18 +79,20 @@ constexpr int kQTileBytes = 2048;
 static_assert(kQTileBytes == 8 * kHeadDim * 2, "bf16 rows of an n-tile");
 __host__ __device__ constexpr int qfrag_tiles(int ntiles) { return ntiles <= 1 ? 0 : ntiles; }
 
-constexpr size_t attend_smem_bytes(int ntiles) {
-  return offsetof(AttnSmem, slot) + (size_t)kStages * kSlotBytes +
+constexpr size_t attend_smem_bytes(int ntiles, int stages = kStages) {
+  return offsetof(AttnSmem, slot) + (size_t)stages * kSlotBytes +
          (size_t)(qfrag_tiles(ntiles) + kItemQ * ntiles) * kQTileBytes + 1024;
 }
 
 // Shared-memory regions after the ring: query fragments (more than one
 // n-tile), then the producer's query-row buffers.
+template <int ST>
 __device__ __forceinline__ uint8_t* after_ring(AttnSmem& sm) {
-  return reinterpret_cast<uint8_t*>(sm.slot) + kStages * kSlotBytes;
+  return reinterpret_cast<uint8_t*>(sm.slot) + ST * kSlotBytes;
 }
+template <int ST>
 __device__ __forceinline__ uint8_t* qrows_buf(AttnSmem& sm, int k, int ntiles) {
-  return after_ring(sm) + (qfrag_tiles(ntiles) + k * ntiles) * kQTileBytes;
+  return after_ring<ST>(sm) + (qfrag_tiles(ntiles) + k * ntiles) * kQTileBytes;
 }
 
 __host__ __device__ size_t attend_part_floats(int ntiles) { return (size_t)ntiles * 8 * (kHeadDim + 2); }
@@ -262,9 +267,8 @@ __device__ __forceinline__ uint2 lds64(uint32_t a) {
 //
 // In a cluster launch rank r < n_heavy takes its pair's heavy item r, the
 // ranks after them (one, or one each) share the pair's light items.
-template <int NTW, bool CLUSTER, class W>
+template <int NTW, int ST, bool CLUSTER, class W>
 __device__ void produce(const W& w, AttnSmem& sm) {
-  constexpr int ST = kStages;
   const AttnParams& p0 = w.call(0);
   int* sched = p0.sched;
   uint32_t seq = 0;
@@ -298,7 +302,7 @@ __device__ void produce(const W& w, AttnSmem& sm) {
     const __nv_bfloat16* qsrc =
         p.q + (size_t)(ii.b * p.n_q_heads + (ii.bh % p.n_kv_heads) * p.group) * p.n_qtok * kHeadDim;
     mbar_arrive_expect_tx(&sm.item_full[k], qbytes);
-    bulk_load(qrows_buf(sm, k, p.mtiles), qsrc, qbytes, &sm.item_full[k]);
+    bulk_load(qrows_buf<ST>(sm, k, p.mtiles), qsrc, qbytes, &sm.item_full[k]);
     for (int t = ii.tb; t < ii.te; ++t, ++seq) {
       const int slot = seq % ST;
       if (seq >= ST && !mbar_wait(&sm.empty[slot], ((seq / ST) - 1) & 1, p.status, 10, p.wait_ns)) {
@@ -364,9 +368,9 @@ __device__ void produce(const W& w, AttnSmem& sm) {
   // longer waits for the copies this producer issued: they land before the
   // CTA leaves. (Otherwise the consumers have waited for every one.)
   const bool failed = stop || (p0.status != nullptr && *reinterpret_cast<volatile int32_t*>(&p0.status->code) != 0);
-  for (int s = 0; failed && s < ST; ++s) {
-    if (seq < (uint32_t)s + 1u) break;
-    const uint32_t sq = seq - 1u - (uint32_t)s;
+  for (uint32_t s = 0; failed && s < ST; ++s) {
+    if (seq < s + 1u) break;
+    const uint32_t sq = seq - 1u - s;
     if (!mbar_wait(&sm.full[sq % ST], (sq / ST) & 1, p0.status, 15, p0.wait_ns)) break;
   }
 }
@@ -976,7 +980,7 @@ __device__ __forceinline__ void merge_weights(const AttnParams& p, float* ml, co
 // back to back, eight items per slot, by bulk copies continuing the consumers'
 // tile sequence, the first ones in flight while the weights are formed.
 // Without `seq` (a merge between items) the threads load them.
-template <int NTW>
+template <int NTW, int ST>
 __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t* seq) {
   const int tid = threadIdx.x;
   const int b = bh / p.n_kv_heads, kvh = bh % p.n_kv_heads;
@@ -989,23 +993,23 @@ __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t*
   const int total = nb * p.mtiles;
   auto issue = [&](int n) {  // batch n: eight items of row block n / nb (thread 0)
     const uint32_t sq = *seq + n;
-    uint64_t* bar = &sm.full[sq % kStages];
+    uint64_t* bar = &sm.full[sq % ST];
     const int i0 = (n % nb) * kPerSlot, cnt = min(kPerSlot, I - i0);
     mbar_arrive_expect_tx(bar, (uint32_t)cnt * 8 * kHeadDim * 4);
     for (int k = 0; k < cnt; ++k)
-      bulk_load(sm.slot[sq % kStages] + k * 8 * kHeadDim * 4, base + (i0 + k) * pf + (size_t)(n / nb) * 8 * kHeadDim,
+      bulk_load(sm.slot[sq % ST] + k * 8 * kHeadDim * 4, base + (i0 + k) * pf + (size_t)(n / nb) * 8 * kHeadDim,
                 8 * kHeadDim * 4, bar);
   };
   if (seq != nullptr && tid == 0) {
     // the partials were written by other CTAs (generic proxy) and acquired
     // at GPU scope; order that acquire before the copy engine's reads
     fence_proxy_async_global();
-    for (int n = 0; n < min(kStages, total); ++n) issue(n);
+    for (int n = 0; n < min(ST, total); ++n) issue(n);
   }
   // rows whose weights are formed at once: every row when the query buffers
   // behind the ring are idle too, else the 8 rows the merge arrays hold
   const int set = NTW == 1 || seq == nullptr ? 8 : rows_pad;
-  float* wts = NTW == 1 || seq == nullptr ? sm.merge_w : reinterpret_cast<float*>(after_ring(sm));  // [I][set]
+  float* wts = NTW == 1 || seq == nullptr ? sm.merge_w : reinterpret_cast<float*>(after_ring<ST>(sm));  // [I][set]
   float* ls = NTW == 1 || seq == nullptr ? sm.merge_l : wts + I * set;
   const int cq = tid & 31, rg = tid >> 5;  // channels 4 cq .. + 3, rows 2 rg, 2 rg + 1 of a block
   for (int s0 = 0; s0 < p.rows; s0 += set) {
@@ -1037,16 +1041,16 @@ __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t*
         for (int j = 0; j < nb; ++j) {
           const int n = r0 / 8 * nb + j, i0 = j * kPerSlot, cnt = min(kPerSlot, I - i0);
           const uint32_t sq = *seq + n;
-          const bool ok = mbar_wait(&sm.full[sq % kStages], (sq / kStages) & 1, p.status, 14, p.wait_ns);
-          const float4* buf = reinterpret_cast<const float4*>(sm.slot[sq % kStages]) + 2 * rg * 32 + cq;
+          const bool ok = mbar_wait(&sm.full[sq % ST], (sq / ST) & 1, p.status, 14, p.wait_ns);
+          const float4* buf = reinterpret_cast<const float4*>(sm.slot[sq % ST]) + 2 * rg * 32 + cq;
           if (ok) {
 #pragma unroll
             for (int k = 0; k < kPerSlot; ++k)
               if (k < cnt) add(i0 + k, buf[k * 256], buf[k * 256 + 32]);
           }
-          if (n + kStages < total) {
+          if (n + ST < total) {
             consumer_sync();  // the slot is read: refill it
-            if (tid == 0) issue(n + kStages);
+            if (tid == 0) issue(n + ST);
           }
         }
       } else {
@@ -1291,14 +1295,14 @@ __device__ __forceinline__ void finish_item(const AttnParams& p, AttnSmem& sm, W
 // All tiles of one item added to a warp's state: bf16 rows (BITS = 16: bf16
 // segments and the tails of packed segments) or packed groups (BITS = 4 / 2).
 // With `keep_last` the item's last slot is not handed back; returns it (-1: none).
-template <int NTW, int BITS>
+template <int NTW, int ST, int BITS>
 __device__ __forceinline__ int run_tiles(const AttnParams& p, AttnSmem& sm, const ItemInfo& ii, int k, uint32_t& seq,
                                          bool& aborted, int KS, int grp, int ks, bool keep_last,
                                          WarpState<NTW>& st) {
   const int lane = threadIdx.x & 31;
   uint32_t* qf = NTW == 1 ? reinterpret_cast<uint32_t*>(sm.merge_w)
-                          : reinterpret_cast<uint32_t*>(after_ring(sm));
-  store_q<BITS>(p, qf, qrows_buf(sm, k, p.mtiles));
+                          : reinterpret_cast<uint32_t*>(after_ring<ST>(sm));
+  store_q<BITS>(p, qf, qrows_buf<ST>(sm, k, p.mtiles));
   consumer_sync();
   if (lane == 0) mbar_arrive(&sm.item_empty[k]);  // the query rows are no longer needed
   const uint32_t qs = smem_u32(qf) + grp * NTW * 2048;
@@ -1306,7 +1310,6 @@ __device__ __forceinline__ int run_tiles(const AttnParams& p, AttnSmem& sm, cons
   if constexpr (BITS != 16) scale_o<NTW>(st, kValueScale);
   int last_slot = -1;
   for (int t = ii.tb; t < ii.te; ++t, ++seq) {
-    constexpr int ST = kStages;
     const int slot = seq % ST;
     if (!aborted && !mbar_wait(&sm.full[slot], (seq / ST) & 1, p.status, 11, p.wait_ns)) aborted = true;
     const uint32_t sbase = smem_u32(sm.slot[slot]);
@@ -1361,12 +1364,12 @@ __device__ __forceinline__ int run_tiles(const AttnParams& p, AttnSmem& sm, cons
   return last_slot;
 }
 
-template <int NTW, int BITS>
+template <int NTW, int ST, int BITS>
 __device__ __forceinline__ void run_item(const AttnParams& p, AttnSmem& sm, const ItemInfo& ii, int it, int k,
                                          uint32_t& seq, bool& aborted, int NG, int KS, int grp, int ks) {
   WarpState<NTW> st;
   state_init<NTW>(st);
-  const int last_slot = run_tiles<NTW, BITS>(p, sm, ii, k, seq, aborted, KS, grp, ks, KS > 1, st);
+  const int last_slot = run_tiles<NTW, ST, BITS>(p, sm, ii, k, seq, aborted, KS, grp, ks, KS > 1, st);
   finish_item<NTW>(p, sm, st, it, last_slot, NG, KS, grp, ks);
 }
 
@@ -1437,11 +1440,11 @@ __device__ __forceinline__ void consume_cluster(const AttnParams& p, AttnSmem& s
     const ItemInfo ii = decode_item(p, pos, &it);
     const SegDev& sd = p.seg[ii.s];
     if (seg_is_bf16(sd.kind) || ii.tail)
-      run_tiles<1, 16>(p, sm, ii, k, seq, aborted, kConsumers, 0, warp, false, st);
+      run_tiles<1, kStages, 16>(p, sm, ii, k, seq, aborted, kConsumers, 0, warp, false, st);
     else if (sd.bits == 4)
-      run_tiles<1, 4>(p, sm, ii, k, seq, aborted, kConsumers, 0, warp, false, st);
+      run_tiles<1, kStages, 4>(p, sm, ii, k, seq, aborted, kConsumers, 0, warp, false, st);
     else
-      run_tiles<1, 2>(p, sm, ii, k, seq, aborted, kConsumers, 0, warp, false, st);
+      run_tiles<1, kStages, 2>(p, sm, ii, k, seq, aborted, kConsumers, 0, warp, false, st);
     reduce_row_sums<1>(st);
     if (g == 0) {
 #pragma unroll
@@ -1559,7 +1562,7 @@ __device__ __forceinline__ void consume_cluster(const AttnParams& p, AttnSmem& s
   cluster_wait();  // no CTA leaves while another may still read its shared memory
 }
 
-template <int NTW, class W>
+template <int NTW, int ST, class W>
 __device__ void consume(const W& w, AttnSmem& sm) {
   const int warp = threadIdx.x >> 5;
   const int mtiles = w.call(0).mtiles;  // the same for every call of a launch
@@ -1581,11 +1584,11 @@ __device__ void consume(const W& w, AttnSmem& sm) {
     const ItemInfo ii = decode_item(p, local, &it);
     const SegDev& sd = p.seg[ii.s];
     if (seg_is_bf16(sd.kind) || ii.tail)
-      run_item<NTW, 16>(p, sm, ii, it, k, seq, aborted, NG, KS, grp, ks);
+      run_item<NTW, ST, 16>(p, sm, ii, it, k, seq, aborted, NG, KS, grp, ks);
     else if (sd.bits == 4)
-      run_item<NTW, 4>(p, sm, ii, it, k, seq, aborted, NG, KS, grp, ks);
+      run_item<NTW, ST, 4>(p, sm, ii, it, k, seq, aborted, NG, KS, grp, ks);
     else
-      run_item<NTW, 2>(p, sm, ii, it, k, seq, aborted, NG, KS, grp, ks);
+      run_item<NTW, ST, 2>(p, sm, ii, it, k, seq, aborted, NG, KS, grp, ks);
 
     // Arrive on the item's counter; the CTA whose arrival completes a
     // (sequence, KV head) owes its merge, done after its last item so that
@@ -1602,7 +1605,7 @@ __device__ void consume(const W& w, AttnSmem& sm) {
       for (int k = 0; k < kMaxPendingMerges; ++k) {
         const AttnParams& pc = w.call(sm.pending[k] >> 16);
         const int bh = sm.pending[k] & 0xffff;
-        final_merge<NTW>(pc, sm, bh, nullptr);
+        final_merge<NTW, ST>(pc, sm, bh, nullptr);
         consumer_sync();
         if (threadIdx.x == 0) pc.counters[bh] = 0;
       }
@@ -1618,14 +1621,14 @@ __device__ void consume(const W& w, AttnSmem& sm) {
   for (int k = 0; k < sm.n_pending; ++k) {
     const AttnParams& pc = w.call(sm.pending[k] >> 16);
     const int bh = sm.pending[k] & 0xffff;
-    final_merge<NTW>(pc, sm, bh, &seq);  // the producer has stopped: the ring is idle
+    final_merge<NTW, ST>(pc, sm, bh, &seq);  // the producer has stopped: the ring is idle
     consumer_sync();
     if (threadIdx.x == 0) pc.counters[bh] = 0;
   }
 }
 
-template <int NTW, class P, bool CLUSTER = false>
-__global__ void __launch_bounds__(kAttnThreads, ctas_for<NTW>()) attend_kernel(const __grid_constant__ P params) {
+template <int NTW, class P, bool CLUSTER = false, int ST = kStages>
+__global__ void __launch_bounds__(kAttnThreads, ctas_for<NTW, ST>()) attend_kernel(const __grid_constant__ P params) {
   const typename WorkOf<P>::type w{params};
   extern __shared__ uint8_t dyn_smem[];
   AttnSmem& sm = *reinterpret_cast<AttnSmem*>(
@@ -1639,7 +1642,7 @@ __global__ void __launch_bounds__(kAttnThreads, ctas_for<NTW>()) attend_kernel(c
   griddep_launch_dependents();
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(&sm.full[s], 1);
       mbar_init(&sm.empty[s], kConsumers);
     }
@@ -1660,13 +1663,13 @@ __global__ void __launch_bounds__(kAttnThreads, ctas_for<NTW>()) attend_kernel(c
           prefetch_tmap(&p.tmap[2 * s + 1]);
         }
       }
-      produce<NTW, CLUSTER>(w, sm);
+      produce<NTW, ST, CLUSTER>(w, sm);
     }
   } else {
     if constexpr (CLUSTER)
       consume_cluster(params, sm);
     else
-      consume<NTW>(w, sm);
+      consume<NTW, ST>(w, sm);
   }
 }
 
@@ -1676,6 +1679,8 @@ static void attend_setup_once() {
     const int one = (int)attend_smem_bytes(1), most = (int)attend_smem_bytes(8);
     cudaFuncSetAttribute(attend_kernel<1, AttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize, one);
     cudaFuncSetAttribute(attend_kernel<2, AttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(attend_kernel<2, AttnParams, false, kMaxStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)attend_smem_bytes(8, kMaxStages));
     cudaFuncSetAttribute(attend_kernel<1, AttnParams, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, one);
     cudaFuncSetAttribute(attend_kernel<1, AttnParams, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaFuncSetAttribute(attend_kernel<1, MultiAttnParams>, cudaFuncAttributeMaxDynamicSharedMemorySize, one);
@@ -1746,9 +1751,11 @@ void launch_attend(const AttnParams& p, int grid, cudaStream_t st) {
     count_launch();
     return;
   }
-  const size_t smem = attend_smem_bytes(p.mtiles);
+  const size_t smem = attend_smem_bytes(p.mtiles, p.stages);
   if (p.mtiles <= 1)
     launch_maybe_pdl(pdl, attend_kernel<1, AttnParams>, grid, kAttnThreads, smem, st, p);
+  else if (p.stages == kMaxStages)
+    launch_maybe_pdl(pdl, attend_kernel<2, AttnParams, false, kMaxStages>, grid, kAttnThreads, smem, st, p);
   else
     launch_maybe_pdl(pdl, attend_kernel<2, AttnParams>, grid, kAttnThreads, smem, st, p);
   count_launch();

@@ -216,6 +216,7 @@ struct AttnParams {
   // > 0: a cluster of this many CTAs per (sequence, KV head) instead of the
   // work queue: one per heavy item, then one for the light items or one each
   int cluster;
+  int stages;       // ring slots of a CTA (uc_attend; batched launches take two)
   int defer_merge;  // 1: the attend launch only leaves partials; a merge kernel follows
   float scale_log2;
   uint64_t wait_ns;  // limit of every bounded wait of the launch (UC_ERR_TIMEOUT past it)

@@ -386,8 +386,11 @@ constexpr int kQuantCtasPerSm = kQuantBufs == 2 ? 2 : 3;
 constexpr int kQuantRowBytes = 272;
 
 struct QuantWarpSmem {
-  uint8_t rows[kQuantBufs][32 * kQuantRowBytes];
-  QuantStats st;
+  alignas(16) uint8_t rows[kQuantBufs][32 * kQuantRowBytes];
+  union {
+    QuantStats st;
+    QuantStats2 st2;
+  };
   uint64_t bar[kQuantBufs];
 };
 constexpr size_t kQuantSmemBytes = kQuantWarps * sizeof(QuantWarpSmem);
@@ -456,7 +459,11 @@ __global__ void __launch_bounds__(kQuantWarps * 32, kQuantCtasPerSm) quantize_gr
       break;
     }
     ph_k ^= 1u;
-    const bool ok = quantize_keys<BITS>(krow, g, out, sm.st);
+    bool ok;
+    if constexpr (BITS == 2)
+      ok = quantize_keys2(sm.rows[0], kQuantRowBytes, g, out, sm.st2);
+    else
+      ok = quantize_keys<BITS>(krow, g, out, sm.st);
     // every lane has read this group's K rows: the buffer takes the next rows
     if constexpr (kQuantBufs == 2) {
       if (next < total) request(next, 0, 0, next_idx);
@@ -469,9 +476,11 @@ __global__ void __launch_bounds__(kQuantWarps * 32, kQuantCtasPerSm) quantize_gr
       break;
     }
     ph_v ^= 1u;
-    if (!ok || !quantize_values<BITS>(vrow, g, out, sm.st)) {
-      if (lane == 0) set_status(a.status, UC_ERR_RANGE, 2);
-    }
+    if constexpr (BITS == 2)
+      ok = ok && quantize_values2(sm.rows[kVBuf], kQuantRowBytes, g, out, sm.st2);
+    else
+      ok = ok && quantize_values<BITS>(vrow, g, out, sm.st);
+    if (!ok && lane == 0) set_status(a.status, UC_ERR_RANGE, 2);
     if constexpr (kQuantBufs == 2) {
       if (next < total) request(next, 1, 1, next_idx);
     } else {

@@ -132,6 +132,39 @@ def test_quantize_zero_scale_and_clamped_codes(bits):
 
 
 @pytest.mark.parametrize("bits", [4, 2])
+def test_quantize_codes_at_their_edges(bits):
+    """Groups of symmetric, tiny, subnormal, offset and huge values: elements
+    on and next to every code's edge, edges next to zero (where bf16 values
+    lie denser than fp32 differences from the zero-point): bit-exact."""
+    B, hkv, n = 2, 4, 256
+    rng = np.random.default_rng(47 + bits)
+    bf = lambda x: torch.from_numpy(np.ascontiguousarray(x, np.float32)).to(torch.bfloat16).float().numpy()
+    qmax = 2 ** bits - 1
+
+    def values(shape):
+        x = rng.standard_normal(shape)
+        a = np.exp2(rng.integers(-18, 13, shape[:-1] + (1,)).astype(np.float64))
+        steps = np.rint(rng.uniform(0, 2 * qmax, shape)) / 2 - qmax / 2       # codes and their edges, centred
+        kind = rng.integers(0, 6, shape[:-1] + (1,))
+        x = np.where(kind == 0, x, np.where(kind == 1, steps, np.where(kind == 2, steps + qmax / 2, np.where(
+            kind == 3, np.sign(x), np.where(kind == 4, x + 40.0, steps * (1 + 2.0 ** -7))))))
+        tiny = rng.random(shape) < 0.2
+        x = np.where(tiny, x * np.exp2(rng.integers(-60, -10, shape).astype(np.float64)), x)
+        return bf(np.clip(x * a, -6e4, 6e4))
+
+    k = values((B, hkv, 128, n)).transpose(0, 1, 3, 2).copy()   # keys: groups along the tokens
+    v = values((B, hkv, n, 128))
+    seg = uc.Segment("quant", bits, B, hkv, n, n, DEV)
+    seg.set_keep([n] * B)
+    ws = uc.Workspace(DEV)
+    uc.compress_segment(dev(k), dev(v), seg, ws=ws)
+    assert ws.status() == 0
+    for b in range(B):
+        for j in range(hkv):
+            _check_quant_block(seg, b, j, oseg.compress(k[b, j], v[b, j], None, "quant", n, bits))
+
+
+@pytest.mark.parametrize("bits", [4, 2])
 def test_evict_quant_parity(bits):
     B, hkv, n = 3, 4, 768
     k, v = synth.make_kv(7 + bits, B, hkv, n)

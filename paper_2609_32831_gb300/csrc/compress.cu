@@ -404,14 +404,30 @@ __global__ void __launch_bounds__(kQuantWarps * 32, kQuantCtasPerSm) quantize_gr
   const int per_bh = a.max_chunks;
   const int total = a.batch * a.n_kv_heads * per_bh;
   const int all = total + a.batch * a.n_kv_heads;  // then one residual tail per (b, kvh)
-  // the first valid group or tail at or after w (groups past a sequence's
-  // full groups and empty tails are skipped)
-  auto valid_from = [&](int w) {
-    for (; w < all; w += n_warps) {
-      const int b = (w < total ? w / per_bh : w - total) / a.n_kv_heads;
-      if (w < total ? w % per_bh < a.keep[b] / kGroup : a.keep[b] % kGroup != 0) break;
+  // A work index w with its (b, kvh) and group (w < total), stepped by the
+  // grid's warps without dividing again.
+  struct Work {
+    int w, bh, g;
+  };
+  const int step_bh = n_warps / per_bh, step_g = n_warps % per_bh;
+  auto stepped = [&](Work k) {
+    k.w += n_warps;
+    k.bh += step_bh;
+    k.g += step_g;
+    if (k.g >= per_bh) {
+      k.g -= per_bh;
+      ++k.bh;
     }
-    return w;
+    return k;
+  };
+  // the first valid group or tail at or after k (groups past a sequence's
+  // full groups and empty tails are skipped)
+  auto valid_from = [&](Work k) {
+    for (; k.w < all; k = stepped(k))
+      if (k.w < total ? k.g < a.keep[k.bh / a.n_kv_heads] / kGroup
+                      : a.keep[(k.w - total) / a.n_kv_heads] % kGroup != 0)
+        break;
+    return k;
   };
   if (a.identity && blockIdx.x == 0 && threadIdx.x < a.batch) a.n_kept[threadIdx.x] = a.keep[threadIdx.x];
   if (lane == 0) {
@@ -421,34 +437,33 @@ __global__ void __launch_bounds__(kQuantWarps * 32, kQuantCtasPerSm) quantize_gr
   __syncwarp();
   // kept index of this lane's row of group w (loaded a group ahead, so that
   // the request does not wait for it)
-  auto row_index = [&](int w) {
-    return w < total ? take_row(a, w / per_bh, (w % per_bh) * kGroup + lane) : 0;
-  };
+  auto row_index = [&](const Work& k) { return k.w < total ? take_row(a, k.bh, k.g * kGroup + lane) : 0; };
   // rows of group w (K if kv == 0, else V) into buffer `buf`
-  auto request = [&](int w, int buf, int kv, int32_t idx) {
-    const int64_t row = (int64_t)(w / per_bh) * a.src_row_stride + a.src_row_offset + idx;
+  auto request = [&](const Work& k, int buf, int kv, int32_t idx) {
+    const int64_t row = (int64_t)k.bh * a.src_row_stride + a.src_row_offset + idx;
     if (lane == 0) mbar_arrive_expect_tx(&sm.bar[buf], kGroup * kHeadDim * 2);
     __syncwarp();
-    if (w == a.withhold && kv == 0 && lane == 0) return;  // test hook: one K row is never copied
+    if (k.w == a.withhold && kv == 0 && lane == 0) return;  // test hook: one K row is never copied
     bulk_load(sm.rows[buf] + lane * kQuantRowBytes, (kv ? a.v_src : a.k_src) + row * kHeadDim, kHeadDim * 2,
               &sm.bar[buf]);
   };
   constexpr int kVBuf = kQuantBufs - 1;
   auto krow = [&](int t) { return reinterpret_cast<const __nv_bfloat16*>(sm.rows[0] + t * kQuantRowBytes); };
   auto vrow = [&](int t) { return reinterpret_cast<const __nv_bfloat16*>(sm.rows[kVBuf] + t * kQuantRowBytes); };
-  int w = valid_from(blockIdx.x * kQuantWarps + (threadIdx.x >> 5));
-  int32_t idx = row_index(w);
-  if (w < total) {
-    request(w, 0, 0, idx);
-    if constexpr (kQuantBufs == 2) request(w, 1, 1, idx);
+  const int w0 = blockIdx.x * kQuantWarps + (threadIdx.x >> 5);
+  Work k = valid_from(Work{w0, w0 / per_bh, w0 % per_bh});
+  int32_t idx = row_index(k);
+  if (k.w < total) {
+    request(k, 0, 0, idx);
+    if constexpr (kQuantBufs == 2) request(k, 1, 1, idx);
   }
   // phase of the next completion of each buffer's barrier
   uint32_t ph_k = 0, ph_v = 0;
   bool failed = false;
-  while (w < total) {
-    const int next = valid_from(w + n_warps);
+  while (k.w < total) {
+    const Work next = valid_from(stepped(k));
     const int32_t next_idx = row_index(next);
-    const int bh = w / per_bh, g = w % per_bh;
+    const int bh = k.bh, g = k.g;
     QuantOut out;
     out.k_codes = a.k_codes + (size_t)bh * a.cap * kHeadDim * BITS / 8;
     out.k_params = a.k_params + (size_t)bh * (a.cap / kGroup) * 512;
@@ -466,9 +481,9 @@ __global__ void __launch_bounds__(kQuantWarps * 32, kQuantCtasPerSm) quantize_gr
       ok = quantize_keys<BITS>(krow, g, out, sm.st);
     // every lane has read this group's K rows: the buffer takes the next rows
     if constexpr (kQuantBufs == 2) {
-      if (next < total) request(next, 0, 0, next_idx);
+      if (next.w < total) request(next, 0, 0, next_idx);
     } else {
-      request(w, 0, 1, idx);
+      request(k, 0, 1, idx);
       ph_v = ph_k;
     }
     if (!__all_sync(0xffffffffu, mbar_wait(&sm.bar[kVBuf], ph_v, a.status, 21, a.wait_ns))) {
@@ -482,13 +497,13 @@ __global__ void __launch_bounds__(kQuantWarps * 32, kQuantCtasPerSm) quantize_gr
       ok = ok && quantize_values<BITS>(vrow, g, out, sm.st);
     if (!ok && lane == 0) set_status(a.status, UC_ERR_RANGE, 2);
     if constexpr (kQuantBufs == 2) {
-      if (next < total) request(next, 1, 1, next_idx);
+      if (next.w < total) request(next, 1, 1, next_idx);
     } else {
-      if (next < total) request(next, 0, 0, next_idx);
+      if (next.w < total) request(next, 0, 0, next_idx);
       ph_k = ph_v;
     }
     idx = next_idx;
-    w = next;
+    k = next;
   }
   if (failed) {
     // copies still in flight must land before the warp's shared memory is
@@ -499,8 +514,8 @@ __global__ void __launch_bounds__(kQuantWarps * 32, kQuantCtasPerSm) quantize_gr
   }
   // the residual tails: the last (n mod 32) kept tokens of a (b, kvh), copied
   // to its bf16 tail block of 32 rows
-  for (; w < all; w = valid_from(w + n_warps)) {
-    const int bh = w - total;
+  for (; k.w < all; k = valid_from(stepped(k))) {
+    const int bh = k.w - total;
     const int n = a.keep[bh / a.n_kv_heads];
     copy_rows(a, bh, n / kGroup * kGroup, n % kGroup, (int64_t)bh * kGroup);
   }

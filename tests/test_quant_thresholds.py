@@ -29,11 +29,11 @@ def _of_order(o):
 def _threshold(z, t_min):
     reaches = lambda x: np.float32(x) - z >= t_min  # noqa: E731
     u = int(_bf16(z + t_min))
-    step = -0x10000 if u & 0x80000000 else 0x10000
     f = lambda v: np.uint32(v & 0xFFFFFFFF).view(np.float32)  # noqa: E731
-    up, down = f(u + step), f(u - step)
-    if u << 1 & 0xFFFFFFFF and not reaches(down) and reaches(up):
-        return f(u) if reaches(f(u)) else up
+    inside = bool(reaches(f(u)))
+    nxt = f(u + (0x10000 if inside == bool(u & 0x80000000) else -0x10000))
+    if u << 1 & 0xFFFFFFFF and bool(reaches(nxt)) != inside:
+        return f(u) if inside else nxt
     lo, hi = 0x007F, 0xFF80
     while hi - lo > 1:
         mid = (lo + hi) >> 1

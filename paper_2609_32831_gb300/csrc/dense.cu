@@ -115,23 +115,26 @@ __device__ __forceinline__ bool dwait_warp(uint64_t* bar, uint32_t parity, DevSt
 }
 
 // ------------------------------------------------------------ materialize
-// Writes fp16 K hi / K lo / V rows of every tile of every (b, kvh). One warp
-// per 32 rows of a tile of kDK rows (a quantization group of a packed
-// segment); a tile never spans two segments. Rows past the sequence's kept
-// count are written as zeros.
+// Writes fp16 K hi / K lo / V rows of every tile of every (b, kvh). One CTA
+// of four warps per 32 rows of a tile of kDK rows (a quantization group of a
+// packed segment); a tile never spans two segments. Rows past the sequence's
+// kept count are written as zeros.
 //
 // A full quantization group of a packed segment (32 tokens) is decoded the
-// way it is stored: each lane reads its own fragment-ordered code words and
-// the parameter entries that belong to exactly its channels (keys) or tokens
-// (values), rebuilds x = code * s + z in fp32, and writes fp16 into a
-// 32-row staging block in shared memory (rows 272 bytes apart: conflict-free
-// for both fragment patterns); the block then goes out as whole rows, 16
-// bytes per lane. bf16 rows, the residual tail and the zero rows past the
-// kept count are converted row by row.
+// way it is stored, by three warps: K hi, K lo (the key codes twice, from
+// cache) and V. Each lane reads its own fragment-ordered code words and the
+// parameter entries that belong to exactly its channels (keys) or tokens
+// (values), rebuilds x = code * s + z in fp32, and writes fp16 into a 32-row
+// staging block in shared memory (rows 272 bytes apart: conflict-free for
+// both fragment patterns); the block then goes out as whole rows, 16 bytes
+// per lane. bf16 rows, the residual tail and the zero rows past the kept
+// count are converted row by row, eight rows of each warp in flight. Short
+// calls are a chain of latencies here (one warp per 32 rows: 11 us before the
+// 45 us of a 1000-query, 2240-key call of batch 1).
 constexpr int kMatWarps = 4;
 constexpr int kMatRow = 136;  // halves per staged row (272 bytes)
 struct MatStage {
-  __half r[2][32][kMatRow];  // K hi, K lo; then V in r[0]
+  __half r[32][kMatRow];
 };
 
 // 32 staged rows -> global rows dst[0 .. 31] (128 halves each), 16 B per lane
@@ -145,112 +148,120 @@ __device__ __forceinline__ void mat_store_rows(__half* dst, const __half (*src)[
   }
 }
 
-template <int BITS>
-__device__ void mat_packed_group(const SegDev& sd, int bh, int g, __half* khi, __half* klo, __half* vv,
-                                 MatStage& st) {
+// Keys of group g, the fp16 hi part or what it leaves (LO): lane (n, j) holds
+// tokens 8 nt + n, channels 16 i + 2 j + {0, 1, 8, 9}.
+template <int BITS, bool LO>
+__device__ void mat_keys(const SegDev& sd, int bh, int g, __half* dst, MatStage& st) {
   const int lane = threadIdx.x & 31;
   constexpr uint32_t mask = (1u << BITS) - 1u;
-  constexpr int kb = 8 / BITS;  // 16-channel (K) / 8-channel (V) blocks per code word
+  constexpr int kb = 8 / BITS;  // 16-channel blocks per code word
   const size_t blk_codes = (size_t)bh * sd.cap * kHeadDim * BITS / 8;
-  // ---- keys: lane (n, j) holds tokens 8 nt + n, channels 16 i + 2 j + {0, 1, 8, 9}
-  {
-    const int n = lane >> 2, j = lane & 3;
-    uint32_t w[4][BITS];
+  const int n = lane >> 2, j = lane & 3;
+  uint32_t w[4][BITS];
+#pragma unroll
+  for (int nt = 0; nt < 4; ++nt) {
+    const uint8_t* src = sd.k_codes + blk_codes + ((size_t)(g * 4 + nt) * 32 + lane) * (BITS * 4);
+    if constexpr (BITS == 4) {
+      const uint4 x = *reinterpret_cast<const uint4*>(src);
+      w[nt][0] = x.x; w[nt][BITS > 1 ? 1 : 0] = x.y; w[nt][BITS > 2 ? 2 : 0] = x.z; w[nt][BITS > 3 ? 3 : 0] = x.w;
+    } else {
+      const uint2 x = *reinterpret_cast<const uint2*>(src);
+      w[nt][0] = x.x; w[nt][BITS > 1 ? 1 : 0] = x.y;
+    }
+  }
+  const uint8_t* kp = sd.k_params + (size_t)bh * (sd.cap / kGroup) * 512 + (size_t)g * 512;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint4 e = *reinterpret_cast<const uint4*>(kp + (i * 4 + j) * 16);  // s01, s89, z01, z89
+    const float2 s01 = __half22float2(*reinterpret_cast<const __half2*>(&e.x));
+    const float2 s89 = __half22float2(*reinterpret_cast<const __half2*>(&e.y));
+    const float2 z01 = __half22float2(*reinterpret_cast<const __half2*>(&e.z));
+    const float2 z89 = __half22float2(*reinterpret_cast<const __half2*>(&e.w));
+    const int q = i / kb, p = 2 * (i % kb);
+    const int c = 16 * i + 2 * j;
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
-      const uint8_t* src = sd.k_codes + blk_codes + ((size_t)(g * 4 + nt) * 32 + lane) * (BITS * 4);
-      if constexpr (BITS == 4) {
-        const uint4 x = *reinterpret_cast<const uint4*>(src);
-        w[nt][0] = x.x; w[nt][BITS > 1 ? 1 : 0] = x.y; w[nt][BITS > 2 ? 2 : 0] = x.z; w[nt][BITS > 3 ? 3 : 0] = x.w;
-      } else {
-        const uint2 x = *reinterpret_cast<const uint2*>(src);
-        w[nt][0] = x.x; w[nt][BITS > 1 ? 1 : 0] = x.y;
+      const uint32_t word = w[nt][q];
+      const float x0 = __fmaf_rn((float)((word >> (BITS * p)) & mask), s01.x, z01.x);
+      const float x1 = __fmaf_rn((float)((word >> (16 + BITS * p)) & mask), s01.y, z01.y);
+      const float x8 = __fmaf_rn((float)((word >> (BITS * (p + 1))) & mask), s89.x, z89.x);
+      const float x9 = __fmaf_rn((float)((word >> (16 + BITS * (p + 1))) & mask), s89.y, z89.y);
+      __half2 h01 = __floats2half2_rn(x0, x1), h89 = __floats2half2_rn(x8, x9);
+      if constexpr (LO) {
+        const float2 f01 = __half22float2(h01), f89 = __half22float2(h89);
+        h01 = __floats2half2_rn(x0 - f01.x, x1 - f01.y);
+        h89 = __floats2half2_rn(x8 - f89.x, x9 - f89.y);
       }
+      const int row = 8 * nt + n;
+      *reinterpret_cast<__half2*>(&st.r[row][c]) = h01;
+      *reinterpret_cast<__half2*>(&st.r[row][c + 8]) = h89;
     }
-    const uint8_t* kp = sd.k_params + (size_t)bh * (sd.cap / kGroup) * 512 + (size_t)g * 512;
+  }
+  __syncwarp();
+  mat_store_rows(dst, st.r);
+}
+
+// Values of group g: lane (gq, j) holds, in 16-token tile kt, tokens
+// 2 j + 8 sub + {0, 1}, channels 8 m + gq.
+template <int BITS>
+__device__ void mat_values(const SegDev& sd, int bh, int g, __half* dst, MatStage& st) {
+  const int lane = threadIdx.x & 31;
+  constexpr uint32_t mask = (1u << BITS) - 1u;
+  constexpr int kb = 8 / BITS;  // 8-channel blocks per code word
+  const size_t blk_codes = (size_t)bh * sd.cap * kHeadDim * BITS / 8;
+  const int gq = lane >> 2, j = lane & 3;
+  const uint8_t* vp = sd.v_params + (size_t)bh * sd.cap * 16;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint4 e = *reinterpret_cast<const uint4*>(kp + (i * 4 + j) * 16);  // s01, s89, z01, z89
-      const float2 s01 = __half22float2(*reinterpret_cast<const __half2*>(&e.x));
-      const float2 s89 = __half22float2(*reinterpret_cast<const __half2*>(&e.y));
+  for (int kt = 0; kt < 2; ++kt) {
+    uint32_t w[2 * BITS];
+    const uint8_t* src = sd.v_codes + blk_codes + ((size_t)(g * 2 + kt) * 32 + lane) * (BITS * 8);
+#pragma unroll
+    for (int q = 0; q < 2 * BITS; q += 4) {
+      const uint4 x = *reinterpret_cast<const uint4*>(src + 4 * q);
+      w[q] = x.x; w[q + 1] = x.y; w[q + 2] = x.z; w[q + 3] = x.w;
+    }
+#pragma unroll
+    for (int grp = 0; grp < 4; ++grp) {
+      const uint4 e = *reinterpret_cast<const uint4*>(vp + (size_t)(g * 2 + kt) * 256 + (grp * 4 + j) * 16);
+      const float2 s01 = __half22float2(*reinterpret_cast<const __half2*>(&e.x));  // tokens 2j, 2j + 1
+      const float2 s89 = __half22float2(*reinterpret_cast<const __half2*>(&e.y));  // 2j + 8, 2j + 9
       const float2 z01 = __half22float2(*reinterpret_cast<const __half2*>(&e.z));
       const float2 z89 = __half22float2(*reinterpret_cast<const __half2*>(&e.w));
-      const int q = i / kb, p = 2 * (i % kb);
-      const int c = 16 * i + 2 * j;
 #pragma unroll
-      for (int nt = 0; nt < 4; ++nt) {
-        const uint32_t word = w[nt][q];
-        const float x0 = __fmaf_rn((float)((word >> (BITS * p)) & mask), s01.x, z01.x);
-        const float x1 = __fmaf_rn((float)((word >> (16 + BITS * p)) & mask), s01.y, z01.y);
-        const float x8 = __fmaf_rn((float)((word >> (BITS * (p + 1))) & mask), s89.x, z89.x);
-        const float x9 = __fmaf_rn((float)((word >> (16 + BITS * (p + 1))) & mask), s89.y, z89.y);
-        const __half2 h01 = __floats2half2_rn(x0, x1), h89 = __floats2half2_rn(x8, x9);
-        const float2 f01 = __half22float2(h01), f89 = __half22float2(h89);
-        const int row = 8 * nt + n;
-        *reinterpret_cast<__half2*>(&st.r[0][row][c]) = h01;
-        *reinterpret_cast<__half2*>(&st.r[0][row][c + 8]) = h89;
-        *reinterpret_cast<__half2*>(&st.r[1][row][c]) = __floats2half2_rn(x0 - f01.x, x1 - f01.y);
-        *reinterpret_cast<__half2*>(&st.r[1][row][c + 8]) = __floats2half2_rn(x8 - f89.x, x9 - f89.y);
+      for (int mm = 0; mm < 4; ++mm) {
+        const int m = 4 * grp + mm;
+        const uint32_t word = w[m / kb];
+        const int p = 2 * (m % kb);
+        const int ch = 8 * m + gq, t0 = 16 * kt + 2 * j;
+        st.r[t0][ch] = __float2half_rn(__fmaf_rn((float)((word >> (BITS * p)) & mask), s01.x, z01.x));
+        st.r[t0 + 1][ch] = __float2half_rn(__fmaf_rn((float)((word >> (16 + BITS * p)) & mask), s01.y, z01.y));
+        st.r[t0 + 8][ch] = __float2half_rn(__fmaf_rn((float)((word >> (BITS * (p + 1))) & mask), s89.x, z89.x));
+        st.r[t0 + 9][ch] = __float2half_rn(__fmaf_rn((float)((word >> (16 + BITS * (p + 1))) & mask), s89.y, z89.y));
       }
     }
-    __syncwarp();
-    mat_store_rows(khi, st.r[0]);
-    mat_store_rows(klo, st.r[1]);
-    __syncwarp();
   }
-  // ---- values: lane (gq, j) holds, in 16-token tile kt, tokens 2 j + 8 sub
-  // + {0, 1}, channels 8 m + gq
-  {
-    const int gq = lane >> 2, j = lane & 3;
-    const uint8_t* vp = sd.v_params + (size_t)bh * sd.cap * 16;
-#pragma unroll
-    for (int kt = 0; kt < 2; ++kt) {
-      uint32_t w[2 * BITS];
-      const uint8_t* src = sd.v_codes + blk_codes + ((size_t)(g * 2 + kt) * 32 + lane) * (BITS * 8);
-#pragma unroll
-      for (int q = 0; q < 2 * BITS; q += 4) {
-        const uint4 x = *reinterpret_cast<const uint4*>(src + 4 * q);
-        w[q] = x.x; w[q + 1] = x.y; w[q + 2] = x.z; w[q + 3] = x.w;
-      }
-#pragma unroll
-      for (int grp = 0; grp < 4; ++grp) {
-        const uint4 e = *reinterpret_cast<const uint4*>(vp + (size_t)(g * 2 + kt) * 256 + (grp * 4 + j) * 16);
-        const float2 s01 = __half22float2(*reinterpret_cast<const __half2*>(&e.x));  // tokens 2j, 2j + 1
-        const float2 s89 = __half22float2(*reinterpret_cast<const __half2*>(&e.y));  // 2j + 8, 2j + 9
-        const float2 z01 = __half22float2(*reinterpret_cast<const __half2*>(&e.z));
-        const float2 z89 = __half22float2(*reinterpret_cast<const __half2*>(&e.w));
-#pragma unroll
-        for (int mm = 0; mm < 4; ++mm) {
-          const int m = 4 * grp + mm;
-          const uint32_t word = w[m / kb];
-          const int p = 2 * (m % kb);
-          const int ch = 8 * m + gq, t0 = 16 * kt + 2 * j;
-          st.r[0][t0][ch] = __float2half_rn(__fmaf_rn((float)((word >> (BITS * p)) & mask), s01.x, z01.x));
-          st.r[0][t0 + 1][ch] = __float2half_rn(__fmaf_rn((float)((word >> (16 + BITS * p)) & mask), s01.y, z01.y));
-          st.r[0][t0 + 8][ch] =
-              __float2half_rn(__fmaf_rn((float)((word >> (BITS * (p + 1))) & mask), s89.x, z89.x));
-          st.r[0][t0 + 9][ch] =
-              __float2half_rn(__fmaf_rn((float)((word >> (16 + BITS * (p + 1))) & mask), s89.y, z89.y));
-        }
-      }
-    }
-    __syncwarp();
-    mat_store_rows(vv, st.r[0]);
-    __syncwarp();
-  }
+  __syncwarp();
+  mat_store_rows(dst, st.r);
+}
+
+template <int BITS>
+__device__ __forceinline__ void mat_part(const SegDev& sd, int part, int bh, int g, __half* khi, __half* klo,
+                                         __half* vv, MatStage& st) {
+  if (part == 0)
+    mat_keys<BITS, false>(sd, bh, g, khi, st);
+  else if (part == 1)
+    mat_keys<BITS, true>(sd, bh, g, klo, st);
+  else if (part == 2)
+    mat_values<BITS>(sd, bh, g, vv, st);
 }
 
 __global__ void __launch_bounds__(32 * kMatWarps) materialize_kernel(const __grid_constant__ DenseParams p) {
-  extern __shared__ __align__(16) uint8_t mat_smem[];
-  MatStage& stg = reinterpret_cast<MatStage*>(mat_smem)[threadIdx.x >> 5];
-  // one warp per (b, kvh, tile, 32-row quarter of the tile)
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int nbh = p.batch * p.n_kv_heads;
+  __shared__ __align__(16) MatStage stages[kMatWarps - 1];
+  griddep_launch_dependents();  // the attention kernel sets up beside this one and waits for its rows
+  const int part = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int kQuarters = kDK / kGroup;
-  if (warp >= nbh * p.n_tiles * kQuarters) return;
-  const int qr = warp % kQuarters;
-  const int bh = warp / (p.n_tiles * kQuarters), ti = (warp / kQuarters) % p.n_tiles;
+  const int qr = blockIdx.x % kQuarters;  // 32-row quarter of the tile
+  const int bh = blockIdx.x / (p.n_tiles * kQuarters), ti = (blockIdx.x / kQuarters) % p.n_tiles;
   const int b = bh / p.n_kv_heads;
   const DenseTile tl = p.tiles[ti];
   const SegDev& sd = p.seg[tl.seg];
@@ -264,55 +275,54 @@ __global__ void __launch_bounds__(32 * kMatWarps) materialize_kernel(const __gri
   const int ng = bf16_kind ? 0 : n / kGroup;
   // a full packed group (quantized segments always have a K lo block)
   if (!bf16_kind && klo != nullptr && (t0 + r_lo) / kGroup < ng) {
+    if (part == kMatWarps - 1) return;
     const int g = (t0 + r_lo) / kGroup;
+    const size_t off = (size_t)r_lo * kHeadDim;
     if (sd.bits == 4)
-      mat_packed_group<4>(sd, bh, g, khi + (size_t)r_lo * kHeadDim, klo + (size_t)r_lo * kHeadDim,
-                          vv + (size_t)r_lo * kHeadDim, stg);
+      mat_part<4>(sd, part, bh, g, khi + off, klo + off, vv + off, stages[part]);
     else
-      mat_packed_group<2>(sd, bh, g, khi + (size_t)r_lo * kHeadDim, klo + (size_t)r_lo * kHeadDim,
-                          vv + (size_t)r_lo * kHeadDim, stg);
+      mat_part<2>(sd, part, bh, g, khi + off, klo + off, vv + off, stages[part]);
     return;
   }
-  const int r_first = r_lo, r_end = r_lo + kGroup;
-  // the rest row by row, eight rows' loads in flight at once: bf16 rows, the
-  // residual tail, zeros past the kept count. Lane: channels 4 lane .. 4 lane + 3.
-  for (int rb = r_first; rb < r_end; rb += 8) {
-    uint2 ka[8], va[8];
+  // the rest row by row, the warp's eight rows in flight at once: bf16 rows,
+  // the residual tail, zeros past the kept count. Lane: channels 4 lane .. 4 lane + 3.
+  constexpr int kRows = kGroup / kMatWarps;
+  const int rb = r_lo + kRows * part;
+  uint2 ka[kRows], va[kRows];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int t = t0 + rb + u;
-      ka[u] = make_uint2(0u, 0u);
-      va[u] = make_uint2(0u, 0u);
-      if (t < n) {
-        int64_t row;
-        if (bf16_kind)
-          row = (int64_t)bh * sd.row_stride + sd.row_offset + t;
-        else
-          row = (int64_t)bh * kGroup + (t - ng * kGroup);  // the residual tail (t >= ng * 32 here)
-        ka[u] = *reinterpret_cast<const uint2*>(p.seg_k[tl.seg] + row * kHeadDim + 4 * lane);
-        va[u] = *reinterpret_cast<const uint2*>(p.seg_v[tl.seg] + row * kHeadDim + 4 * lane);
-      }
+  for (int u = 0; u < kRows; ++u) {
+    const int t = t0 + rb + u;
+    ka[u] = make_uint2(0u, 0u);
+    va[u] = make_uint2(0u, 0u);
+    if (t < n) {
+      int64_t row;
+      if (bf16_kind)
+        row = (int64_t)bh * sd.row_stride + sd.row_offset + t;
+      else
+        row = (int64_t)bh * kGroup + (t - ng * kGroup);  // the residual tail (t >= ng * 32 here)
+      ka[u] = *reinterpret_cast<const uint2*>(p.seg_k[tl.seg] + row * kHeadDim + 4 * lane);
+      va[u] = *reinterpret_cast<const uint2*>(p.seg_v[tl.seg] + row * kHeadDim + 4 * lane);
     }
+  }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int r = rb + u;
-      const float kx[4] = {bf16_lo(ka[u].x), bf16_hi(ka[u].x), bf16_lo(ka[u].y), bf16_hi(ka[u].y)};
-      const float vx[4] = {bf16_lo(va[u].x), bf16_hi(va[u].x), bf16_lo(va[u].y), bf16_hi(va[u].y)};
-      __half hk[4], hv[4], lk[4];
+  for (int u = 0; u < kRows; ++u) {
+    const int r = rb + u;
+    const float kx[4] = {bf16_lo(ka[u].x), bf16_hi(ka[u].x), bf16_lo(ka[u].y), bf16_hi(ka[u].y)};
+    const float vx[4] = {bf16_lo(va[u].x), bf16_hi(va[u].x), bf16_lo(va[u].y), bf16_hi(va[u].y)};
+    __half hk[4], hv[4], lk[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        hk[e] = __float2half_rn(kx[e]);
-        lk[e] = __float2half_rn(kx[e] - __half2float(hk[e]));
-        hv[e] = __float2half_rn(vx[e]);
-      }
-      *reinterpret_cast<uint2*>(khi + r * kHeadDim + 4 * lane) =
-          make_uint2(pack_h2(hk[0], hk[1]), pack_h2(hk[2], hk[3]));
-      *reinterpret_cast<uint2*>(vv + r * kHeadDim + 4 * lane) =
-          make_uint2(pack_h2(hv[0], hv[1]), pack_h2(hv[2], hv[3]));
-      if (klo != nullptr)
-        *reinterpret_cast<uint2*>(klo + r * kHeadDim + 4 * lane) =
-            make_uint2(pack_h2(lk[0], lk[1]), pack_h2(lk[2], lk[3]));
+    for (int e = 0; e < 4; ++e) {
+      hk[e] = __float2half_rn(kx[e]);
+      lk[e] = __float2half_rn(kx[e] - __half2float(hk[e]));
+      hv[e] = __float2half_rn(vx[e]);
     }
+    *reinterpret_cast<uint2*>(khi + r * kHeadDim + 4 * lane) =
+        make_uint2(pack_h2(hk[0], hk[1]), pack_h2(hk[2], hk[3]));
+    *reinterpret_cast<uint2*>(vv + r * kHeadDim + 4 * lane) =
+        make_uint2(pack_h2(hv[0], hv[1]), pack_h2(hv[2], hv[3]));
+    if (klo != nullptr)
+      *reinterpret_cast<uint2*>(klo + r * kHeadDim + 4 * lane) =
+          make_uint2(pack_h2(lk[0], lk[1]), pack_h2(lk[2], lk[3]));
   }
 }
 
@@ -367,6 +377,7 @@ __global__ void __launch_bounds__(kDThreads, 1) dense_kernel(const __grid_consta
       prefetch_tmap(&p.tmap_khi);
       prefetch_tmap(&p.tmap_klo);
       prefetch_tmap(&p.tmap_v);
+      griddep_wait();  // the rebuilt rows; nothing else here reads what the kernel before wrote
       int kc = 0;
       for (int j = 0; j < T && !aborted; ++j) {
         const DenseTile tl = p.tiles[j];
@@ -656,19 +667,16 @@ void launch_dense(const DenseParams& p, cudaStream_t st) {
     cudaFuncSetAttribute(dense_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dense_smem_bytes());
     cudaFuncSetAttribute(dense_kernel<UC_MAX_SEGMENTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)dense_smem_bytes());
-    cudaFuncSetAttribute(materialize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(kMatWarps * sizeof(MatStage)));
   });
   const int nbh = p.batch * p.n_kv_heads;
-  const int warps = nbh * p.n_tiles * (kDK / kGroup);
-  materialize_kernel<<<(warps + kMatWarps - 1) / kMatWarps, 32 * kMatWarps, kMatWarps * sizeof(MatStage), st>>>(p);
+  materialize_kernel<<<nbh * p.n_tiles * (kDK / kGroup), 32 * kMatWarps, 0, st>>>(p);
   count_launch();
   const int n_qp = (p.n_qtok + kDQ * kDQT - 1) / (kDQ * kDQT);
   const int grid = p.batch * p.n_q_heads * n_qp;
   if (p.nseg <= 4)
-    dense_kernel<4><<<grid, kDThreads, dense_smem_bytes(), st>>>(p);
+    launch_maybe_pdl(true, dense_kernel<4>, grid, kDThreads, dense_smem_bytes(), st, p);
   else
-    dense_kernel<UC_MAX_SEGMENTS><<<grid, kDThreads, dense_smem_bytes(), st>>>(p);
+    launch_maybe_pdl(true, dense_kernel<UC_MAX_SEGMENTS>, grid, kDThreads, dense_smem_bytes(), st, p);
   count_launch();
 }
 

@@ -314,12 +314,13 @@ __global__ void dequant_rows_kernel(DequantArgs a) {
 // on to the logical token of that row (every entry has one reader, the lane
 // that also rewrites it), a segment that keeps every token gets its indices
 // here (`identity`: row t is kept token t).
-__device__ __forceinline__ int32_t take_row(const GatherArgs& a, int bh, int t) {
+// With `write` false the entry stays as it is (no src_idx then).
+__device__ __forceinline__ int32_t take_row(const GatherArgs& a, int bh, int t, bool write = true) {
   int32_t* e = a.kept_idx + (int64_t)bh * a.cap + t;
   const int32_t row = a.identity ? t : *e;
   if (a.src_idx != nullptr)
     *e = a.src_idx[(int64_t)bh * a.src_cap + row];
-  else if (a.identity)
+  else if (a.identity && write)
     *e = row;
   return row;
 }
@@ -369,147 +370,141 @@ __global__ void gather_rows_kernel(GatherArgs a) {
 
 // ---------------------------------------------------------- quantization
 
-// Persistent: each warp quantizes the groups gw, gw + W, ... (W warps in the
-// grid), consecutive warps taking consecutive groups of a (b, kvh). A warp
-// stages a group's 32 K rows and 32 V rows in shared memory with one bulk
-// copy per row (rows gathered through the kept-index list, 272 bytes apart
-// so that rows of the fragment-order reads fall in different banks).
-// kQuantBufs = 1 (used): one buffer takes the K rows, then the V rows; each
-// warp waits for every copy, but 10 KB of shared memory per warp fits 21
-// warps per SM, which cover each other's waits (32K layer, batch 16: int2
-// 376 us, int4 383 us). kQuantBufs = 2: K and V rows have buffers of their
-// own and each copy is requested half a group ahead, but only 12 warps fit
-// (403 / 414 us).
-constexpr int kQuantBufs = 1;
-constexpr int kQuantWarps = kQuantBufs == 2 ? 6 : 7;
-constexpr int kQuantCtasPerSm = kQuantBufs == 2 ? 2 : 3;
+// Persistent: each warp takes the units gw, gw + W, ... (W warps in the grid),
+// a unit being a group (32 kept tokens of a (b, kvh)), or its K or V rows
+// (`apart`).
+// A warp stages a unit's rows in shared memory with one bulk copy per row
+// (rows gathered through the kept-index list, 272 bytes apart so that rows of
+// the fragment-order reads fall in different banks). One buffer takes unit
+// after unit; each warp waits for every copy, but 10 KB of shared memory per
+// warp fits 21 warps per SM, which cover each other's waits (buffers of their
+// own for K and V with each copy requested half a group ahead fit 12 and were
+// 7 % slower). K and V apart halve the latency of calls with no more groups
+// than warps (800 tokens, batch 1: 9.6 -> 6.2 us; 7400, batch 1: 10.4 -> 7.8)
+// and the uneven last round of slightly longer ones (7400, batch 4: 24.0 ->
+// 22.7); from kApartRounds groups per warp up the extra unit costs more (7400,
+// batch 8: 39.3 together, 40.9 apart; 32K layer, batch 16: 271 and 280). A re-compression's warp takes
+// both, since its kept indices are rewritten as they are read.
+constexpr int kQuantWarps = 7;
+constexpr int kQuantCtasPerSm = 3;
 constexpr int kQuantRowBytes = 272;
+constexpr int kApartRounds = 2;
 
 struct QuantWarpSmem {
-  alignas(16) uint8_t rows[kQuantBufs][32 * kQuantRowBytes];
+  alignas(16) uint8_t rows[32 * kQuantRowBytes];
   union {
     QuantStats st;
     QuantStats2 st2;
   };
-  uint64_t bar[kQuantBufs];
+  uint64_t bar;
 };
 constexpr size_t kQuantSmemBytes = kQuantWarps * sizeof(QuantWarpSmem);
 
-template <int BITS>
+template <int BITS, bool APART>
 __global__ void __launch_bounds__(kQuantWarps * 32, kQuantCtasPerSm) quantize_groups_kernel(GatherArgs a) {
   extern __shared__ __align__(16) uint8_t quant_smem[];
   QuantWarpSmem& sm = reinterpret_cast<QuantWarpSmem*>(quant_smem)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const int n_warps = gridDim.x * kQuantWarps;
   const int per_bh = a.max_chunks;
-  const int total = a.batch * a.n_kv_heads * per_bh;
-  const int all = total + a.batch * a.n_kv_heads;  // then one residual tail per (b, kvh)
-  // A work index w with its (b, kvh) and group (w < total), stepped by the
-  // grid's warps without dividing again.
+  const int nbh = a.batch * a.n_kv_heads;
+  const int total = (APART ? 2 : 1) * nbh * per_bh;      // apart: every group's K unit, then every V unit
+  const int all = total + nbh;                           // then one residual tail per (b, kvh)
+  // A work index w with its block ((b, kvh), the V units' after the K units')
+  // and group (w < total), stepped by the grid's warps without dividing again.
   struct Work {
-    int w, bh, g;
+    int w, blk, g;
   };
-  const int step_bh = n_warps / per_bh, step_g = n_warps % per_bh;
+  auto is_v = [&](const Work& k) { return APART && k.blk >= nbh; };
+  auto bh_of = [&](const Work& k) { return is_v(k) ? k.blk - nbh : k.blk; };
+  const int step_blk = n_warps / per_bh, step_g = n_warps % per_bh;
   auto stepped = [&](Work k) {
     k.w += n_warps;
-    k.bh += step_bh;
+    k.blk += step_blk;
     k.g += step_g;
     if (k.g >= per_bh) {
       k.g -= per_bh;
-      ++k.bh;
+      ++k.blk;
     }
     return k;
   };
-  // the first valid group or tail at or after k (groups past a sequence's
-  // full groups and empty tails are skipped)
+  // the first valid unit or tail at or after k (groups past a sequence's full
+  // groups and empty tails are skipped)
   auto valid_from = [&](Work k) {
     for (; k.w < all; k = stepped(k))
-      if (k.w < total ? k.g < a.keep[k.bh / a.n_kv_heads] / kGroup
+      if (k.w < total ? k.g < a.keep[bh_of(k) / a.n_kv_heads] / kGroup
                       : a.keep[(k.w - total) / a.n_kv_heads] % kGroup != 0)
         break;
     return k;
   };
   if (a.identity && blockIdx.x == 0 && threadIdx.x < a.batch) a.n_kept[threadIdx.x] = a.keep[threadIdx.x];
   if (lane == 0) {
-    for (int k = 0; k < kQuantBufs; ++k) mbar_init(&sm.bar[k], 1);
+    mbar_init(&sm.bar, 1);
     fence_barrier_init();
   }
   __syncwarp();
-  // kept index of this lane's row of group w (loaded a group ahead, so that
-  // the request does not wait for it)
-  auto row_index = [&](const Work& k) { return k.w < total ? take_row(a, k.bh, k.g * kGroup + lane) : 0; };
-  // rows of group w (K if kv == 0, else V) into buffer `buf`
-  auto request = [&](const Work& k, int buf, int kv, int32_t idx) {
-    const int64_t row = (int64_t)k.bh * a.src_row_stride + a.src_row_offset + idx;
-    if (lane == 0) mbar_arrive_expect_tx(&sm.bar[buf], kGroup * kHeadDim * 2);
+  // kept index of this lane's row of unit k (loaded a unit ahead, so that the
+  // request does not wait for it)
+  auto row_index = [&](const Work& k) {
+    return k.w < total ? take_row(a, bh_of(k), k.g * kGroup + lane, !is_v(k)) : 0;
+  };
+  // K (kv == 0) or V rows of unit k into the buffer
+  auto request = [&](const Work& k, int kv, int32_t idx) {
+    const int64_t row = (int64_t)bh_of(k) * a.src_row_stride + a.src_row_offset + idx;
+    if (lane == 0) mbar_arrive_expect_tx(&sm.bar, kGroup * kHeadDim * 2);
     __syncwarp();
     if (k.w == a.withhold && kv == 0 && lane == 0) return;  // test hook: one K row is never copied
-    bulk_load(sm.rows[buf] + lane * kQuantRowBytes, (kv ? a.v_src : a.k_src) + row * kHeadDim, kHeadDim * 2,
-              &sm.bar[buf]);
+    bulk_load(sm.rows + lane * kQuantRowBytes, (kv ? a.v_src : a.k_src) + row * kHeadDim, kHeadDim * 2, &sm.bar);
   };
-  constexpr int kVBuf = kQuantBufs - 1;
-  auto krow = [&](int t) { return reinterpret_cast<const __nv_bfloat16*>(sm.rows[0] + t * kQuantRowBytes); };
-  auto vrow = [&](int t) { return reinterpret_cast<const __nv_bfloat16*>(sm.rows[kVBuf] + t * kQuantRowBytes); };
+  auto row_of = [&](int t) { return reinterpret_cast<const __nv_bfloat16*>(sm.rows + t * kQuantRowBytes); };
   const int w0 = blockIdx.x * kQuantWarps + (threadIdx.x >> 5);
   Work k = valid_from(Work{w0, w0 / per_bh, w0 % per_bh});
   int32_t idx = row_index(k);
-  if (k.w < total) {
-    request(k, 0, 0, idx);
-    if constexpr (kQuantBufs == 2) request(k, 1, 1, idx);
-  }
-  // phase of the next completion of each buffer's barrier
-  uint32_t ph_k = 0, ph_v = 0;
+  if (k.w < total) request(k, is_v(k), idx);
+  uint32_t ph = 0;  // phase of the next completion of the barrier
   bool failed = false;
+  auto wait = [&](int where) {
+    failed = !__all_sync(0xffffffffu, mbar_wait(&sm.bar, ph, a.status, where, a.wait_ns));
+    if (!failed) ph ^= 1u;
+    return !failed;
+  };
   while (k.w < total) {
     const Work next = valid_from(stepped(k));
     const int32_t next_idx = row_index(next);
-    const int bh = k.bh, g = k.g;
+    const int bh = bh_of(k), g = k.g;
     QuantOut out;
     out.k_codes = a.k_codes + (size_t)bh * a.cap * kHeadDim * BITS / 8;
     out.k_params = a.k_params + (size_t)bh * (a.cap / kGroup) * 512;
     out.v_codes = a.v_codes + (size_t)bh * a.cap * kHeadDim * BITS / 8;
     out.v_params = a.v_params + (size_t)bh * a.cap * 16;
-    if (!__all_sync(0xffffffffu, mbar_wait(&sm.bar[0], ph_k, a.status, 20, a.wait_ns))) {
-      failed = true;
-      break;
+    bool ok = true, values = is_v(k);
+    if (!wait(values ? 21 : 20)) break;
+    if (!values) {
+      if constexpr (BITS == 2)
+        ok = quantize_keys2(sm.rows, kQuantRowBytes, g, out, sm.st2);
+      else
+        ok = quantize_keys<BITS>(row_of, g, out, sm.st);
+      if constexpr (!APART) {  // every lane has read the K rows: the buffer takes the V rows
+        request(k, 1, idx);
+        if (!wait(21)) break;
+        values = true;
+      }
     }
-    ph_k ^= 1u;
-    bool ok;
-    if constexpr (BITS == 2)
-      ok = quantize_keys2(sm.rows[0], kQuantRowBytes, g, out, sm.st2);
-    else
-      ok = quantize_keys<BITS>(krow, g, out, sm.st);
-    // every lane has read this group's K rows: the buffer takes the next rows
-    if constexpr (kQuantBufs == 2) {
-      if (next.w < total) request(next, 0, 0, next_idx);
-    } else {
-      request(k, 0, 1, idx);
-      ph_v = ph_k;
+    if (values && ok) {
+      if constexpr (BITS == 2)
+        ok = quantize_values2(sm.rows, kQuantRowBytes, g, out, sm.st2);
+      else
+        ok = quantize_values<BITS>(row_of, g, out, sm.st);
     }
-    if (!__all_sync(0xffffffffu, mbar_wait(&sm.bar[kVBuf], ph_v, a.status, 21, a.wait_ns))) {
-      failed = true;
-      break;
-    }
-    ph_v ^= 1u;
-    if constexpr (BITS == 2)
-      ok = ok && quantize_values2(sm.rows[kVBuf], kQuantRowBytes, g, out, sm.st2);
-    else
-      ok = ok && quantize_values<BITS>(vrow, g, out, sm.st);
     if (!ok && lane == 0) set_status(a.status, UC_ERR_RANGE, 2);
-    if constexpr (kQuantBufs == 2) {
-      if (next.w < total) request(next, 1, 1, next_idx);
-    } else {
-      if (next.w < total) request(next, 0, 0, next_idx);
-      ph_k = ph_v;
-    }
+    if (next.w < total) request(next, is_v(next), next_idx);
     idx = next_idx;
     k = next;
   }
   if (failed) {
     // copies still in flight must land before the warp's shared memory is
-    // released: wait for each barrier's pending phase (bounded again)
-    mbar_wait(&sm.bar[0], ph_k, nullptr, 0, a.wait_ns);
-    if constexpr (kQuantBufs == 2) mbar_wait(&sm.bar[1], ph_v, nullptr, 0, a.wait_ns);
+    // released: wait for the barrier's pending phase (bounded again)
+    mbar_wait(&sm.bar, ph, nullptr, 0, a.wait_ns);
     return;
   }
   // the residual tails: the last (n mod 32) kept tokens of a (b, kvh), copied
@@ -626,21 +621,25 @@ void launch_gather(const GatherArgs& a, cudaStream_t st) {
   count_launch();
 }
 
+template <int BITS, bool APART>
+static void quantize(const GatherArgs& a, int blocks, cudaStream_t st) {
+  static bool attr = false;
+  if (!attr)
+    attr = cudaFuncSetAttribute(quantize_groups_kernel<BITS, APART>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kQuantSmemBytes) == cudaSuccess;
+  quantize_groups_kernel<BITS, APART><<<blocks, kQuantWarps * 32, kQuantSmemBytes, st>>>(a);
+}
+
 void launch_quantize(const GatherArgs& a, int bits, cudaStream_t st) {
-  static bool attr4 = false, attr2 = false;
-  const int warps = a.batch * a.n_kv_heads * (a.max_chunks + 1);  // groups and tails
-  const int blocks = std::min((warps + kQuantWarps - 1) / kQuantWarps, kQuantCtasPerSm * compress_sms());
-  if (bits == 4) {
-    if (!attr4)
-      attr4 = cudaFuncSetAttribute(quantize_groups_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)kQuantSmemBytes) == cudaSuccess;
-    quantize_groups_kernel<4><<<blocks, kQuantWarps * 32, kQuantSmemBytes, st>>>(a);
-  } else {
-    if (!attr2)
-      attr2 = cudaFuncSetAttribute(quantize_groups_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)kQuantSmemBytes) == cudaSuccess;
-    quantize_groups_kernel<2><<<blocks, kQuantWarps * 32, kQuantSmemBytes, st>>>(a);
-  }
+  const int nbh = a.batch * a.n_kv_heads, slots = kQuantCtasPerSm * compress_sms();
+  const bool apart =
+      a.src_idx == nullptr && (int64_t)nbh * a.max_chunks < (int64_t)kApartRounds * kQuantWarps * slots;
+  const int warps = nbh * ((apart ? 2 : 1) * a.max_chunks + 1);  // units and tails
+  const int blocks = std::min((warps + kQuantWarps - 1) / kQuantWarps, slots);
+  if (bits == 4)
+    apart ? quantize<4, true>(a, blocks, st) : quantize<4, false>(a, blocks, st);
+  else
+    apart ? quantize<2, true>(a, blocks, st) : quantize<2, false>(a, blocks, st);
   count_launch();
 }
 

@@ -766,12 +766,10 @@ struct AttnPlan {
 
 int groups_per_tile(int bits) { return bits == 2 ? 8 : 4; }
 
-// Many items per (sequence, KV head) (a few long sequences): merge them in a
-// kernel of their own, spread over many SMs (the in-launch merge of one
-// (b, kvh) runs on one SM; 128K batch 2, 54 items: 10 us of a 55 us
-// launch). Below 33 items the second launch costs more than it saves.
+// A plan of more items per (sequence, KV head) than this (a few long
+// sequences) is made for the merge kernel alone: there an item costs the
+// attention launch no merge work.
 constexpr int kMergeKernelItems = 32;
-constexpr int kInLaunchMerge = 40;  // items x n-tiles
 
 int seg_tiles_host(const uc_segment* s, int n) {
   if (!is_quant(s->kind)) return (n + 63) / 64;
@@ -850,13 +848,14 @@ double items_us(double item, int h, int nbh) {
   const int n = (h * nbh + 151) / 152;
   return n * item * (n >= 3 ? 1.0 : (n == 2 ? 1.32 : 2.0));
 }
-// The queue's merge (arrival counter, partials through global memory) ends
-// later than the cluster's by about kQueueMergeUs; a cluster has no idle CTAs
-// to take light items and its CTAs lie less evenly over the SMs
-// (kClusterSpread). Cluster / queue, us on the device: 1K batch 1 7.8 / 9.4,
-// 8K batch 8 (int4, bf16) 14.3 / 16.5, and where the rule takes the queue 8K
-// batch 8 int2 20.6 / 19.8, 8K batch 1 int2 12.3 / 11.7, 32K batch 4 int2
-// 39.3 / 31.7.
+// The queue's merge (a kernel behind the call, partials through global
+// memory) ends later than the cluster's by about kQueueMergeUs; a cluster has
+// no idle CTAs to take light items and its CTAs lie less evenly over the SMs
+// (kClusterSpread). Cluster / queue, us on the device: 200 tokens batch 1
+// 7.6 / 8.6, 3000 bf16 batch 8 14.7 / 15.9, 4000 in three packed segments
+// batch 4 11.0 / 11.9; at the line 2000 int2 batch 16 13.1 / 12.9; where the
+// rule takes the queue 8K batch 8 int2 20.6 / 17.3, 32K batch 4 int2
+// 39.3 / 25.3.
 constexpr double kQueueMergeUs = 1.5, kClusterSpread = 1.15;
 constexpr double kLightItemUs = 0.4;  // SM time of a light item's start and end
 
@@ -948,27 +947,6 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
       const int hw = kWholeMergeItems - nl;
       const double all = (double)hw * nbh_launch;
       if (all / (std::ceil(all / slots) * slots) >= 0.8) H = hw;
-    }
-    // Several n-tiles: an in-launch merge takes about 0.2 us per item and
-    // n-tile on the one SM that runs it (4 x 16K tokens, 4 query tokens: 15 of
-    // 46 us). Past kInLaunchMerge of them, where at most twice the items make
-    // it so, the call takes enough, in full rounds, for the merge kernel, which
-    // spreads them over many SMs (that call 45.3 -> 40.6 us, 8 query tokens
-    // 74.3 -> 63.5; from 12 items per pair up, batch 16: 117 -> 135).
-    if (mtiles > 1 && forced_ipb <= 0 && (H + nl) * mtiles > kInLaunchMerge && 2 * (H + nl) > kMergeKernelItems &&
-        H + nl <= kMergeKernelItems) {
-      int tiles = 0;
-      for (int s = 0; s < nseg; ++s) tiles += heavy[s] ? htiles[s] : 0;
-      double best_eff = -1.0;
-      for (int h = kMergeKernelItems + 1 - nl; h <= std::min(hmax, tiles); ++h) {
-        const double all = (double)h * nbh_launch;
-        const double eff = all / (std::ceil(all / slots) * slots);
-        if (eff > best_eff + 1e-9) {
-          best_eff = eff;
-          H = h;
-        }
-        if (eff >= 0.9) break;
-      }
     }
     // calls whose merge is the separate kernel: there an item costs no
     // merge work, so take the most heavy items that still start in the
@@ -1155,6 +1133,14 @@ uc_status check_call(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_
 int decode_mtiles(int n_q_heads, int hkv, int n_qtok) { return (n_q_heads / hkv * n_qtok + 7) / 8; }
 
 int merge_kernel_for(int items_per_bh) { return items_per_bh > kMergeKernelItems ? 1 : 0; }
+
+// Output channels per CTA of the merge kernel: the fewest whose CTAs are all
+// resident at once.
+int merge_width(int pairs, int mtiles) {
+  for (int cw = 32; cw < UC_HEAD_DIM; cw *= 2)
+    if (pairs * mtiles * (UC_HEAD_DIM / cw) <= kMergePerSm * num_sms()) return cw;
+  return UC_HEAD_DIM;
+}
 
 // A decode call's merge counters (one per (b, kvh)) live in a block of fixed
 // size at a fixed place of the workspace, whatever the call's shape: every
@@ -1447,7 +1433,12 @@ uc_status uc_attend(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_s
   if (st != UC_OK) return st;
   // (a device whose clusters fit less well than planned for takes the queue)
   p.cluster = plan.cluster > 0 && attend_clusters(plan.cluster) >= B * hkv ? plan.cluster : 0;
-  p.defer_merge = p.cluster ? 0 : merge_kernel_for(plan.items_per_bh);
+  // Outside clusters the merge is a kernel of its own, also for few items:
+  // launched programmatically it starts as the last items end, while a merge
+  // in the launch streams through the one SM that finishes a pair (one query
+  // token, 16 x 8K 33.0 -> 27.4 us, 4 x 16K 20.1 -> 17.6, 32K int2, batch 16,
+  // 67.1 -> 66.1; four, 4 x 16K 40.8 -> 34.4, 4 x 4K 28.9 -> 17.4; no size was slower).
+  p.defer_merge = p.cluster ? 0 : merge_width(B * hkv, plan.mtiles);
   if (plan.mtiles > 1 && plan.grid <= num_sms()) p.stages = 3;
   launch_attend(p, plan.grid, reinterpret_cast<cudaStream_t>(stream));
   return cuda_check("uc_attend");

@@ -15,11 +15,13 @@
 //               with one LOP3, scales folded into the queries (keys) and the
 //               probabilities (values), S and P V in fp16 with fp32
 //               accumulation.
-// Each item leaves an unnormalised partial (O, m, l); the last CTA to finish
-// a (sequence, KV head) merges its items by log-sum-exp, writes O, lse and
-// the per-segment probability mass, and re-arms the counter. In short calls
-// the items of a (sequence, KV head) run on one thread-block cluster instead,
-// which merges them through distributed shared memory.
+// Each item leaves an unnormalised partial (O, m, l); a merge kernel launched
+// programmatically behind the call merges a (sequence, KV head)'s items by
+// log-sum-exp and writes O, lse and the per-segment probability mass. In
+// short calls the items of a (sequence, KV head) run on one thread-block
+// cluster instead, which merges them through distributed shared memory; in a
+// batch of calls the last CTA to finish a pair merges it and re-arms its
+// counter.
 #include <atomic>
 #include <mutex>
 
@@ -1091,24 +1093,26 @@ __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t*
   if (seq != nullptr) *seq += total;
 }
 
-// Split-K merge as a kernel of its own, for calls with many items per
-// (sequence, KV head) (few long sequences): one CTA per (sequence, KV head,
-// 8-row block, 32 output channels), so the partials of one (b, kvh) are read
-// by several SMs at once instead of streaming through one. Eight warps take
-// every eighth item each, all their loads in flight together; the warps'
-// sums meet in shared memory. The attend launch before it leaves the
-// partials and skips its own merges (`defer_merge`).
-constexpr int kMergeChunks = kHeadDim / 32;
-__global__ void __launch_bounds__(256) merge_partials_kernel(const __grid_constant__ AttnParams p) {
+// Split-K merge as a kernel of its own: a CTA per (sequence, KV head, 8-row
+// block, CW output channels), so the partials of one (b, kvh) are read by
+// several SMs at once instead of streaming through one. A thread has four
+// channels of one row, so 128 / CW groups of threads share the items; the
+// first eight items of each group are fetched before the weights are known.
+// The attend launch before it leaves the partials and skips its own merges
+// (`defer_merge`). What bounds it is the chain launch -> maxima and sums ->
+// weights -> sums; with many pairs every CTA's weights would count too (eight
+// query tokens, 16 x 300: CW 32 took 31.6 us, 20.1 so), so CW grows with the
+// number of CTAs (`merge_width`).
+template <int CW>
+__global__ void __launch_bounds__(256, kMergePerSm) merge_partials_kernel(const __grid_constant__ AttnParams p) {
+  constexpr int kCols = CW / 4, kPos = 8 * kCols, G = 256 / kPos, kPre = 8;
   __shared__ float s_m[kMaxItemsPerBh * 8], s_w[kMaxItemsPerBh * 8];  // m, then the weights; l
-  __shared__ float s_red[8][8][33];
+  __shared__ float4 s_red[G][kPos];
   griddep_wait();  // the attention launch whose partials this merges has completed
   griddep_launch_dependents();
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int rblocks = p.mtiles;
-  const int ch = blockIdx.x % kMergeChunks;
-  const int r0 = ((blockIdx.x / kMergeChunks) % rblocks) * 8;
-  const int bh = blockIdx.x / (kMergeChunks * rblocks);
+  const int tid = threadIdx.x;
+  const int ch = blockIdx.x % (kHeadDim / CW), blk = blockIdx.x / (kHeadDim / CW);
+  const int r0 = (blk % p.mtiles) * 8, bh = blk / p.mtiles;
   const int b = bh / p.n_kv_heads, kvh = bh % p.n_kv_heads;
   const int nr = min(8, p.rows - r0);
   const size_t pf = attend_part_floats(p.mtiles);
@@ -1126,40 +1130,45 @@ __global__ void __launch_bounds__(256) merge_partials_kernel(const __grid_consta
     s_m[x] = m;
     s_w[x] = l;
   }
+  const int pos = tid % kPos, grp = tid / kPos, rr = pos / kCols, c = ch * CW + 4 * (pos % kCols);
+  const float* col = base + (size_t)(r0 + rr) * kHeadDim + c;
+  float4 v[kPre];
+  auto fetch = [&](int i0) {
+#pragma unroll
+    for (int k = 0; k < kPre; ++k) {
+      const int i = i0 + G * k;
+      v[k] = i < I && rr < nr ? __ldg(reinterpret_cast<const float4*>(col + i * pf)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  fetch(grp);
   __syncthreads();
   if (tid < 128) merge_weights<16>(p, s_m, s_w, 8, b, kvh, r0, nr, ch == 0);
   __syncthreads();
-  const int c = ch * 32 + lane;
-  float v[kMaxItemsPerBh / 8][8];
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int i0 = grp; i0 < I; i0 += G * kPre) {
+    if (i0 != grp) fetch(i0);
 #pragma unroll
-  for (int k = 0; k < kMaxItemsPerBh / 8; ++k) {
-    const int i = warp + 8 * k;
-#pragma unroll
-    for (int rr = 0; rr < 8; ++rr)
-      v[k][rr] = (i < I && rr < nr) ? __ldg(base + i * pf + (size_t)(r0 + rr) * kHeadDim + c) : 0.f;
-  }
-  float acc[8];
-#pragma unroll
-  for (int rr = 0; rr < 8; ++rr) acc[rr] = 0.f;
-#pragma unroll
-  for (int k = 0; k < kMaxItemsPerBh / 8; ++k) {
-    const int i = warp + 8 * k;
-    if (i < I)
-#pragma unroll
-      for (int rr = 0; rr < 8; ++rr) acc[rr] += s_m[i * 8 + rr] * v[k][rr];
-  }
-#pragma unroll
-  for (int rr = 0; rr < 8; ++rr) s_red[warp][rr][lane] = acc[rr];
-  __syncthreads();
-  {
-    const int rr = warp;  // 8 warps: one row each
-    float sum = 0.f;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) sum += s_red[w][rr][lane];
-    if (rr < nr) {
-      p.out[out_row(p, b, kvh, r0 + rr) * kHeadDim + c] = __float2bfloat16_rn(sum);
+    for (int k = 0; k < kPre; ++k) {
+      const int i = i0 + G * k;
+      if (i < I) {
+        const float w = s_m[i * 8 + rr];
+        acc.x += w * v[k].x; acc.y += w * v[k].y; acc.z += w * v[k].z; acc.w += w * v[k].w;
+      }
     }
   }
+  if constexpr (G > 1) {
+    s_red[grp][pos] = acc;
+    __syncthreads();
+    if (grp != 0) return;
+#pragma unroll
+    for (int k = 1; k < G; ++k) {
+      const float4 o = s_red[k][pos];
+      acc.x += o.x; acc.y += o.y; acc.z += o.z; acc.w += o.w;
+    }
+  }
+  if (rr < nr)
+    *reinterpret_cast<uint2*>(p.out + out_row(p, b, kvh, r0 + rr) * kHeadDim + c) =
+        make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
 }
 
 // Query rows of every n-tile as Q^T B fragments (bf16 for bf16 rows, else
@@ -1781,7 +1790,13 @@ void launch_attend(const AttnParams& p, int grid, cudaStream_t st) {
     // always launched programmatically: its CTAs take the SM slots the
     // attention CTAs free and wait (griddepcontrol.wait) for that launch to
     // complete, instead of a launch gap after it
-    launch_maybe_pdl(true, merge_partials_kernel, p.batch * p.n_kv_heads * p.mtiles * kMergeChunks, 256, 0, st, p);
+    const int ctas = p.batch * p.n_kv_heads * p.mtiles * (kHeadDim / p.defer_merge);
+    if (p.defer_merge == 32)
+      launch_maybe_pdl(true, merge_partials_kernel<32>, ctas, 256, 0, st, p);
+    else if (p.defer_merge == 64)
+      launch_maybe_pdl(true, merge_partials_kernel<64>, ctas, 256, 0, st, p);
+    else
+      launch_maybe_pdl(true, merge_partials_kernel<128>, ctas, 256, 0, st, p);
     count_launch();
   }
 }

@@ -217,7 +217,9 @@ struct AttnParams {
   // work queue: one per heavy item, then one for the light items or one each
   int cluster;
   int stages;       // ring slots of a CTA (uc_attend; batched launches take two)
-  int defer_merge;  // 1: the attend launch only leaves partials; a merge kernel follows
+  // > 0: the attend launch only leaves partials; a merge kernel follows, whose
+  // CTAs take this many output channels each
+  int defer_merge;
   float scale_log2;
   uint64_t wait_ns;  // limit of every bounded wait of the launch (UC_ERR_TIMEOUT past it)
   int withhold_pos;  // test hook: the first tile of the item at this position is never copied (-1: none)
@@ -273,6 +275,7 @@ int attend_ctas_per_sm(int ntiles);
 constexpr int kMaxClusterItems = 16;  // CTAs of the largest cluster
 int attend_clusters(int c);
 __host__ __device__ size_t attend_part_floats(int mtiles);
+constexpr int kMergePerSm = 3;  // CTAs of the merge kernel per SM
 void launch_attend(const AttnParams& p, int grid, cudaStream_t st);
 void launch_attend_multi(const MultiAttnParams& m, int grid, cudaStream_t st);
 

@@ -375,6 +375,24 @@ def test_attend_query_tiles_many_items(hq, T):
     assert ws.status() == 0
 
 
+@pytest.mark.parametrize("T,B", [(3, 2), (3, 12), (3, 20), (8, 5), (8, 9), (1, 40)])
+def test_attend_merge_widths(T, B):
+    """The merge kernel's CTAs of 32, 64 and 128 channels (more pairs and row
+    blocks), over a last row block of 5 of its 8 rows, items that split
+    unevenly over a CTA's thread groups and sequences that keep one token."""
+    hkv = 4
+    sizes, kinds = [400, 700, 300], ["full", "quant", "evict_quant"]
+    keeps = [400, 700, [1 + (37 * b) % 300 for b in range(B)]]
+    gsegs, osegs = _build_mix(100 * T + B, B, hkv, sizes, kinds, keeps, [16, 4, 2])
+    q = synth.make_q(T + B, B, 28, T)
+    O, lse, mass = uc.attend(dev(q), gsegs)
+    rO, rl, rm = oattn.attend(q, osegs, hkv)
+    assert _packed.attention_error(host(O), rO) <= _packed.ATTN_RTOL
+    bound = _packed.logit_error_bound(q, osegs, hkv, [False, True, True])
+    assert (np.abs(host(lse) - rl) <= bound).all()
+    assert (np.abs(host(mass) - rm) <= 2 * bound[..., None]).all()
+
+
 CLUSTER_MIXES = {
     # (B, Hkv, sizes, kinds, keeps, bits): clusters of 1, few and 16 CTAs, more
     # light items than ranks, eight segments, sequences that hold nothing of a

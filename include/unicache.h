@@ -518,8 +518,9 @@ typedef struct {
   int32_t n_heavy, n_light;             /* heavy / light items per (sequence, KV head) */
   int32_t grid;                         /* CTAs that walk the items as a work queue */
   int32_t merge_kernel;                 /* 1: more items than a merge inside the launch is planned for
-                                         * (> 32); at any count a single call outside clusters merges in
-                                         * a kernel of its own, a batch inside its launch */
+                                         * (> 32); at any count a call outside clusters merges in a
+                                         * kernel of its own, a batch of several query tiles
+                                         * inside its launch */
   int32_t n_chunks[UC_MAX_SEGMENTS];    /* items of each segment */
   int32_t light[UC_MAX_SEGMENTS];       /* 1: every item of the segment is light */
 } uc_attend_plan_info;

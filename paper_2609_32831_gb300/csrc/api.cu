@@ -1136,9 +1136,9 @@ int merge_kernel_for(int items_per_bh) { return items_per_bh > kMergeKernelItems
 
 // Output channels per CTA of the merge kernel: the fewest whose CTAs are all
 // resident at once.
-int merge_width(int pairs, int mtiles) {
+int merge_width(int blocks) {
   for (int cw = 32; cw < UC_HEAD_DIM; cw *= 2)
-    if (pairs * mtiles * (UC_HEAD_DIM / cw) <= kMergePerSm * num_sms()) return cw;
+    if (blocks * (UC_HEAD_DIM / cw) <= kMergePerSm * num_sms()) return cw;
   return UC_HEAD_DIM;
 }
 
@@ -1185,7 +1185,6 @@ uc_status build_decode_call(const void* q, int32_t n_q_heads, int32_t n_qtok, co
     const uc_status st = segment_maps(sg, &p->tmap[2 * s], &p->tmap[2 * s + 1]);
     if (st != UC_OK) return st;
   }
-  const size_t nbh = (size_t)B * hkv;
   p->status = status;
   p->sched = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(status) + 128);
   p->counters = reinterpret_cast<int32_t*>(counters);
@@ -1438,7 +1437,7 @@ uc_status uc_attend(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_s
   // in the launch streams through the one SM that finishes a pair (one query
   // token, 16 x 8K 33.0 -> 27.4 us, 4 x 16K 20.1 -> 17.6, 32K int2, batch 16,
   // 67.1 -> 66.1; four, 4 x 16K 40.8 -> 34.4, 4 x 4K 28.9 -> 17.4; no size was slower).
-  p.defer_merge = p.cluster ? 0 : merge_width(B * hkv, plan.mtiles);
+  p.defer_merge = p.cluster ? 0 : merge_width(B * hkv * plan.mtiles);
   if (plan.mtiles > 1 && plan.grid <= num_sms()) p.stages = 3;
   launch_attend(p, plan.grid, reinterpret_cast<cudaStream_t>(stream));
   return cuda_check("uc_attend");
@@ -1533,6 +1532,7 @@ uc_status uc_attend_batch(const uc_attend_call* calls, int32_t n_calls, void* wo
   m.light_begin[n_calls] = light;
   m.n_calls = n_calls;
   m.n_items = heavy + light;
+  m.merge_width = merge_width(nbh_launch * mtiles);
   const int slots = std::max(1, attend_ctas_per_sm(mtiles)) * num_sms();
   launch_attend_multi(m, std::min(m.n_items, slots), reinterpret_cast<cudaStream_t>(stream));
   return cuda_check("uc_attend_batch");

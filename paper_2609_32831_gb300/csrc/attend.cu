@@ -20,8 +20,8 @@
 // log-sum-exp and writes O, lse and the per-segment probability mass. In
 // short calls the items of a (sequence, KV head) run on one thread-block
 // cluster instead, which merges them through distributed shared memory; in a
-// batch of calls the last CTA to finish a pair merges it and re-arms its
-// counter.
+// batch of calls of several n-tiles the last CTA to finish a pair merges it
+// and re-arms its counter.
 #include <atomic>
 #include <mutex>
 
@@ -59,7 +59,9 @@ constexpr int kMaxPendingMerges = 64;
 constexpr int kItemQ = 2;  // items handed from the producer to the consumers ahead
 
 struct AttnSmem {
-  alignas(16) float merge_w[kMaxItemsPerBh * 8];  // per (item, row of an 8-row block): m, then weight
+  // one n-tile: the query fragments; a cluster's row sums. Several: m, then
+  // weight; l, per (item, row of an 8-row block) of a merge
+  alignas(16) float merge_w[kMaxItemsPerBh * 8];
   float merge_l[kMaxItemsPerBh * 8];
   uint64_t full[kMaxStages];
   uint64_t empty[kMaxStages];
@@ -72,9 +74,8 @@ struct AttnSmem {
 };
 
 // Query fragments of the current item live in shared memory (2 KB per
-// n-tile of 8 query rows): for one n-tile in the merge staging arrays, which
-// are idle while an item runs (merges happen between items), keeping three
-// CTAs per SM; for more n-tiles after the ring. The bf16 query rows of an
+// n-tile of 8 query rows): for one n-tile in `merge_w`, keeping three CTAs
+// per SM; for more n-tiles after the ring. The bf16 query rows of an
 // item as the producer copies them (g * T rows) take as much again per entry
 // of the item queue.
 constexpr int kQTileBytes = 2048;
@@ -185,6 +186,7 @@ struct OneCall {
     *c = 0;
     return p;
   }
+  __device__ const AttnParams& merge_call(int*) const { return p; }
 };
 
 struct ManyCalls {
@@ -206,6 +208,13 @@ struct ManyCalls {
       *local = p.n_heavy * p.batch * p.n_kv_heads + (q - m.light_begin[k]);
     }
     *c = k;
+    return m.call[k];
+  }
+  // the call of row block *blk of the merge (then the block's place in it)
+  __device__ const AttnParams& merge_call(int* blk) const {
+    int k = 0;
+    for (int n; k + 1 < m.n_calls && *blk >= (n = m.call[k].batch * m.call[k].n_kv_heads * m.call[k].mtiles); ++k)
+      *blk -= n;
     return m.call[k];
   }
 };
@@ -991,7 +1000,7 @@ __device__ __forceinline__ void merge_weights(const AttnParams& p, float* ml, co
   }
 }
 
-// The merge runs on the 128 consumer threads of the CTA that finished the
+// A batch's merge with several n-tiles runs on the 128 consumer threads of the CTA that finished the
 // last item of a (sequence, KV head): the weights of every item and row, then
 // per 8-row block the weighted sums of the items' O, four channels of two
 // rows per thread (16-byte shared-memory reads; one 4-byte read per value
@@ -999,7 +1008,9 @@ __device__ __forceinline__ void merge_weights(const AttnParams& p, float* ml, co
 // item the ring is idle (`seq` given): the row blocks of O stream through it
 // back to back, eight items per slot, by bulk copies continuing the consumers'
 // tile sequence, the first ones in flight while the weights are formed.
-// Without `seq` (a merge between items) the threads load them.
+// Without `seq` (a merge between items) the threads load them. (Without these
+// merges in it the kernel's int4 loops came out 3 % slower, so such batches
+// keep them.)
 template <int NTW, int ST>
 __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t* seq) {
   const int tid = threadIdx.x;
@@ -1028,9 +1039,9 @@ __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t*
   }
   // rows whose weights are formed at once: every row when the query buffers
   // behind the ring are idle too, else the 8 rows the merge arrays hold
-  const int set = NTW == 1 || seq == nullptr ? 8 : rows_pad;
-  float* wts = NTW == 1 || seq == nullptr ? sm.merge_w : reinterpret_cast<float*>(after_ring<ST>(sm));  // [I][set]
-  float* ls = NTW == 1 || seq == nullptr ? sm.merge_l : wts + I * set;
+  const int set = seq == nullptr ? 8 : rows_pad;
+  float* wts = seq == nullptr ? sm.merge_w : reinterpret_cast<float*>(after_ring<ST>(sm));  // [I][set]
+  float* ls = seq == nullptr ? sm.merge_l : wts + I * set;
   const int cq = tid & 31, rg = tid >> 5;  // channels 4 cq .. + 3, rows 2 rg, 2 rg + 1 of a block
   for (int s0 = 0; s0 < p.rows; s0 += set) {
     for (int x = tid; x < I * set; x += 128) {
@@ -1041,7 +1052,7 @@ __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t*
     }
     consumer_sync();
     const int nr = min(set, p.rows - s0);
-    if (NTW == 1 || set == 8)
+    if (set == 8)
       merge_weights<16>(p, wts, ls, 8, b, kvh, s0, nr);
     else if (p.mtiles <= 2)
       merge_weights<8>(p, wts, ls, set, b, kvh, s0, nr);
@@ -1098,20 +1109,22 @@ __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t*
 // several SMs at once instead of streaming through one. A thread has four
 // channels of one row, so 128 / CW groups of threads share the items; the
 // first eight items of each group are fetched before the weights are known.
-// The attend launch before it leaves the partials and skips its own merges
-// (`defer_merge`). What bounds it is the chain launch -> maxima and sums ->
+// One launch serves every call of a batch of one n-tile. What bounds it is the chain launch -> maxima and sums ->
 // weights -> sums; with many pairs every CTA's weights would count too (eight
 // query tokens, 16 x 300: CW 32 took 31.6 us, 20.1 so), so CW grows with the
 // number of CTAs (`merge_width`).
-template <int CW>
-__global__ void __launch_bounds__(256, kMergePerSm) merge_partials_kernel(const __grid_constant__ AttnParams p) {
+template <int CW, class P>
+__global__ void __launch_bounds__(256, kMergePerSm) merge_partials_kernel(const __grid_constant__ P params) {
   constexpr int kCols = CW / 4, kPos = 8 * kCols, G = 256 / kPos, kPre = 8;
   __shared__ float s_m[kMaxItemsPerBh * 8], s_w[kMaxItemsPerBh * 8];  // m, then the weights; l
   __shared__ float4 s_red[G][kPos];
   griddep_wait();  // the attention launch whose partials this merges has completed
   griddep_launch_dependents();
   const int tid = threadIdx.x;
-  const int ch = blockIdx.x % (kHeadDim / CW), blk = blockIdx.x / (kHeadDim / CW);
+  const typename WorkOf<P>::type w{params};
+  const int ch = blockIdx.x % (kHeadDim / CW);
+  int blk = blockIdx.x / (kHeadDim / CW);
+  const AttnParams& p = w.merge_call(&blk);
   const int r0 = (blk % p.mtiles) * 8, bh = blk / p.mtiles;
   const int b = bh / p.n_kv_heads, kvh = bh % p.n_kv_heads;
   const int nr = min(8, p.rows - r0);
@@ -1151,8 +1164,8 @@ __global__ void __launch_bounds__(256, kMergePerSm) merge_partials_kernel(const 
     for (int k = 0; k < kPre; ++k) {
       const int i = i0 + G * k;
       if (i < I) {
-        const float w = s_m[i * 8 + rr];
-        acc.x += w * v[k].x; acc.y += w * v[k].y; acc.z += w * v[k].z; acc.w += w * v[k].w;
+        const float wt = s_m[i * 8 + rr];
+        acc.x += wt * v[k].x; acc.y += wt * v[k].y; acc.z += wt * v[k].z; acc.w += wt * v[k].w;
       }
     }
   }
@@ -1231,6 +1244,57 @@ __device__ __forceinline__ void reduce_row_sums(WarpState<NTW>& st) {
     }
 }
 
+// One n-tile: the four consumer warps' states meet in an idle ring slot in one
+// step (rows padded by four floats: the fragments' stores and the row reads
+// are conflict-free), then 16 threads per query row sum them, eight channels
+// each, and store or pass on whole 16-byte pieces. (By a pairwise tree with
+// its barriers and 4-byte stores by the last warp 4K int2, batch 1, took 8.8
+// us, so 8.3; 32K int2, batch 16, 65.8 and 65.2.)
+struct WarpsO {
+  float o[kConsumers][8][kHeadDim + 4];
+  float m[kConsumers][8], l[kConsumers][8];
+};
+static_assert(sizeof(WarpsO) <= kSlotBytes, "in a ring slot");
+
+__device__ __forceinline__ void put_warp(WarpsO& b, int warp, const WarpState<1>& st) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, j = lane & 3;
+#pragma unroll
+  for (int mt = 0; mt < 8; ++mt)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) b.o[warp][2 * j + (e & 1)][16 * mt + g + 8 * (e >> 1)] = st.o[0][mt][e];
+  if (g == 0) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      b.m[warp][2 * j + h] = st.m[0][h];
+      b.l[warp][2 * j + h] = st.l[0][h];
+    }
+  }
+}
+
+// Maximum of row threadIdx.x / 16 over the warps, their weights, and O of
+// channels 4 (threadIdx.x % 16) + {0 .. 3} and the same + 64.
+__device__ __forceinline__ float sum_warps(const WarpsO& b, float (&wt)[kConsumers], float4 (&o)[2]) {
+  const int row = threadIdx.x >> 4, c = 4 * (threadIdx.x & 15);
+  float M = kNegInf;
+#pragma unroll
+  for (int w = 0; w < kConsumers; ++w) M = fmaxf(M, b.m[w][row]);
+#pragma unroll
+  for (int w = 0; w < kConsumers; ++w) {
+    const float m = b.m[w][row];
+    wt[w] = m == kNegInf ? 0.f : exp2f(m - M);
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    o[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < kConsumers; ++w) {
+      const float4 x = *reinterpret_cast<const float4*>(&b.o[w][row][c + 64 * h]);
+      o[h].x += wt[w] * x.x; o[h].y += wt[w] * x.y; o[h].z += wt[w] * x.z; o[h].w += wt[w] * x.w;
+    }
+  }
+  return M;
+}
+
 // Merge the warps that share n-tiles (through the item's last slot), then
 // write this item's partial.
 template <int NTW>
@@ -1240,6 +1304,32 @@ __device__ __forceinline__ void finish_item(const AttnParams& p, AttnSmem& sm, W
   const int g = lane >> 2, j = lane & 3;
   fold_zero_points<NTW>(st);
   reduce_row_sums<NTW>(st);
+  if constexpr (NTW == 1) {
+    float* pi = p.part + (size_t)it * attend_part_floats(1);
+    const int row = threadIdx.x >> 4, c = 4 * (threadIdx.x & 15);
+    float4 o[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+    float M = kNegInf, l = 0.f;
+    if (last_slot >= 0) {
+      WarpsO& b = *reinterpret_cast<WarpsO*>(sm.slot[last_slot]);
+      consumer_sync();  // every warp has read the slot's tile
+      put_warp(b, ks, st);
+      consumer_sync();
+      float wt[kConsumers];
+      M = sum_warps(b, wt, o);
+#pragma unroll
+      for (int w = 0; w < kConsumers; ++w) l += wt[w] * b.l[w][row];
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sm.empty[last_slot]);
+    }
+    *reinterpret_cast<float4*>(pi + row * kHeadDim + c) = o[0];
+    *reinterpret_cast<float4*>(pi + row * kHeadDim + c + 64) = o[1];
+    if (c == 0) {
+      pi[8 * kHeadDim + row] = M;
+      pi[8 * kHeadDim + 8 + row] = l;
+    }
+    return;
+  }
   constexpr int kVals = NTW * 36;
   if (KS > 1 && last_slot >= 0) {
     float* buf = reinterpret_cast<float*>(sm.slot[last_slot]);
@@ -1414,7 +1504,7 @@ struct ClusterPart {
   float l[UC_MAX_SEGMENTS][8];         // row sums per segment
 };
 struct ClusterSmem {
-  float o[kConsumers][8][kHeadDim];    // the warps' O
+  WarpsO warps;
   ClusterPart part;
 };
 static_assert(sizeof(ClusterSmem) <= (size_t)kStages * kSlotBytes, "in the idle ring");
@@ -1488,38 +1578,15 @@ __device__ __forceinline__ void consume_cluster(const AttnParams& p, AttnSmem& s
   fold_zero_points<1>(st);
   ClusterSmem& cs = *reinterpret_cast<ClusterSmem*>(sm.slot[0]);
   consumer_sync();  // every warp is past its last tile: the ring is idle
-#pragma unroll
-  for (int mt = 0; mt < 8; ++mt)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) cs.o[warp][2 * j + (e & 1)][16 * mt + g + 8 * (e >> 1)] = st.o[0][mt][e];
-  float* wm = sm.merge_w;  // the warps' row maxima (the query fragments are no longer needed)
-  if (g == 0) {
-    wm[warp * 8 + 2 * j] = st.m[0][0];
-    wm[warp * 8 + 2 * j + 1] = st.m[0][1];
-  }
+  put_warp(cs.warps, warp, st);
   consumer_sync();
   {
-    const int row = threadIdx.x >> 4;  // 16 threads per row, two float4 each
-    float M = kNegInf, wt[kConsumers];
-#pragma unroll
-    for (int w = 0; w < kConsumers; ++w) M = fmaxf(M, wm[w * 8 + row]);
-#pragma unroll
-    for (int w = 0; w < kConsumers; ++w) {
-      const float m = wm[w * 8 + row];
-      wt[w] = m == kNegInf ? 0.f : exp2f(m - M);
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int c = 4 * (threadIdx.x & 15) + 64 * h;
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int w = 0; w < kConsumers; ++w) {
-        const float4 x = *reinterpret_cast<const float4*>(&cs.o[w][row][c]);
-        a.x += wt[w] * x.x; a.y += wt[w] * x.y; a.z += wt[w] * x.z; a.w += wt[w] * x.w;
-      }
-      *reinterpret_cast<float4*>(&cs.part.o[row][c]) = a;
-    }
-    const int s = threadIdx.x & 15;
+    const int row = threadIdx.x >> 4, c = 4 * (threadIdx.x & 15), s = threadIdx.x & 15;
+    float wt[kConsumers];
+    float4 o[2];
+    const float M = sum_warps(cs.warps, wt, o);
+    *reinterpret_cast<float4*>(&cs.part.o[row][c]) = o[0];
+    *reinterpret_cast<float4*>(&cs.part.o[row][c + 64]) = o[1];
     if (s < p.nseg) {
       float l = 0.f;
 #pragma unroll
@@ -1600,7 +1667,7 @@ __device__ void consume(const W& w, AttnSmem& sm) {
   bool aborted = false;
   // thread 0: the last arrival (call << 16 | bh), checked one item later
   int prev_key = -1, prev_arrivals = -1;
-  if (threadIdx.x == 0) sm.n_pending = 0;
+  if (NTW > 1 && threadIdx.x == 0) sm.n_pending = 0;
   for (uint32_t iseq = 0;; ++iseq) {
     const int k = iseq % kItemQ;
     if (!mbar_wait(&sm.item_full[k], (iseq / kItemQ) & 1, w.call(0).status, 13, w.call(0).wait_ns)) break;
@@ -1617,10 +1684,11 @@ __device__ void consume(const W& w, AttnSmem& sm) {
     else
       run_item<NTW, ST, 2>(p, sm, ii, it, k, seq, aborted, NG, KS, grp, ks);
 
+    consumer_sync();  // the next item's query fragments take this one's place
+    if constexpr (NTW == 1) continue;
     // Arrive on the item's counter; the CTA whose arrival completes a
     // (sequence, KV head) owes its merge, done after its last item so that
     // no warp waits for the atomic here.
-    consumer_sync();
     if (threadIdx.x == 0 && !p.defer_merge) {
       if (prev_key >= 0 && prev_arrivals == w.items_per_bh(prev_key >> 16) - 1)
         sm.pending[sm.n_pending++] = prev_key;
@@ -1640,6 +1708,7 @@ __device__ void consume(const W& w, AttnSmem& sm) {
       consumer_sync();
     }
   }
+  if constexpr (NTW == 1) return;
   if (threadIdx.x == 0) {
     if (prev_key >= 0 && prev_arrivals == w.items_per_bh(prev_key >> 16) - 1)
       sm.pending[sm.n_pending++] = prev_key;
@@ -1768,6 +1837,21 @@ int attend_clusters(int c) {
   return n;
 }
 
+// The merge of `blocks` (pair, row block)s. Always launched programmatically:
+// its CTAs take the SM slots the attention CTAs free and wait
+// (griddepcontrol.wait) for that launch to complete, instead of a launch gap
+// after it.
+template <class P>
+static void launch_merge(const P& p, int blocks, int width, cudaStream_t st) {
+  if (width == 32)
+    launch_maybe_pdl(true, merge_partials_kernel<32, P>, blocks * 4, 256, 0, st, p);
+  else if (width == 64)
+    launch_maybe_pdl(true, merge_partials_kernel<64, P>, blocks * 2, 256, 0, st, p);
+  else
+    launch_maybe_pdl(true, merge_partials_kernel<kHeadDim, P>, blocks, 256, 0, st, p);
+  count_launch();
+}
+
 void launch_attend(const AttnParams& p, int grid, cudaStream_t st) {
   attend_setup_once();
   const bool pdl = pdl_enabled();
@@ -1786,29 +1870,22 @@ void launch_attend(const AttnParams& p, int grid, cudaStream_t st) {
   else
     launch_maybe_pdl(pdl, attend_kernel<2, AttnParams>, grid, kAttnThreads, smem, st, p);
   count_launch();
-  if (p.defer_merge) {
-    // always launched programmatically: its CTAs take the SM slots the
-    // attention CTAs free and wait (griddepcontrol.wait) for that launch to
-    // complete, instead of a launch gap after it
-    const int ctas = p.batch * p.n_kv_heads * p.mtiles * (kHeadDim / p.defer_merge);
-    if (p.defer_merge == 32)
-      launch_maybe_pdl(true, merge_partials_kernel<32>, ctas, 256, 0, st, p);
-    else if (p.defer_merge == 64)
-      launch_maybe_pdl(true, merge_partials_kernel<64>, ctas, 256, 0, st, p);
-    else
-      launch_maybe_pdl(true, merge_partials_kernel<128>, ctas, 256, 0, st, p);
-    count_launch();
-  }
+  launch_merge(p, p.batch * p.n_kv_heads * p.mtiles, p.defer_merge, st);
 }
 
 void launch_attend_multi(const MultiAttnParams& m, int grid, cudaStream_t st) {
   attend_setup_once();
   const size_t smem = attend_smem_bytes(m.call[0].mtiles);
-  if (m.call[0].mtiles <= 1)
-    attend_kernel<1, MultiAttnParams><<<grid, kAttnThreads, smem, st>>>(m);
-  else
+  if (m.call[0].mtiles > 1) {
     attend_kernel<2, MultiAttnParams><<<grid, kAttnThreads, smem, st>>>(m);
+    count_launch();
+    return;
+  }
+  attend_kernel<1, MultiAttnParams><<<grid, kAttnThreads, smem, st>>>(m);
   count_launch();
+  int blocks = 0;
+  for (int c = 0; c < m.n_calls; ++c) blocks += m.call[c].batch * m.call[c].n_kv_heads;
+  launch_merge(m, blocks, m.merge_width, st);
 }
 
 }  // namespace uc

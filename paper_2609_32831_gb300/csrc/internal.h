@@ -232,6 +232,7 @@ struct MultiAttnParams {
   int heavy_begin[UC_MAX_CALLS + 1];  // prefix over calls of n_heavy * B * Hkv
   int light_begin[UC_MAX_CALLS + 1];  // prefix over calls of n_light * B * Hkv
   int n_calls, n_items;
+  int merge_width;  // output channels per CTA of the merge kernel (one n-tile)
 };
 
 // ------------------------------------------------- dense (many queries)

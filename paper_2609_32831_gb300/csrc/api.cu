@@ -940,17 +940,16 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
       }
     }
     H = std::min(std::max(H, nh), hmax);
-    // single-n-tile calls: items that the in-kernel merge stages in one
-    // round trip, if they still keep >= 80 % of the slots busy (8K
-    // understanding layer: 15 -> 14 items, 21.0 -> 19.5 us)
-    if (mtiles == 1 && forced_ipb <= 0 && H + nl > kWholeMergeItems && kWholeMergeItems - nl >= nh) {
-      const int hw = kWholeMergeItems - nl;
+    // single-n-tile calls: few items, if they still keep >= 80 % of the
+    // slots busy
+    if (mtiles == 1 && forced_ipb <= 0 && H + nl > kFewItems && kFewItems - nl >= nh) {
+      const int hw = kFewItems - nl;
       const double all = (double)hw * nbh_launch;
       if (all / (std::ceil(all / slots) * slots) >= 0.8) H = hw;
     }
-    // calls whose merge is the separate kernel: there an item costs no
-    // merge work, so take the most heavy items that still start in the
-    // first round (128K batch 2: 52 -> 56 heavy items, 50.3 -> 47.8 us)
+    // calls of many items (few long sequences): the most heavy items that
+    // still start in the first round (128K batch 2: 52 -> 56 heavy items,
+    // 50.3 -> 47.8 us)
     if (forced_ipb <= 0 && H + nl > kMergeKernelItems) {
       const int hr = std::min(hmax, fill / std::max(1, nbh_launch));
       if (hr > H) H = hr;
@@ -994,13 +993,13 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
       }
     if (!changed) break;
   }
-  // Split them among the heavy segments. Where the launch merges its own
-  // partials, drop then the items that do not shrink a segment's largest
+  // Split them among the heavy segments. In plans of few items, drop then the
+  // items that do not shrink a segment's largest
   // item: each would only bring its start, cross-warp reduction and merge
   // share (8K understanding layer: text 8 tiles as 4 items of 2 instead of 5
   // items of 1-2, 13 items per (b, kvh) instead of 14, 12694 -> 13221
-  // tokens/s). With the separate merge kernel an item is cheap and more of
-  // them even out the SMs' loads.
+  // tokens/s). Many items even out the SMs' loads instead (128K: 58 -> 55
+  // items cost 2 %).
   int hc[UC_MAX_SEGMENTS];
   split_items(H, nseg, heavy, htiles, tcost, hc);
   {

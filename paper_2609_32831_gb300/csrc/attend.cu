@@ -186,7 +186,6 @@ struct OneCall {
     *c = 0;
     return p;
   }
-  __device__ const AttnParams& merge_call(int*) const { return p; }
 };
 
 struct ManyCalls {
@@ -208,13 +207,6 @@ struct ManyCalls {
       *local = p.n_heavy * p.batch * p.n_kv_heads + (q - m.light_begin[k]);
     }
     *c = k;
-    return m.call[k];
-  }
-  // the call of row block *blk of the merge (then the block's place in it)
-  __device__ const AttnParams& merge_call(int* blk) const {
-    int k = 0;
-    for (int n; k + 1 < m.n_calls && *blk >= (n = m.call[k].batch * m.call[k].n_kv_heads * m.call[k].mtiles); ++k)
-      *blk -= n;
     return m.call[k];
   }
 };
@@ -941,17 +933,22 @@ __device__ __forceinline__ void zero_v_rows(uint8_t* slot, int u, int valid) {
 // [rows_pad] l, rows_pad = 8 * (number of n-tiles).
 
 // Output row of query row r of a KV head (r = head * T + token).
-__device__ __forceinline__ size_t out_row(const AttnParams& p, int b, int kvh, int r) {
+template <class P>
+__device__ __forceinline__ size_t out_row(const P& p, int b, int kvh, int r) {
   const int hl = p.n_qtok == 1 ? r : r / p.n_qtok, t = p.n_qtok == 1 ? 0 : r % p.n_qtok;
   return (size_t)(b * p.n_q_heads + kvh * p.group + hl) * p.n_qtok + t;
 }
+
+// First item of segment q.
+__device__ __forceinline__ int segment_begin(const AttnParams& p, int q) { return p.seg[q].chunk_begin; }
+__device__ __forceinline__ int segment_begin(const MergeCall& p, int q) { return p.chunk_begin[q]; }
 
 // Log-sum-exp weights of query rows r0 .. r0 + nr - 1 over every item:
 // ml[i * stride + rr] holds item i's m, ll[...] its l; the normalised weights
 // replace m. PARTS threads per row (128 / PARTS rows at once, stride of them
 // real); lse and the per-segment mass are written for the valid rows.
-template <int PARTS>
-__device__ __forceinline__ void merge_weights(const AttnParams& p, float* ml, const float* ll, int stride, int b,
+template <int PARTS, class P>
+__device__ __forceinline__ void merge_weights(const P& p, float* ml, const float* ll, int stride, int b,
                                               int kvh, int r0, int nr, bool outputs = true) {
   const int I = p.items_per_bh;
   const int rr = threadIdx.x / PARTS, part = threadIdx.x % PARTS;
@@ -974,7 +971,7 @@ __device__ __forceinline__ void merge_weights(const AttnParams& p, float* ml, co
     if (mass) {
       int sg = 0;
 #pragma unroll
-      for (int q = 1; q < UC_MAX_SEGMENTS; ++q) sg += (q < p.nseg && i >= p.seg[q].chunk_begin) ? 1 : 0;
+      for (int q = 1; q < UC_MAX_SEGMENTS; ++q) sg += (q < p.nseg && i >= segment_begin(p, q)) ? 1 : 0;
 #pragma unroll
       for (int q = 0; q < UC_MAX_SEGMENTS; ++q)
         if (q == sg) Ls[q] += lw;
@@ -1113,6 +1110,15 @@ __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t*
 // weights -> sums; with many pairs every CTA's weights would count too (eight
 // query tokens, 16 x 300: CW 32 took 31.6 us, 20.1 so), so CW grows with the
 // number of CTAs (`merge_width`).
+// The call of row block *blk of a merge launch (then the block's place in it).
+__device__ __forceinline__ const MergeCall& merge_call(const MergeCall& p, int*) { return p; }
+__device__ __forceinline__ const MergeCall& merge_call(const MultiMerge& m, int* blk) {
+  int k = 0;
+  for (int n; k + 1 < m.n_calls && *blk >= (n = m.call[k].batch * m.call[k].n_kv_heads * m.call[k].mtiles); ++k)
+    *blk -= n;
+  return m.call[k];
+}
+
 template <int CW, class P>
 __global__ void __launch_bounds__(256, kMergePerSm) merge_partials_kernel(const __grid_constant__ P params) {
   constexpr int kCols = CW / 4, kPos = 8 * kCols, G = 256 / kPos, kPre = 8;
@@ -1121,10 +1127,9 @@ __global__ void __launch_bounds__(256, kMergePerSm) merge_partials_kernel(const 
   griddep_wait();  // the attention launch whose partials this merges has completed
   griddep_launch_dependents();
   const int tid = threadIdx.x;
-  const typename WorkOf<P>::type w{params};
   const int ch = blockIdx.x % (kHeadDim / CW);
   int blk = blockIdx.x / (kHeadDim / CW);
-  const AttnParams& p = w.merge_call(&blk);
+  const MergeCall& p = merge_call(params, &blk);
   const int r0 = (blk % p.mtiles) * 8, bh = blk / p.mtiles;
   const int b = bh / p.n_kv_heads, kvh = bh % p.n_kv_heads;
   const int nr = min(8, p.rows - r0);
@@ -1837,6 +1842,25 @@ int attend_clusters(int c) {
   return n;
 }
 
+static MergeCall merge_of(const AttnParams& p) {
+  MergeCall m;
+  m.part = p.part;
+  m.out = p.out;
+  m.lse = p.lse;
+  m.mass = p.mass;
+  m.nseg = p.nseg;
+  m.batch = p.batch;
+  m.n_kv_heads = p.n_kv_heads;
+  m.n_q_heads = p.n_q_heads;
+  m.n_qtok = p.n_qtok;
+  m.group = p.group;
+  m.rows = p.rows;
+  m.mtiles = p.mtiles;
+  m.items_per_bh = p.items_per_bh;
+  for (int s = 0; s < p.nseg; ++s) m.chunk_begin[s] = p.seg[s].chunk_begin;
+  return m;
+}
+
 // The merge of `blocks` (pair, row block)s. Always launched programmatically:
 // its CTAs take the SM slots the attention CTAs free and wait
 // (griddepcontrol.wait) for that launch to complete, instead of a launch gap
@@ -1870,7 +1894,7 @@ void launch_attend(const AttnParams& p, int grid, cudaStream_t st) {
   else
     launch_maybe_pdl(pdl, attend_kernel<2, AttnParams>, grid, kAttnThreads, smem, st, p);
   count_launch();
-  launch_merge(p, p.batch * p.n_kv_heads * p.mtiles, p.defer_merge, st);
+  launch_merge(merge_of(p), p.batch * p.n_kv_heads * p.mtiles, p.defer_merge, st);
 }
 
 void launch_attend_multi(const MultiAttnParams& m, int grid, cudaStream_t st) {
@@ -1883,9 +1907,14 @@ void launch_attend_multi(const MultiAttnParams& m, int grid, cudaStream_t st) {
   }
   attend_kernel<1, MultiAttnParams><<<grid, kAttnThreads, smem, st>>>(m);
   count_launch();
+  MultiMerge mm;
+  mm.n_calls = m.n_calls;
   int blocks = 0;
-  for (int c = 0; c < m.n_calls; ++c) blocks += m.call[c].batch * m.call[c].n_kv_heads;
-  launch_merge(m, blocks, m.merge_width, st);
+  for (int c = 0; c < m.n_calls; ++c) {
+    mm.call[c] = merge_of(m.call[c]);
+    blocks += m.call[c].batch * m.call[c].n_kv_heads;
+  }
+  launch_merge(mm, blocks, m.merge_width, st);
 }
 
 }  // namespace uc

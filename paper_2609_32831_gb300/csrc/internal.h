@@ -235,6 +235,21 @@ struct MultiAttnParams {
   int merge_width;  // output channels per CTA of the merge kernel (one n-tile)
 };
 
+// What the merge kernel reads of a call (its launch copies no more than that:
+// a batch's full parameters are 24 KB).
+struct MergeCall {
+  const float* part;
+  __nv_bfloat16* out;
+  float* lse;
+  float* mass;
+  int nseg, batch, n_kv_heads, n_q_heads, n_qtok, group, rows, mtiles, items_per_bh;
+  int chunk_begin[UC_MAX_SEGMENTS];
+};
+struct MultiMerge {
+  MergeCall call[UC_MAX_CALLS];
+  int n_calls;
+};
+
 // ------------------------------------------------- dense (many queries)
 struct DenseTile {
   int32_t row;       // first row of the tile inside a (b, kvh) block of khi / v
@@ -244,9 +259,8 @@ struct DenseTile {
 };
 
 // Items per (sequence, KV head) that a single-n-tile decode call takes at most
-// where they still fill the SMs: their partial outputs come into the in-kernel
-// merge in one round trip (two 32 KB ring slots of eight).
-constexpr int kWholeMergeItems = 14;
+// where they still fill the SMs (fewer starts, ends and partial outputs).
+constexpr int kFewItems = 14;
 constexpr int kDenseKeys = 128;     // keys per dense tile
 constexpr int kMaxDenseTiles = 512;  // up to 65536 keys per call
 

@@ -589,8 +589,8 @@ def append_next(seg: Segment, k_new: torch.Tensor, v_new: torch.Tensor, base_pos
 
 
 def set_dense_serial_pv(serial: bool) -> bool:
-    """Issue order of the dense attention kernel (see unicache.h); returns the
-    previous setting."""
+    """A setting of the dense attention kernel kept for its callers, without
+    effect any more (see unicache.h); returns the previous one."""
     return bool(lib().uc_set_dense_serial_pv(1 if serial else 0))
 
 

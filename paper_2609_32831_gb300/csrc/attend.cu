@@ -1109,7 +1109,9 @@ __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t*
 // One launch serves every call of a batch of one n-tile. What bounds it is the chain launch -> maxima and sums ->
 // weights -> sums; with many pairs every CTA's weights would count too (eight
 // query tokens, 16 x 300: CW 32 took 31.6 us, 20.1 so), so CW grows with the
-// number of CTAs (`merge_width`).
+// number of CTAs (`merge_width`). The attention launch writes the partials
+// while this one is resident, so they are read with ordinary (L2) loads behind
+// griddep_wait: the read-only path is for data that no kernel in flight writes.
 // The call of row block *blk of a merge launch (then the block's place in it).
 __device__ __forceinline__ const MergeCall& merge_call(const MergeCall& p, int*) { return p; }
 __device__ __forceinline__ const MergeCall& merge_call(const MultiMerge& m, int* blk) {
@@ -1142,8 +1144,8 @@ __global__ void __launch_bounds__(256, kMergePerSm) merge_partials_kernel(const 
     const int i = x >> 3, rr = x & 7;
     float m = kNegInf, l = 0.f;
     if (rr < nr) {
-      m = __ldg(base + i * pf + rows_pad * kHeadDim + r0 + rr);
-      l = __ldg(base + i * pf + rows_pad * kHeadDim + rows_pad + r0 + rr);
+      m = __ldcg(base + i * pf + rows_pad * kHeadDim + r0 + rr);
+      l = __ldcg(base + i * pf + rows_pad * kHeadDim + rows_pad + r0 + rr);
     }
     s_m[x] = m;
     s_w[x] = l;
@@ -1155,7 +1157,7 @@ __global__ void __launch_bounds__(256, kMergePerSm) merge_partials_kernel(const 
 #pragma unroll
     for (int k = 0; k < kPre; ++k) {
       const int i = i0 + G * k;
-      v[k] = i < I && rr < nr ? __ldg(reinterpret_cast<const float4*>(col + i * pf)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[k] = i < I && rr < nr ? __ldcg(reinterpret_cast<const float4*>(col + i * pf)) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
   fetch(grp);

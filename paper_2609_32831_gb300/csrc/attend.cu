@@ -56,6 +56,7 @@ __host__ __device__ constexpr int quant_groups_per_tile(int bits) { return bits 
 
 constexpr int kMaxItemsPerBh = 64;
 constexpr int kMaxPendingMerges = 64;
+constexpr int kMaxRows = 64;  // query rows of a KV head (eight n-tiles)
 constexpr int kItemQ = 2;  // items handed from the producer to the consumers ahead
 
 struct AttnSmem {
@@ -70,8 +71,11 @@ struct AttnSmem {
   int item_pos[kItemQ];         // processing position, -1: no more work
   int n_pending;                    // (sequence, KV head) merges this CTA owes
   int pending[kMaxPendingMerges];
+  alignas(16) float row_scale[kMaxRows];  // packed items: logit scale of each query row (see store_q)
   alignas(1024) uint8_t slot[kMaxStages][kSlotBytes];  // as many as the launch has
 };
+
+static_assert(offsetof(AttnSmem, row_scale) % 8 == 0, "row scales are read in pairs");
 
 // Query fragments of the current item live in shared memory (2 KB per
 // n-tile of 8 query rows): for one n-tile in `merge_w`, keeping three CTAs
@@ -581,52 +585,53 @@ __device__ __forceinline__ void block_bf16(WarpState<NTW>& st, uint32_t qs,
 // two subnormal fp16 values: a code at bit B is exactly code * 2^(B - 24), one
 // LOP3 per pair and no offset to remove. The tensor cores take subnormal
 // operands as they are; the powers of two are put right elsewhere:
-//   keys    the query of the pair's channels carries 2^(4 - B) and the logit
-//           scale 2^20: int2 copies w << 6, w, w >> 6 with codes at bits 4, 6,
-//           8 (queries times 1, 1/4, 1/16: none overflows for it), int4 copies
-//           w << 4, w, w >> 4, w >> 8 with every code at bit 4 (a query times
-//           1/16 would leave its fp16 lo part too few bits beside codes up to
-//           15: lse of 8192 tokens 3.7e-7 off instead of 4.3e-8);
+//   keys    the query of the pair's channels carries 2^(B0 - B) and the logit
+//           scale 2^(24 - B0). int2: copies w << 6, w << 2, w >> 2, w >> 6 with
+//           the two pairs of a 16-channel step at bits B0 = 6 and 8 (queries
+//           times 1 and 1/4: none overflows for it); int4: copies w << 4, w,
+//           w >> 4, w >> 8 with every code at bit B0 = 4. Each halving costs
+//           the fp16 queries a bit at their small end, which store_q brings
+//           up first, and low codes lose more in the tensor cores' sums. int2
+//           at bits 4, 6 and 8 (queries down to 1/16, two shifts per word
+//           less, no row scales): 32K layer, batch 16, 64.9 us, now 65.9; lse
+//           of 8192 tokens 4.9e-8 off, now 4.3e-8 (bits 4 and 6: 5.7e-8);
+//           with queries of 1e-4 on keys of 1e3, 1024 tokens, 1.4e-5 off, now
+//           2.7e-7;
 //   values  one HFMA2 per pair centres the codes and brings every pair to
 //           2^-9 (code - C): copies w and w >> 10 (int2) or w >> 8 (int4).
 // (With the exponent 2^(10-B) OR-ed in instead, each pair carried an offset of
 // 64, 16 or 4 through the fp32 accumulators, removed by extra rows of the beta
 // MMAs; value copies took two or three shifts per word. One 32K layer, batch
-// 16: int2 70.1 us, now 67.0; lse of 8192 tokens 2.7e-7 (int2) and 1.2e-7
-// (int4) off, now 4.8e-8 and 4.3e-8.)
-template <int BITS>
+// 16: int2 70.1 us; lse of 8192 tokens 2.7e-7 (int2) and 1.2e-7 (int4) off, now
+// 4.3e-8 and 4.4e-8.)
 struct KeyWords {
   uint32_t l, m, r, r2;
 };
 template <int BITS>
-__device__ __forceinline__ KeyWords<BITS> key_words(uint32_t w) {
+__device__ __forceinline__ KeyWords key_words(uint32_t w) {
   if constexpr (BITS == 2)
-    return KeyWords<BITS>{w << 6, w, w >> 6, 0u};
+    return KeyWords{w << 6, w << 2, w >> 2, w >> 6};
   else
-    return KeyWords<BITS>{w << 4, w, w >> 4, w >> 8};
+    return KeyWords{w << 4, w, w >> 4, w >> 8};
 }
 
 // Bit of key pair p in its copy and the class of the pair's channels: queries
 // scaled by 1 / class_scale.
-constexpr int kKeyBit0 = 4;
 template <int BITS>
-__host__ __device__ constexpr int key_bit(int p) {
-  return BITS == 4 ? 4 : (p % 3 == 2 ? 4 : (p % 3 == 0 ? 6 : 8));
-}
+__host__ __device__ constexpr int key_bit0() { return BITS == 4 ? 4 : 6; }
 template <int BITS>
-__host__ __device__ constexpr int key_classes() { return BITS == 4 ? 1 : 3; }
+__host__ __device__ constexpr int key_bit(int p) { return BITS == 4 ? 4 : 6 + 2 * (p & 1); }
 template <int BITS>
-__host__ __device__ constexpr int key_class(int p) { return (key_bit<BITS>(p) - kKeyBit0) / 2; }
-__host__ __device__ constexpr float class_scale(int c) { return (float)(1 << (2 * c)); }  // 2^(B - 4)
+__host__ __device__ constexpr int key_class(int p) { return (key_bit<BITS>(p) - key_bit0<BITS>()) / 2; }
+__host__ __device__ constexpr float class_scale(int c) { return (float)(1 << (2 * c)); }  // 2^(B - B0)
+template <int BITS>
+__host__ __device__ constexpr int key_classes() { return BITS == 4 ? 1 : 2; }
 
 template <int BITS, int P>
-__device__ __forceinline__ uint32_t key_pair(const KeyWords<BITS>& c) {
+__device__ __forceinline__ uint32_t key_pair(const KeyWords& c) {
   constexpr uint32_t code = ((1u << BITS) - 1u) << key_bit<BITS>(P);
-  uint32_t src;
-  if constexpr (BITS == 2)
-    src = P < 2 ? c.l : (P < 5 ? c.m : c.r);
-  else
-    src = P == 0 ? c.l : (P == 1 ? c.m : (P == 2 ? c.r : c.r2));
+  constexpr int copy = BITS == 4 ? P : P / 2;
+  const uint32_t src = copy == 0 ? c.l : (copy == 1 ? c.m : (copy == 2 ? c.r : c.r2));
   return src & (code | (code << 16));
 }
 
@@ -655,7 +660,8 @@ __device__ __forceinline__ uint32_t value_pair(const ValueWords<BITS>& c) {
   return hfma2_u32(x, mul | (mul << 16), add | (add << 16));
 }
 
-// One quantization group (32 keys = two 16-key blocks) of a packed tile.
+// One quantization group (32 keys = two 16-key blocks) of a packed tile;
+// row_scale: shared address of the n-tiles' logit scales by query row.
 // With x_hat = c * s + z (the powers of two of the codes left out):
 //   S^T  = c_K . (s_K (.) Q)^T + beta,  beta = z_K . Q^T
 //          (one MMA per 16 channels: A row r holds z over the channels of
@@ -695,8 +701,7 @@ __device__ __forceinline__ void group_beta_pair(uint32_t qsm, uint32_t base, int
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const uint2 z = lds64(kp + i * 64);  // z(c0 c1), z(c8 c9)
-    const int p0 = BITS == 4 ? 2 * (i & 1) : 2 * (i & 3);
-    const uint32_t az[4] = {gg == key_class<BITS>(p0) ? z.x : 0u, 0u, gg == key_class<BITS>(p0 + 1) ? z.y : 0u, 0u};
+    const uint32_t az[4] = {gg == key_class<BITS>(0) ? z.x : 0u, 0u, gg == key_class<BITS>(1) ? z.y : 0u, 0u};
 #pragma unroll
     for (int nt = 0; nt < NTW; ++nt) {
       const uint2 qv = lds64(qsm + ((nt * 8 + i) * 32 + lane) * 8);
@@ -713,7 +718,7 @@ __device__ __forceinline__ void group_beta_pair(uint32_t qsm, uint32_t base, int
 // instead of its own MMAs.
 template <int NTW, int BITS, bool kBeta = true>
 __device__ __forceinline__ void group_quant(WarpState<NTW>& st, uint32_t qsm,
-                                            uint32_t base, int gl, float scale,
+                                            uint32_t base, int gl, uint32_t row_scale,
                                             const float (&bt_in)[NTW][2]) {
   const int lane = threadIdx.x & 31;
   const int g = lane >> 2, j = lane & 3;
@@ -760,15 +765,14 @@ __device__ __forceinline__ void group_quant(WarpState<NTW>& st, uint32_t qsm,
   for (int i = 0; i < 8; ++i) {
     const uint4 P = lds128(kp + i * 64);  // s(c0 c1), s(c8 c9), z(c0 c1), z(c8 c9)
     // pairs of channels (16i + 2j, +1) and (16i + 2j + 8, +9)
-    const int p0 = BITS == 4 ? 2 * (i & 1) : 2 * (i & 3);
-    const uint32_t az[4] = {kBeta && g == key_class<BITS>(p0) ? P.z : 0u, 0u,
-                            kBeta && g == key_class<BITS>(p0 + 1) ? P.w : 0u, 0u};
+    const uint32_t az[4] = {kBeta && g == key_class<BITS>(0) ? P.z : 0u, 0u,
+                            kBeta && g == key_class<BITS>(1) ? P.w : 0u, 0u};
     // A fragments of both blocks for channels 16 i .. 16 i + 15
     uint32_t af[2][4];
     const int q = BITS == 4 ? (i >> 1) : (i >> 2);
 #pragma unroll
     for (int blk = 0; blk < 2; ++blk) {
-      const KeyWords<BITS> w0 = key_words<BITS>(kw[2 * blk][q]), w1 = key_words<BITS>(kw[2 * blk + 1][q]);
+      const KeyWords w0 = key_words<BITS>(kw[2 * blk][q]), w1 = key_words<BITS>(kw[2 * blk + 1][q]);
       if constexpr (BITS == 4) {
         if ((i & 1) == 0) {
           af[blk][0] = key_pair<4, 0>(w0); af[blk][1] = key_pair<4, 0>(w1);
@@ -814,18 +818,22 @@ __device__ __forceinline__ void group_quant(WarpState<NTW>& st, uint32_t qsm,
     }
   }
   float x[2][NTW][4];
-  const float ks = scale * (float)(1 << (24 - kKeyBit0));  // the codes' power of two
 #pragma unroll
   for (int nt = 0; nt < NTW; ++nt) {
     float bt[2] = {bt_in[nt][0], bt_in[nt][1]};
     if constexpr (kBeta) beta_rows<BITS>(bq[nt], 0, bt);
-    bt[0] *= scale;
-    bt[1] *= scale;
+    const uint2 rs = lds64(row_scale + nt * 32 + j * 8);  // query rows 2j, 2j + 1
+    float ks[2] = {__uint_as_float(rs.x), __uint_as_float(rs.y)};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      bt[h] *= ks[h];
+      ks[h] *= (float)(1 << (24 - key_bit0<BITS>()));  // the codes' power of two
+    }
 #pragma unroll
     for (int blk = 0; blk < 2; ++blk)
 #pragma unroll
       for (int e = 0; e < 4; ++e)
-        x[blk][nt][e] = fmaf(kLoChain ? sa[blk][nt][e] + sl[blk][nt][e] : sa[blk][nt][e], ks, bt[e & 1]);
+        x[blk][nt][e] = fmaf(kLoChain ? sa[blk][nt][e] + sl[blk][nt][e] : sa[blk][nt][e], ks[e & 1], bt[e & 1]);
   }
 
   // ---- softmax over the group's 32 keys
@@ -1191,27 +1199,55 @@ __global__ void __launch_bounds__(256, kMergePerSm) merge_partials_kernel(const 
         make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
 }
 
-// Query rows of every n-tile as Q^T B fragments (bf16 for bf16 rows, else
-// fp16 scaled for the key pairs of their channels)
-// in shared memory: word w of lane (g, j) for channels 16i + 2j (+8) of row
-// 8 nt + g at [((nt * 8 + i) * 32 + lane) * 2 + w], from the bf16 rows the
-// producer copied (row r = head * T + token). All consumer threads.
+// Query rows of every n-tile as Q^T B fragments in shared memory: word w of
+// lane (g, j) for channels 16i + 2j (+8) of row 8 nt + g at
+// [((nt * 8 + i) * 32 + lane) * 2 + w], from the bf16 rows the producer copied
+// (row r = head * T + token). All consumer threads.
+//
+// For bf16 rows the words are the queries as they are. For packed keys they
+// are fp16, whose step stops shrinking at 2^-24: queries of 1e-4 on keys of
+// 1e3 (logits up to 1) lose up to 1e-4 of a logit to it, four times that with
+// a class's 1/4. So a row whose largest element is below 1/2 is brought up to
+// [1/2, 1) by an exact power of two, which its logit scale takes out again.
+// Never above 1: a scaled query q s then stays finite for every fp16 key scale
+// s, and rows from 1/2 up stay as they are.
+constexpr int kMaxRowShift = 60;  // row scales stay normal fp32 values
+
 template <int BITS>
-__device__ __forceinline__ void store_q(const AttnParams& p, uint32_t* qf, const uint8_t* rows) {
-  for (int x = threadIdx.x; x < p.mtiles * 512; x += 128) {
-    const int nt = x >> 9, i = (x >> 6) & 7, ln = (x >> 1) & 31, w = x & 1;
-    const int r = nt * 8 + (ln >> 2);
-    const int c = 16 * i + 2 * (ln & 3) + 8 * w;
-    uint32_t word = 0u;
-    if (r < p.rows) {
-      word = *reinterpret_cast<const uint32_t*>(rows + (r * kHeadDim + c) * 2);
-      if constexpr (BITS != 16) {
-        // 1 / class_scale of the channels' key pair
-        const float f = 1.f / class_scale(key_class<BITS>(BITS == 4 ? 2 * (i & 1) + w : 2 * (i & 3) + w));
-        word = pack_f16(bf16_lo(word) * f, bf16_hi(word) * f);
-      }
+__device__ __forceinline__ void store_q(const AttnParams& p, uint32_t* qf, const uint8_t* rows, float* row_scale) {
+  const int tid = threadIdx.x;
+  if constexpr (BITS == 16) {
+    for (int x = tid; x < p.mtiles * 512; x += 128) {
+      const int nt = x >> 9, i = (x >> 6) & 7, ln = (x >> 1) & 31, w = x & 1;
+      const int r = nt * 8 + (ln >> 2);
+      const int c = 16 * i + 2 * (ln & 3) + 8 * w;
+      qf[x] = r < p.rows ? *reinterpret_cast<const uint32_t*>(rows + (r * kHeadDim + c) * 2) : 0u;
     }
-    qf[x] = word;
+  } else {
+    // words t * 128 + tid of an n-tile: one row per thread, i = 2 t + par; the
+    // row's other words are in the threads that differ in bits 0-2 (and 6)
+    const int ln = (tid >> 1) & 31, w = tid & 1, par = tid >> 6;
+    for (int nt = 0; nt < p.mtiles; ++nt) {
+      const int r = nt * 8 + (ln >> 2);
+      const uint32_t* src = reinterpret_cast<const uint32_t*>(rows) + r * (kHeadDim / 2) + (ln & 3) + 4 * w;
+      uint32_t own[4], mx = 0u;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int i = 2 * t + par;
+        own[t] = r < p.rows ? src[8 * i] : 0u;
+        const uint32_t other = r < p.rows ? src[8 * (i ^ 1)] : 0u;
+        mx = __vmaxu2(mx, __vmaxu2(own[t] & 0x7fff7fffu, other & 0x7fff7fffu));
+      }
+#pragma unroll
+      for (int o = 1; o < 8; o *= 2) mx = __vmaxu2(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      const int ex = (int)(max(mx & 0xffffu, mx >> 16) >> 7);  // the largest element's exponent field
+      const int k = min(max(126 - ex, 0), kMaxRowShift);
+      // 2^k / class_scale of the channels' key pair (pairs alternate with w)
+      const float f = __uint_as_float((uint32_t)(127 + k) << 23) / (w ? class_scale(key_class<BITS>(1)) : 1.f);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) qf[nt * 512 + t * 128 + tid] = pack_f16(bf16_lo(own[t]) * f, bf16_hi(own[t]) * f);
+      if ((tid & 0x47) == 0) row_scale[r] = p.scale_log2 * __uint_as_float((uint32_t)(127 - k) << 23);
+    }
   }
 }
 
@@ -1426,10 +1462,10 @@ __device__ __forceinline__ int run_tiles(const AttnParams& p, AttnSmem& sm, cons
   const int lane = threadIdx.x & 31;
   uint32_t* qf = NTW == 1 ? reinterpret_cast<uint32_t*>(sm.merge_w)
                           : reinterpret_cast<uint32_t*>(after_ring<ST>(sm));
-  store_q<BITS>(p, qf, qrows_buf<ST>(sm, k, p.mtiles));
+  store_q<BITS>(p, qf, qrows_buf<ST>(sm, k, p.mtiles), sm.row_scale);
   consumer_sync();
   if (lane == 0) mbar_arrive(&sm.item_empty[k]);  // the query rows are no longer needed
-  const uint32_t qs = smem_u32(qf) + grp * NTW * 2048;
+  const uint32_t qs = smem_u32(qf) + grp * NTW * 2048, rs = smem_u32(sm.row_scale) + grp * NTW * 32;
   // packed values enter O as kValueScale times theirs
   if constexpr (BITS != 16) scale_o<NTW>(st, kValueScale);
   int last_slot = -1;
@@ -1465,13 +1501,13 @@ __device__ __forceinline__ int run_tiles(const AttnParams& p, AttnSmem& sm, cons
                 bh[nt][0] = h ? bt[1][nt][0] : bt[0][nt][0];
                 bh[nt][1] = h ? bt[1][nt][1] : bt[0][nt][1];
               }
-              group_quant<NTW, BITS, false>(st, qs, sbase, gl, p.scale_log2, bh);
+              group_quant<NTW, BITS, false>(st, qs, sbase, gl, rs, bh);
             }
           }
         }
         const float none[NTW][2] = {};
 #pragma unroll 1
-        for (; gl < ngt; gl += KS) group_quant<NTW, BITS>(st, qs, sbase, gl, p.scale_log2, none);
+        for (; gl < ngt; gl += KS) group_quant<NTW, BITS>(st, qs, sbase, gl, rs, none);
       }
     }
     if (t + 1 < ii.te || !keep_last) {

@@ -354,6 +354,46 @@ def test_attend_parity(mix, T):
     assert (np.abs(host(mass) - rm) <= 2 * bound[..., None]).all()
 
 
+@pytest.mark.parametrize("T", [1, 4])
+@pytest.mark.parametrize("bits", [4, 2])
+@pytest.mark.parametrize("qmag,kmag", [(1e-4, 1e2), (1e-4, 1e3), (1e-2, 1.0), (1.0, 1.0), (1.0, 0.02), (100.0, 0.01)])
+def test_attend_query_and_key_magnitudes(qmag, kmag, bits, T):
+    """Queries far from 1 against packed keys far from 1, the heads of a KV
+    head up to six decades apart: the fp16 query fragments must not lose the
+    small ends that the fp32 logits still hold. One group of keys, so that a
+    logit error is not averaged away in lse."""
+    B, hkv, n = 2, 4, 32
+    k, v = synth.make_kv(int(1e6 * qmag) + bits, B, hkv, n)
+    k = synth.bf16_round(k * np.float32(kmag))
+    q = synth.make_q(T + bits, B, 28, T) * np.float32(qmag)
+    q = synth.bf16_round(q * np.exp2(-10.0 * (np.arange(28) % 3)).astype(np.float32)[None, :, None, None])
+    seg = uc.Segment("quant", bits, B, hkv, n, n, DEV)
+    seg.set_keep([n] * B)
+    uc.compress_segment(dev(k), dev(v), seg)
+    ref = [[oseg.compress(k[b, j], v[b, j], None, "quant", n, bits) for j in range(hkv)] for b in range(B)]
+    O, lse, _ = uc.attend(dev(q), [seg])
+    rO, rl, _ = oattn.attend(q, [ref], hkv)
+    # A row's largest element enters as 1/2 or more, int2's second channel class
+    # at 1/4 of that: a stored query, and its product with the key scale, are
+    # off by fp16's half step 2^-25 times 4 (int2), times 2 rowmax outside that
+    # scale. The query's error meets the key, the product's a code <= qmax.
+    # Products also carry 2^-22 of themselves; fp32 sums of 128 channels, exp2
+    # and log2: 2^-20 of the terms.
+    qmax, g = 2.0 ** bits - 1, 7
+    step = 2.0 ** -25 * (4 if bits == 2 else 1)
+    for b in range(B):
+        for j in range(hkv):
+            rows = np.abs(q[b, j * g:(j + 1) * g].reshape(-1, 128).astype(np.float64))
+            s, keys = ref[b][j].k_scale[0].astype(np.float64), np.abs(ref[b][j].kv()[0])
+            floor = step * 2 * rows.max(1) * (keys.max(0) + qmax).sum()
+            terms = rows @ keys.max(0) + rows @ (qmax * s)
+            bound = ((floor + 2.0 ** -20 * terms) / np.sqrt(128)).reshape(g, T)
+            got, want = host(lse)[b, j * g:(j + 1) * g], rl[b, j * g:(j + 1) * g]
+            assert (np.abs(got - want) <= bound + 2.0 ** -21 * np.abs(want) + 5e-7).all(), \
+                (b, j, np.abs(got - want).max(), bound.min())
+    assert _packed.attention_error(host(O), rO) <= _packed.ATTN_RTOL
+
+
 @pytest.mark.parametrize("hq,T", [(28, 3), (28, 4), (28, 6), (32, 8), (24, 8), (8, 8)])
 def test_attend_query_tiles_many_items(hq, T):
     """2 to 8 query n-tiles with enough items per (b, kvh) that their merge

@@ -516,16 +516,25 @@ size_t uc_attend_workspace_size(const uc_segment* const* segs, int32_t n_seg, in
 typedef struct {
   int32_t items_per_bh;                 /* partials per (sequence, KV head), <= 64 */
   int32_t n_heavy, n_light;             /* heavy / light items per (sequence, KV head) */
-  int32_t grid;                         /* CTAs that walk the items as a work queue */
-  int32_t merge_kernel;                 /* 1: more items than a merge inside the launch is planned for
-                                         * (> 32); at any count a call outside clusters merges in a
-                                         * kernel of its own, a batch of several query tiles
-                                         * inside its launch */
+  int32_t grid;                         /* CTAs that would walk the items as a work queue */
+  int32_t merge_kernel;                 /* 1: more items (> 32) than a merge inside a launch is planned
+                                         * for; uc_attend_launch says how the call is launched */
   int32_t n_chunks[UC_MAX_SEGMENTS];    /* items of each segment */
   int32_t light[UC_MAX_SEGMENTS];       /* 1: every item of the segment is light */
 } uc_attend_plan_info;
 uc_status uc_attend_plan(const uc_segment* const* segs, int32_t n_seg, int32_t n_q_heads, int32_t n_qtok,
                          int32_t slots, uc_attend_plan_info* out);
+
+/* What uc_attend launches for that plan (same arguments and errors). */
+typedef struct {
+  int32_t cluster;       /* > 0: one cluster of this many CTAs per (sequence, KV head), merged inside it;
+                          * 0: CTAs on a work queue, then the merge kernel */
+  int32_t ctas;          /* CTAs of the attention kernel */
+  int32_t stages;        /* ring slots of each */
+  int32_t merge_width;   /* output channels per CTA of the merge kernel (32, 64 or 128); 0: none */
+} uc_attend_launch_info;
+uc_status uc_attend_launch(const uc_segment* const* segs, int32_t n_seg, int32_t n_q_heads, int32_t n_qtok,
+                           int32_t slots, uc_attend_launch_info* out);
 
 /*
  * Several independent decode-shaped attention calls in one launch (App. E,

@@ -71,6 +71,10 @@ class UcAttendPlanInfo(C.Structure):
     ]
 
 
+class UcAttendLaunchInfo(C.Structure):
+    _fields_ = [("cluster", C.c_int32), ("ctas", C.c_int32), ("stages", C.c_int32), ("merge_width", C.c_int32)]
+
+
 MAX_CALLS = 8
 
 # uc_allocator: stream-ordered device memory hooks for library-owned segments
@@ -124,6 +128,7 @@ _SIGS = {
     "uc_attend": (C.c_int, [_P, C.c_int32, C.c_int32, _P, C.c_int32, _P, _P, _P, _P, C.c_size_t, _P]),
     "uc_attend_workspace_size": (C.c_size_t, [_P, C.c_int32, C.c_int32, C.c_int32]),
     "uc_attend_plan": (C.c_int, [_P, C.c_int32, C.c_int32, C.c_int32, C.c_int32, _P]),
+    "uc_attend_launch": (C.c_int, [_P, C.c_int32, C.c_int32, C.c_int32, C.c_int32, _P]),
     "uc_attend_batch": (C.c_int, [_P, C.c_int32, _P, C.c_size_t, _P]),
     "uc_attend_batch_workspace_size": (C.c_size_t, [_P, C.c_int32]),
     "uc_attend_static": (C.c_int, [_P, C.c_int32, C.c_int32, _P, C.c_int32, _P, _P, _P, _P]),

@@ -760,6 +760,7 @@ namespace {
 struct AttnPlan {
   int items_per_bh, n_items, grid, mtiles, n_heavy, n_light;
   int cluster;  // > 0: short call, a cluster of this many CTAs per (sequence, KV head)
+  int stages, merge_width;  // uc_attend's launch: ring slots of a CTA; channels per merge CTA (0: cluster)
   int chunk_begin[UC_MAX_SEGMENTS], n_chunks[UC_MAX_SEGMENTS];
   int16_t heavy_local[128], light_local[2 * UC_MAX_SEGMENTS];
 };
@@ -859,6 +860,14 @@ double items_us(double item, int h, int nbh) {
 constexpr double kQueueMergeUs = 1.5, kClusterSpread = 1.15;
 constexpr double kLightItemUs = 0.4;  // SM time of a light item's start and end
 
+// Output channels per CTA of the merge kernel: the fewest whose CTAs are all
+// resident at once.
+int merge_width(int blocks, int sms) {
+  for (int cw = 32; cw < UC_HEAD_DIM; cw *= 2)
+    if (blocks * (UC_HEAD_DIM / cw) <= kMergePerSm * sms) return cw;
+  return UC_HEAD_DIM;
+}
+
 // nbh_launch: (sequence, KV head) pairs of every call sharing the launch.
 // forced_ipb > 0 fixes the items per (sequence, KV head) instead of
 // searching for the count that fills whole rounds of CTA slots.
@@ -871,6 +880,7 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
   const int B = segs[0]->batch, hkv = segs[0]->n_kv_heads;
   const int nbh = B * hkv;
   const int slots = slots_in > 0 ? slots_in : std::max(1, attend_ctas_per_sm(mtiles)) * num_sms();
+  const int sms = slots_in > 0 ? std::max(1, slots_in / (mtiles <= 1 ? 3 : (mtiles < 8 ? 2 : 1))) : num_sms();
   // heavy tiles of each segment (a packed segment's bf16 tail is a light
   // item of its own) and their cost
   int htiles[UC_MAX_SEGMENTS];
@@ -1044,6 +1054,15 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
   p.items_per_bh = assigned;  // at most 64 (the merge staging)
   p.n_items = assigned * nbh;
   p.grid = std::min(p.n_items, slots);
+  // Several n-tiles on no more CTAs than SMs take three ring slots each.
+  p.stages = mtiles > 1 && p.grid <= sms ? 3 : 2;
+  // Outside clusters uc_attend's merge is a kernel of its own, also for few
+  // items: launched programmatically it starts as the last items end, while a
+  // merge in the launch streams through the one SM that finishes a pair (one
+  // query token, 16 x 8K 33.0 -> 27.4 us, 4 x 16K 20.1 -> 17.6, 32K int2, batch
+  // 16, 67.1 -> 66.1; four, 4 x 16K 40.8 -> 34.4, 4 x 4K 28.9 -> 17.4; no size
+  // was slower).
+  p.merge_width = p.cluster ? 0 : merge_width(nbh * mtiles, sms);
   return p;
 }
 
@@ -1133,14 +1152,6 @@ int decode_mtiles(int n_q_heads, int hkv, int n_qtok) { return (n_q_heads / hkv 
 
 int merge_kernel_for(int items_per_bh) { return items_per_bh > kMergeKernelItems ? 1 : 0; }
 
-// Output channels per CTA of the merge kernel: the fewest whose CTAs are all
-// resident at once.
-int merge_width(int blocks) {
-  for (int cw = 32; cw < UC_HEAD_DIM; cw *= 2)
-    if (blocks * (UC_HEAD_DIM / cw) <= kMergePerSm * num_sms()) return cw;
-  return UC_HEAD_DIM;
-}
-
 // A decode call's merge counters (one per (b, kvh)) live in a block of fixed
 // size at a fixed place of the workspace, whatever the call's shape: every
 // counter a call uses is re-armed to zero by its merge, so a block that calls
@@ -1209,7 +1220,7 @@ uc_status build_decode_call(const void* q, int32_t n_q_heads, int32_t n_qtok, co
   p->scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)UC_HEAD_DIM));
   p->wait_ns = uc::wait_limit_ns();
   p->withhold_pos = uc::take_withhold_pos();
-  p->stages = 2;
+  p->stages = 2;  // (a batch's launch)
   return UC_OK;
 }
 
@@ -1298,47 +1309,57 @@ size_t uc_attend_workspace_size(const uc_segment* const* segs, int32_t n_seg, in
   return decode_workspace(plan_attend(segs, n_seg, mtiles, segs[0]->batch * hkv));
 }
 
-uc_status uc_attend_plan(const uc_segment* const* segs, int32_t n_seg, int32_t n_q_heads, int32_t n_qtok,
-                         int32_t slots, uc_attend_plan_info* out) {
-  UC_TRACE();
+// The checks of the planner's entry points, which read no device array;
+// *mtiles: the call's 8-row query tiles.
+static uc_status check_plan_call(const uc_segment* const* segs, int32_t n_seg, int32_t n_q_heads, int32_t n_qtok,
+                                 const void* out, const char* name, int* mtiles) {
   if (segs == nullptr || out == nullptr) {
-    set_error("uc_attend_plan: null pointer");
+    set_error("%s: null pointer", name);
     return UC_ERR_ARG;
   }
   if (n_seg < 1 || n_seg > UC_MAX_SEGMENTS || n_qtok < 1 || n_qtok > UC_MAX_QTOKENS) {
-    set_error("uc_attend_plan: need 1..%d segments and 1..%d query tokens", UC_MAX_SEGMENTS, UC_MAX_QTOKENS);
+    set_error("%s: need 1..%d segments and 1..%d query tokens", name, UC_MAX_SEGMENTS, UC_MAX_QTOKENS);
     return UC_ERR_SHAPE;
   }
   for (int s = 0; s < n_seg; ++s) {
     const uc_segment* g = segs[s];
     if (g == nullptr) {
-      set_error("uc_attend_plan: segment %d is null", s);
+      set_error("%s: segment %d is null", name, s);
       return UC_ERR_ARG;
     }
     const bool q = is_quant(g->kind);
     if (g->batch < 1 || g->batch > UC_MAX_BATCH || g->n_kv_heads < 1 || g->batch != segs[0]->batch ||
         g->n_kv_heads != segs[0]->n_kv_heads || g->kind < UC_KIND_FULL || g->kind > UC_KIND_EVICT_QUANT ||
         (q && g->bits != 2 && g->bits != 4)) {
-      set_error("uc_attend_plan: segment %d has an invalid kind, width, batch or head count", s);
+      set_error("%s: segment %d has an invalid kind, width, batch or head count", name, s);
       return UC_ERR_SHAPE;
     }
     for (int b = 0; b < g->batch; ++b)
       if (g->n_kept_host[b] < 0) {
-        set_error("uc_attend_plan: segment %d holds a negative count", s);
+        set_error("%s: segment %d holds a negative count", name, s);
         return UC_ERR_SHAPE;
       }
   }
   const int hkv = segs[0]->n_kv_heads;
   if (n_q_heads < hkv || n_q_heads % hkv) {
-    set_error("uc_attend_plan: query heads %d not a multiple of KV heads %d", n_q_heads, hkv);
+    set_error("%s: query heads %d not a multiple of KV heads %d", name, n_q_heads, hkv);
     return UC_ERR_SHAPE;
   }
-  const int mtiles = decode_mtiles(n_q_heads, hkv, n_qtok);
-  if (mtiles > 8) {
-    set_error("uc_attend_plan: (Hq / Hkv) * T = %d rows exceed 64", n_q_heads / hkv * n_qtok);
+  *mtiles = decode_mtiles(n_q_heads, hkv, n_qtok);
+  if (*mtiles > 8) {
+    set_error("%s: (Hq / Hkv) * T = %d rows exceed 64", name, n_q_heads / hkv * n_qtok);
     return UC_ERR_SHAPE;
   }
-  const AttnPlan p = plan_attend(segs, n_seg, mtiles, segs[0]->batch * hkv, 0, slots);
+  return UC_OK;
+}
+
+uc_status uc_attend_plan(const uc_segment* const* segs, int32_t n_seg, int32_t n_q_heads, int32_t n_qtok,
+                         int32_t slots, uc_attend_plan_info* out) {
+  UC_TRACE();
+  int mtiles = 0;
+  const uc_status st = check_plan_call(segs, n_seg, n_q_heads, n_qtok, out, "uc_attend_plan", &mtiles);
+  if (st != UC_OK) return st;
+  const AttnPlan p = plan_attend(segs, n_seg, mtiles, segs[0]->batch * segs[0]->n_kv_heads, 0, slots);
   memset(out, 0, sizeof(*out));
   out->items_per_bh = p.items_per_bh;
   out->n_heavy = p.n_heavy;
@@ -1352,6 +1373,21 @@ uc_status uc_attend_plan(const uc_segment* const* segs, int32_t n_seg, int32_t n
       any_heavy |= p.heavy_local[i] >= p.chunk_begin[s] && p.heavy_local[i] < p.chunk_begin[s] + p.n_chunks[s];
     out->light[s] = any_heavy ? 0 : 1;
   }
+  return UC_OK;
+}
+
+uc_status uc_attend_launch(const uc_segment* const* segs, int32_t n_seg, int32_t n_q_heads, int32_t n_qtok,
+                           int32_t slots, uc_attend_launch_info* out) {
+  UC_TRACE();
+  int mtiles = 0;
+  const uc_status st = check_plan_call(segs, n_seg, n_q_heads, n_qtok, out, "uc_attend_launch", &mtiles);
+  if (st != UC_OK) return st;
+  const int nbh = segs[0]->batch * segs[0]->n_kv_heads;
+  const AttnPlan p = plan_attend(segs, n_seg, mtiles, nbh, 0, slots);
+  out->cluster = p.cluster;
+  out->ctas = p.cluster ? p.cluster * nbh : p.grid;
+  out->stages = p.stages;
+  out->merge_width = p.merge_width;
   return UC_OK;
 }
 
@@ -1431,13 +1467,8 @@ uc_status uc_attend(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_s
   if (st != UC_OK) return st;
   // (a device whose clusters fit less well than planned for takes the queue)
   p.cluster = plan.cluster > 0 && attend_clusters(plan.cluster) >= B * hkv ? plan.cluster : 0;
-  // Outside clusters the merge is a kernel of its own, also for few items:
-  // launched programmatically it starts as the last items end, while a merge
-  // in the launch streams through the one SM that finishes a pair (one query
-  // token, 16 x 8K 33.0 -> 27.4 us, 4 x 16K 20.1 -> 17.6, 32K int2, batch 16,
-  // 67.1 -> 66.1; four, 4 x 16K 40.8 -> 34.4, 4 x 4K 28.9 -> 17.4; no size was slower).
-  p.defer_merge = p.cluster ? 0 : merge_width(B * hkv * plan.mtiles);
-  if (plan.mtiles > 1 && plan.grid <= num_sms()) p.stages = 3;
+  p.defer_merge = p.cluster ? 0 : merge_width(B * hkv * plan.mtiles, num_sms());
+  p.stages = plan.stages;
   launch_attend(p, plan.grid, reinterpret_cast<cudaStream_t>(stream));
   return cuda_check("uc_attend");
 }
@@ -1531,7 +1562,7 @@ uc_status uc_attend_batch(const uc_attend_call* calls, int32_t n_calls, void* wo
   m.light_begin[n_calls] = light;
   m.n_calls = n_calls;
   m.n_items = heavy + light;
-  m.merge_width = merge_width(nbh_launch * mtiles);
+  m.merge_width = merge_width(nbh_launch * mtiles, num_sms());
   const int slots = std::max(1, attend_ctas_per_sm(mtiles)) * num_sms();
   launch_attend_multi(m, std::min(m.n_items, slots), reinterpret_cast<cudaStream_t>(stream));
   return cuda_check("uc_attend_batch");

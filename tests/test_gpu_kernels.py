@@ -415,8 +415,19 @@ def test_attend_query_tiles_many_items(hq, T):
     assert ws.status() == 0
 
 
-@pytest.mark.parametrize("T,B", [(3, 2), (3, 12), (3, 20), (8, 5), (8, 9), (1, 40)])
-def test_attend_merge_widths(T, B):
+def _attend_as_planned(q, gsegs, plan, **kw):
+    """One attend call, checked to launch what the plan says: the attention
+    kernel alone for clusters, else it and the merge kernel."""
+    n0 = uc.launch_count()
+    res = uc.attend(dev(q), gsegs, **kw)
+    assert uc.launch_count() - n0 == (1 if plan["cluster"] else 2)
+    assert (plan["merge_width"] == 0) == (plan["cluster"] > 0)
+    return res
+
+
+@pytest.mark.parametrize("T,B,width,stages", [(3, 2, 32, 3), (3, 12, 64, 2), (3, 20, 128, 2), (8, 5, 64, 2),
+                                              (8, 9, 128, 2), (1, 40, 64, 2)])
+def test_attend_merge_widths(T, B, width, stages):
     """The merge kernel's CTAs of 32, 64 and 128 channels (more pairs and row
     blocks), over a last row block of 5 of its 8 rows, items that split
     unevenly over a CTA's thread groups and sequences that keep one token."""
@@ -425,7 +436,9 @@ def test_attend_merge_widths(T, B):
     keeps = [400, 700, [1 + (37 * b) % 300 for b in range(B)]]
     gsegs, osegs = _build_mix(100 * T + B, B, hkv, sizes, kinds, keeps, [16, 4, 2])
     q = synth.make_q(T + B, B, 28, T)
-    O, lse, mass = uc.attend(dev(q), gsegs)
+    plan = uc.attend_plan(gsegs, 28, T)
+    assert (plan["cluster"], plan["merge_width"], plan["stages"]) == (0, width, stages)
+    O, lse, mass = _attend_as_planned(q, gsegs, plan)
     rO, rl, rm = oattn.attend(q, osegs, hkv)
     assert _packed.attention_error(host(O), rO) <= _packed.ATTN_RTOL
     bound = _packed.logit_error_bound(q, osegs, hkv, [False, True, True])
@@ -434,19 +447,22 @@ def test_attend_merge_widths(T, B):
 
 
 CLUSTER_MIXES = {
-    # (B, Hkv, sizes, kinds, keeps, bits): clusters of 1, few and 16 CTAs, more
-    # light items than ranks, eight segments, sequences that hold nothing of a
-    # segment, 64 pairs (six CTAs each), and one pair too many for any cluster
+    # (B, Hkv, sizes, kinds, keeps, bits): clusters of 1, few and 16 CTAs, light
+    # items with a rank each and two that share one, eight segments, sequences
+    # that hold nothing of a segment's packed groups, 64 pairs (six CTAs each);
+    # one long pair and one pair too many for any cluster take the queue
     "one_token": (1, 1, [1], ["full"], [1], [16]),
     "tails_only": (2, 2, [20, 33, 31], ["quant", "quant", "quant"], [20, 33, 31], [4, 2, 4]),
     "eight_segments": (1, 4, [40, 64, 100, 33, 257, 7, 90, 300],
                        ["full", "quant", "evict", "quant", "evict_quant", "full", "quant", "evict_quant"],
                        [40, 64, 20, 33, 130, 7, 90, 250], [16, 4, 16, 2, 2, 16, 4, 4]),
-    "sixteen_ranks": (1, 1, [3000, 4100], ["full", "quant"], [3000, 4100], [16, 4]),
+    "shared_light_rank": (8, 4, [300, 700, 200], ["full", "evict_quant", "quant"], [300, 600, 200], [16, 4, 2]),
+    "one_long_pair": (1, 1, [3000, 4100], ["full", "quant"], [3000, 4100], [16, 4]),
     "ragged": (5, 4, [700, 900], ["evict", "evict_quant"], [[1, 700, 64, 65, 128], [900, 1, 32, 64, 31]], [16, 2]),
     "pairs_64": (8, 8, [300, 1000], ["full", "quant"], [300, 1000], [16, 2]),
     "pairs_512": (64, 8, [70], ["full"], [70], [16]),
 }
+QUEUED = ("one_long_pair", "pairs_512")
 
 
 @pytest.mark.parametrize("mix", list(CLUSTER_MIXES))
@@ -458,9 +474,12 @@ def test_attend_short_calls(mix):
     rO, rl, rm = oattn.attend(q, osegs, hkv)
     bound = _packed.logit_error_bound(q, osegs, hkv, [kd in ("quant", "evict_quant") for kd in kinds])
     ws = uc.Workspace(DEV)
+    plan = uc.attend_plan(gsegs, hq, 1)
+    if mix != "ragged":   # (16 CTAs for each of 20 pairs: not on every GB300's GPCs)
+        assert (plan["cluster"] > 0) == (mix not in QUEUED)
     first = None
     for _ in range(2):
-        O, lse, mass = uc.attend(dev(q), gsegs, ws=ws)
+        O, lse, mass = _attend_as_planned(q, gsegs, plan, ws=ws)
         assert _packed.attention_error(host(O), rO) <= _packed.ATTN_RTOL
         assert (np.abs(host(lse) - rl) <= bound).all()
         assert (np.abs(host(mass) - rm) <= 2 * bound[..., None]).all()

@@ -64,19 +64,18 @@ def test_understanding_8k_hand_worked():
     assert _tiles(_lib.KIND_QUANT, 2, 512) == (2, 0)
     p = api.attend_plan([text, vit, gen], 28, 1, SLOTS)
     # 13 heavy items would fill 416 of 456 slots (>= 90 %), but with the two
-    # packed tails that is 15 > 14 items, more than one merge stages whole;
-    # 12 still fill 384 (84 % >= 80 %). Largest item smallest, one item at a
-    # time: image 6 items (3 tiles, 60 KB), text 5 (2 tiles, 64 KB),
-    # generated 1 (48 KB). The fifth text item leaves the largest text item
-    # at 2 tiles, so it is dropped: text 4, image 6 + tail, generated 1 +
-    # tail (empty here) = 13 items, 11 of them heavy.
+    # packed tails that is 15 > 14 items, and 12 still fill 384 (84 % >= 80
+    # %). Largest item smallest, one item at a time: image 6 items (3 tiles, 60
+    # KB), text 5 (2 tiles, 64 KB), generated 1 (48 KB). The fifth text item
+    # leaves the largest text item at 2 tiles, so it is dropped: text 4, image
+    # 6 + tail, generated 1 + tail (empty here) = 13 items, 11 of them heavy.
     assert p["n_chunks"] == [4, 7, 2]
     assert p["n_heavy"] == 11 and p["n_light"] == 2 and p["items_per_bh"] == 13
     assert p["grid"] == 13 * 32 and not p["merge_kernel"]
 
 
 def test_no_item_leaves_a_segments_largest_item_as_it_was():
-    # merged inside the launch, a segment of 8 tiles takes 4 items of 2 rather
+    # in a plan of few items a segment of 8 tiles takes 4 items of 2 rather
     # than 5 of 1-2, whatever count the slot fill asked for
     for tiles, kind, bits, n in [(8, _lib.KIND_FULL, 16, 512), (17, _lib.KIND_QUANT, 4, 2144)]:
         seg = _seg(kind, bits, [n] * 2, hkv=1)
@@ -143,13 +142,60 @@ def test_plan_invariants_random_mixes(seed):
         else:
             # a heavy packed segment ends with its (light) tail item
             assert p["n_chunks"][s] >= (2 if packed else 1)
-            # and, where the launch merges its own partials, takes no item
-            # that leaves its largest item as large
+            # and, in a plan of few items, takes no item that leaves its
+            # largest item as large
             tiles = _tiles(seg.kind, seg.bits, max(seg.n_kept_host[b] for b in range(B)))[0]
             hc = p["n_chunks"][s] - (1 if packed else 0)
             per = -(-tiles // hc)
             if not p["merge_kernel"]:
                 assert hc == -(-tiles // per)
+
+
+# cluster CTAs, merge width of the short-call mixes on 456 slots
+CLUSTERS = {"one_token": (1, 0), "tails_only": (4, 0), "eight_segments": (14, 0), "shared_light_rank": (12, 0),
+            "one_long_pair": (0, 32), "ragged": (16, 0), "pairs_64": (6, 0), "pairs_512": (0, 128)}
+
+
+def test_short_calls_and_their_clusters():
+    """One rank per heavy item and one for every light item, or a single one
+    for all of them where a cluster of more would not fit often enough; the
+    GPU tests run the same mixes."""
+    from tests.test_gpu_kernels import CLUSTER_MIXES
+    assert set(CLUSTERS) == set(CLUSTER_MIXES)
+    kind_of = api.KIND_NAMES
+    for mix, (B, hkv, _, kinds, keeps, bits) in CLUSTER_MIXES.items():
+        segs = [_seg(kind_of[k], bt, kp if hasattr(kp, "__len__") else [kp] * B, hkv)
+                for k, kp, bt in zip(kinds, keeps, bits)]
+        p = api.attend_plan(segs, 7 * hkv, 1, SLOTS)
+        assert (p["cluster"], p["merge_width"]) == CLUSTERS[mix], mix
+        if p["cluster"]:
+            assert p["cluster"] - p["n_heavy"] in (0 if p["n_light"] == 0 else 1, p["n_light"]), mix
+            assert p["ctas"] == p["cluster"] * B * hkv <= SLOTS and p["stages"] == 2
+        else:
+            assert p["ctas"] == p["grid"]
+    # two light items, one rank for both
+    B, hkv, _, kinds, keeps, bits = CLUSTER_MIXES["shared_light_rank"]
+    p = api.attend_plan([_seg(kind_of[k], bt, [kp] * B, hkv) for k, kp, bt in zip(kinds, keeps, bits)], 28, 1, SLOTS)
+    assert p["n_light"] == 2 and p["cluster"] == p["n_heavy"] + 1
+
+
+def test_launches_of_the_hand_worked_calls():
+    """The 32K layer walks its items as a queue and merges 64 pairs by CTAs of
+    32 channels; the 8K layer's 32 pairs are clusters of 12."""
+    seg32 = [_seg(_lib.KIND_QUANT, 2, [3276] * 16), _seg(_lib.KIND_QUANT, 2, [29492] * 16),
+             _seg(_lib.KIND_EVICT, 16, [128] * 16)]
+    p = api.attend_plan(seg32, 28, 1, SLOTS)
+    assert (p["cluster"], p["ctas"], p["stages"], p["merge_width"]) == (0, SLOTS, 2, 32)
+    seg8 = [_seg(_lib.KIND_FULL, 16, [512] * 8), _seg(_lib.KIND_EVICT_QUANT, 4, [2150] * 8),
+            _seg(_lib.KIND_QUANT, 2, [512] * 8)]
+    p = api.attend_plan(seg8, 28, 1, SLOTS)
+    assert (p["cluster"], p["ctas"], p["merge_width"]) == (12, 12 * 32, 0)
+    # four query tokens: four row blocks of each pair, three ring slots only
+    # where the CTAs are no more than the SMs
+    p = api.attend_plan([_seg(_lib.KIND_FULL, 16, [43000])], 28, 4, 2 * 152)
+    assert (p["cluster"], p["stages"]) == (0, 3) and p["ctas"] <= 152
+    p = api.attend_plan(seg8, 28, 4, 2 * 152)
+    assert (p["cluster"], p["stages"], p["merge_width"]) == (0, 2, 64)   # 128 (pair, row block)s
 
 
 def test_plan_rejects_bad_calls():
@@ -163,4 +209,7 @@ def test_plan_rejects_bad_calls():
     assert h.uc_attend_plan(C.cast(arr, C.c_void_p), 1, 30, 1, SLOTS, C.byref(info)) == _lib.UC_ERR_SHAPE
     seg.bits = 3
     assert h.uc_attend_plan(C.cast(arr, C.c_void_p), 1, 28, 1, SLOTS, C.byref(info)) == _lib.UC_ERR_SHAPE
+    run = _lib.UcAttendLaunchInfo()
+    assert h.uc_attend_launch(None, 1, 28, 1, SLOTS, C.byref(run)) == _lib.UC_ERR_ARG
+    assert h.uc_attend_launch(C.cast(arr, C.c_void_p), 1, 28, 1, SLOTS, C.byref(run)) == _lib.UC_ERR_SHAPE
     assert h.uc_launch_count() == n0

@@ -832,8 +832,11 @@ void split_items(int h, int nseg, const bool* heavy, const int* htiles, const do
   }
 }
 
-// Clusters of c CTAs that a GB300 runs at once with three CTAs per SM (the
-// occupancy query's answer: clusters stay inside a GPC, so not slots / c).
+// Clusters of c CTAs that a GB300 of kClusterSlots CTA slots runs at once
+// (clusters stay inside a GPC, so not slots / c), for plans made without a
+// device. With one, its own occupancy answers: GPCs may differ from chip to
+// chip, and a plan for clusters that do not fit would leave the queue with
+// the cluster's items.
 constexpr int kClusterFit[kMaxClusterItems + 1] = {0,  456, 228, 148, 110, 87, 74, 59, 51,
                                                    46, 43,  36,  36,  28,  26, 26, 21};
 constexpr int kClusterSlots = 456;
@@ -845,8 +848,8 @@ double tile_us(const uc_segment* s) { return !is_quant(s->kind) ? 0.75 : (s->bit
 // Time until a single-n-tile call's longest items (`item` us of SM time each,
 // h per pair) end: the CTAs of the busiest SM share it, and one or two of
 // them leave part of its rate unused.
-double items_us(double item, int h, int nbh) {
-  const int n = (h * nbh + 151) / 152;
+double items_us(double item, int h, int nbh, int sms) {
+  const int n = (h * nbh + sms - 1) / sms;
   return n * item * (n >= 3 ? 1.0 : (n == 2 ? 1.32 : 2.0));
 }
 // The queue's merge (a kernel behind the call, partials through global
@@ -881,6 +884,10 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
   const int nbh = B * hkv;
   const int slots = slots_in > 0 ? slots_in : std::max(1, attend_ctas_per_sm(mtiles)) * num_sms();
   const int sms = slots_in > 0 ? std::max(1, slots_in / (mtiles <= 1 ? 3 : (mtiles < 8 ? 2 : 1))) : num_sms();
+  // clusters are planned for three CTAs per SM (tile_us)
+  const bool clusters =
+      mtiles == 1 && forced_ipb <= 0 && (slots_in > 0 ? slots_in == kClusterSlots : slots == 3 * sms);
+  auto cluster_fit = [&](int c) { return slots_in > 0 ? kClusterFit[c] : attend_clusters(c); };
   // heavy tiles of each segment (a packed segment's bf16 tail is a light
   // item of its own) and their cost
   int htiles[UC_MAX_SEGMENTS];
@@ -967,7 +974,7 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
     // short calls: the items of a pair on one cluster where that, with the
     // number of items a cluster can have, is expected to end sooner
     p.cluster = 0;
-    if (mtiles == 1 && forced_ipb <= 0 && slots == kClusterSlots && nh > 0) {
+    if (clusters && nh > 0) {
       auto longest_us = [&](int h) {
         int hc[UC_MAX_SEGMENTS];
         split_items(h, nseg, heavy, htiles, tcost, hc);
@@ -976,16 +983,17 @@ AttnPlan plan_attend(const uc_segment* const* segs, int nseg, int mtiles, int nb
           if (heavy[s]) us = std::max(us, ((htiles[s] + hc[s] - 1) / hc[s]) * tile_us(segs[s]));
         return us;
       };
-      double best = items_us(longest_us(H), H, nbh_launch) + kQueueMergeUs;
+      double best = items_us(longest_us(H), H, nbh_launch, sms) + kQueueMergeUs;
       double light = nl * kLightItemUs;
       for (int s = 0; s < nseg; ++s)
         if (!heavy[s] && htiles[s] > 1) light += htiles[s] * tile_us(segs[s]);
       // ranks for the light items: one each, or one for all of them
       for (int lr = nl;; lr = 1) {
         int h = std::min(kMaxClusterItems - lr, hmax);
-        while (h >= nh && kClusterFit[h + lr] < nbh_launch) --h;
+        while (h >= nh && cluster_fit(h + lr) < nbh_launch) --h;
         if (h >= nh) {
-          const double us = kClusterSpread * items_us(std::max(light / std::max(1, lr), longest_us(h)), h + lr, nbh_launch);
+          const double us =
+              kClusterSpread * items_us(std::max(light / std::max(1, lr), longest_us(h)), h + lr, nbh_launch, sms);
           if (us < best) {
             best = us;
             p.cluster = lr + 1;
@@ -1465,9 +1473,8 @@ uc_status uc_attend(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_s
   st = build_decode_call(q, n_q_heads, n_qtok, segs, n_seg, out, lse, mass, &plan, ws + 256,
                          ws + 256 + kCounterBlock, reinterpret_cast<DevStatus*>(ws), &p);
   if (st != UC_OK) return st;
-  // (a device whose clusters fit less well than planned for takes the queue)
-  p.cluster = plan.cluster > 0 && attend_clusters(plan.cluster) >= B * hkv ? plan.cluster : 0;
-  p.defer_merge = p.cluster ? 0 : merge_width(B * hkv * plan.mtiles, num_sms());
+  p.cluster = plan.cluster;
+  p.defer_merge = plan.merge_width;
   p.stages = plan.stages;
   launch_attend(p, plan.grid, reinterpret_cast<cudaStream_t>(stream));
   return cuda_check("uc_attend");

@@ -34,7 +34,11 @@ def _mix(seed, B, hkv, spec):
     N = sum(s[0] for s in spec)
     k, v = synth.make_kv(seed, B, hkv, N)
     sc = synth.make_scores(seed, (B, hkv, N))
-    kd, vd, sd = dev(k), dev(v), torch.from_numpy(sc).to(DEV)
+    return _segments(k, v, sc, dev(k), dev(v), torch.from_numpy(sc).to(DEV), spec)
+
+
+def _segments(k, v, sc, kd, vd, sd, spec):
+    B, hkv = k.shape[:2]
     gs, os_ = [], []
     off = 0
     for n, kind, keep, bits in spec:
@@ -80,9 +84,8 @@ def test_dense_parity(case):
 
 
 def test_dense_issue_orders_agree_bitwise():
-    """P(j) shares tensor memory with S(j+1) of its Q tile; the default issue
-    order relies on the tensor pipe reading P before the next Q K^T writes
-    there. Waiting for P V to complete first must give the same bits."""
+    """The issue-order setting is kept for its callers and has no effect: both
+    values run the same code, so they give the same bits."""
     B, T, spec = 2, 700, CASES["editing_mix"][2]
     gs, _ = _mix(99, B, 4, spec)
     q = dev(synth.make_q(8, B, 28, T))
@@ -97,6 +100,46 @@ def test_dense_issue_orders_agree_bitwise():
             uc.set_dense_serial_pv(prev)
     for r in runs[1:]:
         assert all(torch.equal(a, b) for a, b in zip(runs[0], r))
+
+
+SHARED_S = {
+    # (T, spec): both query tiles' S go through one tensor-memory buffer, handed
+    # over twice per key tile. One key tile, no row in the second query tile;
+    # two key tiles, one of them with a K lo part, one row in that query tile;
+    # an odd count, all with K lo parts, all rows but one; more tiles than
+    # either ring has slots, kinds mixed, over two CTAs with a ragged last one
+    "one_tile": (9, [(40, "full", 40, 16)]),
+    "two_tiles": (129, [(128, "full", 128, 16), (100, "quant", 100, 4)]),
+    "odd_tiles_lo": (255, [(300, "quant", 300, 2)]),
+    "mixed_tiles": (300, [(64, "full", 64, 16), (260, "quant", 260, 4), (200, "full", 200, 16),
+                          (150, "evict_quant", 33, 2), (129, "evict", 129, 16), (31, "quant", 31, 4)]),
+}
+
+
+@pytest.mark.parametrize("case", list(SHARED_S))
+def test_dense_shared_s_buffer(case):
+    """Keys that grow along the context move the softmax reference (and so
+    rescale O) on many key tiles; against the oracle, and the same bits again
+    and again."""
+    T, spec = SHARED_S[case]
+    B, hkv, N = 2, 4, sum(s[0] for s in spec)
+    k, v = synth.make_kv(len(case), B, hkv, N)
+    k = synth.bf16_round(k * np.linspace(0.1, 3.0, N, dtype=np.float32)[:, None])
+    sc = synth.make_scores(len(case), (B, hkv, N))
+    kd, vd, sd = dev(k), dev(v), torch.from_numpy(sc).to(DEV)
+    gs, os_ = _segments(k, v, sc, kd, vd, sd, spec)
+    q = synth.make_q(3, B, 28, T)
+    rO, rl, rm = oattn.attend(q, os_, hkv)
+    bound = _packed.logit_error_bound(q, os_, hkv, [False] * len(spec))
+    first = None
+    for _ in range(4):
+        O, lse, mass = uc.attend(dev(q), gs)
+        if first is None:
+            assert _packed.attention_error(host(O), rO) <= _packed.ATTN_RTOL
+            assert (np.abs(host(lse) - rl) <= bound + 1e-5).all()
+            assert (np.abs(host(mass) - rm) <= 2 * bound[..., None] + 1e-5).all()
+            first = (O, lse, mass)
+        assert all(torch.equal(a, b) for a, b in zip(first, (O, lse, mass)))
 
 
 @pytest.mark.parametrize("name", ["denoise_4k", "edit_4k"])

@@ -532,7 +532,7 @@ def attend_batch(calls, ws: Optional[Workspace] = None, stream=None):
     n = len(calls)
     given = [(list(call[2:5]) + [None, None, None])[:3] for call in calls]
     shapes = [(B, hq, T, len(call[1])) for call in calls for B, hq, T, _ in [call[0].shape]]
-    dev = calls[0][0].device
+    dev = calls[0][0].device if n else None   # (an empty batch with a workspace is the library's to refuse)
     if n > 1 and all(g[1] is None and g[2] is None for g in given) and all(x == shapes[0] for x in shapes) \
             and all(call[0].device == dev for call in calls):
         # one allocation each for the calls' lse and masses
@@ -555,7 +555,7 @@ def attend_batch(calls, ws: Optional[Workspace] = None, stream=None):
                                          mass.data_ptr()))
         results.append((out, lse, mass))
     arr = (_lib.UcAttendCall * n)(*structs)
-    ws = ws or default_workspace(dev)
+    ws = ws or default_workspace(calls[0][0].device)
     L = lib()
     buf = ws.bufs.get("attend_batch")   # as in attend(): the size is asked for only when the call needs more
     wp, wn = (buf.data_ptr(), buf.numel()) if buf is not None else \

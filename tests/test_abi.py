@@ -323,3 +323,14 @@ def test_wait_limit_setting_round_trips():
         assert api.set_wait_limit(prev) == 2_000_000_000
     finally:
         api.set_wait_limit(prev)
+
+
+def test_attend_batch_without_calls_is_the_librarys_error():
+    """An empty batch with a workspace at hand is refused by the library's
+    argument checks, not by an index into the calls."""
+    class Stream:
+        cuda_stream = 0
+    n0 = api.launch_count()
+    with pytest.raises(api.UniCacheError):
+        api.attend_batch([], ws=api.Workspace("cpu"), stream=Stream())
+    assert api.launch_count() == n0

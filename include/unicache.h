@@ -488,8 +488,8 @@ uc_status uc_attention_mass(const float* mass, int32_t batch, int32_t n_q_heads,
  * tensor cores, 128 keys per tile; at most 512 tiles per sequence, each
  * segment padded to a multiple of 128 tokens.
  * workspace: uc_attend_workspace_size() bytes, zero-filled once before first
- * use and used by uc_attend only (it holds merge counters that every call
- * leaves at zero again); calls sharing one workspace must not overlap.
+ * use and used by uc_attend only (it holds the work queue's counters, which
+ * every call leaves at zero again); calls sharing one workspace must not overlap.
  */
 uc_status uc_attend(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_segment* const* segs,
                     int32_t n_seg, void* out, float* lse, float* mass, void* workspace,
@@ -582,7 +582,7 @@ size_t uc_attend_batch_workspace_size(const uc_attend_call* calls, int32_t n_cal
  *  - All calls share the one array: calls that overlap on the GPU (for
  *    example on two streams at once) race and give wrong results; order them
  *    on one stream or through events. Each call clears the array's status
- *    word and merge counters before it launches.
+ *    word and work-queue counters before it launches.
  */
 uc_status uc_attend_static(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_segment* const* segs,
                            int32_t n_seg, void* out, float* lse, float* mass, void* stream);

@@ -41,7 +41,7 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 class Workspace:
     """Zero-filled device scratch, grown on demand and reused across calls.
 
-    ``uc_attend`` and ``uc_attend_batch`` keep self-resetting merge counters
+    ``uc_attend`` and ``uc_attend_batch`` keep self-resetting counters
     in their workspaces, so each gets a buffer of its own ("attend",
     "attend_batch"); every other entry point shares the "scratch" buffer."""
 

@@ -1160,8 +1160,9 @@ int decode_mtiles(int n_q_heads, int hkv, int n_qtok) { return (n_q_heads / hkv 
 
 int merge_kernel_for(int items_per_bh) { return items_per_bh > kMergeKernelItems ? 1 : 0; }
 
-// A decode call's merge counters (one per (b, kvh)) live in a block of fixed
-// size at a fixed place of the workspace, whatever the call's shape: every
+// The merge counters (one per (b, kvh)) of a batch's call of several n-tiles
+// live in a block of fixed size at a fixed place of the workspace, whatever
+// the call's shape (uc_attend's workspace keeps one, unused): every
 // counter a call uses is re-armed to zero by its merge, so a block that calls
 // of any layout share stays zero between calls (counters placed by the
 // call's own layout could land on an earlier call's partial outputs).
@@ -1282,8 +1283,6 @@ namespace uc {
 // Everything uc_attend checks before it looks at its workspace, in the same
 // order and with the same statuses; *need receives the workspace bytes the
 // call takes. Shared with uc_attend_static, which has no workspace.
-size_t attend_counter_bytes() { return kCounterBlock; }
-
 uc_status attend_precheck(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_segment* const* segs,
                           int32_t n_seg, const void* out, const char* name, size_t* need) {
   AttnPlan plan;
@@ -1474,7 +1473,7 @@ uc_status uc_attend(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_s
                          ws + 256 + kCounterBlock, reinterpret_cast<DevStatus*>(ws), &p);
   if (st != UC_OK) return st;
   p.cluster = plan.cluster;
-  p.defer_merge = plan.merge_width;
+  p.merge_width = plan.merge_width;
   p.stages = plan.stages;
   launch_attend(p, plan.grid, reinterpret_cast<cudaStream_t>(stream));
   return cuda_check("uc_attend");

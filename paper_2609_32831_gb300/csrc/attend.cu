@@ -180,6 +180,7 @@ __device__ __forceinline__ ItemInfo decode_item(const AttnParams& p, int pos, in
 // light tail items. locate() maps a processing position to its call's
 // parameters and to the position inside that call's own order.
 struct OneCall {
+  static constexpr bool kMany = false;
   const AttnParams& p;
   __device__ int n_items() const { return p.n_items; }
   __device__ int n_calls() const { return 1; }
@@ -193,6 +194,7 @@ struct OneCall {
 };
 
 struct ManyCalls {
+  static constexpr bool kMany = true;
   const MultiAttnParams& m;
   __device__ int n_items() const { return m.n_items; }
   __device__ int n_calls() const { return m.n_calls; }
@@ -1005,17 +1007,18 @@ __device__ __forceinline__ void merge_weights(const P& p, float* ml, const float
   }
 }
 
-// A batch's merge with several n-tiles runs on the 128 consumer threads of the CTA that finished the
-// last item of a (sequence, KV head): the weights of every item and row, then
-// per 8-row block the weighted sums of the items' O, four channels of two
+// A batch's merge with several n-tiles runs on the 128 consumer threads of the
+// CTA that finished the last item of a (sequence, KV head): the weights of
+// every item and row, then per 8-row block the weighted sums of the items' O, four channels of two
 // rows per thread (16-byte shared-memory reads; one 4-byte read per value
 // with its weight held the merge of 13 items for 5 us). After the CTA's last
 // item the ring is idle (`seq` given): the row blocks of O stream through it
 // back to back, eight items per slot, by bulk copies continuing the consumers'
 // tile sequence, the first ones in flight while the weights are formed.
-// Without `seq` (a merge between items) the threads load them. (Without these
-// merges in it the kernel's int4 loops came out 3 % slower, so such batches
-// keep them.)
+// Without `seq` (a merge between items) the threads load them. Only batches
+// merge here: single calls are faster with the merge kernel, and their kernel
+// without this code in it (four query tokens, 4 x 16K int2 36.4 -> 35.2 us, 8 x
+// 20K int4 70.4 -> 69.3; two, 1 x 300 10.6 -> 10.1; mixed 4 x 16K 33.7 -> 34.1).
 template <int NTW, int ST>
 __device__ void final_merge(const AttnParams& p, AttnSmem& sm, int bh, uint32_t* seq) {
   const int tid = threadIdx.x;
@@ -1701,6 +1704,7 @@ __device__ __forceinline__ void consume_cluster(const AttnParams& p, AttnSmem& s
 
 template <int NTW, int ST, class W>
 __device__ void consume(const W& w, AttnSmem& sm) {
+  constexpr bool kMerges = NTW > 1 && W::kMany;  // else the merge kernel does
   const int warp = threadIdx.x >> 5;
   const int mtiles = w.call(0).mtiles;  // the same for every call of a launch
   const int NG = (mtiles + NTW - 1) / NTW <= 1 ? 1 : ((mtiles + NTW - 1) / NTW <= 2 ? 2 : 4);
@@ -1710,7 +1714,7 @@ __device__ void consume(const W& w, AttnSmem& sm) {
   bool aborted = false;
   // thread 0: the last arrival (call << 16 | bh), checked one item later
   int prev_key = -1, prev_arrivals = -1;
-  if (NTW > 1 && threadIdx.x == 0) sm.n_pending = 0;
+  if (kMerges && threadIdx.x == 0) sm.n_pending = 0;
   for (uint32_t iseq = 0;; ++iseq) {
     const int k = iseq % kItemQ;
     if (!mbar_wait(&sm.item_full[k], (iseq / kItemQ) & 1, w.call(0).status, 13, w.call(0).wait_ns)) break;
@@ -1728,11 +1732,11 @@ __device__ void consume(const W& w, AttnSmem& sm) {
       run_item<NTW, ST, 2>(p, sm, ii, it, k, seq, aborted, NG, KS, grp, ks);
 
     consumer_sync();  // the next item's query fragments take this one's place
-    if constexpr (NTW == 1) continue;
-    // Arrive on the item's counter; the CTA whose arrival completes a
+    if constexpr (!kMerges) continue;
+    // A batch: arrive on the item's counter; the CTA whose arrival completes a
     // (sequence, KV head) owes its merge, done after its last item so that
     // no warp waits for the atomic here.
-    if (threadIdx.x == 0 && !p.defer_merge) {
+    if (threadIdx.x == 0) {
       if (prev_key >= 0 && prev_arrivals == w.items_per_bh(prev_key >> 16) - 1)
         sm.pending[sm.n_pending++] = prev_key;
       prev_arrivals = counter_arrive_acq_rel(&p.counters[ii.bh]);
@@ -1751,7 +1755,7 @@ __device__ void consume(const W& w, AttnSmem& sm) {
       consumer_sync();
     }
   }
-  if constexpr (NTW == 1) return;
+  if constexpr (!kMerges) return;
   if (threadIdx.x == 0) {
     if (prev_key >= 0 && prev_arrivals == w.items_per_bh(prev_key >> 16) - 1)
       sm.pending[sm.n_pending++] = prev_key;
@@ -1932,7 +1936,7 @@ void launch_attend(const AttnParams& p, int grid, cudaStream_t st) {
   else
     launch_maybe_pdl(pdl, attend_kernel<2, AttnParams>, grid, kAttnThreads, smem, st, p);
   count_launch();
-  launch_merge(merge_of(p), p.batch * p.n_kv_heads * p.mtiles, p.defer_merge, st);
+  launch_merge(merge_of(p), p.batch * p.n_kv_heads * p.mtiles, p.merge_width, st);
 }
 
 void launch_attend_multi(const MultiAttnParams& m, int grid, cudaStream_t st) {
@@ -1960,7 +1964,7 @@ void launch_attend_multi(const MultiAttnParams& m, int grid, cudaStream_t st) {
 // ------------------------------------------------------ no-allocation variant
 //
 // uc_attend_static: decode attention for callers that cannot hand the
-// library a workspace. Its scratch (status word, merge counters, partial
+// library a workspace. Its scratch (status word, work queue, partial
 // outputs) is this file-scope device array, reserved on every GPU that loads
 // the library for as long as the process lives.
 namespace uc {
@@ -2018,8 +2022,8 @@ extern "C" uc_status uc_attend_static(const void* q, int32_t n_q_heads, int32_t 
     return UC_ERR_OOM;
   }
   // The array keeps the previous call's contents: clear the status word and
-  // the merge counters, which must start at zero.
-  const size_t clear = 256 + attend_counter_bytes();
+  // the work queue's counters (the first 256 bytes), which must start at zero.
+  const size_t clear = 256;
   if (cudaMemsetAsync(scratch, 0, clear, reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess) {
     set_error("uc_attend_static: clearing the scratch failed: %s", cudaGetErrorString(cudaGetLastError()));
     return UC_ERR_CUDA;

@@ -63,9 +63,6 @@ int take_withhold_pos();
 // statuses); *need: the workspace bytes the call takes.
 uc_status attend_precheck(const void* q, int32_t n_q_heads, int32_t n_qtok, const uc_segment* const* segs,
                           int32_t n_seg, const void* out, const char* name, size_t* need);
-// Bytes of a uc_attend call's merge counters in its workspace (after the
-// 256-byte status word): a block of fixed size that must start at zero.
-size_t attend_counter_bytes();
 
 // ------------------------------------------------------------ compression
 struct TopkArgs {
@@ -201,7 +198,7 @@ struct AttnParams {
   float* lse;
   float* mass;
   float* part;       // per item: [rows_pad][128] O, then [rows_pad] m, [rows_pad] l
-  int32_t* counters; // [B*Hkv]
+  int32_t* counters; // [B*Hkv], batches of several n-tiles
   int32_t* sched;    // launch-wide work queue: [0] next item, [1] CTAs done (re-armed to 0)
   DevStatus* status;
   int nseg, batch, n_kv_heads, n_q_heads, n_qtok, group, rows, mtiles, items_per_bh, n_items;
@@ -217,9 +214,7 @@ struct AttnParams {
   // work queue: one per heavy item, then one for the light items or one each
   int cluster;
   int stages;       // ring slots of a CTA (uc_attend; batched launches take two)
-  // > 0: the attend launch only leaves partials; a merge kernel follows, whose
-  // CTAs take this many output channels each
-  int defer_merge;
+  int merge_width;  // output channels per CTA of the merge kernel behind the call (uc_attend; 0: a cluster)
   float scale_log2;
   uint64_t wait_ns;  // limit of every bounded wait of the launch (UC_ERR_TIMEOUT past it)
   int withhold_pos;  // test hook: the first tile of the item at this position is never copied (-1: none)

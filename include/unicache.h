@@ -189,9 +189,12 @@ int32_t uc_set_dense_serial_pv(int32_t serial);
  * value. */
 uint64_t uc_set_wait_limit(uint64_t ns);
 
-/* Programmatic dependent launch of the decode kernels (uc_attend's attention
- * and merge kernels, uc_append / uc_append_next), process-wide, read when a
- * call launches (a captured graph keeps what its capture saw). With 1, the
+/* Programmatic dependent launch of uc_attend's decode attention kernel and of
+ * uc_append / uc_append_next, process-wide, read when a call launches (a
+ * captured graph keeps what its capture saw). Whatever it says, the merge
+ * kernel behind a decode attention and the dense attention kernel behind the
+ * launch that rebuilds its rows are launched programmatically: both wait for
+ * the launch before them, which belongs to the same call. With 1, the
  * next kernel in the stream may start while the current one's last CTAs are
  * finishing: an attention kernel still waits for the kernel before it (so
  * its layer's append is complete), but an append waits for nothing. The

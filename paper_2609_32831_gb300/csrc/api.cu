@@ -841,8 +841,12 @@ constexpr int kClusterFit[kMaxClusterItems + 1] = {0,  456, 228, 148, 110, 87, 7
                                                    46, 43,  36,  36,  28,  26, 26, 21};
 constexpr int kClusterSlots = 456;
 
-// Time (us) of a tile on an SM that runs three CTAs (one 32K layer by the
-// planner at 3, 2 and 1 CTAs per SM: int2 75, 83, 124 us, int4 84, 93, 146).
+// Time (us) of a tile on an SM that runs three CTAs, for comparing clusters
+// with the queue. These and the two constants below were fitted together when
+// an int2 layer took 75 us; only the comparison's outcome counts (see there).
+// One layer now at 3, 2 and 1 CTAs per SM: int2 (16 x 32K) 63.6, 71.6, 94.5 us,
+// int4 69.3, 79.7, 110.4, bf16 (16 x 8K) 45.8, 46.3, 55.3, which is 1.03, 0.57
+// and 0.70 us per tile.
 double tile_us(const uc_segment* s) { return !is_quant(s->kind) ? 0.75 : (s->bits == 4 ? 0.68 : 1.16); }
 
 // Time until a single-n-tile call's longest items (`item` us of SM time each,
@@ -855,11 +859,12 @@ double items_us(double item, int h, int nbh, int sms) {
 // The queue's merge (a kernel behind the call, partials through global
 // memory) ends later than the cluster's by about kQueueMergeUs; a cluster has
 // no idle CTAs to take light items and its CTAs lie less evenly over the SMs
-// (kClusterSpread). Cluster / queue, us on the device: 200 tokens batch 1
-// 7.6 / 8.6, 3000 bf16 batch 8 14.7 / 15.9, 4000 in three packed segments
-// batch 4 11.0 / 11.9; at the line 2000 int2 batch 16 13.1 / 12.9; where the
-// rule takes the queue 8K batch 8 int2 20.6 / 17.3, 32K batch 4 int2
-// 39.3 / 25.3.
+// (kClusterSpread). Cluster / queue, us on the device, where the rule takes the
+// cluster: 200 int2 tokens batch 1 7.3 / 7.5, 3000 bf16 batch 8 14.1 / 15.2, 512
+// bf16 + 2150 int4 + 512 int2 batch 8 12.9 / 13.6, and past its line 2000 int2
+// batch 16 12.9 / 12.3, 4000 int2 batch 8 12.7 / 11.8; where it takes the queue:
+// 4000 int2 batch 2 9.6 / 8.7, 8000 int4 batch 4 14.9 / 12.7, 32K int2 batch 4
+// 33.9 / 24.3, and on its line 8000 int2 batch 8 16.0 / 16.5.
 constexpr double kQueueMergeUs = 1.5, kClusterSpread = 1.15;
 constexpr double kLightItemUs = 0.4;  // SM time of a light item's start and end
 

@@ -5,6 +5,9 @@ The kernel finds, for each group, the smallest bf16 value that reaches code 1,
 steps in numpy are compared with the oracle's quantizer for every finite bf16
 value: random fp16 scales and zero-points, and the relations where a
 threshold lies near zero, where bf16 values are denser than fp32 differences.
+This pins the argument only; the kernel's own codes are compared with the
+oracle's in test_gpu_kernels (test_quantize_codes_at_their_edges and the
+parity cases).
 """
 import numpy as np
 import pytest
